@@ -125,46 +125,53 @@ class _Maker:
         return self.normal(rank, k, scale=0.02), self.normal(n, rank, scale=0.02)
 
 
-def _layers(m, x, idx, ns, rank, sigma, capacity):
-    """Layers that read x [tokens, K]: their weights, one smoothing vector, factors of their own."""
-    k = x.shape[1]
-    s, out = None, []
+def _group(m, tokens, k, ns, rank, gain, sigma, gated=False):
+    """Layers that read one x [tokens, K]: x, its smoothing vector, and each layer's weights and factors."""
+    idx = m.outliers(k)
+    x = m.activations(tokens, k, idx, gain, gated)
+    s, layers = None, []
     for n in ns:
         w = m.normal(n, k, scale=sigma)
         if s is None:
             s = m.smoothing(x, w, idx)
-        la, lb = m.factors(k, n, rank)
-        out.append(aser.AserLinear(w, s, la, lb, capacity))
-    return out
+        layers.append((w, *m.factors(k, n, rank)))
+    return x, s, layers
+
+
+def _inputs(case, seed):
+    """The groups of layers that a pass goes through, one after the other."""
+    m = _Maker(seed)
+    gain, sigma, rank = case.get("gain", 30.0), case.get("sigma", 0.02), case.get("rank", 0)
+    if case["kind"] == "block":
+        for k, ns in ((HIDDEN, (HIDDEN, KV, KV)), (HIDDEN, (HIDDEN,)), (HIDDEN, (MLP, MLP)), (MLP, (HIDDEN,))):
+            yield _group(m, case["tokens"], k, ns, rank, gain, sigma, gated=k == MLP)
+    elif case["kind"] in ("pack", "construct"):
+        yield _group(m, case.get("calibration", 64), case["k"], (case["n"],), 0, gain, sigma)
+    else:
+        yield _group(m, case["tokens"], case["k"], (case["n"],) * case.get("layers", 1), rank, gain, sigma,
+                     case.get("gated", False))
 
 
 def prepare(case, seed):
-    m = _Maker(seed)
     kind = case["kind"]
-    gain, sigma = case.get("gain", 30.0), case.get("sigma", 0.02)
     tokens, rank = case.get("tokens", 0), case.get("rank", 0)
     st = {"kind": kind}
+
+    def built(group, capacity):
+        x, s, layers = group
+        return x, [aser.AserLinear(w, s, la, lb, capacity) for w, la, lb in layers]
+
     if kind == "block":
-        def group(k, ns, gated=False):
-            idx = m.outliers(k)
-            x = m.activations(tokens, k, idx, gain, gated)
-            return x, _layers(m, x, idx, ns, rank, sigma, tokens)
-        x_qkv, qkv = group(HIDDEN, (HIDDEN, KV, KV))
-        x_o, o = group(HIDDEN, (HIDDEN,))
-        x_mlp, mlp = group(HIDDEN, (MLP, MLP))
-        x_down, down = group(MLP, (HIDDEN,), gated=True)
+        (x_qkv, qkv), (x_o, o), (x_mlp, mlp), (x_down, down) = [built(g, tokens) for g in _inputs(case, seed)]
         st["steps"] = [(aser.AserSharedInputCat(qkv, tokens), x_qkv), (o[0], x_o),
                        (aser.AserSharedInput(mlp, tokens), x_mlp), (down[0], x_down)]
         return st
     k, n = case["k"], case["n"]
-    idx = m.outliers(k)
+    group, = _inputs(case, seed)
     if kind in ("pack", "construct"):
-        x = m.activations(case.get("calibration", 64), k, idx, gain)
-        w = m.normal(n, k, scale=sigma)
-        st.update(W=w, s=m.smoothing(x, w, idx), X=x, rank=rank)
+        st.update(W=group[2][0][0], s=group[1], X=group[0], rank=rank)
         return st
-    x = m.activations(tokens, k, idx, gain, case.get("gated", False))
-    layers = _layers(m, x, idx, (n,) * case.get("layers", 1), rank, sigma, case.get("capacity", tokens))
+    x, layers = built(group, case.get("capacity", tokens))
     st["X"] = x
     if kind == "shared":
         st["call"] = aser.AserSharedInput(layers, tokens)
@@ -211,6 +218,58 @@ def run(st):
     # the factors are determined up to sign and rotation: their product is what a layer uses
     return {"Wq": out["Wq"], "scale": out["w_scale"], "sigma": out["sigma"],
             "product": out["L_B"].float() @ out["L_A"].float()}
+
+
+# ----------------------------------------------------------------------------
+# the same outputs in plain torch: codes and their scales by single fp32 steps, as the format
+# defines them, everything summed in fp64
+# ----------------------------------------------------------------------------
+def _codes(v, qmax, low):
+    scale = v.abs().amax(1) / float(qmax)
+    q = (v / torch.where(scale > 0, scale, 1.0)[:, None]).round_().clamp_(low, qmax)
+    return q, scale
+
+
+def _exact_pass(x, s, layers, qmax=127):
+    xs = x.float() / s
+    q, a_scale = _codes(xs, qmax, -qmax)
+    out = []
+    for w, la, lb in layers:
+        wq, w_scale = _codes(w.float() * s, 7, -8)
+        y = q.double() @ wq.double().T * a_scale.double()[:, None] * w_scale.double()
+        if la is not None:
+            y += (xs.double() @ la.double().T) @ lb.double().T
+        out.append(y)
+    return out, a_scale
+
+
+def exact(case, seed):
+    kind = case["kind"]
+    groups = _inputs(case, seed)
+    if kind == "block":
+        outs = [_exact_pass(*g)[0] for g in groups]
+        return [outs[0], outs[1][0], outs[2], outs[3][0]]
+    (x, s, layers), = groups
+    if kind in ("linear", "host"):
+        return _exact_pass(x, s, layers)[0][0]
+    if kind == "shared":
+        return _exact_pass(x, s, layers)[0]
+    if kind == "variant":
+        y, a_scale = _exact_pass(x, s, layers, 2 ** (case["act_bits"] - 1) - 1)
+        return {"Y": y[0], "codes": None, "scale": a_scale.double()}
+    ws = layers[0][0].float() * s
+    if kind == "pack":
+        return {"Wq": None, "scale": ws.double().abs().amax(1) / 7, "Wk": None}
+    q, scale = _codes(ws, 7, -8)
+    error = ws.double() - q.double() * scale.double()[:, None]
+    xs = (x.float() / s).double()
+    gram = xs.T @ xs
+    gram.diagonal().add_(0.01 * gram.trace() / gram.shape[0])
+    a = error @ torch.linalg.cholesky(gram)
+    values, u = torch.linalg.eigh(a @ a.T)               # ascending: the squared singular values of E S
+    u = u[:, -case["rank"]:]
+    # U_r U_r^T (E S) S^-1
+    return {"Wq": None, "scale": scale.double(), "sigma": values[-case["rank"]:].flip(0).sqrt(), "product": u @ (u.T @ error)}
 
 
 # ----------------------------------------------------------------------------
