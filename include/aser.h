@@ -319,8 +319,9 @@ int aser_forward_host(const void* X_host_f16, void* Y_host_f16,
  * of E S (Eq. 6) and split them into L_B = U_r Sigma_r [N, r] and L_A = V_r^T S^-1 [r, K] (the
  * paper's L_A and L_B, in that order).  fp64 throughout, factors rounded to fp16 at the end.
  *   W_f16 [N, K], s [K] or NULL, Xcal_f16 [n_cal, K] calibration tokens (NOT yet smoothed).
- *   iterations: subspace iterations for the singular subspace (<= 0: 48); p = r + max(32, r/2)
- *   vectors are iterated, so the r-th triplet converges like (sigma_{p+1} / sigma_r)^(2 iterations).
+ *   iterations: subspace iterations for the singular subspace (<= 0: 22, with the accuracy of 48
+ *   plain ones and more); p = r + max(32, r/2) vectors are iterated, two plain steps and then Chebyshev
+ *   steps, so the r-th triplet converges at least like (sigma_{p+1} / sigma_r)^(2 iterations).
  *   Outputs: Wq [N, K/2] canonical, w_scale [N], LA_f16 [r, K], LB_f16 [N, r]; optional
  *   sigma_out [r] (fp64 singular values, descending) and S_out [K, K] (fp64, lower, row-major).
  *   split_idx [n_split] (device, int32; NULL with n_split = 0): the outlier columns of the

@@ -314,7 +314,7 @@ int aser_construct(const void* W_f16, const float* s, const void* Xcal_f16, int 
     int rc = check_device();
     if (rc != ASER_OK) return rc;
     return launch_construct(static_cast<const __half*>(W_f16), s, static_cast<const __half*>(Xcal_f16), N, K,
-                            n_cal, r, damping, iterations > 0 ? iterations : 48, Wq, w_scale,
+                            n_cal, r, damping, iterations > 0 ? iterations : kConstructIterations, Wq, w_scale,
                             static_cast<__half*>(LA_f16), static_cast<__half*>(LB_f16), sigma_out, S_out,
                             split_idx, n_split, workspace, static_cast<cudaStream_t>(stream));
 }

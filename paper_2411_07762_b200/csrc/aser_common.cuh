@@ -45,6 +45,7 @@ int launch_quant_act_ws(const __half* X, const float* s, const __half* LA, int M
                         int8_t* Xq, float* a_scale, __nv_bfloat16* T, void* scratch, size_t scratch_bytes,
                         cudaStream_t st, int act_bits = 8, bool t_pair = false);
 // Device-side construction of a layer's factors (construct.cu); synchronises the stream.
+constexpr int kConstructIterations = 22;     // applications of A A^T unless the caller says otherwise
 size_t construct_workspace_bytes(int N, int K, int Tcal, int r, int n_split);
 int launch_construct(const __half* W, const float* s, const __half* Xcal, int N, int K, int Tcal, int r,
                      double damping, int iters, uint8_t* Wq, float* w_scale, __half* LA, __half* LB,

@@ -5,16 +5,37 @@
 //   S   = lower Cholesky factor of G                              (whitening, Eq. 5)
 //   A   = E S,  A ~ U_r Sigma_r V_r^T                             (truncated SVD, Eq. 6)
 //   L_B = U_r Sigma_r  [N, r],   L_A = V_r^T S^-1  [r, K]
-// All in fp64 on CUDA cores (an offline step: a few hundred GFLOP at the largest shapes).
+// All in fp64.
 //
-// The top-r singular triplets come from subspace iteration on A^T A with p = r + oversampling
-// vectors kept as ROWS (Qt [p, K]): Yt = Qt A^T, Zt = Yt A, Qt = orthonormalised Zt (Cholesky of
-// Zt Zt^T and a forward substitution, done twice), then Rayleigh-Ritz by one-sided Jacobi
-// rotations applied to the rows of Bt = Qt A^T and of Qt together: when the rows of Bt are
-// orthogonal their norms are the singular values, the r longest rows of Bt are (U_r Sigma_r)^T
-// and the matching rows of Qt are V_r^T.  The whitened spectrum of a quantization error decays,
-// so a few dozen iterations reach the singular subspace to near machine precision.
+// S is not needed for the factors.  With u a left singular vector of A, sigma its value,
+//   A A^T = E G E^T = F F^T,  F = [ sqrt(lambda) E | E X~^T ]   [N, K + tokens],
+// so F has the singular values and left vectors of A, and since A = E S,
+//   v^T S^-1 = sigma^-1 u^T A S^-1 = sigma^-1 u^T E:  L_A = Sigma_r^-1 U_r^T E.
+// With no more tokens than channels F takes the place of A: no Gram matrix, no Cholesky factor, no
+// triangular solve (4096 x 4096 with 512 tokens: 17 GFLOP instead of 180).  The factor S is computed
+// when the caller asks for it, when there are more tokens than channels (then A is the smaller
+// matrix), and when lambda is so small that the damped Gram matrix may turn out singular, which
+// the Cholesky factorisation has to report.
+//
+// The r leading left vectors come from subspace iteration on F F^T with p = r + oversampling
+// vectors as rows (Ut [p, N]): Y = Ut F, Z = Y F^T, normalised by the Cholesky factor of Z Z^T.
+// After two plain steps the steps follow the Chebyshev recurrence T' = 2 (2/b F F^T - I) T - T"
+// on [0, b], b the smallest Ritz value (from below an estimate of sigma_p^2, so nothing wanted is
+// damped): the recurrence is linear in the rows, so both of its terms may be multiplied by the
+// inverse Cholesky factor after every step and it keeps its accuracy whatever the spread of the
+// spectrum.  b is estimated anew every dozen steps.  With x = sigma_r^2 / sigma_p^2, a step of the
+// recurrence gains exp(acosh(2 x - 1)), a plain one x: at x = 1.2 ... 1.6, where quantization errors
+// lie, 22 steps reach what 60 to 90 plain ones would.  Measured against the exact triplets (2048 x
+// 2048, 512 tokens, r = 64): product 5e-5 after 18 such steps, 9e-5 after 48 plain ones.
+// The final Rayleigh-Ritz step works on the p x p Cholesky factor L of (Ut F)(Ut F)^T: one-sided
+// Jacobi rotations of its rows until they are orthogonal; their norms are the singular values.
+//
+// 4096 x 4096, 512 tokens, r = 64 took 236.8 ms with plain iteration on A, a 64 x 64 fma product
+// (157 ms), one thread per column in the triangular solves (46 ms) and one launch per Jacobi round
+// (11 ms); now 11.0 ms: Y and Z 5.8 (at 28 of 37 TFLOP/s), Cholesky factors 1.1, Jacobi 1.4.  2048 x
+// 1024, r = 256: 784 -> 46 ms.
 #include "aser_common.cuh"
+#include "gemm64.cuh"
 
 namespace aser {
 
@@ -161,55 +182,31 @@ __global__ void zero_upper_kernel(double* __restrict__ A, long long lda, int n) 
 }
 
 // ---------------------------------------------------------------------------
-// Z [p, ncols] <- L^-1 Z with L lower p x p: thread per column, forward substitution down the rows.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128)
-left_solve_lower_kernel(const double* __restrict__ L, long long ldl, int p, double* __restrict__ Z, long long ldz, int ncols) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= ncols) return;
-    for (int i = 0; i < p; ++i) {
-        double v = Z[(long long)i * ldz + c];
-        const double* Li = L + (long long)i * ldl;
-        for (int j = 0; j < i; ++j) v -= Li[j] * Z[(long long)j * ldz + c];
-        Z[(long long)i * ldz + c] = v / Li[i];
-    }
-}
-
-// Rows of X [rows, nb] (leading dimension ld): X <- X L^-1 with L the nb x nb lower block, i.e.
-// solve x L = b backwards along the row; one thread per row.
-__global__ void __launch_bounds__(128)
-right_solve_lower_kernel(double* __restrict__ X, long long ld, int rows, const double* __restrict__ L, long long ldl, int nb) {
-    __shared__ double Ls[kCB][kCB + 1];
-    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) Ls[e / nb][e % nb] = L[(long long)(e / nb) * ldl + e % nb];
-    __syncthreads();
-    const int row = blockIdx.x * blockDim.x + threadIdx.x;
-    if (row >= rows) return;
-    double x[kCB];
-    double* p = X + (long long)row * ld;
-#pragma unroll 1
-    for (int c = nb - 1; c >= 0; --c) {
-        double v = p[c];
-        for (int k = c + 1; k < nb; ++k) v -= x[k] * Ls[k][c];
-        x[c] = v / Ls[c][c];
-        p[c] = x[c];
-    }
-}
-
-// ---------------------------------------------------------------------------
 // operands
 // ---------------------------------------------------------------------------
-// E = fp32(W) * s (one fp32 multiply, as the quantizer sees it) - q * w_scale, in fp64.
-__global__ void build_error_kernel(const __half* __restrict__ W, const float* __restrict__ s,
-                                   const uint8_t* __restrict__ Wq, const float* __restrict__ w_scale,
-                                   int N, int K, double* __restrict__ E) {
+// E = fp32(W) * s (one fp32 multiply, as the quantizer sees it) - q * w_scale, in fp64, times *mul
+// (or 1); eight columns per thread, rows of E ld apart.
+__global__ void __launch_bounds__(256)
+build_error_kernel(const __half* __restrict__ W, const float* __restrict__ s, const uint8_t* __restrict__ Wq,
+                   const float* __restrict__ w_scale, int N, int K, double* __restrict__ E, long long ld,
+                   const double* __restrict__ mul) {
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (long long)N * K) return;
-    const int n = (int)(e / K), k = (int)(e % K);
-    const float ws = __fmul_rn(__half2float(W[e]), s ? s[k] : 1.f);
-    const uint8_t byte = Wq[(long long)n * (K / 2) + k / 2];
-    int q = (k & 1) ? (byte >> 4) : (byte & 0xF);
-    q = (q ^ 8) - 8;                                    // sign-extend the nibble
-    E[e] = (double)ws - (double)q * (double)w_scale[n];
+    if (e >= (long long)N * (K / 8)) return;
+    const int n = (int)(e / (K / 8)), k = (int)(e % (K / 8)) * 8;
+    const uint4 raw = *reinterpret_cast<const uint4*>(W + (long long)n * K + k);
+    const uint32_t codes = *reinterpret_cast<const uint32_t*>(Wq + (long long)n * (K / 2) + k / 2);
+    const __half* h = reinterpret_cast<const __half*>(&raw);
+    const double sc = (double)w_scale[n], f = mul ? *mul : 1.0;
+    double v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float ws = __fmul_rn(__half2float(h[i]), s ? s[k + i] : 1.f);
+        const int q = (int)(((codes >> (4 * i)) & 0xF) ^ 8) - 8;        // sign-extend the nibble
+        v[i] = ((double)ws - (double)q * sc) * f;
+    }
+    double2* o = reinterpret_cast<double2*>(E + (long long)n * ld + k);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) o[i] = make_double2(v[2 * i], v[2 * i + 1]);
 }
 
 // Copy of W with the columns of the outlier set zeroed: what the quantizer sees under the outlier
@@ -224,17 +221,47 @@ __global__ void mask_columns_kernel(const __half* __restrict__ W, int N, int K, 
     Wm[e] = out ? __float2half(0.f) : W[e];
 }
 
-// X~ = fp32(X) / s (one fp32 division), in fp64.
-__global__ void build_xs_kernel(const __half* __restrict__ X, const float* __restrict__ s, int T, int K,
-                                double* __restrict__ Xs) {
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (long long)T * K) return;
-    const float x = __half2float(X[e]);
-    Xs[e] = (double)(s ? __fdiv_rn(x, s[e % K]) : x);
+// X~ = fp32(X) / s (one fp32 division), in fp64; rows past T (up to the grid) are zero.  The sum of
+// squares of each row goes to row_sq.
+__global__ void __launch_bounds__(256)
+build_xs_kernel(const __half* __restrict__ X, const float* __restrict__ s, int T, int K, double* __restrict__ Xs,
+                double* __restrict__ row_sq) {
+    __shared__ double red[256];
+    const int row = blockIdx.x;
+    double sum = 0.0;
+    for (int k = threadIdx.x; k < K; k += 256) {
+        double v = 0.0;
+        if (row < T) {
+            const float x = __half2float(X[(long long)row * K + k]);
+            v = (double)(s ? __fdiv_rn(x, s[k]) : x);
+        }
+        Xs[(long long)row * K + k] = v;
+        sum = fma(v, v, sum);
+    }
+    red[threadIdx.x] = sum;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) row_sq[row] = red[0];
+}
+
+// lambda = damping * trace(X~^T X~) / K, its root and the root's inverse.  A trace that is zero or
+// not finite has no positive definite damped Gram matrix.
+__global__ void lambda_kernel(const double* __restrict__ row_sq, int rows, int K, double damping,
+                              double* __restrict__ out, int* __restrict__ fail) {
+    double t = 0.0;
+    for (int i = threadIdx.x; i < rows; i += 32) t += row_sq[i];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (threadIdx.x != 0) return;
+    double lam = damping * t / K;
+    if (!(lam > 0.0) || !(lam < 1e300)) { *fail = 1; lam = 1.0; }
+    out[0] = lam; out[1] = sqrt(lam); out[2] = 1.0 / sqrt(lam);
 }
 
 // G += lambda I with lambda = damping * trace(G) / K; one CTA (the trace is summed in a fixed order).
-__global__ void __launch_bounds__(256) damp_kernel(double* __restrict__ G, int K, double damping, double* __restrict__ lambda_out) {
+__global__ void __launch_bounds__(256) damp_kernel(double* __restrict__ G, int K, double damping) {
     __shared__ double red[256];
     double t = 0.0;
     for (int i = threadIdx.x; i < K; i += 256) t += G[(long long)i * K + i];
@@ -246,7 +273,6 @@ __global__ void __launch_bounds__(256) damp_kernel(double* __restrict__ G, int K
     }
     const double lam = damping * red[0] / K;
     for (int i = threadIdx.x; i < K; i += 256) G[(long long)i * K + i] += lam;
-    if (threadIdx.x == 0 && lambda_out) *lambda_out = lam;
 }
 
 // Start vectors: a fixed hash of the index mapped to (-1, 1) (any full-rank start works).
@@ -262,7 +288,8 @@ __global__ void init_basis_kernel(double* __restrict__ Qt, long long n) {
 
 // ---------------------------------------------------------------------------
 // One round of one-sided Jacobi: CTA b rotates rows (i, j) = pairs[b] of Bt [p, N] so that they
-// become orthogonal, and applies the same rotation to rows i, j of Qt [p, K].
+// become orthogonal, and applies the same rotation to rows i, j of Qt [p, K].  For more vectors than
+// one CTA's shared memory holds.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
 jacobi_round_kernel(double* __restrict__ Bt, int N, double* __restrict__ Qt, int K, int p, int round) {
@@ -309,53 +336,242 @@ jacobi_round_kernel(double* __restrict__ Bt, int N, double* __restrict__ Qt, int
     }
 }
 
-// Squared norms of the rows of Bt, then (one thread) the indices of the r largest in descending
-// order: order[0..r).  p <= 1024.
-__global__ void __launch_bounds__(256) row_norms_kernel(const double* __restrict__ Bt, int N, double* __restrict__ norms) {
-    __shared__ double red[256];
-    const double* b = Bt + (long long)blockIdx.x * N;
-    double a = 0.0;
-    for (int k = threadIdx.x; k < N; k += 256) a = fma(b[k], b[k], a);
-    red[threadIdx.x] = a;
+// ---------------------------------------------------------------------------
+// Small matrices (p <= kMaxP), one CTA with everything in registers or shared memory.
+// ---------------------------------------------------------------------------
+constexpr int kMaxP = 112;
+
+// H [p, p] symmetric -> Linv = L^-1 (lower, zeros above) with H = L L^T, and L itself if G is given.
+// 16 x 16 threads hold the matrix cyclically (row ti + 16 a, column tj + 16 b).  Elimination step j
+// needs row j alone (the multipliers of column j are its entries, by symmetry): its owners write it to
+// shared memory, then every thread updates its T x T entries; columns below j, done with, hold the
+// rows of the inverse instead.  One barrier per step: 40 us for p = 96 (one thread per row and three
+// barriers took 74 for each block of 64, and the inverse another 310).
+template <int T>
+__global__ void __launch_bounds__(256)
+chol_inverse_kernel(const double* __restrict__ H, long long ldh, int p, double* __restrict__ Linv, long long ldl,
+                    double* __restrict__ G, long long ldg, int* __restrict__ fail) {
+    __shared__ double row[2][16 * T];
+    __shared__ double piv[16 * T];
+    const int ti = threadIdx.x >> 4, tj = threadIdx.x & 15;
+    double w[T][T];
+#pragma unroll
+    for (int a = 0; a < T; ++a)
+#pragma unroll
+        for (int b = 0; b < T; ++b) {
+            const int i = ti + 16 * a, j = tj + 16 * b;
+            w[a][b] = (i < p && j < p) ? H[(long long)i * ldh + j] : (i == j ? 1.0 : 0.0);
+        }
+    bool bad = false;
+#pragma unroll
+    for (int ja = 0; ja < T; ++ja) {
+#pragma unroll 1
+        for (int jj = 0; jj < 16; ++jj) {
+            const int j = 16 * ja + jj, buf = jj & 1;
+            if (ti == jj) {
+#pragma unroll
+                for (int b = 0; b < T; ++b) row[buf][tj + 16 * b] = w[ja][b];
+            }
+            __syncthreads();
+            double d = row[buf][j];
+            if (!(d > 0.0)) { bad = true; d = 1.0; }
+            if (threadIdx.x == 0) piv[j] = d;
+            const double inv = 1.0 / d;
+            double v[T];
+#pragma unroll
+            for (int b = 0; b < T; ++b) v[b] = (tj + 16 * b == j) ? 1.0 : row[buf][tj + 16 * b];
+#pragma unroll
+            for (int a = ja; a < T; ++a) {
+                const int i = ti + 16 * a;
+                if (i <= j) continue;
+                const double l = row[buf][i] * inv;
+#pragma unroll
+                for (int b = 0; b < T; ++b) {
+                    if (tj + 16 * b == j) w[a][b] = 0.0;
+                    w[a][b] = fma(-l, v[b], w[a][b]);
+                }
+            }
+        }
+    }
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    if (bad && threadIdx.x == 0) *fail = 1;
+    if (threadIdx.x < 16 * T) piv[threadIdx.x] = 1.0 / sqrt(piv[threadIdx.x]);
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < T; ++a)
+#pragma unroll
+        for (int b = 0; b < T; ++b) {
+            const int i = ti + 16 * a, j = tj + 16 * b;
+            if (i >= p || j >= p) continue;
+            Linv[(long long)i * ldl + j] = (j < i) ? w[a][b] * piv[i] : (j == i ? piv[i] : 0.0);
+            if (G) {        // row i froze at step i: its entries right of the diagonal are d_i l_ji
+                G[(long long)j * ldg + i] = (j >= i) ? w[a][b] * piv[i] : 0.0;
+            }
+        }
+}
+
+// *b = the smallest eigenvalue of H = L L^T, from above, by twelve inverse iterations with L^-1.
+__global__ void __launch_bounds__(1024)
+smallest_eigenvalue_kernel(const double* __restrict__ Linv, long long ldl, int p, double* __restrict__ b) {
+    __shared__ double v[512], u[512], red[32];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    auto sum_squares = [&](const double* x) {
+        double s = 0.0;
+        for (int i = tid; i < p; i += 1024) s = fma(x[i], x[i], s);
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) red[warp] = s;
+        __syncthreads();
+        s = 0.0;
+        for (int i = 0; i < 32; ++i) s += red[i];
+        __syncthreads();
+        return s;
+    };
+    for (int i = tid; i < p; i += 1024) v[i] = 1.0;
+    __syncthreads();
+    double last = 1.0;
+    for (int it = 0; it < 12; ++it) {
+        const double nv = 1.0 / sqrt(sum_squares(v));
+        for (int i = warp; i < p; i += 32) {                 // u = Linv v / |v|
+            double s = 0.0;
+            for (int j = lane; j <= i; j += 32) s = fma(Linv[(long long)i * ldl + j], v[j], s);
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) u[i] = s * nv;
+        }
+        __syncthreads();
+        last = sum_squares(u);                               // v^T H^-1 v / v^T v
+        // v = Linv^T u: 32 columns per warp, the rows dealt over the warps of a column group
+        const int groups = (p + 31) / 32, per = 32 / groups, grp = warp % groups, part = warp / groups;
+        const int j = grp * 32 + lane;
+        double s = 0.0;
+        if (part < per && j < p)
+            for (int i = j + part; i < p; i += per) s = fma(Linv[(long long)i * ldl + j], u[i], s);
+        __shared__ double acc[32][33];
+        acc[warp][lane] = s;
+        __syncthreads();
+        if (warp < groups && j < p) {
+            double t = 0.0;
+            for (int q = 0; q < per; ++q) t += acc[q * groups + warp][lane];
+            v[j] = t;
+        }
         __syncthreads();
     }
-    if (threadIdx.x == 0) norms[blockIdx.x] = red[0];
-}
-__global__ void select_top_kernel(double* __restrict__ norms, int p, int r, int* __restrict__ order, double* __restrict__ sigma_out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    for (int t = 0; t < r; ++t) {
-        int best = 0;
-        for (int i = 1; i < p; ++i) if (norms[i] > norms[best]) best = i;
-        order[t] = best;
-        if (sigma_out) sigma_out[t] = sqrt(norms[best]);
-        norms[best] = -1.0;
-    }
+    if (tid == 0) *b = 1.0 / last;
 }
 
-// L_B[n, t] = fp16(Bt[order[t], n]);  Vt[t, k] = Qt[order[t], k] (fp64, input of the last solve).
-__global__ void gather_kernel(const double* __restrict__ Bt, int N, const double* __restrict__ Qt, int K,
-                              const int* __restrict__ order, int r, __half* __restrict__ LB, double* __restrict__ Vt) {
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < (long long)N * r) {
-        const int n = (int)(e / r), t = (int)(e % r);
-        LB[e] = __double2half(Bt[(long long)order[t] * N + n]);
+// One-sided Jacobi on the rows of G [p, p], the rotations applied to V (the identity at first):
+// V G has orthogonal rows.  All rounds in one CTA, rows in shared memory, half a warp per pair; ends
+// with the first sweep that finds every pair orthogonal to rounding.  The tangent of an angle is
+// taken in fp32 (its error only leaves the pair for a later sweep), cosine and sine in fp64, so the
+// rotations are orthogonal to fp64 rounding.
+constexpr int kJacobiThreads = 896;          // kMaxP / 2 half warps
+static_assert(kJacobiThreads / 16 >= kMaxP / 2, "a half warp per pair");
+__global__ void __launch_bounds__(kJacobiThreads)
+jacobi_kernel(double* __restrict__ G, double* __restrict__ V, int p) {
+    extern __shared__ __align__(16) double jsm[];
+    double* g = jsm;
+    double* v = jsm + p * p;
+    __shared__ int rotated;
+    const int pair = threadIdx.x >> 4, lane = threadIdx.x & 15;
+    for (int e = threadIdx.x; e < p * p; e += kJacobiThreads) { g[e] = G[e]; v[e] = (e / p == e % p) ? 1.0 : 0.0; }
+    const int m = p - 1;
+    for (int sweep = 0; sweep < 20; ++sweep) {
+        __syncthreads();
+        if (threadIdx.x == 0) rotated = 0;
+        __syncthreads();
+        for (int round = 0; round < m; ++round) {
+            // round-robin tournament over p (even) players: player p - 1 stays, the others rotate
+            const int i = (pair == 0) ? round : (round + pair) % m;
+            const int j = (pair == 0) ? m : (round + m - pair) % m;
+            const bool have = pair < p / 2;
+            double* gi = g + i * p;
+            double* gj = g + j * p;
+            double a = 0.0, b = 0.0, c = 0.0;
+            if (have)
+                for (int k = lane; k < p; k += 16) {
+                    const double x = gi[k], y = gj[k];
+                    a = fma(x, x, a); b = fma(y, y, b); c = fma(x, y, c);
+                }
+            for (int o = 8; o > 0; o >>= 1) {
+                a += __shfl_xor_sync(0xffffffffu, a, o);
+                b += __shfl_xor_sync(0xffffffffu, b, o);
+                c += __shfl_xor_sync(0xffffffffu, c, o);
+            }
+            if (have && c * c > 1e-28 * a * b) {
+                if (lane == 0) rotated = 1;
+                const float zeta = (float)((b - a) / (2.0 * c)), z = fabsf(zeta);
+                const float tf = z > 1e9f ? 0.5f / z : 1.f / (z + sqrtf(1.f + z * z));
+                const double t = zeta >= 0.f ? (double)tf : -(double)tf;
+                const double cs = rsqrt(1.0 + t * t), sn = cs * t;
+                double* vi = v + i * p;
+                double* vj = v + j * p;
+                for (int k = lane; k < p; k += 16) {
+                    const double x = gi[k], y = gj[k], w = vi[k], u = vj[k];
+                    gi[k] = cs * x - sn * y; gj[k] = sn * x + cs * y;
+                    vi[k] = cs * w - sn * u; vj[k] = sn * w + cs * u;
+                }
+            }
+            __syncthreads();
+        }
+        if (!rotated) break;
     }
-    if (e < (long long)r * K) {
-        const int t = (int)(e / K), k = (int)(e % K);
-        Vt[e] = Qt[(long long)order[t] * K + k];
+    for (int e = threadIdx.x; e < p * p; e += kJacobiThreads) { G[e] = g[e]; V[e] = v[e]; }
+}
+
+__global__ void identity_kernel(double* __restrict__ V, int p) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < p * p) V[e] = (e / p == e % p) ? 1.0 : 0.0;
+}
+
+// The r longest rows of G [p, p] in descending order (equal ones by index): their norms to sigma
+// and sigma_out, the matching rows of V to Vsel [r, p].  One CTA, p <= 512.
+__global__ void __launch_bounds__(512)
+select_top_kernel(const double* __restrict__ G, const double* __restrict__ V, int p, int r, double* __restrict__ Vsel,
+                  double* __restrict__ sigma, double* __restrict__ sigma_out) {
+    __shared__ double norm[512];
+    __shared__ int order[512];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int i = warp; i < p; i += 16) {
+        double s = 0.0;
+        for (int k = lane; k < p; k += 32) s = fma(G[(long long)i * p + k], G[(long long)i * p + k], s);
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) norm[i] = s;
     }
+    __syncthreads();
+    for (int i = threadIdx.x; i < p; i += 512) {
+        int rank = 0;
+        for (int k = 0; k < p; ++k) rank += (norm[k] > norm[i] || (norm[k] == norm[i] && k < i)) ? 1 : 0;
+        order[rank] = i;
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < r; t += 512) {
+        const double s = sqrt(norm[order[t]]);
+        sigma[t] = s;
+        if (sigma_out) sigma_out[t] = s;
+    }
+    for (int e = threadIdx.x; e < r * p; e += 512) Vsel[e] = V[(long long)order[e / p] * p + e % p];
 }
-__global__ void to_half_kernel(const double* __restrict__ src, long long n, __half* __restrict__ dst) {
+
+// L_B[n, t] = fp16(sigma[t] * U[t, n])
+__global__ void up_factor_kernel(const double* __restrict__ U, const double* __restrict__ sigma, int N, int r, __half* __restrict__ LB) {
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < n) dst[e] = __double2half(src[e]);
+    if (e >= (long long)N * r) return;
+    const int n = (int)(e / r), t = (int)(e % r);
+    LB[e] = __double2half(sigma[t] * U[(long long)t * N + n]);
 }
+// L_A[t, k] = fp16(src[t, k] / sigma[t] * *mul)
+__global__ void down_factor_kernel(const double* __restrict__ src, const double* __restrict__ sigma, int K, int r,
+                                   const double* __restrict__ mul, __half* __restrict__ LA) {
+    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < (long long)r * K) LA[e] = __double2half(src[e] / sigma[e / K] * (mul ? *mul : 1.0));
+}
+
+// Splits of k are chosen for a fixed SM count, so that the workspace size needs no device.
+constexpr int kSplitSms = 148;
 
 struct ConstructLayout {
-    int p;
-    size_t E, A, G, Xs, Qt, Zt, Yt, C, Vt, norms, lambda, order, fail, Wm, total;     // byte offsets
+    int p, tokens;                // tokens padded to 16 rows
+    long long lda;                // columns of the wide error matrix, at most
+    size_t A, E, G, Xs, T[4], Y, part, C, L, V, Vsel, sigma, row_sq, scalars, fail, Wm, total;     // byte offsets
 };
 
 ConstructLayout construct_layout(int N, int K, int Tcal, int r, int n_split) {
@@ -365,20 +581,37 @@ ConstructLayout construct_layout(int N, int K, int Tcal, int r, int n_split) {
     const int lim = (N < K ? N : K) & ~1;
     if (p > lim) p = lim;
     L.p = p;
+    L.tokens = (Tcal + 15) / 16 * 16;
+    const int wide = L.tokens <= K ? K + L.tokens : K;
+    L.lda = wide;
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t o = off; off += (bytes + 255) / 256 * 256; return o; };
+    L.A = take((size_t)N * wide * 8);
     L.E = take((size_t)N * K * 8);
-    L.A = take((size_t)N * K * 8);
     L.G = take((size_t)K * K * 8);
-    L.Xs = take((size_t)Tcal * K * 8);
-    L.Qt = take((size_t)p * K * 8);
-    L.Zt = take((size_t)p * K * 8);
-    L.Yt = take((size_t)p * N * 8);
+    L.Xs = take((size_t)L.tokens * K * 8);
+    for (int i = 0; i < 4; ++i) L.T[i] = take((size_t)p * N * 8);
+    L.Y = take((size_t)p * wide * 8);
+    size_t part = 0;
+    auto need = [&](int m, int n, int k) {
+        const size_t b = gemm64::partial_bytes(m, n, k, kSplitSms);
+        if (b > part) part = b;
+    };
+    need(N, L.tokens, K); need(N, K, K);
+    for (int kc : {K, wide}) { need(p, kc, N); need(p, N, kc); need(p, p, kc); }
+    need(p, p, N); need(p, N, p); need(r, N, p); need(r, K, N);
+    for (int i0 = kMaxP; i0 < p; i0 += kMaxP) {
+        const int nb = p - i0 < kMaxP ? p - i0 : kMaxP;
+        need(p - i0, kMaxP, kMaxP); need(p - i0, p - i0, kMaxP); need(nb, i0, i0); need(nb, i0, nb);
+    }
+    L.part = take(part);
     L.C = take((size_t)p * p * 8);
-    L.Vt = take((size_t)(r > 0 ? r : 1) * K * 8);
-    L.norms = take((size_t)p * 8);
-    L.lambda = take(8);
-    L.order = take((size_t)(r > 0 ? r : 1) * 4);
+    L.L = take((size_t)p * p * 8);
+    L.V = take((size_t)p * p * 8);
+    L.Vsel = take((size_t)(r > 0 ? r : 1) * p * 8);
+    L.sigma = take((size_t)(r > 0 ? r : 1) * 8);
+    L.row_sq = take((size_t)L.tokens * 8);
+    L.scalars = take(64);
     L.fail = take(4);
     L.Wm = take(n_split > 0 ? (size_t)N * K * 2 : 0);
     L.total = off;
@@ -387,17 +620,65 @@ ConstructLayout construct_layout(int N, int K, int Tcal, int r, int n_split) {
 
 inline int blocks_for(long long n, int threads) { return (int)((n + threads - 1) / threads); }
 
-// Rows of Z [p, K] made orthonormal: C = Z Z^T = L L^T, Z <- L^-1 Z, twice (the second pass
-// removes what rounding left of the first).
-int orthonormalize_rows(cudaStream_t st, double* Z, int p, int K, double* C, int* fail) {
-    for (int pass = 0; pass < 2; ++pass) {
-        int rc = dgemm(st, p, p, K, 1.0, Z, K, 1, Z, 1, K, 0.0, C, p);
-        if (rc != ASER_OK) return rc;
-        rc = potrf_lower(st, C, p, p, fail);
-        if (rc != ASER_OK) return rc;
-        left_solve_lower_kernel<<<blocks_for(K, 128), 128, 0, st>>>(C, p, p, Z, K, K);
+// What the steps share: stream, pieces of split products, failure flag.
+struct Ctx {
+    cudaStream_t st;
+    double* part;
+    int* fail;
+};
+
+// C[m, n] = a0 / *div * A B (+ a1 X1 + a2 X2)
+int product(const Ctx& c, bool tb, int m, int n, int k, const double* A, long long lda, const double* B, long long ldb,
+            double* C, long long ldc, double a0 = 1.0, const double* div = nullptr, const double* X1 = nullptr, double a1 = 0.0,
+            const double* X2 = nullptr, double a2 = 0.0) {
+    gemm64::Args g = {};
+    g.A = A; g.B = B; g.C = C; g.lda = lda; g.ldb = ldb; g.ldc = ldc; g.m = m; g.n = n; g.k = k;
+    g.a0 = a0; g.a0_div = div; g.X1 = X1; g.a1 = a1; g.X2 = X2; g.a2 = a2;
+    return gemm64::run(g, tb, c.part, kSplitSms, c.st);
+}
+
+#define ASER_STEP(call)                        \
+    do {                                       \
+        const int step_rc = (call);            \
+        if (step_rc != ASER_OK) return step_rc; \
+    } while (0)
+
+int chol_inverse_block(const Ctx& c, const double* H, long long ldh, int p, double* Linv, long long ldl, double* G, long long ldg) {
+    switch ((p + 15) / 16) {
+        case 1: chol_inverse_kernel<1><<<1, 256, 0, c.st>>>(H, ldh, p, Linv, ldl, G, ldg, c.fail); break;
+        case 2: chol_inverse_kernel<2><<<1, 256, 0, c.st>>>(H, ldh, p, Linv, ldl, G, ldg, c.fail); break;
+        case 3: chol_inverse_kernel<3><<<1, 256, 0, c.st>>>(H, ldh, p, Linv, ldl, G, ldg, c.fail); break;
+        case 4: chol_inverse_kernel<4><<<1, 256, 0, c.st>>>(H, ldh, p, Linv, ldl, G, ldg, c.fail); break;
+        case 5: chol_inverse_kernel<5><<<1, 256, 0, c.st>>>(H, ldh, p, Linv, ldl, G, ldg, c.fail); break;
+        case 6: chol_inverse_kernel<6><<<1, 256, 0, c.st>>>(H, ldh, p, Linv, ldl, G, ldg, c.fail); break;
+        default: chol_inverse_kernel<7><<<1, 256, 0, c.st>>>(H, ldh, p, Linv, ldl, G, ldg, c.fail); break;
     }
-    return check_launch("orthonormalize_rows");
+    return check_launch("chol_inverse_kernel");
+}
+
+// H [p, p] (overwritten where p > kMaxP) = L L^T: Linv = L^-1, G = L (both pitch p, zeros above the
+// diagonal).  Larger matrices in blocks of kMaxP rows.
+int chol_inverse(const Ctx& c, double* H, int p, double* Linv, double* G) {
+    if (p <= kMaxP) return chol_inverse_block(c, H, p, p, Linv, p, G, p);
+    cudaError_t e = cudaMemsetAsync(Linv, 0, (size_t)p * p * 8, c.st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(G, 0, (size_t)p * p * 8, c.st);
+    if (e != cudaSuccess) return record_cuda_error(e, "construct: memset");
+    for (int i0 = 0; i0 < p; i0 += kMaxP) {
+        const int nb = p - i0 < kMaxP ? p - i0 : kMaxP, rest = p - i0 - nb;
+        const long long d = (long long)i0 * p + i0, below = d + (long long)nb * p;
+        ASER_STEP(chol_inverse_block(c, H + d, p, nb, Linv + d, p, G + d, p));
+        if (rest > 0) {
+            // rows below: L_ib = H_ib Linv_bb^T, then their Schur complement
+            ASER_STEP(product(c, true, rest, nb, nb, H + below, p, Linv + d, p, G + below, p));
+            ASER_STEP(product(c, true, rest, rest, nb, G + below, p, G + below, p, H + below + nb, p, -1.0, nullptr,
+                              H + below + nb, 1.0));
+        }
+        if (i0 > 0) {       // row block of the inverse: -Linv_bb (L_b,0..i0 Linv_0..i0); H's rows are scratch by now
+            ASER_STEP(product(c, false, nb, i0, i0, G + (long long)i0 * p, p, Linv, p, H + (long long)i0 * p, p));
+            ASER_STEP(product(c, false, nb, i0, nb, Linv + d, p, H + (long long)i0 * p, p, Linv + (long long)i0 * p, p, -1.0));
+        }
+    }
+    return ASER_OK;
 }
 
 }  // namespace
@@ -412,19 +693,11 @@ int launch_construct(const __half* W, const float* s, const __half* Xcal, int N,
                      cudaStream_t st) {
     const ConstructLayout L = construct_layout(N, K, Tcal, r, n_split);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    double* E = reinterpret_cast<double*>(ws + L.E);
-    double* A = reinterpret_cast<double*>(ws + L.A);
-    double* G = reinterpret_cast<double*>(ws + L.G);
-    double* Xs = reinterpret_cast<double*>(ws + L.Xs);
-    double* Qt = reinterpret_cast<double*>(ws + L.Qt);
-    double* Zt = reinterpret_cast<double*>(ws + L.Zt);
-    double* Yt = reinterpret_cast<double*>(ws + L.Yt);
-    double* C = reinterpret_cast<double*>(ws + L.C);
-    double* Vt = reinterpret_cast<double*>(ws + L.Vt);
-    double* norms = reinterpret_cast<double*>(ws + L.norms);
-    double* lambda = reinterpret_cast<double*>(ws + L.lambda);
-    int* order = reinterpret_cast<int*>(ws + L.order);
+    auto at = [&](size_t off) { return reinterpret_cast<double*>(ws + off); };
+    double *A = at(L.A), *G = at(L.G), *Xs = at(L.Xs), *Y = at(L.Y), *C = at(L.C), *Li = at(L.L), *V = at(L.V);
+    double *Vsel = at(L.Vsel), *sigma = at(L.sigma), *lambda = at(L.scalars), *bound = lambda + 3;
     int* fail = reinterpret_cast<int*>(ws + L.fail);
+    const Ctx ctx{st, at(L.part), fail};
     const int p = L.p;
 
     const __half* Wquant = W;
@@ -433,64 +706,111 @@ int launch_construct(const __half* W, const float* s, const __half* Xcal, int N,
         mask_columns_kernel<<<blocks_for((long long)N * K, 256), 256, 0, st>>>(W, N, K, split_idx, n_split, Wm);
         Wquant = Wm;
     }
-    int rc = launch_pack_w4(Wquant, s, N, K, Wq, w_scale, st);
-    if (rc != ASER_OK) return rc;
+    ASER_STEP(launch_pack_w4(Wquant, s, N, K, Wq, w_scale, st));
     if (r == 0) return ASER_OK;
     cudaError_t e = cudaMemsetAsync(fail, 0, sizeof(int), st);
     if (e != cudaSuccess) return record_cuda_error(e, "construct: memset");
-    build_error_kernel<<<blocks_for((long long)N * K, 256), 256, 0, st>>>(W, s, Wq, w_scale, N, K, E);
-    build_xs_kernel<<<blocks_for((long long)Tcal * K, 256), 256, 0, st>>>(Xcal, s, Tcal, K, Xs);
-    // G = X~^T X~ (the paper's X X^T), damped, then its Cholesky factor in place
-    rc = dgemm(st, K, K, Tcal, 1.0, Xs, 1, K, Xs, K, 1, 0.0, G, K);
-    if (rc != ASER_OK) return rc;
-    damp_kernel<<<1, 256, 0, st>>>(G, K, damping, lambda);
-    rc = potrf_lower(st, G, K, K, fail);
-    if (rc != ASER_OK) return rc;
-    zero_upper_kernel<<<blocks_for((long long)K * K, 256), 256, 0, st>>>(G, K, K);
-    if (S_out) {
-        e = cudaMemcpyAsync(S_out, G, (size_t)K * K * 8, cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return record_cuda_error(e, "construct: copy S");
-    }
-    // A = E S
-    rc = dgemm(st, N, K, K, 1.0, E, K, 1, G, K, 1, 0.0, A, K);
-    if (rc != ASER_OK) return rc;
-    // subspace iteration on A^T A with the basis as rows
-    init_basis_kernel<<<blocks_for((long long)p * K, 256), 256, 0, st>>>(Qt, (long long)p * K);
-    rc = orthonormalize_rows(st, Qt, p, K, C, fail);
-    if (rc != ASER_OK) return rc;
-    for (int it = 0; it < iters; ++it) {
-        rc = dgemm(st, p, N, K, 1.0, Qt, K, 1, A, 1, K, 0.0, Yt, N);          // Yt = Qt A^T
-        if (rc != ASER_OK) return rc;
-        rc = dgemm(st, p, K, N, 1.0, Yt, N, 1, A, K, 1, 0.0, Zt, K);          // Zt = Yt A
-        if (rc != ASER_OK) return rc;
-        double* t = Qt; Qt = Zt; Zt = t;
-        rc = orthonormalize_rows(st, Qt, p, K, C, fail);
-        if (rc != ASER_OK) return rc;
-    }
-    // Rayleigh-Ritz: rotate the rows of Bt = Qt A^T (and of Qt with them) until they are orthogonal
-    rc = dgemm(st, p, N, K, 1.0, Qt, K, 1, A, 1, K, 0.0, Yt, N);
-    if (rc != ASER_OK) return rc;
-    for (int sweep = 0; sweep < 12; ++sweep)
-        for (int round = 0; round < p - 1; ++round)
-            jacobi_round_kernel<<<p / 2, 256, 0, st>>>(Yt, N, Qt, K, p, round);
-    row_norms_kernel<<<p, 256, 0, st>>>(Yt, N, norms);
-    select_top_kernel<<<1, 32, 0, st>>>(norms, p, r, order, sigma_out);
-    const long long ge = (long long)(N > K ? N : K) * r;
-    gather_kernel<<<blocks_for(ge, 256), 256, 0, st>>>(Yt, N, Qt, K, order, r, LB, Vt);
-    // L_A S = V_r^T: solve backwards over 64-column blocks, in place in Vt
-    for (int c0 = ((K - 1) / kCB) * kCB; c0 >= 0; c0 -= kCB) {
-        const int nb = (K - c0 < kCB) ? (K - c0) : kCB;
-        const int done = K - c0 - nb;           // columns behind the block, already solved
-        if (done > 0) {
-            rc = dgemm(st, r, nb, done, -1.0, Vt + c0 + nb, K, 1, G + (long long)(c0 + nb) * K + c0, K, 1, 1.0,
-                       Vt + c0, K);
-            if (rc != ASER_OK) return rc;
+    build_xs_kernel<<<L.tokens, 256, 0, st>>>(Xcal, s, Tcal, K, Xs, at(L.row_sq));
+    lambda_kernel<<<1, 32, 0, st>>>(at(L.row_sq), L.tokens, K, damping, lambda, fail);
+
+    // The matrix A [N, kc] to be decomposed, and the error matrix E (times *e_mul^-1) inside or beside it.
+    // Above a damping of 1e-6 the smallest eigenvalue of the damped Gram matrix is far above the
+    // rounding of its Cholesky factorisation at every supported K, so nothing is left to report.
+    const bool factor = S_out != nullptr || damping < 1e-6 || L.tokens > K;
+    const int kc = factor ? K : K + L.tokens;
+    const double *E, *e_mul;
+    long long lde;
+    const int error_blocks = blocks_for((long long)N * (K / 8), 256);
+    if (factor) {
+        // G = X~^T X~ (the paper's X X^T), damped, its Cholesky factor in place, A = E S
+        double* Ef = at(L.E);
+        build_error_kernel<<<error_blocks, 256, 0, st>>>(W, s, Wq, w_scale, N, K, Ef, K, nullptr);
+        ASER_STEP(dgemm(st, K, K, Tcal, 1.0, Xs, 1, K, Xs, K, 1, 0.0, G, K));
+        damp_kernel<<<1, 256, 0, st>>>(G, K, damping);
+        ASER_STEP(potrf_lower(st, G, K, K, fail));
+        zero_upper_kernel<<<blocks_for((long long)K * K, 256), 256, 0, st>>>(G, K, K);
+        if (S_out) {
+            e = cudaMemcpyAsync(S_out, G, (size_t)K * K * 8, cudaMemcpyDeviceToDevice, st);
+            if (e != cudaSuccess) return record_cuda_error(e, "construct: copy S");
         }
-        right_solve_lower_kernel<<<blocks_for(r, 128), 128, 0, st>>>(Vt + c0, K, r, G + (long long)c0 * K + c0, K, nb);
+        ASER_STEP(product(ctx, false, N, K, K, Ef, K, G, K, A, K));
+        E = Ef; lde = K; e_mul = nullptr;
+    } else {
+        // A = [ sqrt(lambda) E | E X~^T ]
+        build_error_kernel<<<error_blocks, 256, 0, st>>>(W, s, Wq, w_scale, N, K, A, kc, lambda + 1);
+        ASER_STEP(product(ctx, true, N, L.tokens, K, A, kc, Xs, K, A + K, kc, 1.0, lambda + 1));
+        E = A; lde = kc; e_mul = lambda + 2;
     }
-    to_half_kernel<<<blocks_for((long long)r * K, 256), 256, 0, st>>>(Vt, (long long)r * K, LA);
-    rc = check_launch("construct");
-    if (rc != ASER_OK) return rc;
+
+    // subspace iteration on A A^T with the basis as rows: t0 the current basis, t1 the term before it
+    double *t0 = at(L.T[0]), *t1 = at(L.T[1]), *f0 = at(L.T[2]), *f1 = at(L.T[3]);
+    auto swap = [](double*& x, double*& y) { double* t = x; x = y; y = t; };
+    // t0 <- L^-1 t0 with L L^T = t0 t0^T; the same factor applied to t1 if it is still needed
+    auto normalize = [&](bool both) {
+        ASER_STEP(product(ctx, true, p, p, N, t0, N, t0, N, C, p));
+        ASER_STEP(chol_inverse(ctx, C, p, Li, V));
+        gemm64::Args g = {};
+        g.A = Li; g.lda = p; g.B = t0; g.ldb = N; g.C = f0; g.ldc = N; g.m = p; g.n = N; g.k = p; g.a0 = 1.0;
+        if (both) { g.B2 = t1; g.C2 = f1; }
+        if (both) { ASER_STEP(gemm64::run(g, false, ctx.part, kSplitSms, st)); swap(t1, f1); }
+        else { ASER_STEP(product(ctx, false, p, N, p, Li, p, t0, N, f0, N)); }
+        swap(t0, f0);
+        return (int)ASER_OK;
+    };
+    init_basis_kernel<<<blocks_for((long long)p * N, 256), 256, 0, st>>>(t0, (long long)p * N);
+    ASER_STEP(normalize(false));
+    ASER_STEP(normalize(false));
+    int done = 0;
+    for (; done < iters && done < 2; ++done) {
+        ASER_STEP(product(ctx, false, p, kc, N, t0, N, A, kc, Y, kc));
+        ASER_STEP(product(ctx, true, p, N, kc, Y, kc, A, kc, f0, N));
+        swap(t0, f0);
+        ASER_STEP(normalize(false));
+    }
+    const int cycles = (iters - done + 11) / 12;
+    for (int cycle = 0; cycle < cycles; ++cycle) {
+        const int steps = (iters - done) / (cycles - cycle);
+        for (int i = 0; i < steps; ++i, ++done) {
+            ASER_STEP(product(ctx, false, p, kc, N, t0, N, A, kc, Y, kc));
+            if (i == 0) {       // the basis is orthonormal here: Y Y^T holds its Ritz values
+                ASER_STEP(product(ctx, true, p, p, kc, Y, kc, Y, kc, C, p));
+                ASER_STEP(chol_inverse(ctx, C, p, Li, V));
+                smallest_eigenvalue_kernel<<<1, 1024, 0, st>>>(Li, p, p, bound);
+                ASER_STEP(product(ctx, true, p, N, kc, Y, kc, A, kc, f0, N, 2.0, bound, t0, -1.0));
+            } else {
+                ASER_STEP(product(ctx, true, p, N, kc, Y, kc, A, kc, f0, N, 4.0, bound, t0, -2.0, t1, -1.0));
+            }
+            swap(t1, f0);       // the new term to t1 ...
+            swap(t0, t1);       // ... and into its place, the old basis behind it
+            ASER_STEP(normalize(i + 1 < steps));
+        }
+    }
+    ASER_STEP(normalize(false));
+
+    // Rayleigh-Ritz: rotate the rows of the Cholesky factor of (Ut A)(Ut A)^T until they are orthogonal
+    ASER_STEP(product(ctx, false, p, kc, N, t0, N, A, kc, Y, kc));
+    ASER_STEP(product(ctx, true, p, p, kc, Y, kc, Y, kc, C, p));
+    ASER_STEP(chol_inverse(ctx, C, p, Li, V));
+    double* Lrows = V;          // L, then the rotated rows
+    double* Vrot = Li;          // the rotations (the inverse is not needed here)
+    if (p <= kMaxP) {
+        const int smem = 2 * p * p * 8;
+        e = cudaFuncSetAttribute(jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kMaxP * kMaxP * 8);
+        if (e != cudaSuccess) return record_cuda_error(e, "jacobi smem attribute");
+        jacobi_kernel<<<1, kJacobiThreads, smem, st>>>(Lrows, Vrot, p);
+    } else {
+        identity_kernel<<<blocks_for((long long)p * p, 256), 256, 0, st>>>(Vrot, p);
+        for (int sweep = 0; sweep < 12; ++sweep)
+            for (int round = 0; round < p - 1; ++round)
+                jacobi_round_kernel<<<p / 2, 256, 0, st>>>(Lrows, p, Vrot, p, p, round);
+    }
+    select_top_kernel<<<1, 512, 0, st>>>(Lrows, Vrot, p, r, Vsel, sigma, sigma_out);
+    // U_r^T = Vsel Ut;  L_B = U_r Sigma_r,  L_A = Sigma_r^-1 U_r^T E
+    ASER_STEP(product(ctx, false, r, N, p, Vsel, p, t0, N, f0, N));
+    up_factor_kernel<<<blocks_for((long long)N * r, 256), 256, 0, st>>>(f0, sigma, N, r, LB);
+    ASER_STEP(product(ctx, false, r, K, N, f0, N, E, lde, Y, K));
+    down_factor_kernel<<<blocks_for((long long)r * K, 256), 256, 0, st>>>(Y, sigma, K, r, e_mul, LA);
+    ASER_STEP(check_launch("construct"));
     // an offline step: wait for it and report a failed factorisation
     int host_fail = 0;
     e = cudaMemcpyAsync(&host_fail, fail, sizeof(int), cudaMemcpyDeviceToHost, st);

@@ -104,3 +104,30 @@ def test_construct_config2_full_size(aser):
     """The 4096 x 4096 attention projection with 512 calibration tokens, rank 64 (configuration 2)."""
     lay, r = synth.config2_decode(8)
     _check(aser, lay, r)
+
+
+@pytest.mark.parametrize("N,K,r,n_cal", [
+    (384, 512, 32, 256),       # 64 vectors, k split over CTAs
+    (520, 768, 48, 5),         # ragged N, token rows padded from 5 to 16
+    (1160, 256, 16, 256),      # 48 vectors, as many tokens as channels
+    (512, 512, 80, 600),       # 120 vectors (two row blocks), more tokens than channels: through S
+    (648, 640, 128, 100),      # 192 vectors
+])
+def test_construct_without_the_whitening_factor(aser, N, K, r, n_cal):
+    """No S asked for: the decomposed matrix is [sqrt(lambda) E | E X~^T] with at most K tokens, and L_A comes
+    from the error matrix instead of a triangular solve.  Bounds as in _check: the product differs by
+    two fp16 roundings a side, the singular values by fp64 rounding and the unconverged remainder."""
+    lay = synth.make_layer(4, N, K, seed=synth.seed_for(2, N + K + r), n_cal=n_cal)
+    s = Cn.smoothing_vector_config(lay.X_cal, lay.W, lay.outlier_idx)
+    L = Cn.construct_layer(lay.W, lay.X_cal, s, r=r)
+    out = aser.construct(to_dev(lay.W), to_dev(s), to_dev(lay.X_cal), r)
+    assert out["S"] is None
+    assert np.array_equal(out["Wq"].cpu().numpy(), L.Wq)
+    assert np.allclose(out["sigma"].cpu().numpy(), L.sigma[:r], rtol=1e-6)
+    prod_gpu = out["L_B"].cpu().numpy().astype(np.float64) @ out["L_A"].cpu().numpy().astype(np.float64)
+    prod_ref = L.L_B.astype(np.float64) @ L.L_A.astype(np.float64)
+    assert np.linalg.norm(prod_gpu - prod_ref) < 2e-3 * np.linalg.norm(prod_ref)
+    # a zero calibration set has no positive definite damped Gram matrix
+    with pytest.raises(aser.AserError) as err:
+        aser.construct(to_dev(lay.W), to_dev(s), torch.zeros_like(to_dev(lay.X_cal)), r)
+    assert err.value.code == -3
