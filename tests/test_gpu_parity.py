@@ -50,6 +50,26 @@ def test_pack_w4_bit_exact(aser, N, K, smooth):
     assert torch.equal(back, Wq)
 
 
+@pytest.mark.parametrize("N,K", [(16, 2176), (8, 4224), (136, 6272), (24, 8320), (8, 16384), (16, 16512), (8, 24704), (8, 32768)])
+def test_pack_w4_chunks_per_thread(aser, N, K):
+    """A row length for every chunk count a thread may hold (its last chunk partly missing where the
+    length allows), with a row of exact ties and smoothing factors so small that the scale is below
+    the range where its reciprocal is used."""
+    lay = synth.make_layer(1, N, K, seed=300 + N + K, n_cal=8)
+    W = lay.W.copy()
+    W[1] = (np.arange(K) % 15 - 7).astype(np.float16) / 2      # halves, so ties against a scale of 1
+    W[1, 0] = np.float16(7)
+    W[2] = np.float16(2.0 ** -24)
+    s = synth.standin_smoothing_vector(K, lay.outlier_idx, 11.5)
+    for sv in (None, s, (s * np.float32(2.0 ** -120)).astype(np.float32)):
+        q, w_scale = F.quant_w4(W, sv)
+        Wq, wsc = aser.pack_w4(to_dev(W), None if sv is None else to_dev(sv))
+        assert np.array_equal(Wq.cpu().numpy(), F.pack_w4(q))
+        assert np.array_equal(bits(wsc.cpu().numpy()), bits(w_scale))
+    Wk = aser.repack_w4(Wq)
+    assert torch.equal(aser.unrepack_w4(Wk, N, K), Wq)
+
+
 def test_repack_layout_by_definition(aser):
     """Word w of sub-block `sub`, row `row` covers columns 32*sub + 8*w .. +7 with column
     c0+i in nibble 2i and column c0+4+i in nibble 2i+1."""
