@@ -82,6 +82,12 @@ int launch_linear_decode(const int8_t* Xq, const float* a_scale, const uint8_t* 
                          const float* w_scale, const __nv_bfloat16* T, const __half* LB,
                          int M, int N, int K, int r, __half* Y, int32_t* acc_debug,
                          cudaStream_t st, bool overlap_prev = false, int ldt = 0, CatSplit cat = CatSplit());
+// Many-token kernel on pairs of CTAs (linear_pair.cu); uses the workspace's status word only.
+constexpr int kLinearPairMinTokens = 192;
+bool linear_pair_prefers(int M, int N, int K, int r, const CatSplit& cat);
+int launch_linear_pair(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const float* w_scale,
+                       const __nv_bfloat16* T, const __half* LB, int M, int N, int K, int r, __half* Y,
+                       int32_t* acc_debug, void* workspace, cudaStream_t st, bool overlap_prev, int ldt, CatSplit cat);
 size_t linear_tc_workspace_bytes(int M, int N, int K, int r);
 // The range checks launch_linear_tc makes before it launches (workspace size, index widths), for
 // callers that must reject a call before they enqueue anything else.  Records the error text.

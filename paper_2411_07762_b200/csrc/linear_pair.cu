@@ -1,0 +1,678 @@
+// Tensor-core kernel of the ASER linear for many tokens (Sec. 4.2, "W_q X + L_A L_B X"), on pairs of CTAs:
+//   acc = Xq Wq^T (int8 x int4 -> int32),  Y = fp16(acc * a_scale[m] * w_scale[n] + T L_B^T).
+//
+// As in linear_tc.cu the tile is computed transposed, D[n, token]: packed int4 weights are streamed to
+// shared memory, turned into int8 (value 16 q) in registers and written to TENSOR MEMORY as the A
+// operand; the int8 activations are the B operand in shared memory.  What bounds that kernel at many
+// tokens is not arithmetic (tensor pipe busy 41 to 55 %) but the hand-over of A blocks: they are unpacked
+// for 128 tokens at a time, two accumulators and the fp32 low-rank accumulator leave tensor memory for
+// four of them, and a 128 x 128 tile asks 192 bytes of shared memory per cycle at full rate.  Here:
+//  * two CTAs share a tile of 256 output channels x 256 tokens (cta_group::2): each holds 128 rows of
+//    A and of D, and half the tokens' activations.  An A block serves 256 tokens instead of 128, an SM
+//    loads 24 KB per 128 columns of K for twice the products, 96 bytes of shared memory per cycle;
+//  * the tile's tokens are two halves, each with an accumulator of 128 columns and a thread of its own
+//    in the leader CTA that issues the half's MMAs.  The other 256 columns of tensor memory are EIGHT A
+//    blocks, in four stages of two;
+//  * there is no low-rank accumulator.  When a half's integer sums are complete the epilogue takes them
+//    into registers (64 per thread) and hands the columns back at once; the half's low-rank product
+//    (kind::f16) is computed into THE SAME columns, read and added to the scaled sums.  One half's
+//    turn-around is covered by the other half's MMAs;
+//  * A blocks and activations of a stage share one barrier each way, so an issuer waits once and commits
+//    once per eight MMAs (75 cycles each; a wait or a commit costs as much as one to four of them);
+//  * the packed words of a group's next stage are in registers before its slot is free;
+//  * both halves' outputs stay in registers as fp16 until both accumulators are free, then leave through
+//    shared memory as tensor stores (two-byte stores, 64 bytes per warp and token, took 4300 cycles a half
+//    and held up the other half's turn-around);
+//  * arrivals on the other CTA's barriers are plain arrivals: with .release.cluster each cost its thread
+//    a cluster-wide fence, in the unpack groups' loop of all places (4096 x 4096 x 14336: 229 -> 178 us);
+//  * warpgroups of their own register budget (setmaxnreg): one of producers and issuers, two that
+//    unpack (alternate stages), two of epilogue.
+//
+// Work: whole tiles, dealt round robin to the pairs; a remainder of at most half a wave is dealt as half
+// tiles (one half each, the other issuer only hands slots on).  No tile is shared, so there are no
+// partial sums and no workspace beyond the status word.
+// Every wait is bounded: on expiry the CTA sets the status word and winds down.
+//
+// Measured against linear_tc_kernel<128> (tokens x channels x K, rank; us): 2048 x 14336 x 4096, 64: 136 -> 123;
+// 4096 x 14336 x 4096, 128: 271 -> 230; 4096 x 4096 x 14336, 128: 233 -> 178 (2.7 POP/s); 4096 x 28672 x 8192,
+// 256: 1188 -> 896; 1024 x 4096 x 4096, 128: 44 -> 28; 333 x 14336 x 4096, 64: 49 -> 41; 192 x 8192 x 8192, 32:
+// 35 -> 33.
+#include "aser_common.cuh"
+#include "sm100_ptx.cuh"
+
+namespace aser {
+
+namespace {
+
+constexpr int kThreads = 640;                  // five warpgroups
+constexpr int kRegsLaunch = 96;                // per thread at launch: 640 x 96 = 128 x (48 + 2 x 72 + 2 x 144)
+constexpr int kKS = 2;                         // 128-column blocks per stage
+constexpr int kNS = 4, kNW = 2;                // stages of the operand ring (A blocks and activations) and of the weight ring
+constexpr int kMaxHalf = 128;                  // tokens per half, at most
+constexpr int kWStage = kKS * kWkBlockBytes;
+constexpr int kXStage = kKS * kMaxHalf * 128;  // a CTA holds half of each half's tokens
+constexpr int kLbBytes = 128 * 128, kTBytes = (kMaxHalf / 2) * 128;
+constexpr int kYRow = 256;                     // bytes of a staged output row: 128 channels
+constexpr int kOffX = 0, kOffW = kOffX + kNS * kXStage, kOffLr = kOffW + kNW * kWStage,
+              kOffT = kOffLr + 2 * kLbBytes,             // T chunks: [half][slot]
+              kOffBar = kOffT + 4 * kTBytes, kOffScale = kOffBar + 256;
+constexpr int kSmemBytes = kOffScale + 2 * kMaxHalf * 4 + 1024;
+static_assert(2 * kMaxHalf * kYRow <= kOffBar - kOffLr, "the outputs of a tile are staged where its low-rank operands were");
+static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
+constexpr long long kWaitClocks = 400000000ll; // about 0.2 s of SM clocks per wait
+
+// Barriers.  "leader": waited on by the leader CTA's issuers, arrived on from both CTAs; "pair": arrived
+// on in both CTAs by a commit of the leader's issuers; the others are local to a CTA.
+//   W_FULL, W_FREE[s]    weight bytes landed -> unpack; in registers (count 4) -> weight producer
+//   FULL[s]              leader, count 3: both CTAs' activation bytes landed, both CTAs' A blocks written -> issuers
+//   FREE[s]              pair, count 2: both halves' MMAs of the stage retired -> unpack, activation producer
+//   ACC_FULL[h]          pair: integer sums complete -> epilogue
+//   D_READ[h]            leader: integer sums in registers -> issuer (the low-rank product may overwrite them)
+//   LR_DONE[h]           pair: low-rank product complete -> epilogue
+//   ACC_EMPTY[h]         leader: everything read -> issuer (next tile)
+//   LR_FULL              a set of low-rank operands landed -> epilogue (converts T)
+//   LR_CONV              leader, count 2: set converted in both CTAs -> issuers
+//   LR_PART              pair: first of two sets multiplied by a half -> epilogue (loads the next set)
+constexpr int B_W_FULL = 0, B_W_FREE = B_W_FULL + kNW, B_FULL = B_W_FREE + kNW, B_FREE = B_FULL + kNS,
+              B_ACC_FULL = B_FREE + kNS, B_D_READ = B_ACC_FULL + 2, B_LR_DONE = B_D_READ + 2,
+              B_ACC_EMPTY = B_LR_DONE + 2, B_LR_FULL = B_ACC_EMPTY + 2, B_LR_CONV = B_LR_FULL + 1,
+              B_LR_PART = B_LR_CONV + 1, kNumBars = B_LR_PART + 1;
+static_assert(kNumBars * 8 + 8 <= 256, "barrier area");
+constexpr int kEpiWarps = 8, kEpiThreads = 256;
+
+struct Params {
+    const uint8_t* Wk;
+    const float* a_scale;
+    const float* w_scale;
+    int32_t* acc_debug;
+    uint32_t* status;
+    int M, N, r;
+    int KB, NB;            // 128-column blocks, 128-row blocks
+    int NT, TT, half;      // tiles of 256 rows, tiles of 2 half tokens
+    int full, items;       // items [0, full) are whole tiles, the rest single halves, two per tile
+    int tt_outer;          // tile numbering: 1 = token tile outer
+    CatSplit cat;
+};
+
+// `step` tokens lie between the rows of the two CTAs: a whole tile's tokens are [CTA][half][rows], a
+// single half's [CTA][rows].
+struct Item { int nt, tok0, halves, step; };
+
+__device__ __forceinline__ Item get_item(const Params& p, int i) {
+    int tile = i, part = 0;
+    const bool single = i >= p.full;
+    if (single) { tile = p.full + ((i - p.full) >> 1); part = (i - p.full) & 1; }
+    Item w;
+    int tt;
+    if (p.tt_outer) { tt = tile / p.NT; w.nt = tile - tt * p.NT; }
+    else { w.nt = tile / p.TT; tt = tile - w.nt * p.TT; }
+    w.tok0 = (2 * tt + part) * p.half;
+    const int left = p.M - w.tok0;
+    w.halves = left <= 0 ? 0 : (single || left <= p.half) ? 1 : 2;
+    w.step = w.halves == 1 ? p.half / 2 : p.half;
+    return w;
+}
+
+struct Stop {
+    volatile int* flag;    // shared
+    uint32_t* status;      // global
+};
+
+// Bounded wait on a barrier phase: false after the limit or when another role of this CTA gave up.
+// (In line: a call would keep the compiler from giving each warpgroup its register budget.)
+__device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity, const Stop& stop) {
+    uint32_t spins = 0;
+    long long t0 = 0;
+    while (!mbar_try_wait(bar, parity)) {
+        if ((++spins & 255u) == 0) {
+            if (*stop.flag) return false;
+            const long long now = clock64();
+            if (t0 == 0) {
+                t0 = now;
+            } else if (now - t0 > kWaitClocks) {
+                *stop.flag = 1;
+                atomicOr(stop.status, 1u);
+                if (atomicCAS(stop.status + 1, 0u, 0x80000000u | threadIdx.x) == 0u) {    // which wait it was
+                    stop.status[2] = blockIdx.x;
+                    stop.status[3] = (bar & 1023u) >> 3;
+                    stop.status[4] = parity;
+                }
+                return false;
+            }
+        }
+    }
+    return true;
+}
+
+__device__ __forceinline__ bool group_wait(uint32_t bar, uint32_t parity, const Stop& stop, bool leader, int group) {
+    bool ok = true;
+    if (leader) ok = wait(bar, parity, stop);
+    return group == 0 ? named_bar_all(3, 128, ok) : named_bar_all(4, 128, ok);
+}
+
+// Copies in flight land before a CTA that gave up lets go of its shared memory.
+__device__ __forceinline__ void let_copies_land() {
+    const long long t0 = clock64();
+    while (clock64() - t0 < 2000000) {}
+}
+
+template <bool DEBUG_ACC>
+__global__ void __launch_bounds__(kThreads, 1)
+linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_lb,
+                   const __grid_constant__ CUtensorMap map_t, const __grid_constant__ CUtensorMap map_y,
+                   const Params p) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    const uint32_t sbase = smem_u32(smem), bar0 = sbase + kOffBar;
+    auto bar = [&](int i) { return bar0 + 8u * i; };
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kOffBar + kNumBars * 8);
+    volatile int* stop_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_rank();
+    const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+    const Stop stop{stop_flag, p.status};
+    const int chunks = (p.r + 63) / 64;
+    const int stages = (p.KB + kKS - 1) / kKS;      // per item
+
+    if (warp == 0) {
+        for (int i = lane; i < kNumBars; i += 32) {
+            uint32_t count = 1;
+            if (i >= B_W_FREE && i < B_FULL) count = 4;
+            if (i >= B_FULL && i < B_FREE) count = 3;
+            if ((i >= B_FREE && i < B_ACC_FULL) || i == B_LR_CONV) count = 2;
+            if ((i >= B_D_READ && i < B_LR_DONE) || (i >= B_ACC_EMPTY && i < B_LR_FULL)) count = 2 * kEpiWarps;
+            mbar_init(bar(i), count);
+        }
+        if (lane == 0) *stop_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_proxy_async_smem();
+    }
+    if (warp == 2) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    if (warp == 1 && lane == 0) {
+        prefetch_tensormap(&map_x);
+        prefetch_tensormap(&map_y);
+        if (p.r > 0) { prefetch_tensormap(&map_lb); prefetch_tensormap(&map_t); }
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_arrive();          // both CTAs' barriers are in place before anything is sent across
+    cluster_wait();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    const uint32_t tm_a = tmem + 2 * kMaxHalf;
+
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+        if (warp == 0 && lane == 0) {
+            // =================== weight producer ===================
+            uint32_t c = 0;
+            bool ok = true;
+            for (int i = pair; i < p.items && ok; i += pairs) {
+                const Item w = get_item(p, i);
+                if (w.halves == 0) continue;
+                int nb = 2 * w.nt + (int)rank;
+                if (nb >= p.NB) nb = p.NB - 1;         // rows past N: any weights, the results are dropped
+                const uint8_t* src = p.Wk + (size_t)nb * p.KB * kWkBlockBytes;
+                for (int kb = 0; kb < p.KB; kb += kKS, ++c) {
+                    const int nkb = p.KB - kb < kKS ? p.KB - kb : kKS, s = c % kNW;
+                    ok = wait(bar(B_W_FREE + s), ((c / kNW) & 1) ^ 1, stop);
+                    if (!ok) break;
+                    mbar_arrive_expect_tx(bar(B_W_FULL + s), nkb * kWkBlockBytes);
+                    bulk_copy_g2s(sbase + kOffW + s * kWStage, src + (size_t)kb * kWkBlockBytes, nkb * kWkBlockBytes, bar(B_W_FULL + s));
+                }
+            }
+            if (!ok || *stop_flag) let_copies_land();
+        } else if (warp == 1 && lane == 0) {
+            // =================== activation producer ===================
+            grid_dep_wait();       // Xq comes from the kernel launched before this one
+            const uint32_t full0 = map_to_rank(bar(B_FULL), 0);
+            uint32_t c = 0;
+            bool ok = true;
+            for (int i = pair; i < p.items && ok; i += pairs) {
+                const Item w = get_item(p, i);
+                if (w.halves == 0) continue;
+                for (int kb = 0; kb < p.KB; kb += kKS, ++c) {
+                    const uint32_t s = c % kNS;
+                    ok = wait(bar(B_FREE + s), ((c / kNS) & 1) ^ 1, stop);
+                    if (!ok) break;
+                    // both CTAs' bytes are counted on the leader's barrier; blocks past K and tokens past M read as zero
+                    if (rank == 0) mbar_arrive_expect_tx(bar(B_FULL + s), 2 * kKS * p.half * 128);
+                    tma_load_3d_pair(sbase + kOffX + s * kXStage, &map_x, 0, w.tok0 + (int)rank * w.step, kb, full0 + 8u * s);
+                }
+            }
+            if (!ok || *stop_flag) let_copies_land();
+        } else if (warp >= 2 && lane == 0 && rank == 0) {
+            // =================== MMA issuer of one half (leader CTA) ===================
+            const int h = warp - 2;
+            const uint32_t d = tmem + h * kMaxHalf;
+            const uint32_t idesc_i8 = make_idesc(2, 1, 256, p.half), idesc_f16 = make_idesc(1, 0, 256, p.half);
+            const uint32_t xblock = (p.half * 128) >> 4;                 // descriptor step between a stage's blocks
+            const uint32_t xoff = h * (p.half / 2) * 128;
+            uint32_t ca = 0, done = 0, conv = 0;
+            bool ok = true;
+            // the chunks [c0, c1) of the set that occupies the slots
+            auto multiply = [&](int c0, int c1, bool fresh) {
+                tc_fence_after();
+                for (int c = c0; c < c1; ++c) {
+                    const uint64_t ad = smem_desc_sw128(sbase + kOffLr + (c & 1) * kLbBytes);
+                    const uint64_t bd = smem_desc_sw128(sbase + kOffT + (h * 2 + (c & 1)) * kTBytes);
+                    int steps = (p.r - c * 64) / 16;
+                    if (steps > 4) steps = 4;
+                    for (int kk = 0; kk < steps; ++kk)
+                        mma_f16_ss_pair(d, ad + 2 * kk, bd + 2 * kk, idesc_f16, (fresh && c == c0 && kk == 0) ? 0u : 1u);
+                }
+            };
+            for (int i = pair; i < p.items && ok; i += pairs) {
+                const Item w = get_item(p, i);
+                if (w.halves == 0) continue;
+                const bool mine = h < w.halves;
+                if (mine) ok = wait(bar(B_ACC_EMPTY + h), (done & 1) ^ 1, stop);
+                for (int kb = 0; kb < p.KB && ok; kb += kKS, ++ca) {
+                    const int s = ca % kNS;
+                    ok = wait(bar(B_FULL + s), (ca / kNS) & 1, stop);
+                    if (!ok) break;
+                    if (mine) {
+                        const int nkb = p.KB - kb < kKS ? p.KB - kb : kKS;
+                        tc_fence_after();
+                        const uint64_t xdesc = smem_desc_sw128(sbase + kOffX + s * kXStage + xoff);
+                        const uint32_t a = tm_a + s * (kKS * 32);
+#pragma unroll
+                        for (int j = 0; j < kKS; ++j)
+                            if (j < nkb) {
+#pragma unroll
+                                for (int kk = 0; kk < 4; ++kk)
+                                    mma_i8_ts_pair(d, a + j * 32 + kk * 8, xdesc + j * xblock + 2 * kk, idesc_i8,
+                                                   (kb | j | kk) != 0 ? 1u : 0u);
+                            }
+                    }
+                    tc_commit_pair(bar(B_FREE + s));       // a half without tokens only hands the slot on
+                }
+                if (!ok) break;
+                if (mine) {
+                    tc_commit_pair(bar(B_ACC_FULL + h));
+                    if (chunks > 0) {
+                        // the low-rank product into the same columns, once their sums are in registers.  Up to two
+                        // chunks: one set for both halves.  More: the first half multiplies chunks 0, 1 and then
+                        // 2, 3, the second half 2, 3 (still there) and then 0, 1 (loaded again).
+                        ok = wait(bar(B_D_READ + h), done & 1, stop);
+                        const uint32_t first = conv + (chunks > 2 ? h : 0);
+                        ok = ok && wait(bar(B_LR_CONV), first & 1, stop);
+                        if (!ok) break;
+                        if (chunks <= 2) {
+                            multiply(0, chunks, true);
+                        } else {
+                            if (h == 0) multiply(0, 2, true);
+                            else multiply(2, chunks, true);
+                            tc_commit_pair(bar(B_LR_PART));
+                            ok = wait(bar(B_LR_CONV), (first + 1) & 1, stop);
+                            if (!ok) break;
+                            if (h == 0) multiply(2, chunks, false);
+                            else multiply(0, 2, false);
+                        }
+                        tc_commit_pair(bar(B_LR_DONE + h));
+                    }
+                    ++done;
+                }
+                if (chunks > 0) conv += chunks <= 2 ? 1 : 1 + w.halves;      // sets per item
+            }
+        }
+    } else if (warp < 12) {
+        // =================== unpack: int4 -> int8 (x16) into tensor memory ===================
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+        const int q = warp & 3, row = q * 32 + lane, group = (warp - 4) >> 2;
+        const bool leader = (threadIdx.x & 127) == 0;
+        const uint32_t full0 = map_to_rank(bar(B_FULL), 0);
+        int items = 0;
+        for (int i = pair; i < p.items; i += pairs) items += get_item(p, i).halves > 0 ? 1 : 0;
+        const uint32_t total = (uint32_t)items * (uint32_t)stages;
+        // the packed words of this group's next stage are fetched while the MMAs still use its slot
+        uint4 raw[kKS][4];
+        auto fetch = [&](uint32_t c) {
+            const uint32_t s = c % kNW;                     // = group
+            if (!group_wait(bar(B_W_FULL + s), (c / kNW) & 1, stop, leader, group)) return false;
+            const uint8_t* src = smem + kOffW + s * kWStage + row * 16;
+#pragma unroll
+            for (int j = 0; j < kKS; ++j)                   // a ragged stage's second block: whatever is there
+#pragma unroll
+                for (int s4 = 0; s4 < 4; ++s4) raw[j][s4] = *reinterpret_cast<const uint4*>(src + j * kWkBlockBytes + s4 * 2048);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(B_W_FREE + s));
+            return true;
+        };
+        bool ok = (uint32_t)group < total ? fetch(group) : true;
+        for (uint32_t c = group; c < total && ok; c += 2) {
+            const uint32_t s = c % kNS;
+            const uint32_t a = tm_a + s * (kKS * 32) + ((uint32_t)(q * 32) << 16);
+            ok = group_wait(bar(B_FREE + s), ((c / kNS) & 1) ^ 1, stop, leader, group);
+            if (!ok) break;
+            tc_fence_after();
+#pragma unroll
+            for (int j = 0; j < 2 * kKS; ++j) {              // 64 columns at a time
+                uint32_t v[16];
+#pragma unroll
+                for (int s4 = 0; s4 < 2; ++s4) {
+                    const uint4 x = raw[j >> 1][(j & 1) * 2 + s4];
+                    const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        v[s4 * 8 + 2 * e] = (xs[e] << 4) & 0xF0F0F0F0u;      // columns c0 .. c0+3
+                        v[s4 * 8 + 2 * e + 1] = xs[e] & 0xF0F0F0F0u;         // columns c0+4 .. c0+7
+                    }
+                }
+                tmem_st16(a + j * 16, v);
+            }
+            tmem_wait_st();
+            tc_fence_before();
+            if (group == 0) named_bar_sync(3, 128);
+            else named_bar_sync(4, 128);
+            if (leader) mbar_arrive_cluster(full0 + 8u * s);
+            if (c + 2 < total) ok = fetch(c + 2);
+        }
+    } else {
+        // =================== epilogue ===================
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 144;");
+        const int q = warp & 3, side = (warp - 12) >> 2;      // side: the CTA whose tokens this warp's columns are
+        const int et = threadIdx.x - 12 * 32;
+        const int hw = p.half / 2, nch = hw / 16;             // columns per warp and half, in chunks of 16
+        const uint32_t lane_sel = (uint32_t)(q * 32) << 16;
+        const uint32_t dread0 = map_to_rank(bar(B_D_READ), 0), empty0 = map_to_rank(bar(B_ACC_EMPTY), 0),
+                       conv0 = map_to_rank(bar(B_LR_CONV), 0);
+        float* scales = reinterpret_cast<float*>(smem + kOffScale);
+        uint32_t done = 0, sets = 0, parts = 0;               // done: bit h = parity of the half's items
+        bool ok = true;
+        grid_dep_wait();           // a_scale and T come from the kernel launched before this one
+        // a set of low-rank operands: chunks [c0, c1), T of the halves in the mask (one thread)
+        auto load_set = [&](const Item& w, int c0, int c1, int mask) {
+            const int row0 = (2 * w.nt + (int)rank) * 128, layer = cat_layer(p.cat, w.nt * 256) * p.r;
+            mbar_arrive_expect_tx(bar(B_LR_FULL), (c1 - c0) * (kLbBytes + ((mask & 1) + (mask >> 1)) * hw * 128));
+            for (int c = c0; c < c1; ++c) {
+                tma_load_2d(sbase + kOffLr + (c & 1) * kLbBytes, &map_lb, c * 64, row0, bar(B_LR_FULL));
+                for (int h = 0; h < 2; ++h)
+                    if (mask >> h & 1)
+                        tma_load_2d(sbase + kOffT + (h * 2 + (c & 1)) * kTBytes, &map_t, c * 64 + layer,
+                                    w.tok0 + (int)rank * w.step + h * hw, bar(B_LR_FULL));
+            }
+        };
+        // ... of an item's first set
+        auto load_first = [&](const Item& w) {
+            if (chunks <= 2) load_set(w, 0, chunks, w.halves == 2 ? 3 : 1);
+            else load_set(w, 0, 2, 1);
+        };
+        // T of the set just landed: bf16 -> fp16 in place (exact in the fp16 normal range)
+        auto convert_set = [&](int c0, int c1, int mask) {
+            bool landed = true;
+            if (et == 0) landed = wait(bar(B_LR_FULL), sets & 1, stop);
+            ++sets;
+            if (!named_bar_all(1, kEpiThreads, landed)) return false;
+            for (int h = 0; h < 2; ++h) {
+                if (!(mask >> h & 1)) continue;
+                for (int i = et; i < (c1 - c0) * hw * 8; i += kEpiThreads) {
+                    const int c = i >= hw * 8 ? 1 : 0, e = i - c * hw * 8;
+                    uint4* t = reinterpret_cast<uint4*>(smem + kOffT + (h * 2 + c) * kTBytes) + e;
+                    const uint4 raw = *t;
+                    const uint32_t in[4] = {raw.x, raw.y, raw.z, raw.w};
+                    uint32_t out[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const __half2 v = __floats2half2_rn(__uint_as_float(in[k] << 16), __uint_as_float(in[k] & 0xFFFF0000u));
+                        out[k] = *reinterpret_cast<const uint32_t*>(&v);
+                    }
+                    *t = make_uint4(out[0], out[1], out[2], out[3]);
+                }
+            }
+            fence_proxy_async_smem();
+            named_bar_sync(1, kEpiThreads);
+            if (et == 0) mbar_arrive_cluster(conv0);
+            return true;
+        };
+        int i = pair;
+        Item w = {0, 0, 0, 0};
+        while (i < p.items && (w = get_item(p, i)).halves == 0) i += pairs;
+        if (chunks > 0 && i < p.items && et == 0) load_first(w);
+        while (i < p.items && ok) {
+            // the item after this one (its first operands are loaded as soon as their place is free)
+            int i_next = i + pairs;
+            Item next = {0, 0, 0, 0};
+            while (i_next < p.items && (next = get_item(p, i_next)).halves == 0) i_next += pairs;
+            const int n0 = (2 * w.nt + (int)rank) * 128, n = n0 + q * 32 + lane;
+            const float ws16 = (n < p.N ? __ldg(p.w_scale + n) : 0.f) * 0.0625f;      // the sums hold 16 q x
+            {   // token scales in the order of the accumulator's columns: [half][CTA][rows]
+                const int h = et >= p.half ? 1 : 0, col = et - h * p.half, cta = col >= hw ? 1 : 0;
+                const int tok = w.tok0 + cta * w.step + h * hw + (col - cta * hw);
+                if (et < 2 * p.half) scales[et] = (h < w.halves && tok < p.M) ? __ldg(p.a_scale + tok) : 0.f;
+            }
+            if (chunks > 0) ok = convert_set(0, chunks < 2 ? chunks : 2, chunks <= 2 && w.halves == 2 ? 3 : 1);
+            if (!ok) break;
+            uint32_t y[2][4][8];           // fp16 pairs of both halves: stored when both accumulators are free
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (h >= w.halves || !ok) continue;
+                const uint32_t d = tmem + h * kMaxHalf + lane_sel + side * hw;
+                bool full = true;
+                if (lane == 0) full = wait(bar(B_ACC_FULL + h), (done >> h) & 1, stop);
+                ok = named_bar_all(1, kEpiThreads, full);
+                if (!ok) continue;
+                tc_fence_after();
+                uint32_t v[4][16];
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (c < nch) tmem_ld16(d + c * 16, v[c]);
+                tmem_wait_ld_all();
+#pragma unroll
+                for (int c = 0; c < 4; ++c) tmem_use(v[c]);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster((chunks > 0 ? dread0 : empty0) + 8u * h);
+                if (DEBUG_ACC) {
+                    const int tok = w.tok0 + side * w.step + h * hw;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            if (c < nch && tok + c * 16 + j < p.M && n < p.N)
+                                p.acc_debug[(size_t)(tok + c * 16 + j) * p.N + n] = ((int)v[c][j]) >> 4;
+                }
+                if (chunks > 0) {
+                    if (chunks > 2 && (h == 0 || w.halves == 2)) {
+                        // the half's second set
+                        bool free = true;
+                        const int c0 = h == 0 ? 2 : 0, c1 = h == 0 ? chunks : 2, mask = h == 0 ? (w.halves == 2 ? 3 : 1) : 2;
+                        if (et == 0) {
+                            free = wait(bar(B_LR_PART), parts & 1, stop);
+                            if (free) load_set(w, c0, c1, mask);
+                        }
+                        ++parts;
+                        ok = named_bar_all(1, kEpiThreads, free) && convert_set(c0, c1, mask);
+                        if (!ok) continue;
+                    }
+                    bool lr = true;
+                    if (lane == 0) lr = wait(bar(B_LR_DONE + h), (done >> h) & 1, stop);
+                    ok = __shfl_sync(0xffffffffu, lr ? 1 : 0, 0) != 0;
+                    if (!ok) continue;
+                    tc_fence_after();
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    if (c >= nch) continue;
+                    uint32_t f[16];
+                    if (chunks > 0) {
+                        tmem_ld16(d + c * 16, f);
+                        tmem_wait_ld(f);
+                    }
+                    const float4* ap = reinterpret_cast<const float4*>(scales + h * p.half + side * hw + c * 16);
+#pragma unroll
+                    for (int j4 = 0; j4 < 4; ++j4) {
+                        const float4 a4 = ap[j4];
+                        const float as[4] = {a4.x, a4.y, a4.z, a4.w};
+                        float o[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            o[j] = fmaf((float)(int)v[c][4 * j4 + j], as[j] * ws16, chunks > 0 ? __uint_as_float(f[4 * j4 + j]) : 0.f);
+                        const __half2 h0 = __floats2half2_rn(o[0], o[1]), h1 = __floats2half2_rn(o[2], o[3]);
+                        y[h][c][2 * j4] = *reinterpret_cast<const uint32_t*>(&h0);
+                        y[h][c][2 * j4 + 1] = *reinterpret_cast<const uint32_t*>(&h1);
+                    }
+                }
+                if (chunks > 0) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_cluster(empty0 + 8u * h);
+                }
+                done ^= 1u << h;
+            }
+            if (!ok) break;
+            // The outputs, [half][CTA][token][128 channels], are staged where the low-rank operands were: every warp
+            // has seen the item's last low-rank product retire.  They leave as tensor stores, which clip at M and N.
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (h >= w.halves) continue;
+                uint16_t* stage = reinterpret_cast<uint16_t*>(smem + kOffLr) + ((h * 2 + side) * hw) * (kYRow / 2) + q * 32 + lane;
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (c < nch) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            stage[(c * 16 + 2 * j) * (kYRow / 2)] = (uint16_t)(y[h][c][j] & 0xFFFFu);
+                            stage[(c * 16 + 2 * j + 1) * (kYRow / 2)] = (uint16_t)(y[h][c][j] >> 16);
+                        }
+                    }
+            }
+            fence_proxy_async_smem();
+            named_bar_sync(1, kEpiThreads);
+            if (et == 0) {
+                if (n0 < p.N) {
+                    for (int b = 0; b < 2 * w.halves; ++b) {
+                        const int tok = w.tok0 + (b & 1) * w.step + (b >> 1) * hw;
+                        if (tok < p.M) tma_store_2d_tile(&map_y, n0, tok, sbase + kOffLr + b * hw * kYRow);
+                    }
+                    bulk_store_commit();
+                    bulk_store_wait_read();
+                }
+                if (chunks > 0 && i_next < p.items) load_first(next);
+            }
+            if (chunks == 0) named_bar_sync(1, kEpiThreads);      // the staging area has been read
+            w = next;
+            i = i_next;
+        }
+        if (et == 0) {
+            bulk_store_wait_all();
+            if (!ok || *stop_flag) let_copies_land();
+        }
+    }
+
+    // =================== teardown ===================
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    cluster_arrive();          // nothing is sent to a CTA that has left
+    cluster_wait();
+    if (warp == 2) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+    }
+}
+
+struct Plan { int half, NT, TT, full, items; };
+
+// Tokens per half and the deal of the tiles.  Cost of a stage: its MMAs (4 cycles per token of the tile and
+// 128 columns), but no less than the unpacking of its weights; estimated for whole waves of pairs.
+Plan make_plan(int M, int N, int pairs) {
+    Plan best = {};
+    long long best_cost = -1;
+    const int NT = (N + 255) / 256;
+    for (int half = kMaxHalf; half >= 32; half -= 32) {
+        Plan c;
+        c.half = half;
+        c.NT = NT;
+        c.TT = (M + 2 * half - 1) / (2 * half);
+        const int tiles = c.NT * c.TT, rest = tiles % pairs;
+        const bool split = rest > 0 && 2 * rest <= pairs;
+        c.full = split ? tiles - rest : tiles;
+        c.items = split ? c.full + 2 * rest : tiles;
+        auto cost_of = [](int tokens) { return (long long)(tokens > 160 ? tokens : 160); };
+        const long long cost = (long long)((c.full + pairs - 1) / pairs) * cost_of(2 * half) + (split ? cost_of(half) : 0);
+        if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = c; }
+    }
+    return best;
+}
+
+template <bool DEBUG_ACC>
+int configure(int dev) {
+    static bool configured[kMaxDevices] = {false};
+    if (configured[dev]) return ASER_OK;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, linear_pair_kernel<DEBUG_ACC>);
+    if (e != cudaSuccess) return record_cuda_error(e, "linear_pair attributes");
+    // the warpgroups' budgets add up to what the block is launched with, and to nothing else
+    if (a.numRegs != kRegsLaunch) return record_error(ASER_ERR_LAUNCH, "linear_pair: built with an unexpected register count");
+    e = cudaFuncSetAttribute(linear_pair_kernel<DEBUG_ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e != cudaSuccess) return record_cuda_error(e, "linear_pair smem attribute");
+    configured[dev] = true;
+    return ASER_OK;
+}
+
+}  // namespace
+
+bool linear_pair_prefers(int M, int N, int K, int r, const CatSplit& cat) {
+    (void)K; (void)N; (void)r;
+    if (cat.layers > 1 && ((cat.b1 | (cat.layers > 2 ? cat.b2 : 0) | (cat.layers > 3 ? cat.b3 : 0)) & 255)) return false;
+    return M >= kLinearPairMinTokens;
+}
+
+int launch_linear_pair(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const float* w_scale,
+                       const __nv_bfloat16* T, const __half* LB, int M, int N, int K, int r, __half* Y,
+                       int32_t* acc_debug, void* workspace, cudaStream_t st, bool overlap_prev, int ldt, CatSplit cat) {
+    int num_sms = 0, dev = 0;
+    int rc = device_sm_count(&num_sms);
+    if (rc == ASER_OK) rc = current_device(&dev);
+    if (rc == ASER_OK) rc = acc_debug ? configure<true>(dev) : configure<false>(dev);
+    if (rc != ASER_OK) return rc;
+    const int pairs = num_sms / 2 > 0 ? num_sms / 2 : 1;
+    const Plan plan = make_plan(M, N, pairs);
+    CUtensorMap mx, mlb, mt, my;
+    rc = encode_map_2d(&my, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, Y, M, N, plan.half / 2, 128, CU_TENSOR_MAP_SWIZZLE_NONE);
+    if (rc != ASER_OK) return rc;
+    rc = encode_map_blocks(&mx, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Xq, M, K, plan.half, kKS);
+    if (rc != ASER_OK) return rc;
+    if (r > 0) {
+        rc = encode_map_2d(&mlb, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, LB, N, r, 128, 64, CU_TENSOR_MAP_SWIZZLE_128B);
+        if (rc != ASER_OK) return rc;
+        rc = encode_map_2d_ld(&mt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, T, M, r * cat.layers, ldt > 0 ? ldt : r * cat.layers,
+                              plan.half / 2, 64, CU_TENSOR_MAP_SWIZZLE_128B);
+        if (rc != ASER_OK) return rc;
+    } else {
+        mlb = mx;
+        mt = mx;
+    }
+    Params p = {};
+    p.Wk = Wk; p.a_scale = a_scale; p.w_scale = w_scale; p.acc_debug = acc_debug;
+    p.status = static_cast<uint32_t*>(workspace);
+    p.M = M; p.N = N; p.r = r;
+    p.KB = K / kWkCols; p.NB = (N + kWkRows - 1) / kWkRows;
+    p.NT = plan.NT; p.TT = plan.TT; p.half = plan.half; p.full = plan.full; p.items = plan.items;
+    // the smaller of the two operand sets stays in L2 while the other is streamed (as in linear_tc.cu)
+    p.tt_outer = ((long long)M * K > (long long)N * K / 2) ? 1 : 0;
+    p.cat = cat;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * (plan.items < pairs ? plan.items : pairs), 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = overlap_prev ? 2 : 1;
+    const cudaError_t e = acc_debug ? cudaLaunchKernelEx(&cfg, linear_pair_kernel<true>, mx, mlb, mt, my, p)
+                                    : cudaLaunchKernelEx(&cfg, linear_pair_kernel<false>, mx, mlb, mt, my, p);
+    if (e != cudaSuccess) return record_cuda_error(e, "linear_pair_kernel");
+    return check_launch("linear_pair_kernel");
+}
+
+}  // namespace aser

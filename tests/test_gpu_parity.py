@@ -291,6 +291,26 @@ def test_path_parity_small(aser, impl, M, N, K, r):
     run_path(aser, lay, s, Wq, w_scale, L_A, L_B, impl, timed_config=(impl == "tc"))
 
 
+PAIR_CASES = [  # M, N, K, r: the kernel on CTA pairs (256 channels x up to 256 tokens, 256 columns per stage)
+    (192, 8, 128, 16),          # fewest tokens; one column block: half a stage; no second row block
+    (333, 264, 384, 48),        # odd column blocks, ragged channels and tokens
+    (260, 640, 512, 0),         # no low-rank term; odd number of 128-row blocks
+    (700, 1544, 1152, 80),      # two chunks, the second 16 wide
+    (1000, 4104, 256, 144),     # three chunks; whole tiles and a remainder of single halves
+    (513, 768, 640, 256),       # four chunks
+    (2100, 5000, 256, 64),      # more than a wave of whole tiles, then single halves
+]
+
+
+@pytest.mark.parametrize("M,N,K,r", PAIR_CASES)
+def test_pair_kernel_edges(aser, M, N, K, r):
+    lay = synth.make_layer(M, N, K, seed=900 + M + N + K + r, n_cal=16, n_out=max(1, K // 100))
+    s, Wq, w_scale, L_A, L_B = oracle_layer(lay, r, construct=False)
+    if r == 0:
+        L_A = L_B = None
+    run_path(aser, lay, s, Wq, w_scale, L_A, L_B, "tc", timed_config=True, use_dgemm=True)
+
+
 @pytest.mark.parametrize("impl", ["simt", "tc"])
 def test_config1_tiny_with_constructed_factors(aser, impl):
     lay, r = synth.config1_tiny()
