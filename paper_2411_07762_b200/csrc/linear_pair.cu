@@ -88,8 +88,8 @@ struct Params {
     uint32_t* status;
     int M, N, r;
     int KB, NB;            // 128-column blocks, 128-row blocks
-    int NT, TT, half;      // tiles of 256 rows, tiles of 2 half tokens
-    int full, items;       // items [0, full) are whole tiles, the rest single halves, two per tile
+    int NT, TT, half;      // tiles of 256 rows, tiles of 2 half tokens (whole ones; see Plan)
+    int full, cut, items;  // items [0, full): whole tiles; [full, full + 2 cut): the halves of further tiles; then the short ones
     int tt_outer;          // tile numbering: 1 = token tile outer
     CatSplit cat;
 };
@@ -99,17 +99,21 @@ struct Params {
 struct Item { int nt, tok0, halves, step; };
 
 __device__ __forceinline__ Item get_item(const Params& p, int i) {
-    int tile = i, part = 0;
-    const bool single = i >= p.full;
-    if (single) { tile = p.full + ((i - p.full) >> 1); part = (i - p.full) & 1; }
     Item w;
-    int tt;
-    if (p.tt_outer) { tt = tile / p.NT; w.nt = tile - tt * p.NT; }
-    else { w.nt = tile / p.TT; tt = tile - w.nt * p.TT; }
+    int tt, part = 0;
+    bool single = i >= p.full;
+    if (i >= p.full + 2 * p.cut) {          // the last, short column of tokens
+        w.nt = i - p.full - 2 * p.cut;
+        tt = p.TT;
+    } else {
+        int tile = i;
+        if (single) { tile = p.full + ((i - p.full) >> 1); part = (i - p.full) & 1; }
+        if (p.tt_outer) { tt = tile / p.NT; w.nt = tile - tt * p.NT; }
+        else { w.nt = tile / p.TT; tt = tile - w.nt * p.TT; }
+    }
     w.tok0 = (2 * tt + part) * p.half;
-    const int left = p.M - w.tok0;
-    w.halves = left <= 0 ? 0 : (single || left <= p.half) ? 1 : 2;
-    w.step = w.halves == 1 ? p.half / 2 : p.half;
+    w.halves = single ? 1 : 2;
+    w.step = single ? p.half / 2 : p.half;
     return w;
 }
 
@@ -174,6 +178,17 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     const int chunks = (p.r + 63) / 64;
     const int stages = (p.KB + kKS - 1) / kKS;      // per item
 
+    auto weights_of = [&](int item) {
+        int nb = 2 * get_item(p, item).nt + (int)rank;
+        if (nb >= p.NB) nb = p.NB - 1;             // rows past N: any weights, the results are dropped
+        return p.Wk + (size_t)nb * p.KB * kWkBlockBytes;
+    };
+    auto load_weights = [&](const uint8_t* src, int kb, uint32_t s) {
+        const uint32_t bytes = (p.KB - kb < kKS ? p.KB - kb : kKS) * kWkBlockBytes;
+        mbar_arrive_expect_tx(bar(B_W_FULL + s), bytes);
+        bulk_copy_g2s(sbase + kOffW + s * kWStage, src + (size_t)kb * kWkBlockBytes, bytes, bar(B_W_FULL + s));
+    };
+
     if (warp == 0) {
         for (int i = lane; i < kNumBars; i += 32) {
             uint32_t count = 1;
@@ -186,6 +201,11 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         if (lane == 0) *stop_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {           // the first stages of weights leave before tensor memory is there
+            const uint8_t* src = weights_of(pair);
+            for (int c = 0; c < kNW && c < stages; ++c) load_weights(src, c * kKS, c);
+        }
     }
     if (warp == 2) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -212,17 +232,12 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             uint32_t c = 0;
             bool ok = true;
             for (int i = pair; i < p.items && ok; i += pairs) {
-                const Item w = get_item(p, i);
-                if (w.halves == 0) continue;
-                int nb = 2 * w.nt + (int)rank;
-                if (nb >= p.NB) nb = p.NB - 1;         // rows past N: any weights, the results are dropped
-                const uint8_t* src = p.Wk + (size_t)nb * p.KB * kWkBlockBytes;
+                const uint8_t* src = weights_of(i);
                 for (int kb = 0; kb < p.KB; kb += kKS, ++c) {
-                    const int nkb = p.KB - kb < kKS ? p.KB - kb : kKS, s = c % kNW;
-                    ok = wait(bar(B_W_FREE + s), ((c / kNW) & 1) ^ 1, stop);
+                    if (i == pair && kb < kNW * kKS) continue;     // already on its way
+                    ok = wait(bar(B_W_FREE + c % kNW), ((c / kNW) & 1) ^ 1, stop);
                     if (!ok) break;
-                    mbar_arrive_expect_tx(bar(B_W_FULL + s), nkb * kWkBlockBytes);
-                    bulk_copy_g2s(sbase + kOffW + s * kWStage, src + (size_t)kb * kWkBlockBytes, nkb * kWkBlockBytes, bar(B_W_FULL + s));
+                    load_weights(src, kb, c % kNW);
                 }
             }
             if (!ok || *stop_flag) let_copies_land();
@@ -234,7 +249,6 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             bool ok = true;
             for (int i = pair; i < p.items && ok; i += pairs) {
                 const Item w = get_item(p, i);
-                if (w.halves == 0) continue;
                 for (int kb = 0; kb < p.KB; kb += kKS, ++c) {
                     const uint32_t s = c % kNS;
                     ok = wait(bar(B_FREE + s), ((c / kNS) & 1) ^ 1, stop);
@@ -253,7 +267,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             const uint32_t xblock = (p.half * 128) >> 4;                 // descriptor step between a stage's blocks
             const uint32_t xoff = h * (p.half / 2) * 128;
             uint32_t ca = 0, done = 0, conv = 0;
-            bool ok = true;
+            bool ok = true, ready = false;     // ready: stage ca was seen complete already
             // the chunks [c0, c1) of the set that occupies the slots
             auto multiply = [&](int c0, int c1, bool fresh) {
                 tc_fence_after();
@@ -268,26 +282,26 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             };
             for (int i = pair; i < p.items && ok; i += pairs) {
                 const Item w = get_item(p, i);
-                if (w.halves == 0) continue;
                 const bool mine = h < w.halves;
                 if (mine) ok = wait(bar(B_ACC_EMPTY + h), (done & 1) ^ 1, stop);
-                for (int kb = 0; kb < p.KB && ok; kb += kKS, ++ca) {
-                    const int s = ca % kNS;
-                    ok = wait(bar(B_FULL + s), (ca / kNS) & 1, stop);
+                if (!ok) break;
+                for (int kb = 0; kb < p.KB; kb += kKS, ++ca) {
+                    const int s = ca % kNS, s1 = (ca + 1) % kNS;
+                    if (!ready) ok = wait(bar(B_FULL + s), (ca / kNS) & 1, stop);
                     if (!ok) break;
+                    ready = false;
                     if (mine) {
-                        const int nkb = p.KB - kb < kKS ? p.KB - kb : kKS;
                         tc_fence_after();
                         const uint64_t xdesc = smem_desc_sw128(sbase + kOffX + s * kXStage + xoff);
                         const uint32_t a = tm_a + s * (kKS * 32);
+                        if (kb + kKS <= p.KB) {
+                            ready = mma_i8_stage_pair(d, a, xdesc, xblock, idesc_i8, kb != 0 ? 1u : 0u, bar(B_FULL + s1),
+                                                      ((ca + 1) / kNS) & 1);
+                        } else {
 #pragma unroll
-                        for (int j = 0; j < kKS; ++j)
-                            if (j < nkb) {
-#pragma unroll
-                                for (int kk = 0; kk < 4; ++kk)
-                                    mma_i8_ts_pair(d, a + j * 32 + kk * 8, xdesc + j * xblock + 2 * kk, idesc_i8,
-                                                   (kb | j | kk) != 0 ? 1u : 0u);
-                            }
+                            for (int kk = 0; kk < 4; ++kk)
+                                mma_i8_ts_pair(d, a + kk * 8, xdesc + 2 * kk, idesc_i8, (kb | kk) != 0 ? 1u : 0u);
+                        }
                     }
                     tc_commit_pair(bar(B_FREE + s));       // a half without tokens only hands the slot on
                 }
@@ -326,8 +340,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         const int q = warp & 3, row = q * 32 + lane, group = (warp - 4) >> 2;
         const bool leader = (threadIdx.x & 127) == 0;
         const uint32_t full0 = map_to_rank(bar(B_FULL), 0);
-        int items = 0;
-        for (int i = pair; i < p.items; i += pairs) items += get_item(p, i).halves > 0 ? 1 : 0;
+        const int items = (p.items - pair + pairs - 1) / pairs;
         const uint32_t total = (uint32_t)items * (uint32_t)stages;
         // the packed words of this group's next stage are fetched while the MMAs still use its slot
         uint4 raw[kKS][4];
@@ -431,13 +444,13 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         };
         int i = pair;
         Item w = {0, 0, 0, 0};
-        while (i < p.items && (w = get_item(p, i)).halves == 0) i += pairs;
+        if (i < p.items) w = get_item(p, i);
         if (chunks > 0 && i < p.items && et == 0) load_first(w);
         while (i < p.items && ok) {
             // the item after this one (its first operands are loaded as soon as their place is free)
-            int i_next = i + pairs;
+            const int i_next = i + pairs;
             Item next = {0, 0, 0, 0};
-            while (i_next < p.items && (next = get_item(p, i_next)).halves == 0) i_next += pairs;
+            if (i_next < p.items) next = get_item(p, i_next);
             const int n0 = (2 * w.nt + (int)rank) * 128, n = n0 + q * 32 + lane;
             const float ws16 = (n < p.N ? __ldg(p.w_scale + n) : 0.f) * 0.0625f;      // the sums hold 16 q x
             {   // token scales in the order of the accumulator's columns: [half][CTA][rows]
@@ -576,26 +589,40 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     }
 }
 
-struct Plan { int half, NT, TT, full, items; };
+// The deal of the work.  A token column is `whole` when it has more than `half` tokens, at most one is
+// `short`; short columns give single halves.  Items go to the pairs round robin, whole tiles first.
+struct Plan { int half, NT, TT, full, cut, items; };
 
-// Tokens per half and the deal of the tiles.  Cost of a stage: its MMAs (4 cycles per token of the tile and
-// 128 columns), but no less than the unpacking of its weights; estimated for whole waves of pairs.
+// Tokens per half, and whether the tiles of the last, incomplete wave are cut into halves.  The estimate
+// is the load of the busiest pair in cycles per stage of 256 columns: a whole tile takes its MMAs' 8 cycles
+// per token of a half plus about 480 (hand-over; its epilogue spread over 16 stages), a single half 4 and 480,
+// neither less than about 950, which the unpacking takes.
 Plan make_plan(int M, int N, int pairs) {
     Plan best = {};
     long long best_cost = -1;
     const int NT = (N + 255) / 256;
     for (int half = kMaxHalf; half >= 32; half -= 32) {
-        Plan c;
-        c.half = half;
-        c.NT = NT;
-        c.TT = (M + 2 * half - 1) / (2 * half);
-        const int tiles = c.NT * c.TT, rest = tiles % pairs;
-        const bool split = rest > 0 && 2 * rest <= pairs;
-        c.full = split ? tiles - rest : tiles;
-        c.items = split ? c.full + 2 * rest : tiles;
-        auto cost_of = [](int tokens) { return (long long)(tokens > 160 ? tokens : 160); };
-        const long long cost = (long long)((c.full + pairs - 1) / pairs) * cost_of(2 * half) + (split ? cost_of(half) : 0);
-        if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = c; }
+        const int columns = (M + 2 * half - 1) / (2 * half), last = M - (columns - 1) * 2 * half;
+        const bool has_short = last <= half;
+        const int TT = has_short ? columns - 1 : columns, tiles = NT * TT, shorts = has_short ? NT : 0;
+        auto at_least = [](int c) { return (long long)(c > 950 ? c : 950); };
+        const long long whole = at_least(8 * half + 480), single = at_least(4 * half + 480);
+        for (int cut = 0; cut <= 1; ++cut) {
+            Plan c;
+            c.half = half; c.NT = NT; c.TT = TT;
+            c.cut = cut ? tiles % pairs : 0;
+            c.full = tiles - c.cut;
+            c.items = c.full + 2 * c.cut + shorts;
+            // the busiest pair: all have full / pairs whole tiles, the first full % pairs one more; the singles are
+            // dealt on from there
+            const int rest = c.full % pairs, singles = c.items - c.full;
+            const int free_pairs = pairs - rest;                              // pairs without the extra tile
+            const int second = singles > free_pairs ? (singles - free_pairs + pairs - 1) / pairs : 0;
+            const long long with_extra = rest > 0 ? whole + second * single : 0;
+            const long long without = (singles > 0 ? 1 + (singles > pairs ? (singles - 1) / pairs : 0) : 0) * single;
+            const long long cost = (long long)(c.full / pairs) * whole + (with_extra > without ? with_extra : without);
+            if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = c; }
+        }
     }
     return best;
 }
@@ -653,7 +680,7 @@ int launch_linear_pair(const int8_t* Xq, const float* a_scale, const uint8_t* Wk
     p.status = static_cast<uint32_t*>(workspace);
     p.M = M; p.N = N; p.r = r;
     p.KB = K / kWkCols; p.NB = (N + kWkRows - 1) / kWkRows;
-    p.NT = plan.NT; p.TT = plan.TT; p.half = plan.half; p.full = plan.full; p.items = plan.items;
+    p.NT = plan.NT; p.TT = plan.TT; p.half = plan.half; p.full = plan.full; p.cut = plan.cut; p.items = plan.items;
     // the smaller of the two operand sets stays in L2 while the other is streamed (as in linear_tc.cu)
     p.tt_outer = ((long long)M * K > (long long)N * K / 2) ? 1 : 0;
     p.cat = cat;

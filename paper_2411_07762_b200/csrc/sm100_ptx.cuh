@@ -147,6 +147,37 @@ __device__ __forceinline__ void mma_i8_ts_pair(uint32_t d, uint32_t a, uint64_t 
         ::"r"(d), "r"(a), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// The eight products of a stage of two 128-column blocks (A at a, a + 32; B at bdesc, bdesc + bstep; `accumulate`
+// is for the first), with a look at a barrier phase that is issued before them and read after them: a look
+// costs its thread about 300 cycles of latency under copy traffic, here the MMAs are issued meanwhile.
+__device__ __forceinline__ bool mma_i8_stage_pair(uint32_t d, uint32_t a, uint64_t bdesc, uint64_t bstep, uint32_t idesc,
+                                                  uint32_t accumulate, uint32_t bar, uint32_t parity) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred w, p, t;\n\t.reg .b32 x;\n\t.reg .b64 y, z;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 w, [%7], %8;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::i8 [%1], [%2], %3, %5, p;\n\t"
+        "add.u32 x, %2, 8;\n\tadd.u64 y, %3, 2;\n\t"
+        "tcgen05.mma.cta_group::2.kind::i8 [%1], [x], y, %5, t;\n\t"
+        "add.u32 x, %2, 16;\n\tadd.u64 y, %3, 4;\n\t"
+        "tcgen05.mma.cta_group::2.kind::i8 [%1], [x], y, %5, t;\n\t"
+        "add.u32 x, %2, 24;\n\tadd.u64 y, %3, 6;\n\t"
+        "tcgen05.mma.cta_group::2.kind::i8 [%1], [x], y, %5, t;\n\t"
+        "add.u32 x, %2, 32;\n\tadd.u64 z, %3, %4;\n\t"
+        "tcgen05.mma.cta_group::2.kind::i8 [%1], [x], z, %5, t;\n\t"
+        "add.u32 x, %2, 40;\n\tadd.u64 y, z, 2;\n\t"
+        "tcgen05.mma.cta_group::2.kind::i8 [%1], [x], y, %5, t;\n\t"
+        "add.u32 x, %2, 48;\n\tadd.u64 y, z, 4;\n\t"
+        "tcgen05.mma.cta_group::2.kind::i8 [%1], [x], y, %5, t;\n\t"
+        "add.u32 x, %2, 56;\n\tadd.u64 y, z, 6;\n\t"
+        "tcgen05.mma.cta_group::2.kind::i8 [%1], [x], y, %5, t;\n\t"
+        "selp.u32 %0, 1, 0, w;\n\t}"
+        : "=r"(done)
+        : "r"(d), "r"(a), "l"(bdesc), "l"(bstep), "r"(idesc), "r"(accumulate), "r"(bar), "r"(parity)
+        : "memory");
+    return done != 0;
+}
 __device__ __forceinline__ void mma_f16_ss_pair(uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                                 uint32_t accumulate) {
     asm volatile(
@@ -197,6 +228,19 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
           "=r"(v[14]), "=r"(v[15])
         : "r"(taddr)
         : "memory");
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+        : "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld8(uint32_t (&v)[8]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7])
+                 :
+                 : "memory");
 }
 // Waits for all tensor-memory loads of the warp; what they wrote must not be read before it (tie each
 // register array to the wait with tmem_use).
