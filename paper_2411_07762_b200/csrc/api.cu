@@ -118,7 +118,7 @@ int linear_common(const int8_t* Xq, const float* a_scale, const void* Wk, const 
                                     static_cast<const __half*>(LB_f16), M, N, K, r,
                                     static_cast<__half*>(Y_f16), acc_debug,
                                     static_cast<cudaStream_t>(stream), overlap_prev, ldt, cat);
-    if (linear_pair_prefers(M, N, K, r, cat)) {
+    if (linear_pair_prefers(M, N, K, cat)) {
         rc = linear_tc_check(M, N, K, r, workspace_bytes);      // the limits are the same for both kernels
         if (rc != ASER_OK) return rc;
         return launch_linear_pair(Xq, a_scale, static_cast<const uint8_t*>(Wk), w_scale,

@@ -83,11 +83,15 @@ int launch_linear_decode(const int8_t* Xq, const float* a_scale, const uint8_t* 
                          int M, int N, int K, int r, __half* Y, int32_t* acc_debug,
                          cudaStream_t st, bool overlap_prev = false, int ldt = 0, CatSplit cat = CatSplit());
 // Many-token kernel on pairs of CTAs (linear_pair.cu); uses the workspace's status word only.
-constexpr int kLinearPairMinTokens = 192;
-bool linear_pair_prefers(int M, int N, int K, int r, const CatSplit& cat);
+// linear_pair_prefers: the shapes for which it is faster than linear_tc (estimates of both, in cycles).
+constexpr int kLinearPairMinTokens = 65;
+bool linear_pair_prefers(int M, int N, int K, const CatSplit& cat);
 int launch_linear_pair(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const float* w_scale,
                        const __nv_bfloat16* T, const __half* LB, int M, int N, int K, int r, __half* Y,
                        int32_t* acc_debug, void* workspace, cudaStream_t st, bool overlap_prev, int ldt, CatSplit cat);
+// Estimated cycles of launch_linear_tc with 128-token tiles (M > 64): 530 per 128 x 128 x 128 unit of the
+// fullest CTA, and 8000 of fixed cost, or where tiles are shared between CTAs as much as 32 to 64 more units.
+long long linear_tc_estimate(int M, int N, int K, int num_sms);
 size_t linear_tc_workspace_bytes(int M, int N, int K, int r);
 // The range checks launch_linear_tc makes before it launches (workspace size, index widths), for
 // callers that must reject a call before they enqueue anything else.  Records the error text.

@@ -33,10 +33,12 @@
 // partial sums and no workspace beyond the status word.
 // Every wait is bounded: on expiry the CTA sets the status word and winds down.
 //
-// Measured against linear_tc_kernel<128> (tokens x channels x K, rank; us): 2048 x 14336 x 4096, 64: 136 -> 123;
-// 4096 x 14336 x 4096, 128: 271 -> 230; 4096 x 4096 x 14336, 128: 233 -> 178 (2.7 POP/s); 4096 x 28672 x 8192,
-// 256: 1188 -> 896; 1024 x 4096 x 4096, 128: 44 -> 28; 333 x 14336 x 4096, 64: 49 -> 41; 192 x 8192 x 8192, 32:
-// 35 -> 33.
+// Measured against linear_tc_kernel<128> (tokens x channels x K, rank; us): 2048 x 14336 x 4096, 64: 136 -> 112;
+// 4096 x 14336 x 4096, 128: 271 -> 211; 4096 x 4096 x 14336, 128: 233 -> 170 (2.8 POP/s); 4096 x 28672 x 8192,
+// 256: 1188 -> 851; 1024 x 4096 x 4096, 128: 44 -> 27; 333 x 14336 x 4096, 64: 49 -> 37.  A stage takes 1230 cycles
+// against 1024 of MMAs (4096 x 4096 x 14336, rank 0); a tile of K = 4096 pays 5000 more for its turn-around, 11000
+// with a low-rank term.  Sixteen epilogue warps (72 registers at launch) or both halves' sums read at once cost
+// more in spilled registers than they saved there (gate projection 116 -> 122 ... 139 us).
 #include "aser_common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -48,16 +50,16 @@ constexpr int kThreads = 640;                  // five warpgroups
 constexpr int kRegsLaunch = 96;                // per thread at launch: 640 x 96 = 128 x (48 + 2 x 72 + 2 x 144)
 constexpr int kKS = 2;                         // 128-column blocks per stage
 constexpr int kNS = 4, kNW = 2;                // stages of the operand ring (A blocks and activations) and of the weight ring
-constexpr int kMaxHalf = 128;                  // tokens per half, at most
+constexpr int kHalf = 128, kHw = kHalf / 2;    // tokens per half; a CTA holds half of them
 constexpr int kWStage = kKS * kWkBlockBytes;
-constexpr int kXStage = kKS * kMaxHalf * 128;  // a CTA holds half of each half's tokens
-constexpr int kLbBytes = 128 * 128, kTBytes = (kMaxHalf / 2) * 128;
+constexpr int kXStage = kKS * kHalf * 128;  // a CTA holds half of each half's tokens
+constexpr int kLbBytes = 128 * 128, kTBytes = (kHalf / 2) * 128;
 constexpr int kYRow = 256;                     // bytes of a staged output row: 128 channels
 constexpr int kOffX = 0, kOffW = kOffX + kNS * kXStage, kOffLr = kOffW + kNW * kWStage,
               kOffT = kOffLr + 2 * kLbBytes,             // T chunks: [half][slot]
               kOffBar = kOffT + 4 * kTBytes, kOffScale = kOffBar + 256;
-constexpr int kSmemBytes = kOffScale + 2 * kMaxHalf * 4 + 1024;
-static_assert(2 * kMaxHalf * kYRow <= kOffBar - kOffLr, "the outputs of a tile are staged where its low-rank operands were");
+constexpr int kSmemBytes = kOffScale + 2 * kHalf * 4 + 1024;
+static_assert(2 * kHalf * kYRow <= kOffBar - kOffLr, "the outputs of a tile are staged where its low-rank operands were");
 static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
 constexpr long long kWaitClocks = 400000000ll; // about 0.2 s of SM clocks per wait
 
@@ -88,7 +90,7 @@ struct Params {
     uint32_t* status;
     int M, N, r;
     int KB, NB;            // 128-column blocks, 128-row blocks
-    int NT, TT, half;      // tiles of 256 rows, tiles of 2 half tokens (whole ones; see Plan)
+    int NT, TT;            // tiles of 256 rows, whole token columns (see Plan)
     int full, cut, items;  // items [0, full): whole tiles; [full, full + 2 cut): the halves of further tiles; then the short ones
     int tt_outer;          // tile numbering: 1 = token tile outer
     CatSplit cat;
@@ -111,9 +113,9 @@ __device__ __forceinline__ Item get_item(const Params& p, int i) {
         if (p.tt_outer) { tt = tile / p.NT; w.nt = tile - tt * p.NT; }
         else { w.nt = tile / p.TT; tt = tile - w.nt * p.TT; }
     }
-    w.tok0 = (2 * tt + part) * p.half;
+    w.tok0 = (2 * tt + part) * kHalf;
     w.halves = single ? 1 : 2;
-    w.step = single ? p.half / 2 : p.half;
+    w.step = single ? kHw : kHalf;
     return w;
 }
 
@@ -223,7 +225,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     cluster_wait();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const uint32_t tm_a = tmem + 2 * kMaxHalf;
+    const uint32_t tm_a = tmem + 2 * kHalf;
 
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
@@ -254,7 +256,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                     ok = wait(bar(B_FREE + s), ((c / kNS) & 1) ^ 1, stop);
                     if (!ok) break;
                     // both CTAs' bytes are counted on the leader's barrier; blocks past K and tokens past M read as zero
-                    if (rank == 0) mbar_arrive_expect_tx(bar(B_FULL + s), 2 * kKS * p.half * 128);
+                    if (rank == 0) mbar_arrive_expect_tx(bar(B_FULL + s), 2 * kKS * kHalf * 128);
                     tma_load_3d_pair(sbase + kOffX + s * kXStage, &map_x, 0, w.tok0 + (int)rank * w.step, kb, full0 + 8u * s);
                 }
             }
@@ -262,10 +264,10 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         } else if (warp >= 2 && lane == 0 && rank == 0) {
             // =================== MMA issuer of one half (leader CTA) ===================
             const int h = warp - 2;
-            const uint32_t d = tmem + h * kMaxHalf;
-            const uint32_t idesc_i8 = make_idesc(2, 1, 256, p.half), idesc_f16 = make_idesc(1, 0, 256, p.half);
-            const uint32_t xblock = (p.half * 128) >> 4;                 // descriptor step between a stage's blocks
-            const uint32_t xoff = h * (p.half / 2) * 128;
+            const uint32_t d = tmem + h * kHalf;
+            constexpr uint32_t idesc_i8 = make_idesc(2, 1, 256, kHalf), idesc_f16 = make_idesc(1, 0, 256, kHalf);
+            constexpr uint32_t xblock = (kHalf * 128) >> 4;                 // descriptor step between a stage's blocks
+            const uint32_t xoff = h * (kHw) * 128;
             uint32_t ca = 0, done = 0, conv = 0;
             bool ok = true, ready = false;     // ready: stage ca was seen complete already
             // the chunks [c0, c1) of the set that occupies the slots
@@ -390,7 +392,6 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         asm volatile("setmaxnreg.inc.sync.aligned.u32 144;");
         const int q = warp & 3, side = (warp - 12) >> 2;      // side: the CTA whose tokens this warp's columns are
         const int et = threadIdx.x - 12 * 32;
-        const int hw = p.half / 2, nch = hw / 16;             // columns per warp and half, in chunks of 16
         const uint32_t lane_sel = (uint32_t)(q * 32) << 16;
         const uint32_t dread0 = map_to_rank(bar(B_D_READ), 0), empty0 = map_to_rank(bar(B_ACC_EMPTY), 0),
                        conv0 = map_to_rank(bar(B_LR_CONV), 0);
@@ -401,13 +402,13 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         // a set of low-rank operands: chunks [c0, c1), T of the halves in the mask (one thread)
         auto load_set = [&](const Item& w, int c0, int c1, int mask) {
             const int row0 = (2 * w.nt + (int)rank) * 128, layer = cat_layer(p.cat, w.nt * 256) * p.r;
-            mbar_arrive_expect_tx(bar(B_LR_FULL), (c1 - c0) * (kLbBytes + ((mask & 1) + (mask >> 1)) * hw * 128));
+            mbar_arrive_expect_tx(bar(B_LR_FULL), (c1 - c0) * (kLbBytes + ((mask & 1) + (mask >> 1)) * kHw * 128));
             for (int c = c0; c < c1; ++c) {
                 tma_load_2d(sbase + kOffLr + (c & 1) * kLbBytes, &map_lb, c * 64, row0, bar(B_LR_FULL));
                 for (int h = 0; h < 2; ++h)
                     if (mask >> h & 1)
                         tma_load_2d(sbase + kOffT + (h * 2 + (c & 1)) * kTBytes, &map_t, c * 64 + layer,
-                                    w.tok0 + (int)rank * w.step + h * hw, bar(B_LR_FULL));
+                                    w.tok0 + (int)rank * w.step + h * kHw, bar(B_LR_FULL));
             }
         };
         // ... of an item's first set
@@ -423,8 +424,8 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             if (!named_bar_all(1, kEpiThreads, landed)) return false;
             for (int h = 0; h < 2; ++h) {
                 if (!(mask >> h & 1)) continue;
-                for (int i = et; i < (c1 - c0) * hw * 8; i += kEpiThreads) {
-                    const int c = i >= hw * 8 ? 1 : 0, e = i - c * hw * 8;
+                for (int i = et; i < (c1 - c0) * kHw * 8; i += kEpiThreads) {
+                    const int c = i >= kHw * 8 ? 1 : 0, e = i - c * kHw * 8;
                     uint4* t = reinterpret_cast<uint4*>(smem + kOffT + (h * 2 + c) * kTBytes) + e;
                     const uint4 raw = *t;
                     const uint32_t in[4] = {raw.x, raw.y, raw.z, raw.w};
@@ -454,9 +455,9 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             const int n0 = (2 * w.nt + (int)rank) * 128, n = n0 + q * 32 + lane;
             const float ws16 = (n < p.N ? __ldg(p.w_scale + n) : 0.f) * 0.0625f;      // the sums hold 16 q x
             {   // token scales in the order of the accumulator's columns: [half][CTA][rows]
-                const int h = et >= p.half ? 1 : 0, col = et - h * p.half, cta = col >= hw ? 1 : 0;
-                const int tok = w.tok0 + cta * w.step + h * hw + (col - cta * hw);
-                if (et < 2 * p.half) scales[et] = (h < w.halves && tok < p.M) ? __ldg(p.a_scale + tok) : 0.f;
+                const int h = et >= kHalf ? 1 : 0, col = et - h * kHalf, cta = col >= kHw ? 1 : 0;
+                const int tok = w.tok0 + cta * w.step + h * kHw + (col - cta * kHw);
+                if (et < 2 * kHalf) scales[et] = (h < w.halves && tok < p.M) ? __ldg(p.a_scale + tok) : 0.f;
             }
             if (chunks > 0) ok = convert_set(0, chunks < 2 ? chunks : 2, chunks <= 2 && w.halves == 2 ? 3 : 1);
             if (!ok) break;
@@ -464,7 +465,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 if (h >= w.halves || !ok) continue;
-                const uint32_t d = tmem + h * kMaxHalf + lane_sel + side * hw;
+                const uint32_t d = tmem + h * kHalf + lane_sel + side * kHw;
                 bool full = true;
                 if (lane == 0) full = wait(bar(B_ACC_FULL + h), (done >> h) & 1, stop);
                 ok = named_bar_all(1, kEpiThreads, full);
@@ -473,7 +474,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                 uint32_t v[4][16];
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
-                    if (c < nch) tmem_ld16(d + c * 16, v[c]);
+                    tmem_ld16(d + c * 16, v[c]);
                 tmem_wait_ld_all();
 #pragma unroll
                 for (int c = 0; c < 4; ++c) tmem_use(v[c]);
@@ -481,12 +482,12 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster((chunks > 0 ? dread0 : empty0) + 8u * h);
                 if (DEBUG_ACC) {
-                    const int tok = w.tok0 + side * w.step + h * hw;
+                    const int tok = w.tok0 + side * w.step + h * kHw;
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
 #pragma unroll
                         for (int j = 0; j < 16; ++j)
-                            if (c < nch && tok + c * 16 + j < p.M && n < p.N)
+                            if (tok + c * 16 + j < p.M && n < p.N)
                                 p.acc_debug[(size_t)(tok + c * 16 + j) * p.N + n] = ((int)v[c][j]) >> 4;
                 }
                 if (chunks > 0) {
@@ -510,13 +511,12 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                 }
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
-                    if (c >= nch) continue;
                     uint32_t f[16];
                     if (chunks > 0) {
                         tmem_ld16(d + c * 16, f);
                         tmem_wait_ld(f);
                     }
-                    const float4* ap = reinterpret_cast<const float4*>(scales + h * p.half + side * hw + c * 16);
+                    const float4* ap = reinterpret_cast<const float4*>(scales + h * kHalf + side * kHw + c * 16);
 #pragma unroll
                     for (int j4 = 0; j4 < 4; ++j4) {
                         const float4 a4 = ap[j4];
@@ -543,10 +543,10 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 if (h >= w.halves) continue;
-                uint16_t* stage = reinterpret_cast<uint16_t*>(smem + kOffLr) + ((h * 2 + side) * hw) * (kYRow / 2) + q * 32 + lane;
+                uint16_t* stage = reinterpret_cast<uint16_t*>(smem + kOffLr) + ((h * 2 + side) * kHw) * (kYRow / 2) + q * 32 + lane;
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
-                    if (c < nch) {
+                    {
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
                             stage[(c * 16 + 2 * j) * (kYRow / 2)] = (uint16_t)(y[h][c][j] & 0xFFFFu);
@@ -559,8 +559,8 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             if (et == 0) {
                 if (n0 < p.N) {
                     for (int b = 0; b < 2 * w.halves; ++b) {
-                        const int tok = w.tok0 + (b & 1) * w.step + (b >> 1) * hw;
-                        if (tok < p.M) tma_store_2d_tile(&map_y, n0, tok, sbase + kOffLr + b * hw * kYRow);
+                        const int tok = w.tok0 + (b & 1) * w.step + (b >> 1) * kHw;
+                        if (tok < p.M) tma_store_2d_tile(&map_y, n0, tok, sbase + kOffLr + b * kHw * kYRow);
                     }
                     bulk_store_commit();
                     bulk_store_wait_read();
@@ -589,40 +589,32 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     }
 }
 
-// The deal of the work.  A token column is `whole` when it has more than `half` tokens, at most one is
-// `short`; short columns give single halves.  Items go to the pairs round robin, whole tiles first.
-struct Plan { int half, NT, TT, full, cut, items; };
+// The deal of the work.  A column of 256 tokens is whole when it has more than 128, the last may be short:
+// short columns give single halves, and the tiles of the last, incomplete wave may be cut into single
+// halves.  Items go to the pairs round robin, whole tiles first.  The cost is the load of the busiest pair in
+// cycles per stage of 256 columns: 1500 for a whole tile, 1300 for a single half (measured, the epilogue
+// spread over the stages; narrower tiles, bound by the unpacking, cost no less).
+struct Plan { int NT, TT, full, cut, items; long long cost; };
 
-// Tokens per half, and whether the tiles of the last, incomplete wave are cut into halves.  The estimate
-// is the load of the busiest pair in cycles per stage of 256 columns: a whole tile takes its MMAs' 8 cycles
-// per token of a half plus about 480 (hand-over; its epilogue spread over 16 stages), a single half 4 and 480,
-// neither less than about 950, which the unpacking takes.
 Plan make_plan(int M, int N, int pairs) {
+    constexpr long long whole = 1500, single = 1300;
+    const int columns = (M + 2 * kHalf - 1) / (2 * kHalf), last = M - (columns - 1) * 2 * kHalf;
+    const int NT = (N + 255) / 256, TT = last <= kHalf ? columns - 1 : columns, tiles = NT * TT;
+    const int shorts = last <= kHalf ? NT : 0;
     Plan best = {};
-    long long best_cost = -1;
-    const int NT = (N + 255) / 256;
-    for (int half = kMaxHalf; half >= 32; half -= 32) {
-        const int columns = (M + 2 * half - 1) / (2 * half), last = M - (columns - 1) * 2 * half;
-        const bool has_short = last <= half;
-        const int TT = has_short ? columns - 1 : columns, tiles = NT * TT, shorts = has_short ? NT : 0;
-        auto at_least = [](int c) { return (long long)(c > 950 ? c : 950); };
-        const long long whole = at_least(8 * half + 480), single = at_least(4 * half + 480);
-        for (int cut = 0; cut <= 1; ++cut) {
-            Plan c;
-            c.half = half; c.NT = NT; c.TT = TT;
-            c.cut = cut ? tiles % pairs : 0;
-            c.full = tiles - c.cut;
-            c.items = c.full + 2 * c.cut + shorts;
-            // the busiest pair: all have full / pairs whole tiles, the first full % pairs one more; the singles are
-            // dealt on from there
-            const int rest = c.full % pairs, singles = c.items - c.full;
-            const int free_pairs = pairs - rest;                              // pairs without the extra tile
-            const int second = singles > free_pairs ? (singles - free_pairs + pairs - 1) / pairs : 0;
-            const long long with_extra = rest > 0 ? whole + second * single : 0;
-            const long long without = (singles > 0 ? 1 + (singles > pairs ? (singles - 1) / pairs : 0) : 0) * single;
-            const long long cost = (long long)(c.full / pairs) * whole + (with_extra > without ? with_extra : without);
-            if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = c; }
-        }
+    for (int cut = 0; cut <= 1; ++cut) {
+        Plan c;
+        c.NT = NT; c.TT = TT;
+        c.cut = cut ? tiles % pairs : 0;
+        c.full = tiles - c.cut;
+        c.items = c.full + 2 * c.cut + shorts;
+        // all pairs have full / pairs whole tiles, the first full % pairs one more; singles are dealt on from there
+        const int rest = c.full % pairs, singles = c.items - c.full, free_pairs = pairs - rest;
+        const int second = singles > free_pairs ? (singles - free_pairs + pairs - 1) / pairs : 0;
+        const long long with_extra = rest > 0 ? whole + second * single : 0;
+        const long long without = (singles > 0 ? 1 + (singles > pairs ? (singles - 1) / pairs : 0) : 0) * single;
+        c.cost = (long long)(c.full / pairs) * whole + (with_extra > without ? with_extra : without);
+        if (cut == 0 || c.cost < best.cost) best = c;
     }
     return best;
 }
@@ -644,10 +636,17 @@ int configure(int dev) {
 
 }  // namespace
 
-bool linear_pair_prefers(int M, int N, int K, int r, const CatSplit& cat) {
-    (void)K; (void)N; (void)r;
+// The estimates were fitted to whole forward passes (M 48 ... 2048, seven layer shapes): pairs win from about
+// 600 tokens on nearly everywhere and below that where they fill the part or where linear_tc would have to
+// share its tiles (333 x 2048 x 2048: 24 against 38 us, 160 x 8192 x 28672: 81 / 91), linear_tc where few long
+// tiles have to be split over the part (256 x 4096 x 14336: 50 against 60 us), which pairs do not do.
+bool linear_pair_prefers(int M, int N, int K, const CatSplit& cat) {
+    if (M < kLinearPairMinTokens) return false;
     if (cat.layers > 1 && ((cat.b1 | (cat.layers > 2 ? cat.b2 : 0) | (cat.layers > 3 ? cat.b3 : 0)) & 255)) return false;
-    return M >= kLinearPairMinTokens;
+    int num_sms = 0;
+    if (device_sm_count(&num_sms) != ASER_OK || num_sms < 2) return false;
+    const long long stages = (K / kWkCols + kKS - 1) / kKS;
+    return make_plan(M, N, num_sms / 2).cost * stages + 12000 < linear_tc_estimate(M, N, K, num_sms);
 }
 
 int launch_linear_pair(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const float* w_scale,
@@ -661,15 +660,15 @@ int launch_linear_pair(const int8_t* Xq, const float* a_scale, const uint8_t* Wk
     const int pairs = num_sms / 2 > 0 ? num_sms / 2 : 1;
     const Plan plan = make_plan(M, N, pairs);
     CUtensorMap mx, mlb, mt, my;
-    rc = encode_map_2d(&my, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, Y, M, N, plan.half / 2, 128, CU_TENSOR_MAP_SWIZZLE_NONE);
+    rc = encode_map_2d(&my, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, Y, M, N, kHw, 128, CU_TENSOR_MAP_SWIZZLE_NONE);
     if (rc != ASER_OK) return rc;
-    rc = encode_map_blocks(&mx, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Xq, M, K, plan.half, kKS);
+    rc = encode_map_blocks(&mx, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Xq, M, K, kHalf, kKS);
     if (rc != ASER_OK) return rc;
     if (r > 0) {
         rc = encode_map_2d(&mlb, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, LB, N, r, 128, 64, CU_TENSOR_MAP_SWIZZLE_128B);
         if (rc != ASER_OK) return rc;
         rc = encode_map_2d_ld(&mt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, T, M, r * cat.layers, ldt > 0 ? ldt : r * cat.layers,
-                              plan.half / 2, 64, CU_TENSOR_MAP_SWIZZLE_128B);
+                              kHw, 64, CU_TENSOR_MAP_SWIZZLE_128B);
         if (rc != ASER_OK) return rc;
     } else {
         mlb = mx;
@@ -680,7 +679,7 @@ int launch_linear_pair(const int8_t* Xq, const float* a_scale, const uint8_t* Wk
     p.status = static_cast<uint32_t*>(workspace);
     p.M = M; p.N = N; p.r = r;
     p.KB = K / kWkCols; p.NB = (N + kWkRows - 1) / kWkRows;
-    p.NT = plan.NT; p.TT = plan.TT; p.half = plan.half; p.full = plan.full; p.cut = plan.cut; p.items = plan.items;
+    p.NT = plan.NT; p.TT = plan.TT; p.full = plan.full; p.cut = plan.cut; p.items = plan.items;
     // the smaller of the two operand sets stays in L2 while the other is streamed (as in linear_tc.cu)
     p.tt_outer = ((long long)M * K > (long long)N * K / 2) ? 1 : 0;
     p.cat = cat;

@@ -973,6 +973,46 @@ Layout make_layout(int M, int N, int K, int r) {
     return L;
 }
 
+// CTAs of the persistent grid.
+int pick_grid(const Layout& L, int num_sms) {
+    int grid = num_sms < kMaxCtas ? num_sms : kMaxCtas;
+    long long want = (L.units + 1) / 2;   // at least two units per CTA on tiny problems
+    if (want < 1) want = 1;
+    if (grid > want) grid = (int)want;
+    // Tiles that have to be split anyway are split evenly: with a grid that divides the units
+    // into equal shares of a whole fraction of a tile, every CTA has exactly one (partial) work
+    // item instead of up to three, at the price of a few idle SMs.
+    {
+        const long long KBl = L.KB;
+        for (int g = grid; g >= grid - grid / 6 && g >= 1; --g) {
+            if (L.units % g) continue;
+            const long long share = L.units / g;
+            if (share < KBl && KBl % share == 0) { grid = g; break; }
+        }
+        // 128-token tiles: a grid that gives every CTA WHOLE tiles has no shared tile at all.  A
+        // shared 128 x 128 tile costs a 128 KB partial (int32 + fp32) per contributor through the
+        // workspace and a serial tail in the last CTA while the accumulators wait; measured, a
+        // launch with shared tiles pays about as much as 64 more column blocks per CTA (20 us at
+        // K = 4096; about half of that where tiles are long and hide it).  So: the smallest
+        // whole-tile share among the grids down to a third of the SM count, taken if it beats the
+        // split share plus that fee.  Measured at 128 against 148 CTAs: 2 tiles of 32 blocks
+        // -28 %, 8 x 32 -6 %, 14 x 32 -3 %, 4 x 64 -2 %; at 112 CTAs 2 x 64 -27 %; 28 x 32,
+        // 16 x 64 and 4 x 112 are faster split and stay so.
+        if (L.BT == 128) {
+            const long long fee = (KBl <= 64) ? 64 : 32;
+            long long best = (L.units + grid - 1) / grid + fee;
+            int best_g = 0;
+            for (int g = num_sms < kMaxCtas ? num_sms : kMaxCtas; g >= num_sms / 3 && g >= 1; --g) {
+                if (L.units % ((long long)g * KBl)) continue;
+                const long long share = L.units / g;
+                if (share < best) { best = share; best_g = g; }
+            }
+            if (best_g) grid = best_g;
+        }
+    }
+    return grid;
+}
+
 template <int BT, bool MID>
 int launch_bt(const CUtensorMap& mx, const CUtensorMap& mlb, const CUtensorMap& mt, const Params& p,
               int grid, cudaStream_t st, bool overlap_prev) {
@@ -1021,6 +1061,15 @@ int linear_tc_check(int M, int N, int K, int r, size_t workspace_bytes) {
     return ASER_OK;
 }
 
+long long linear_tc_estimate(int M, int N, int K, int num_sms) {
+    const Layout L = make_layout(M, N, K, 0);
+    const int grid = pick_grid(L, num_sms);
+    const bool shared = L.KB > 1 && L.units % ((long long)grid * L.KB) != 0;
+    const long long share = (L.units + grid - 1) / grid;
+    const long long sharing = L.KB < 64 ? 64 : L.KB < 96 ? 56 : 32;     // less where long tiles hide it
+    return 530 * (share + (shared ? sharing : 0)) + (shared ? 0 : 8000);
+}
+
 int launch_linear_tc(const int8_t* Xq, const float* a_scale, const uint8_t* Wk,
                      const float* w_scale, const __nv_bfloat16* T, const __half* LB,
                      int M, int N, int K, int r, __half* Y, int32_t* acc_debug,
@@ -1035,41 +1084,7 @@ int launch_linear_tc(const int8_t* Xq, const float* a_scale, const uint8_t* Wk,
         const int rc = device_sm_count(&num_sms);
         if (rc != ASER_OK) return rc;
     }
-    int grid = num_sms < kMaxCtas ? num_sms : kMaxCtas;
-    long long want = (L.units + 1) / 2;   // at least two units per CTA on tiny problems
-    if (want < 1) want = 1;
-    if (grid > want) grid = (int)want;
-    // Tiles that have to be split anyway are split evenly: with a grid that divides the units
-    // into equal shares of a whole fraction of a tile, every CTA has exactly one (partial) work
-    // item instead of up to three, at the price of a few idle SMs.
-    {
-        const long long KBl = K / 128;
-        for (int g = grid; g >= grid - grid / 6 && g >= 1; --g) {
-            if (L.units % g) continue;
-            const long long share = L.units / g;
-            if (share < KBl && KBl % share == 0) { grid = g; break; }
-        }
-        // 128-token tiles: a grid that gives every CTA WHOLE tiles has no shared tile at all.  A
-        // shared 128 x 128 tile costs a 128 KB partial (int32 + fp32) per contributor through the
-        // workspace and a serial tail in the last CTA while the accumulators wait; measured, a
-        // launch with shared tiles pays about as much as 64 more column blocks per CTA (20 us at
-        // K = 4096; about half of that where tiles are long and hide it).  So: the smallest
-        // whole-tile share among the grids down to a third of the SM count, taken if it beats the
-        // split share plus that fee.  Measured at 128 against 148 CTAs: 2 tiles of 32 blocks
-        // -28 %, 8 x 32 -6 %, 14 x 32 -3 %, 4 x 64 -2 %; at 112 CTAs 2 x 64 -27 %; 28 x 32,
-        // 16 x 64 and 4 x 112 are faster split and stay so.
-        if (L.BT == 128) {
-            const long long fee = (KBl <= 64) ? 64 : 32;
-            long long best = (L.units + grid - 1) / grid + fee;
-            int best_g = 0;
-            for (int g = num_sms < kMaxCtas ? num_sms : kMaxCtas; g >= num_sms / 3 && g >= 1; --g) {
-                if (L.units % ((long long)g * KBl)) continue;
-                const long long share = L.units / g;
-                if (share < best) { best = share; best_g = g; }
-            }
-            if (best_g) grid = best_g;
-        }
-    }
+    const int grid = pick_grid(L, num_sms);
 
     CUtensorMap mx, mlb, mt;
     const int ks = L.BT == 16 ? Cfg<16>::KS : L.BT == 32 ? Cfg<32>::KS : L.BT == 64 ? Cfg<64>::KS : Cfg<128>::KS;

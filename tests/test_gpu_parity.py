@@ -291,14 +291,13 @@ def test_path_parity_small(aser, impl, M, N, K, r):
     run_path(aser, lay, s, Wq, w_scale, L_A, L_B, impl, timed_config=(impl == "tc"))
 
 
-PAIR_CASES = [  # M, N, K, r: the kernel on CTA pairs (256 channels x up to 256 tokens, 256 columns per stage)
-    (192, 8, 128, 16),          # fewest tokens; one column block: half a stage; no second row block
-    (333, 264, 384, 48),        # odd column blocks, ragged channels and tokens
-    (260, 640, 512, 0),         # no low-rank term; odd number of 128-row blocks
-    (700, 1544, 1152, 80),      # two chunks, the second 16 wide
-    (1000, 4104, 256, 144),     # three chunks; whole tiles and a remainder of single halves
-    (513, 768, 640, 256),       # four chunks
-    (2100, 5000, 256, 64),      # more than a wave of whole tiles, then single halves
+PAIR_CASES = [  # M, N, K, r: shapes the kernel on CTA pairs serves (256 channels x 256 tokens, 256 columns per stage)
+    (333, 264, 384, 48),        # odd column blocks (half a stage), ragged channels, a whole and a short token column
+    (260, 640, 512, 0),         # no low-rank term; odd number of 128-row blocks; four tokens in the short column
+    (100, 520, 512, 80),        # a single half; two chunks, the second 16 wide
+    (1300, 2056, 512, 144),     # three chunks; whole tiles, then single halves
+    (513, 768, 640, 256),       # four chunks; tiles cut into single halves; one token in the short column
+    (2100, 4104, 512, 64),      # more than one item per pair: whole, cut and short
 ]
 
 
