@@ -82,12 +82,15 @@ def version() -> int:
     return lib.aser_version()
 
 
+# A pass of a few tokens is shorter on the GPU than its call from Python, so the call is kept lean: addresses
+# and the stream go to ctypes as plain integers (a c_void_p object each and torch.cuda.current_stream()
+# took 6 of the 15 us of a one-token pass).
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _chk(rc: int, where: str):
@@ -374,11 +377,14 @@ class AserLinear:
         M = X.shape[0]
         assert M <= self.max_tokens
         r = self.r if lowrank else 0       # the plain W4A8 control: the same entry point at rank 0
-        _chk(lib.aser_forward(_ptr(X), _ptr(self.s), _ptr(self.L_A) if r else None, _ptr(self.Wk),
-                              _ptr(self.w_scale), _ptr(self.L_B) if r else None, M, self.N, self.K, r,
-                              _ptr(self.Xq), _ptr(self.a_scale), _ptr(self.T) if r else None,
-                              _ptr(self.Y), _ptr(self.ws), self.ws.numel(), _stream()), "aser_forward")
-        return self.Y[:M]
+        s, Y, ws = self.s, self.Y, self.ws
+        rc = lib.aser_forward(X.data_ptr(), None if s is None else s.data_ptr(), self.L_A.data_ptr() if r else None,
+                              self.Wk.data_ptr(), self.w_scale.data_ptr(), self.L_B.data_ptr() if r else None,
+                              M, self.N, self.K, r, self.Xq.data_ptr(), self.a_scale.data_ptr(),
+                              self.T.data_ptr() if r else None, Y.data_ptr(), ws.data_ptr(), ws.numel(), _stream())
+        if rc != 0:
+            raise AserError(rc, "aser_forward")
+        return Y.narrow(0, 0, M)
 
     def forward_host(self, X_host: torch.Tensor, Y_host: torch.Tensor):
         """Host fp16 X [M,K] (pinned) -> host fp16 Y [M,N] through aser_forward_host."""
@@ -437,12 +443,11 @@ class AserSharedInput:
         """Returns the layers' outputs [M, N_l] (views of preallocated buffers)."""
         M = X.shape[0]
         assert M <= self.max_tokens
-        T = self.T if M == self.max_tokens else self.T[:M]
         _chk(lib.aser_forward_shared(_ptr(X), _ptr(self.s), _ptr(self.L_A), self.n, self._Wk, self._ws,
                                      self._LB, self._N, self._r, M, self.K, _ptr(self.Xq),
                                      _ptr(self.a_scale), _ptr(self.T) if self.r_total else None, self._Y,
                                      _ptr(self.ws), self.ws.numel(), _stream()), "aser_forward_shared")
-        return [y[:M] for y in self.Y]
+        return [y.narrow(0, 0, M) for y in self.Y]
 
 
 
@@ -473,7 +478,7 @@ class AserSharedInputCat(AserSharedInput):
     def _views(self, M: int):
         out, col = [], 0
         for n in self.N:
-            out.append(self.Y_cat[:M, col:col + n])
+            out.append((self.Y_cat if M == self.max_tokens else self.Y_cat[:M]).narrow(1, col, n))
             col += n
         return out
 

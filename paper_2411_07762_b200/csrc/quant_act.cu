@@ -43,96 +43,159 @@ __device__ __forceinline__ uint2 quant8(const float (&v)[8], float sc, bool nonz
 // ---------------------------------------------------------------------------
 // few tokens
 // ---------------------------------------------------------------------------
-constexpr int kSmallThreads = 256;
 constexpr int kRowsPerCta = 4;  // L_A rows handled by one projection CTA
 
-// grid = (1 + ceil(r / kRowsPerCta), M).  blockIdx.x == 0 quantizes token blockIdx.y,
-// the others compute kRowsPerCta entries of T for that token.
-// dynamic smem: K floats (the smoothed row; used by the quantizing CTA).
-__global__ void __launch_bounds__(kSmallThreads)
+// CTAs 0 .. M - 1 quantize one token each, the others compute kRowsPerCta entries of T for TOK tokens.
+// What bounds it is the chain of loads: launch, one round trip per batch of chunks, a reduction.  So a thread
+// has at most CPT 8-column chunks of a row (TH threads by the row length), the quantizing CTA keeps them in
+// registers, and a projection CTA uses the L_A chunks it loads for TOK tokens (one token per CTA read L_A
+// from L2 M times: 16 tokens x 384 rows 10.9 us; K = 14336 took 9.1 us at one token because 256 threads went
+// through seven dependent rounds).
+template <int TH, int CPT, int TOK>
+__global__ void __launch_bounds__(TH)
 quant_act_small_kernel(const __half* __restrict__ X, const float* __restrict__ s,
                        const __half* __restrict__ LA, int M, int K, int r,
                        int8_t* __restrict__ Xq, float* __restrict__ a_scale,
                        __nv_bfloat16* __restrict__ T, int ldt, int lo_off, float qmax) {
-    extern __shared__ __align__(16) float xs[];
-    grid_dep_launch();      // a dependent linear kernel may start streaming its weights
-    __shared__ float red[kRowsPerCta][kSmallThreads / 32];
-    const int m = blockIdx.y;
-    const int chunks = K / 8;
-    const __half* row = X + (size_t)m * K;
+    constexpr int kWarps = TH / 32;
+    // Launched as a programmatic dependent of whatever precedes it on the stream.  The wait comes first: a
+    // dependent linear kernel may start streaming its weights only when everything before this kernel is done.
+    grid_dep_wait();
+    grid_dep_launch();
+    __shared__ float red[kRowsPerCta * TOK][kWarps];
+    const int chunks = K / 8, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    if (blockIdx.x == 0) {
-        // ---- quantize this token: x~ to shared memory with the row maximum, then the codes ----
-        float amax = 0.f;
-        for (int c = threadIdx.x; c < chunks; c += kSmallThreads) {
-            RawChunk rc = load_raw(row, s, c * 8, true);
-            float v[8];
-            smooth8(rc, v);
+    if ((int)blockIdx.x < M) {
+        // ---- quantize a token: x~ in registers, the row maximum, the codes ----
+        const int m = blockIdx.x;
+        const __half* row = X + (size_t)m * K;
+        RawChunk rc[CPT];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) amax = fmaxf(amax, fabsf(v[i]));
-            *reinterpret_cast<float4*>(xs + c * 8) = make_float4(v[0], v[1], v[2], v[3]);
-            *reinterpret_cast<float4*>(xs + c * 8 + 4) = make_float4(v[4], v[5], v[6], v[7]);
+        for (int i = 0; i < CPT; ++i) {
+            const int c = threadIdx.x + i * TH;
+            if (c < chunks) rc[i] = load_raw(row, s, c * 8, true);
+        }
+        float v[CPT][8], amax = 0.f;
+#pragma unroll
+        for (int i = 0; i < CPT; ++i) {
+            if ((int)threadIdx.x + i * TH >= chunks) continue;
+            smooth8(rc[i], v[i]);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) amax = fmaxf(amax, fabsf(v[i][e]));
         }
         amax = warp_max(amax);
-        if ((threadIdx.x & 31) == 0) red[0][threadIdx.x >> 5] = amax;
+        if (lane == 0) red[0][warp] = amax;
         __syncthreads();
         amax = red[0][0];
 #pragma unroll
-        for (int i = 1; i < kSmallThreads / 32; ++i) amax = fmaxf(amax, red[0][i]);
+        for (int i = 1; i < kWarps; ++i) amax = fmaxf(amax, red[0][i]);
         const float sc = __fdiv_rn(amax, qmax);
         if (threadIdx.x == 0) a_scale[m] = sc;
         int8_t* out = Xq + (size_t)m * K;
-        for (int c = threadIdx.x; c < chunks; c += kSmallThreads) {
-            float v[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = xs[c * 8 + i];
-            *reinterpret_cast<uint2*>(out + c * 8) = quant8(v, sc, amax > 0.f, qmax);
+        for (int i = 0; i < CPT; ++i) {
+            const int c = threadIdx.x + i * TH;
+            if (c < chunks) *reinterpret_cast<uint2*>(out + c * 8) = quant8(v[i], sc, amax > 0.f, qmax);
         }
         return;
     }
 
-    // ---- down projection: kRowsPerCta rows of L_A against the smoothed token.  A thread
+    // ---- down projection: kRowsPerCta rows of L_A against TOK smoothed tokens.  A thread
     // smooths the chunks it multiplies, so all of its loads (activations, divisors, L_A rows)
     // are in flight together and no barrier separates them. ----
-    const int j0 = (blockIdx.x - 1) * kRowsPerCta;
-    float acc[kRowsPerCta];
+    const int groups = (r + kRowsPerCta - 1) / kRowsPerCta, idx = (int)blockIdx.x - M;
+    const int j0 = (idx % groups) * kRowsPerCta, m0 = (idx / groups) * TOK;
+    float acc[kRowsPerCta][TOK];
 #pragma unroll
-    for (int jj = 0; jj < kRowsPerCta; ++jj) acc[jj] = 0.f;
+    for (int jj = 0; jj < kRowsPerCta; ++jj)
+#pragma unroll
+        for (int k = 0; k < TOK; ++k) acc[jj][k] = 0.f;
 #pragma unroll 2
-    for (int c = threadIdx.x; c < chunks; c += kSmallThreads) {
-        const RawChunk rc = load_raw(row, s, c * 8, true);
+    for (int c = threadIdx.x; c < chunks; c += TH) {
+        RawChunk rc[TOK];
+        rc[0] = load_raw(X + (size_t)m0 * K, s, c * 8, true);
+#pragma unroll
+        for (int k = 1; k < TOK; ++k) {
+            rc[k].s0 = rc[0].s0; rc[k].s1 = rc[0].s1;
+            rc[k].x = m0 + k < M ? *reinterpret_cast<const uint4*>(X + (size_t)(m0 + k) * K + c * 8) : make_uint4(0, 0, 0, 0);
+        }
         uint4 la[kRowsPerCta];
 #pragma unroll
         for (int jj = 0; jj < kRowsPerCta; ++jj)
             la[jj] = (j0 + jj < r) ? *reinterpret_cast<const uint4*>(LA + (size_t)(j0 + jj) * K + c * 8)
                                    : make_uint4(0, 0, 0, 0);
-        float v[8];
-        smooth8(rc, v);
+        // Reciprocals of the divisors, once for all tokens (T is a sum of fp32 products: one rounding more or
+        // less of a factor is not what limits it; the codes below a scale are divided).
+        const float sv[8] = {rc[0].s0.x, rc[0].s0.y, rc[0].s0.z, rc[0].s0.w, rc[0].s1.x, rc[0].s1.y, rc[0].s1.z, rc[0].s1.w};
+        float inv[8];
+        bool ones = true;
 #pragma unroll
-        for (int jj = 0; jj < kRowsPerCta; ++jj) {
-            const __half2* h2 = reinterpret_cast<const __half2*>(&la[jj]);
-            const float2 a = __half22float2(h2[0]), b = __half22float2(h2[1]);
-            const float2 cc = __half22float2(h2[2]), d = __half22float2(h2[3]);
-            float t = acc[jj];
-            t = fmaf(a.x, v[0], t); t = fmaf(a.y, v[1], t);
-            t = fmaf(b.x, v[2], t); t = fmaf(b.y, v[3], t);
-            t = fmaf(cc.x, v[4], t); t = fmaf(cc.y, v[5], t);
-            t = fmaf(d.x, v[6], t); t = fmaf(d.y, v[7], t);
-            acc[jj] = t;
+        for (int i = 0; i < 8; ++i) { ones = ones && sv[i] == 1.f; inv[i] = 1.f; }
+        if (!ones) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) inv[i] = __frcp_rn(sv[i]);
+        }
+#pragma unroll
+        for (int k = 0; k < TOK; ++k) {
+            const __half2* xh = reinterpret_cast<const __half2*>(&rc[k].x);
+            float v[8];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 x2 = __half22float2(xh[i]);
+                v[2 * i] = x2.x * inv[2 * i]; v[2 * i + 1] = x2.y * inv[2 * i + 1];
+            }
+#pragma unroll
+            for (int jj = 0; jj < kRowsPerCta; ++jj) {
+                const __half2* h2 = reinterpret_cast<const __half2*>(&la[jj]);
+                float t = acc[jj][k];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float2 a = __half22float2(h2[i]);
+                    t = fmaf(a.x, v[2 * i], t); t = fmaf(a.y, v[2 * i + 1], t);
+                }
+                acc[jj][k] = t;
+            }
         }
     }
 #pragma unroll
-    for (int jj = 0; jj < kRowsPerCta; ++jj) {
-        float t = warp_sum(acc[jj]);
-        if ((threadIdx.x & 31) == 0) red[jj][threadIdx.x >> 5] = t;
-    }
+    for (int jj = 0; jj < kRowsPerCta; ++jj)
+#pragma unroll
+        for (int k = 0; k < TOK; ++k) {
+            const float t = warp_sum(acc[jj][k]);
+            if (lane == 0) red[jj * TOK + k][warp] = t;
+        }
     __syncthreads();
-    if (threadIdx.x < kRowsPerCta && j0 + threadIdx.x < r) {
+    if (threadIdx.x < kRowsPerCta * TOK) {
+        const int j = j0 + (int)threadIdx.x / TOK, m = m0 + (int)threadIdx.x % TOK;
         float t = 0.f;
 #pragma unroll
-        for (int i = 0; i < kSmallThreads / 32; ++i) t += red[threadIdx.x][i];
-        store_t(T + (size_t)m * ldt, j0 + threadIdx.x, t, lo_off);
+        for (int i = 0; i < kWarps; ++i) t += red[threadIdx.x][i];
+        if (j < r && m < M) store_t(T + (size_t)m * ldt, j, t, lo_off);
     }
+}
+
+template <int TH, int CPT>
+int launch_small(const __half* X, const float* s, const __half* LA, int M, int K, int r, int8_t* Xq, float* a_scale,
+                 __nv_bfloat16* T, int ldt, int lo_off, float qmax, cudaStream_t st) {
+    // tokens per projection CTA: as many as leave about a CTA for every SM
+    const int groups = (r + kRowsPerCta - 1) / kRowsPerCta;
+    auto ctas = [&](int tok) { return groups * ((M + tok - 1) / tok); };
+    const int tok = (M > 2 && ctas(4) >= 128) ? 4 : (M > 1 && ctas(2) >= 128) ? 2 : 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(M + ctas(tok), 1, 1);
+    cfg.blockDim = dim3(TH, 1, 1);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e;
+    if (tok == 4) e = cudaLaunchKernelEx(&cfg, quant_act_small_kernel<TH, CPT, 4>, X, s, LA, M, K, r, Xq, a_scale, T, ldt, lo_off, qmax);
+    else if (tok == 2) e = cudaLaunchKernelEx(&cfg, quant_act_small_kernel<TH, CPT, 2>, X, s, LA, M, K, r, Xq, a_scale, T, ldt, lo_off, qmax);
+    else e = cudaLaunchKernelEx(&cfg, quant_act_small_kernel<TH, CPT, 1>, X, s, LA, M, K, r, Xq, a_scale, T, ldt, lo_off, qmax);
+    if (e != cudaSuccess) return record_cuda_error(e, "quant_act_small_kernel");
+    return check_launch("quant_act_small_kernel");
 }
 
 // ---------------------------------------------------------------------------
@@ -1116,20 +1179,11 @@ int launch_quant_act(const __half* X, const float* s, const __half* LA, int M, i
     if (M == 0) return ASER_OK;
     const int ldt = t_pair ? 2 * r : r, lo_off = t_pair ? r : 0;
     if (M <= 32) {
-        size_t smem = (size_t)K * sizeof(float);
-        static size_t configured[kMaxDevices] = {0};   // beyond the 48 KiB every kernel may use
-        int dev = 0;
-        const int drc = current_device(&dev);
-        if (drc != ASER_OK) return drc;
-        if (smem > 48 * 1024 && smem > configured[dev]) {
-            cudaError_t e = cudaFuncSetAttribute(quant_act_small_kernel,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return record_cuda_error(e, "quant_act_small smem attribute");
-            configured[dev] = smem;
-        }
-        dim3 grid(1 + (r + kRowsPerCta - 1) / kRowsPerCta, M);
-        quant_act_small_kernel<<<grid, kSmallThreads, smem, st>>>(X, s, LA, M, K, r, Xq, a_scale, T, ldt, lo_off, qmax);
-        return check_launch("quant_act_small_kernel");
+        // threads by the row length: two chunks of eight columns each up to 8192, then four and eight (K <= 32768)
+        if (K <= 4096) return launch_small<256, 2>(X, s, LA, M, K, r, Xq, a_scale, T, ldt, lo_off, qmax, st);
+        if (K <= 8192) return launch_small<512, 2>(X, s, LA, M, K, r, Xq, a_scale, T, ldt, lo_off, qmax, st);
+        if (K <= 16384) return launch_small<512, 4>(X, s, LA, M, K, r, Xq, a_scale, T, ldt, lo_off, qmax, st);
+        return launch_small<512, 8>(X, s, LA, M, K, r, Xq, a_scale, T, ldt, lo_off, qmax, st);
     }
     bool unsupported = false;
     if (r > kTMaxRank && r <= 2 * kTMaxRank) {
