@@ -94,6 +94,8 @@ act_proj_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     const int la_box_rows = r / la_boxes;
     const uint32_t la_stage_bytes = (uint32_t)r * 128u;
     extern __shared__ uint8_t smem_raw[];
+    // a programmatic dependent of whatever precedes it; what depends on it starts only after its wait
+    grid_dep_wait();
     grid_dep_launch();
     const uint32_t sraw = smem_u32(smem_raw);
     const uint32_t sb = (sraw + 1023u) & ~1023u;
@@ -646,17 +648,22 @@ int launch_quant_act_ws(const __half* X, const float* s, const __half* LA, int M
     for (int m_first = 0; m_first < M; m_first += plan.Mc) {
         const int Mc = (M - m_first < plan.Mc) ? (M - m_first) : plan.Mc;
         const int tiles = (Mc + kPTok - 1) / kPTok;
-        act_proj_kernel<<<dim3(plan.KS, tiles, 1), kPThreads, smem, st>>>(mx, mla, s, m_first, Mc, K, Kc, r,
-                                                                          amax_part, t_part);
-        rc = check_launch("act_proj_kernel");
-        if (rc != ASER_OK) return rc;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t pcfg = {};
+        pcfg.gridDim = dim3(plan.KS, tiles, 1);
+        pcfg.blockDim = dim3(kPThreads, 1, 1);
+        pcfg.dynamicSmemBytes = smem;
+        pcfg.stream = st;
+        pcfg.attrs = attr;
+        pcfg.numAttrs = 1;
+        cudaError_t pe = cudaLaunchKernelEx(&pcfg, act_proj_kernel, mx, mla, s, m_first, Mc, K, Kc, r, amax_part, t_part);
+        if (pe != cudaSuccess) return record_cuda_error(pe, "act_proj_kernel");
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((Mc + kQRows - 1) / kQRows, 1, 1);
         cfg.blockDim = dim3(256, 1, 1);
         cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         cudaError_t e = cudaLaunchKernelEx(&cfg, act_quant_kernel, X, s, m_first, Mc, K, r, plan.KS,

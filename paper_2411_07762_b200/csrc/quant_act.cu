@@ -562,7 +562,10 @@ quant_act_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
                      int M, int K, int Kc, int r, int CK, float* __restrict__ a_scale,
                      __nv_bfloat16* __restrict__ T, int ldt, int lo_off, float qmax) {
     extern __shared__ uint8_t smem_raw[];
-    grid_dep_launch();      // a dependent linear kernel may start streaming its weights
+    // a programmatic dependent of whatever precedes it; a dependent linear kernel may start streaming its weights
+    // only after the wait
+    grid_dep_wait();
+    grid_dep_launch();
     const uint32_t sraw = smem_u32(smem_raw);
     const uint32_t sb = (sraw + 1023u) & ~1023u;            // swizzled tiles need 1 KiB alignment
     uint8_t* smem = smem_raw + (sb - sraw);
@@ -1137,13 +1140,15 @@ int launch_tma(const __half* X, const float* s, const __half* LA, int M, int K, 
     cfg.blockDim = dim3(kTThreads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = ck;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     cudaError_t e = cudaLaunchKernelEx(&cfg, quant_act_tma_kernel, mx, mla, mq, s, M, K, kc, r, ck, a_scale, T, ldt, lo_off, qmax);
     if (e != cudaSuccess) return record_cuda_error(e, "quant_act_tma_kernel");
     return check_launch("quant_act_tma_kernel");
