@@ -302,7 +302,9 @@ int aser_forward_shared_cat(const void* X_f16, const float* s, const void* LA_st
  * ideally pinned) to the device staging buffer X_dev, runs aser_forward, and copies Y back to Y_host,
  * all enqueued on `stream`; returns without synchronising.  Device-side operands and
  * staging buffers are the caller's.  All arguments are checked before the first copy is
- * enqueued.
+ * enqueued.  With pinned buffers and 256 tokens or more the pass is cut into up to four parts of tokens
+ * whose copies run on streams of the library's own (a few per calling thread), begun behind `stream` and
+ * joined to it at the end; each part is an aser_forward of its own.
  */
 int aser_forward_host(const void* X_host_f16, void* Y_host_f16,
                       void* X_dev, int8_t* Xq_dev, float* a_scale_dev, void* T_dev, void* Y_dev,

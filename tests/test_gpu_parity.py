@@ -715,3 +715,58 @@ def test_quant_act_bits_rejects_other_widths(aser):
         with pytest.raises(aser.AserError) as err:
             aser.quant_act(X, None, None, act_bits=bad)
         assert err.value.code == -3
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M", [200, 256, 333, 700, 1030])
+def test_forward_host_in_parts(aser, M):
+    """Pinned buffers: one part below 256 tokens, then two to four parts of whole 128-token groups with a ragged
+    last one; pageable buffers take the undivided path.  Both against the oracle, and again on two streams in turn
+    and from two threads at once (each with a layer of its own)."""
+    import threading
+    N, K, r = 264, 512, 32
+    lay = synth.make_layer(M, N, K, seed=1200 + M, n_cal=8)
+    s, Wq, w_scale, L_A, L_B = oracle_layer(lay, r, construct=False)
+    ref = F.forward(lay.X, s, Wq, w_scale, L_A, L_B, use_dgemm=True)
+    X = torch.from_numpy(lay.X.copy())
+
+    def make():
+        return (aser.AserLinear(to_dev(lay.W), to_dev(s), to_dev(L_A), to_dev(L_B), M), X.pin_memory(),
+                torch.zeros((M, N), dtype=torch.float16).pin_memory())
+
+    layer, X_pin, Y_pin = make()
+    torch.cuda.synchronize()
+    layer.forward_host(X_pin, Y_pin)
+    torch.cuda.current_stream().synchronize()
+    assert_rows_close(Y_pin.numpy(), ref.y)
+    Y_page = torch.zeros((M, N), dtype=torch.float16)
+    layer.forward_host(X, Y_page)
+    torch.cuda.current_stream().synchronize()
+    assert_rows_close(Y_page.numpy(), ref.y)
+
+    sets = [make(), make()]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for _ in range(3):
+        for st, (l, x, y) in zip(streams, sets):
+            with torch.cuda.stream(st):
+                l.forward_host(x, y)
+    for st in streams:
+        st.synchronize()
+    for _, _, y in sets:
+        assert_rows_close(y.numpy(), ref.y)
+        y.zero_()
+
+    def work(st, l, x, y):
+        with torch.cuda.stream(st):
+            for _ in range(5):
+                l.forward_host(x, y)
+            st.synchronize()
+    threads = [threading.Thread(target=work, args=(st, *t)) for st, t in zip(streams, sets)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for l, _, y in sets:
+        assert_rows_close(y.numpy(), ref.y)
+        aser.check_status(l.ws)
