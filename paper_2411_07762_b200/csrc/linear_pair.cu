@@ -314,9 +314,12 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                         // the low-rank product into the same columns, once their sums are in registers.  Up to two
                         // chunks: one set for both halves.  More: the first half multiplies chunks 0, 1 and then
                         // 2, 3, the second half 2, 3 (still there) and then 0, 1 (loaded again).
-                        ok = wait(bar(B_D_READ + h), done & 1, stop);
                         const uint32_t first = conv + (chunks > 2 ? h : 0);
-                        ok = ok && wait(bar(B_LR_CONV), first & 1, stop);
+                        // one set: converted long ago, so it is looked at while the epilogue reads the sums.  (With more
+                        // sets a half skips phases of LR_CONV, and only D_READ says that those are over.)
+                        if (chunks <= 2) ok = wait(bar(B_LR_CONV), first & 1, stop);
+                        ok = ok && wait(bar(B_D_READ + h), done & 1, stop);
+                        if (chunks > 2) ok = ok && wait(bar(B_LR_CONV), first & 1, stop);
                         if (!ok) break;
                         if (chunks <= 2) {
                             multiply(0, chunks, true);
