@@ -311,32 +311,28 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                 if (mine) {
                     tc_commit_pair(bar(B_ACC_FULL + h));
                     if (chunks > 0) {
-                        // the low-rank product into the same columns, once their sums are in registers.  Up to two
-                        // chunks: one set for both halves.  More: the first half multiplies chunks 0, 1 and then
-                        // 2, 3, the second half 2, 3 (still there) and then 0, 1 (loaded again).
-                        const uint32_t first = conv + (chunks > 2 ? h : 0);
+                        // The low-rank product into the same columns, once their sums are in registers.  Up to two chunks
+                        // are one set for both halves; more are two sets for each half in turn, so that every half
+                        // adds its chunks in order (the same sums as linear_tc.cu, whichever kernel serves a shape).
+                        const uint32_t first = conv + (chunks > 2 ? 2 * h : 0);
                         // one set: converted long ago, so it is looked at while the epilogue reads the sums.  (With more
                         // sets a half skips phases of LR_CONV, and only D_READ says that those are over.)
                         if (chunks <= 2) ok = wait(bar(B_LR_CONV), first & 1, stop);
                         ok = ok && wait(bar(B_D_READ + h), done & 1, stop);
                         if (chunks > 2) ok = ok && wait(bar(B_LR_CONV), first & 1, stop);
                         if (!ok) break;
-                        if (chunks <= 2) {
-                            multiply(0, chunks, true);
-                        } else {
-                            if (h == 0) multiply(0, 2, true);
-                            else multiply(2, chunks, true);
+                        multiply(0, chunks < 2 ? chunks : 2, true);
+                        if (chunks > 2) {
                             tc_commit_pair(bar(B_LR_PART));
                             ok = wait(bar(B_LR_CONV), (first + 1) & 1, stop);
                             if (!ok) break;
-                            if (h == 0) multiply(2, chunks, false);
-                            else multiply(0, 2, false);
+                            multiply(2, chunks, false);
                         }
                         tc_commit_pair(bar(B_LR_DONE + h));
                     }
                     ++done;
                 }
-                if (chunks > 0) conv += chunks <= 2 ? 1 : 1 + w.halves;      // sets per item
+                if (chunks > 0) conv += chunks <= 2 ? 1 : 2 * w.halves;      // sets per item
             }
         }
     } else if (warp < 12) {
@@ -469,6 +465,8 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             for (int h = 0; h < 2; ++h) {
                 if (h >= w.halves || !ok) continue;
                 const uint32_t d = tmem + h * kHalf + lane_sel + side * kHw;
+                if (h == 1 && chunks > 2) ok = convert_set(0, 2, 2);
+                if (!ok) continue;
                 bool full = true;
                 if (lane == 0) full = wait(bar(B_ACC_FULL + h), (done >> h) & 1, stop);
                 ok = named_bar_all(1, kEpiThreads, full);
@@ -494,16 +492,15 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                                 p.acc_debug[(size_t)(tok + c * 16 + j) * p.N + n] = ((int)v[c][j]) >> 4;
                 }
                 if (chunks > 0) {
-                    if (chunks > 2 && (h == 0 || w.halves == 2)) {
+                    if (chunks > 2) {
                         // the half's second set
                         bool free = true;
-                        const int c0 = h == 0 ? 2 : 0, c1 = h == 0 ? chunks : 2, mask = h == 0 ? (w.halves == 2 ? 3 : 1) : 2;
                         if (et == 0) {
                             free = wait(bar(B_LR_PART), parts & 1, stop);
-                            if (free) load_set(w, c0, c1, mask);
+                            if (free) load_set(w, 2, chunks, 1 << h);
                         }
                         ++parts;
-                        ok = named_bar_all(1, kEpiThreads, free) && convert_set(c0, c1, mask);
+                        ok = named_bar_all(1, kEpiThreads, free) && convert_set(2, chunks, 1 << h);
                         if (!ok) continue;
                     }
                     bool lr = true;
@@ -511,6 +508,8 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                     ok = __shfl_sync(0xffffffffu, lr ? 1 : 0, 0) != 0;
                     if (!ok) continue;
                     tc_fence_after();
+                    // the first half is through: the second half's first set
+                    if (chunks > 2 && h == 0 && w.halves == 2 && et == 0) load_set(w, 0, 2, 2);
                 }
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {

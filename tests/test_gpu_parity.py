@@ -770,3 +770,31 @@ def test_forward_host_in_parts(aser, M):
     for l, _, y in sets:
         assert_rows_close(y.numpy(), ref.y)
         aser.check_status(l.ws)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("r", [128, 192])
+def test_fused_group_is_bit_identical_across_the_two_tensor_core_kernels(aser, r):
+    """1024 tokens, K = 4096, two layers of 2048 channels: the fused launch (4096 channels) is served by CTA pairs,
+    a layer alone by the kernel that may share tiles.  Both add the low-rank chunks in order, so the bits agree."""
+    import ctypes as C
+    M, K, N = 1024, 4096, 2048
+    g = torch.Generator(device="cuda")
+    g.manual_seed(77 + r)
+    Xq = torch.randint(-127, 128, (M, K), device="cuda", dtype=torch.int8, generator=g)
+    a = torch.rand(M, device="cuda", generator=g) * 1e-3
+    T = torch.randn(M, 2 * r, device="cuda", generator=g).bfloat16()
+    packed = [aser.pack_w4(torch.randn(N, K, device="cuda", generator=g).half(), None) for _ in range(2)]
+    Wk = [aser.repack_w4(w) for w, _ in packed]
+    LB = [torch.randn(N, r, device="cuda", generator=g).half() * 0.1 for _ in range(2)]
+    ws = aser.new_workspace(M, 2 * N, K, r)
+    Y = torch.empty((M, 2 * N), device="cuda", dtype=torch.float16)
+    wk, sc, lb = torch.cat(Wk), torch.cat([s for _, s in packed]), torch.cat(LB).contiguous()
+    P = lambda t: C.c_void_p(t.data_ptr())
+    rc = aser.lib.aser_linear_w4a8_lr_cat(P(Xq), P(a), P(wk), P(sc), P(T), P(lb), 2, (C.c_int * 2)(N, N), r, M, K, P(Y),
+                                          P(ws), ws.numel(), C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert rc == 0
+    for i in range(2):
+        y = aser.linear_w4a8_lr_ld(Xq, a, Wk[i], packed[i][1], T, i * r, LB[i], N, ws)
+        assert torch.equal(Y[:, i * N:(i + 1) * N], y)
+    aser.check_status(ws)
