@@ -140,15 +140,16 @@ bool act_shape_ok(int M, int K, int r) {
 
 // Which activation kernels a forward pass runs.  The two-kernel path with scratch reads X once
 // from HBM whatever the rank; it is the only one above rank 128 (stacked down projections of a
-// shared-input group) and the faster one from about a thousand tokens on (measured at rank 128,
-// two-kernel against cluster kernel: 1024 x 4096 21 against 27 us, 4096 x 4096 34 against 42 us,
-// 2048 x 14336 52 against 65 us, 4096 x 14336 95 against 134 us, 8192 x 8192 107 against 159 us).
-// Below that the one-launch cluster kernel is faster (256 x 4096: 23 against 17 us), and up to 32
-// tokens the few-token kernel serves every rank.
+// shared-input group).  The one-launch cluster kernel reads X twice (the second time from L2) and has one
+// launch less of fixed cost.  Measured at rank 128, cluster against two-kernel path: 400 x 4096 11.4 / 13.6 us, 512 x
+// 4096 14.9 / 14.0, 1000 x 4096 23 / 16, 400 x 14336 22.5 / 22.5, 512 x 14336 35 / 25, 1000 x 14336 63 / 30, 4096 x 14336
+// 125 / 83; rows of 1024 columns 9.1 / 11.3 at 512 tokens and still 16.3 / 16.8 at 4096.  Up to 32 tokens the few-token
+// kernel serves every rank.
 bool forward_act_uses_scratch(int M, int K, int r) {
     if (M <= 32) return false;
     if (r > 128) return true;
-    (void)K;
+    if (K >= 4096) return M >= 448;
+    if (K <= 1024) return M > 4096;
     return M >= 1024;
 }
 
