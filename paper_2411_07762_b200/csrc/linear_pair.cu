@@ -459,58 +459,63 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                 if (et < 2 * kHalf) scales[et] = (h < w.halves && tok < p.M) ? __ldg(p.a_scale + tok) : 0.f;
             }
             if (chunks > 0) ok = convert_set(0, chunks < 2 ? chunks : 2, chunks <= 2 && w.halves == 2 ? 3 : 1);
+            else named_bar_sync(1, kEpiThreads);          // the scales are there
             if (!ok) break;
             uint32_t y[2][4][8];           // fp16 pairs of both halves: stored when both accumulators are free
+            // A warp whose wait gave up does no more work but still takes part in every barrier of the item, which
+            // ends with all warps going on or giving up together.
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                if (h >= w.halves || !ok) continue;
+                if (h >= w.halves) continue;
                 const uint32_t d = tmem + h * kHalf + lane_sel + side * kHw;
-                if (h == 1 && chunks > 2) ok = convert_set(0, 2, 2);
-                if (!ok) continue;
-                bool full = true;
-                if (lane == 0) full = wait(bar(B_ACC_FULL + h), (done >> h) & 1, stop);
-                ok = named_bar_all(1, kEpiThreads, full);
-                if (!ok) continue;
-                tc_fence_after();
-                uint32_t v[4][16];
-#pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    tmem_ld16(d + c * 16, v[c]);
-                tmem_wait_ld_all();
-#pragma unroll
-                for (int c = 0; c < 4; ++c) tmem_use(v[c]);
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive_cluster((chunks > 0 ? dread0 : empty0) + 8u * h);
-                if (DEBUG_ACC) {
-                    const int tok = w.tok0 + side * w.step + h * kHw;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c)
-#pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            if (tok + c * 16 + j < p.M && n < p.N)
-                                p.acc_debug[(size_t)(tok + c * 16 + j) * p.N + n] = ((int)v[c][j]) >> 4;
+                if (h == 1 && chunks > 2) {
+                    const bool converted = convert_set(0, 2, 2);
+                    ok = ok && converted;
                 }
-                if (chunks > 0) {
-                    if (chunks > 2) {
-                        // the half's second set
-                        bool free = true;
-                        if (et == 0) {
-                            free = wait(bar(B_LR_PART), parts & 1, stop);
-                            if (free) load_set(w, 2, chunks, 1 << h);
-                        }
-                        ++parts;
-                        ok = named_bar_all(1, kEpiThreads, free) && convert_set(2, chunks, 1 << h);
-                        if (!ok) continue;
+                if (ok) {
+                    if (lane == 0) ok = wait(bar(B_ACC_FULL + h), (done >> h) & 1, stop);
+                    ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                }
+                uint32_t v[4][16];
+                if (ok) {
+                    tc_fence_after();
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) tmem_ld16(d + c * 16, v[c]);
+                    tmem_wait_ld_all();
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) tmem_use(v[c]);
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_cluster((chunks > 0 ? dread0 : empty0) + 8u * h);
+                    if (DEBUG_ACC) {
+                        const int tok = w.tok0 + side * w.step + h * kHw;
+#pragma unroll
+                        for (int c = 0; c < 4; ++c)
+#pragma unroll
+                            for (int j = 0; j < 16; ++j)
+                                if (tok + c * 16 + j < p.M && n < p.N)
+                                    p.acc_debug[(size_t)(tok + c * 16 + j) * p.N + n] = ((int)v[c][j]) >> 4;
                     }
-                    bool lr = true;
-                    if (lane == 0) lr = wait(bar(B_LR_DONE + h), (done >> h) & 1, stop);
-                    ok = __shfl_sync(0xffffffffu, lr ? 1 : 0, 0) != 0;
-                    if (!ok) continue;
+                }
+                if (chunks > 2) {
+                    // the half's second set
+                    bool free = ok;
+                    if (et == 0 && free) {
+                        free = wait(bar(B_LR_PART), parts & 1, stop);
+                        if (free) load_set(w, 2, chunks, 1 << h);
+                    }
+                    ++parts;
+                    ok = named_bar_all(1, kEpiThreads, free);
+                    if (ok) ok = convert_set(2, chunks, 1 << h);
+                }
+                if (chunks > 0 && ok) {
+                    if (lane == 0) ok = wait(bar(B_LR_DONE + h), (done >> h) & 1, stop);
+                    ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
                     tc_fence_after();
                     // the first half is through: the second half's first set
-                    if (chunks > 2 && h == 0 && w.halves == 2 && et == 0) load_set(w, 0, 2, 2);
+                    if (ok && chunks > 2 && h == 0 && w.halves == 2 && et == 0) load_set(w, 0, 2, 2);
                 }
+                if (!ok) continue;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     uint32_t f[16];
@@ -539,25 +544,23 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                 }
                 done ^= 1u << h;
             }
-            if (!ok) break;
             // The outputs, [half][CTA][token][128 channels], are staged where the low-rank operands were: every warp
             // has seen the item's last low-rank product retire.  They leave as tensor stores, which clip at M and N.
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                if (h >= w.halves) continue;
+                if (h >= w.halves || !ok) continue;
                 uint16_t* stage = reinterpret_cast<uint16_t*>(smem + kOffLr) + ((h * 2 + side) * kHw) * (kYRow / 2) + q * 32 + lane;
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
-                    {
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            stage[(c * 16 + 2 * j) * (kYRow / 2)] = (uint16_t)(y[h][c][j] & 0xFFFFu);
-                            stage[(c * 16 + 2 * j + 1) * (kYRow / 2)] = (uint16_t)(y[h][c][j] >> 16);
-                        }
+                    for (int j = 0; j < 8; ++j) {
+                        stage[(c * 16 + 2 * j) * (kYRow / 2)] = (uint16_t)(y[h][c][j] & 0xFFFFu);
+                        stage[(c * 16 + 2 * j + 1) * (kYRow / 2)] = (uint16_t)(y[h][c][j] >> 16);
                     }
             }
             fence_proxy_async_smem();
-            named_bar_sync(1, kEpiThreads);
+            ok = named_bar_all(1, kEpiThreads, ok);
+            if (!ok) break;
             if (et == 0) {
                 if (n0 < p.N) {
                     for (int b = 0; b < 2 * w.halves; ++b) {
