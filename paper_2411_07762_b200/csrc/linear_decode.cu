@@ -186,35 +186,23 @@ linear_decode_kernel(const int8_t* Xq, const float* a_scale, const uint8_t* __re
         x_ok[nt] = g + 8 * nt < M;
         xrow[nt] = Xq + (size_t)(x_ok[nt] ? g + 8 * nt : 0) * K + t * 32;
     }
-    // Up to eight tokens the fragment of the next block is loaded before this block's products (it comes from
-    // L2 on its first use by an SM): 8192 x 8192, one token 10.6 -> 9.9 us.  With sixteen the second
-    // fragment does not fit the registers (12.8 -> 19 us).
-    constexpr bool kAhead = NT == 1;
-    auto load_x = [&](int kbi, uint32_t (&b)[NT][8]) {
+    for (int kb0 = warp; kb0 < KB; kb0 += kDecWarps * BATCH) {
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-            uint4 lo = make_uint4(0, 0, 0, 0), hi = make_uint4(0, 0, 0, 0);
-            if (x_ok[nt] && kbi < KB) {
-                const uint4* xp = reinterpret_cast<const uint4*>(xrow[nt] + kbi * kWkCols);
-                lo = xp[0];
-                hi = xp[1];
-            }
-            b[nt][0] = lo.x; b[nt][1] = lo.y; b[nt][2] = lo.z; b[nt][3] = lo.w;
-            b[nt][4] = hi.x; b[nt][5] = hi.y; b[nt][6] = hi.z; b[nt][7] = hi.w;
-        }
-    };
-    uint32_t bx[kAhead ? 2 : 1][NT][8];
-    if (kAhead) load_x(warp, bx[0]);
-    constexpr int UNROLL = BATCH % 2 ? 2 : 1;          // the two fragments alternate: an even number of blocks per turn
-    for (int kb0 = warp; kb0 < KB; kb0 += kDecWarps * BATCH * UNROLL) {
-#pragma unroll
-        for (int iu = 0; iu < BATCH * UNROLL; ++iu) {
-            const int i = iu % BATCH;
-            const int kbi = kb0 + iu * kDecWarps;
+        for (int i = 0; i < BATCH; ++i) {
+            const int kbi = kb0 + i * kDecWarps;
             if (kbi < KB) {
-                uint32_t (&b)[NT][8] = bx[kAhead ? iu & 1 : 0];
-                if (kAhead) load_x(kbi + kDecWarps, bx[kAhead ? (iu + 1) & 1 : 0]);
-                else load_x(kbi, b);
+                uint32_t b[NT][8];
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt) {
+                    uint4 lo = make_uint4(0, 0, 0, 0), hi = make_uint4(0, 0, 0, 0);
+                    if (x_ok[nt]) {
+                        const uint4* xp = reinterpret_cast<const uint4*>(xrow[nt] + kbi * kWkCols);
+                        lo = xp[0];
+                        hi = xp[1];
+                    }
+                    b[nt][0] = lo.x; b[nt][1] = lo.y; b[nt][2] = lo.z; b[nt][3] = lo.w;
+                    b[nt][4] = hi.x; b[nt][5] = hi.y; b[nt][6] = hi.z; b[nt][7] = hi.w;
+                }
                 const int kbn = kbi + kDecWarps * BATCH;
 #pragma unroll
                 for (int rt = 0; rt < R; ++rt) {
@@ -316,9 +304,11 @@ int launch_nt(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const f
         if (rc != ASER_OK) return rc;
     }
     // (Four blocks in flight per warp at 32 rows, i.e. 256 bytes per thread and two CTAs per SM,
-    // measured 7 % slower at 8192 x 8192 than two blocks and three CTAs per SM.)  Where the tiles are a few too
-    // many for three CTAs per SM, four with half the bytes in flight each take them in one wave (14336 x 4096:
-    // 448 tiles for 444 places, 12.9 -> 8.8 us at one token, 12.6 -> 10.2 at eight).
+    // measured 7 % slower at 8192 x 8192 than two blocks and three CTAs per SM.  Loading the next block's
+    // activation fragment ahead made the kernel alone up to 8 % faster and a whole step of 4096 x 4096 9 % slower:
+    // its first load is then two deep behind the dependency wait.)  Up to eight tokens, where the tiles are a few
+    // too many for three CTAs per SM, four with half the bytes in flight each take them in one wave (14336 x 4096:
+    // 448 tiles for 444 places; a step of eight tokens 14.5 -> 12.9 us).
     const int tiles = (N + 31) / 32;
     if (NT == 1 && tiles > 3 * num_sms && tiles <= 4 * num_sms)
         return launch_cfg<1, 2, 1>(Xq, a_scale, Wk, w_scale, T, LB, M, N, K, r, Y, acc_debug, st, overlap_prev, ldt, cat);
