@@ -304,7 +304,8 @@ int aser_forward_shared_cat(const void* X_f16, const float* s, const void* LA_st
  * staging buffers are the caller's.  All arguments are checked before the first copy is
  * enqueued.  With pinned buffers and 256 tokens or more the pass is cut into up to four parts of tokens
  * whose copies run on streams of the library's own (a few per calling thread), begun behind `stream` and
- * joined to it at the end; each part is an aser_forward of its own.
+ * joined to it at the end; each part is an aser_forward of its own.  A thread whose last passes went to three
+ * streams or more overlaps them itself: its passes are not cut.
  */
 int aser_forward_host(const void* X_host_f16, void* Y_host_f16,
                       void* X_dev, int8_t* Xq_dev, float* a_scale_dev, void* T_dev, void* Y_dev,
