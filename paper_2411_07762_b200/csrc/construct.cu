@@ -523,7 +523,9 @@ __global__ void identity_kernel(double* __restrict__ V, int p) {
 }
 
 // The r longest rows of G [p, p] in descending order (equal ones by index): their norms to sigma
-// and sigma_out, the matching rows of V to Vsel [r, p].  One CTA, p <= 512.
+// and sigma_out, the matching rows of V to Vsel [r, p].  One CTA, p <= 512.  Weights or tokens with NaN or
+// infinity make norms that are NaN; those rank behind every number, so that the ranks are a permutation
+// and every index read below has been written (the call then reports the failed factorisation).
 __global__ void __launch_bounds__(512)
 select_top_kernel(const double* __restrict__ G, const double* __restrict__ V, int p, int r, double* __restrict__ Vsel,
                   double* __restrict__ sigma, double* __restrict__ sigma_out) {
@@ -534,7 +536,7 @@ select_top_kernel(const double* __restrict__ G, const double* __restrict__ V, in
         double s = 0.0;
         for (int k = lane; k < p; k += 32) s = fma(G[(long long)i * p + k], G[(long long)i * p + k], s);
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) norm[i] = s;
+        if (lane == 0) norm[i] = s >= 0.0 ? s : -1.0;
     }
     __syncthreads();
     for (int i = threadIdx.x; i < p; i += 512) {

@@ -131,3 +131,17 @@ def test_construct_without_the_whitening_factor(aser, N, K, r, n_cal):
     with pytest.raises(aser.AserError) as err:
         aser.construct(to_dev(lay.W), to_dev(s), torch.zeros_like(to_dev(lay.X_cal)), r)
     assert err.value.code == -3
+
+
+@pytest.mark.parametrize("where", ["W nan", "W inf", "X nan", "s nan"])
+def test_construct_reports_operands_that_are_not_numbers(aser, where):
+    """Every norm of the decomposition is NaN then: the call ends with the error of a failed factorisation, and the
+    order of the singular values is still a permutation (no index is left unwritten)."""
+    lay = synth.make_layer(4, 384, 512, seed=77, n_cal=64)
+    ops = dict(W=lay.W.copy(), s=np.ones(512, np.float32), X=lay.X_cal.copy())
+    name, value = where.split()
+    ops[name].flat[5] = float(value)
+    for damping in (0.01, 1e-8):            # without the whitening factor, and through it
+        with pytest.raises(aser.AserError) as err:
+            aser.construct(to_dev(ops["W"]), to_dev(ops["s"]), to_dev(ops["X"]), 32, damping=damping)
+        assert err.value.code == -3
