@@ -110,6 +110,7 @@ quant_act_small_kernel(const __half* __restrict__ X, const float* __restrict__ s
     for (int jj = 0; jj < kRowsPerCta; ++jj)
 #pragma unroll
         for (int k = 0; k < TOK; ++k) acc[jj][k] = 0.f;
+    bool far = false;           // a divisor so far from 1 that the parts of its reciprocal may leave the normal range
 #pragma unroll 2
     for (int c = threadIdx.x; c < chunks; c += TH) {
         RawChunk rc[TOK];
@@ -124,16 +125,25 @@ quant_act_small_kernel(const __half* __restrict__ X, const float* __restrict__ s
         for (int jj = 0; jj < kRowsPerCta; ++jj)
             la[jj] = (j0 + jj < r) ? *reinterpret_cast<const uint4*>(LA + (size_t)(j0 + jj) * K + c * 8)
                                    : make_uint4(0, 0, 0, 0);
-        // Reciprocals of the divisors, once for all tokens (T is a sum of fp32 products: one rounding more or
-        // less of a factor is not what limits it; the codes below a scale are divided).
+        // x~ = fp32(x) / s as for the codes, without a division per token: the reciprocal of a divisor as two numbers
+        // (the first truncated, so the remainder has its sign and an infinite x stays infinite), once for all tokens;
+        // x * high + x * low is rounded once and differs from the quotient only where that lies within 2^-20 of a
+        // unit in the last place from a tie.  A remainder of zero is replaced by one that no sum sees.
         const float sv[8] = {rc[0].s0.x, rc[0].s0.y, rc[0].s0.z, rc[0].s0.w, rc[0].s1.x, rc[0].s1.y, rc[0].s1.z, rc[0].s1.w};
-        float inv[8];
+        constexpr float kUnseen = 0x1p-40f;
+        float inv[8], low[8];
         bool ones = true;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) { ones = ones && sv[i] == 1.f; inv[i] = 1.f; }
+        for (int i = 0; i < 8; ++i) { ones = ones && sv[i] == 1.f; inv[i] = 1.f; low[i] = kUnseen; }
         if (!ones) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) inv[i] = __frcp_rn(sv[i]);
+            for (int i = 0; i < 8; ++i) {
+                const float a = fabsf(sv[i]);
+                far = far || !(a > 0x1p-80f && a < 0x1p80f);
+                inv[i] = __frcp_rz(sv[i]);
+                const float rem = fmaf(-sv[i], inv[i], 1.f);
+                low[i] = inv[i] * (rem > 0.f ? rem : kUnseen);
+            }
         }
 #pragma unroll
         for (int k = 0; k < TOK; ++k) {
@@ -142,7 +152,9 @@ quant_act_small_kernel(const __half* __restrict__ X, const float* __restrict__ s
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const float2 x2 = __half22float2(xh[i]);
-                v[2 * i] = x2.x * inv[2 * i]; v[2 * i + 1] = x2.y * inv[2 * i + 1];
+                const float2 v2 = __ffma2_rn(x2, make_float2(inv[2 * i], inv[2 * i + 1]),
+                                             __fmul2_rn(x2, make_float2(low[2 * i], low[2 * i + 1])));
+                v[2 * i] = v2.x; v[2 * i + 1] = v2.y;
             }
 #pragma unroll
             for (int jj = 0; jj < kRowsPerCta; ++jj) {
@@ -154,6 +166,21 @@ quant_act_small_kernel(const __half* __restrict__ X, const float* __restrict__ s
                     t = fmaf(a.x, v[2 * i], t); t = fmaf(a.y, v[2 * i + 1], t);
                 }
                 acc[jj][k] = t;
+            }
+        }
+    }
+    if (far) {                  // the thread's sums once more, every column divided
+#pragma unroll
+        for (int k = 0; k < TOK; ++k) {
+#pragma unroll
+            for (int jj = 0; jj < kRowsPerCta; ++jj) acc[jj][k] = 0.f;
+            if (m0 + k >= M) continue;
+            const __half* row = X + (size_t)(m0 + k) * K;
+            for (int col = threadIdx.x * 8; col < K; col += (col & 7) == 7 ? TH * 8 - 7 : 1) {
+                const float v = __fdiv_rn(__half2float(row[col]), __ldg(s + col));
+#pragma unroll
+                for (int jj = 0; jj < kRowsPerCta; ++jj)
+                    if (j0 + jj < r) acc[jj][k] = fmaf(__half2float(LA[(size_t)(j0 + jj) * K + col]), v, acc[jj][k]);
             }
         }
     }

@@ -136,6 +136,27 @@ def test_quant_act_dense_smoothing_vector(aser, M, K, r):
     assert_T_close(T.float().cpu().numpy(), F.down_proj(xs, L_A), xs, L_A)
 
 
+@pytest.mark.parametrize("M,r", [(1, 32), (3, 256), (7, 256)])       # one, two and four tokens per projection CTA
+@pytest.mark.parametrize("K", [512, 8320])
+def test_quant_act_few_tokens_extreme_divisors(aser, M, r, K):
+    """Divisors whose reciprocal is infinite (below 2^-128) or subnormal (above 2^126), with zeros and
+    the smallest activations against them: x~ is the quotient, for the codes and for T alike."""
+    lay = synth.make_layer(M, 8, K, seed=450 + M + r, n_cal=8)
+    s = np.ones(K, np.float32)
+    X = lay.X.copy()
+    s[3], s[70], s[300], s[301] = 1e-40, 1e-40, 3e38, 7.0
+    X[:, 3] = 0
+    X[:, 70] = np.where(np.arange(M) % 2, 0, 2.0 ** -24).astype(np.float16)
+    L_A = synth.standin_factors(8, K, r, seed=M, scale_a=0.05)[0]
+    xs = F.smooth_act(X, s)
+    assert np.isfinite(xs).all()
+    Xq_ref, sc_ref = F.quant_act(xs)
+    Xq, sc, T = aser.quant_act(to_dev(X), to_dev(s), to_dev(L_A))
+    assert np.array_equal(Xq.cpu().numpy(), Xq_ref)
+    assert np.array_equal(bits(sc.cpu().numpy()), bits(sc_ref))
+    assert_T_close(T.float().cpu().numpy(), F.down_proj(xs, L_A), xs, L_A)
+
+
 @pytest.mark.parametrize("path,M,K,r", [("cluster", 4096, 4096, 64), ("ws", 4800, 8192, 16)])
 def test_quant_act_dense_smoothing_long_slices(aser, path, M, K, r):
     """Every divisor differs from 1 on slices long enough that a CTA meets more units with a
