@@ -242,8 +242,19 @@ CopyLane* copy_lane(cudaStream_t st) {
     return &l;
 }
 
-int host_parts(const void* X_host, const void* Y_host, int M, cudaStream_t st) {
+bool overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + b_bytes && y < x + a_bytes;
+}
+
+int host_parts(const void* X_host, const void* Y_host, const void* X_dev, const void* Y_dev, int M, int N, int K,
+               cudaStream_t st) {
     if (M < 256) return 1;
+    // Y in the place of X (on either side) asks for all of X to be read before the first of Y is written, unless each
+    // row of Y takes the place of its own row of X
+    const size_t x_bytes = (size_t)M * K * 2, y_bytes = (size_t)M * N * 2;
+    if (overlap(X_host, x_bytes, Y_host, y_bytes) && !(X_host == Y_host && N == K)) return 1;
+    if (overlap(X_dev, x_bytes, Y_dev, y_bytes) && !(X_dev == Y_dev && N == K)) return 1;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { cudaGetLastError(); return 1; }
     if (cap != cudaStreamCaptureStatusNone) return 1;
@@ -712,7 +723,7 @@ int aser_forward_host(const void* X_host_f16, void* Y_host_f16, void* X_dev, int
                               T_dev, Y_dev, workspace, workspace_bytes);
     if (rc != ASER_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int parts = host_parts(X_host_f16, Y_host_f16, M, st);
+    const int parts = host_parts(X_host_f16, Y_host_f16, X_dev, Y_dev, M, N, K, st);
     CopyLane* lane = parts > 1 ? copy_lane(st) : nullptr;
     if (lane == nullptr) {
         cudaError_t e = cudaMemcpyAsync(X_dev, X_host_f16, (size_t)M * K * 2, cudaMemcpyHostToDevice, st);

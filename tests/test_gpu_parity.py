@@ -794,6 +794,30 @@ def test_forward_host_in_parts(aser, M):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("host,device", [(True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("N,K", [(1024, 512), (512, 1024), (512, 512)])
+def test_forward_host_output_in_the_place_of_the_input(aser, N, K, host, device):
+    """Y over X in the pinned host buffer, in the device staging buffer, or both: no row of X is overwritten before it
+    is read, whether or not the pass is cut into parts."""
+    M, r = 512, 32
+    lay = synth.make_layer(M, N, K, seed=1300 + N + K, n_cal=8)
+    s, Wq, w_scale, L_A, L_B = oracle_layer(lay, r, construct=False)
+    ref = F.forward(lay.X, s, Wq, w_scale, L_A, L_B, use_dgemm=True)
+    layer = aser.AserLinear(to_dev(lay.W), to_dev(s), to_dev(L_A), to_dev(L_B), M)
+    if device:
+        both = torch.empty((M * max(N, K),), dtype=torch.float16, device="cuda")
+        layer.X_dev, layer.Y = both[:M * K].view(M, K), both[:M * N].view(M, N)
+    X = torch.empty((M * max(N, K),), dtype=torch.float16).pin_memory()
+    Y = X if host else torch.empty((M * N,), dtype=torch.float16).pin_memory()
+    for _ in range(3):
+        X[:M * K] = torch.from_numpy(lay.X.copy()).view(-1)
+        layer.forward_host(X[:M * K].view(M, K), Y[:M * N].view(M, N))
+        torch.cuda.current_stream().synchronize()
+        assert_rows_close(Y[:M * N].view(M, N).numpy(), ref.y)
+    aser.check_status(layer.ws)
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("r", [128, 192])
 def test_fused_group_is_bit_identical_across_the_two_tensor_core_kernels(aser, r):
     """1024 tokens, K = 4096, two layers of 2048 channels: the fused launch (4096 channels) is served by CTA pairs,
