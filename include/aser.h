@@ -302,11 +302,15 @@ int aser_forward_shared_cat(const void* X_f16, const float* s, const void* LA_st
  * ideally pinned) to the device staging buffer X_dev, runs aser_forward, and copies Y back to Y_host,
  * all enqueued on `stream`; returns without synchronising.  Device-side operands and
  * staging buffers are the caller's.  All arguments are checked before the first copy is
- * enqueued.  With pinned buffers and 256 tokens or more the pass is cut into up to four parts of tokens
+ * enqueued.  With pinned buffers a large pass is cut into up to four parts of at least 128 tokens
  * whose copies run on streams of the library's own (a few per calling thread), begun behind `stream` and
- * joined to it at the end; each part is an aser_forward of its own.  A thread whose last passes went to three
+ * joined to it at the end; each part is an aser_forward of its own.  A pass is not cut while `stream` is being
+ * captured, nor where Y lies over X with rows of another length.  A thread whose last passes went to three
  * streams or more overlaps them itself: its passes are not cut.
+ * aser_forward_host_parts: the number of parts that a pass of this size is cut into where its buffers allow it, and
+ * (first_token not NULL, of five entries) the first token of each part, then M.
  */
+int aser_forward_host_parts(int M, int N, int K, int* first_token);
 int aser_forward_host(const void* X_host_f16, void* Y_host_f16,
                       void* X_dev, int8_t* Xq_dev, float* a_scale_dev, void* T_dev, void* Y_dev,
                       const float* s, const void* LA_f16, const void* Wk, const float* w_scale,

@@ -169,12 +169,16 @@ int quant_with_workspace(const void* X_f16, const float* s, const void* LA_f16, 
 }
 
 // ---- aser_forward_host: copies beside the computation ----
-// From 256 tokens on with pinned buffers, a pass is cut into up to four parts of at least 128 tokens whose copies
-// in both directions overlap each other and the computation (1024 x 4096 -> 4096: 155 us in, 40 us of kernels
-// and 150 us out, one after the other 377 us).  The copies need streams of their own: each thread keeps a few pairs
+// With pinned buffers a pass is cut into up to four parts whose copies in both directions overlap each other and the
+// computation (1024 x 4096 -> 4096: 155 us in, 40 us of kernels and 150 us out, one after the other 361 us, in parts
+// 285).  A part costs about 12 us of calls, so it has at least 1.5 MiB to hide in the smaller direction (undivided /
+// parts of 1 / 1.5 / 2 MiB, seven layers of a block on one stream: 512 tokens 1965 / 1749 / 1742 / 1738 us, 256 tokens 1131 /
+// 1051 / 1127 / 1126; on four streams 1247 / 1252 / 1175 / 1171 and 620 / 662 / 620 / 620; parts of any size made 512 tokens of
+// 512 x 264 99 us instead of 57).  The copies need streams of their own: each thread keeps a few pairs
 // per device, one for each of the caller's streams it has seen lately (so those do not queue behind each other), and
 // gives them back when it ends.
 constexpr int kHostParts = 4, kCopyLanes = 4;
+constexpr size_t kPartBytes = 3 << 19;
 
 struct CopyLane {
     int device = -1;
@@ -242,29 +246,38 @@ CopyLane* copy_lane(cudaStream_t st) {
     return &l;
 }
 
+// Parts that a pass of this size is cut into, where its buffers allow it: at least 128 tokens each, and at least
+// kPartBytes each in the smaller direction, which is what the overlap can hide.
+int host_parts(int M, int N, int K) {
+    const size_t row = (size_t)(N < K ? N : K) * 2, by_bytes = M * row / kPartBytes, by_tokens = (size_t)M / 128;
+    const size_t parts = by_bytes < by_tokens ? by_bytes : by_tokens;
+    return parts < 1 ? 1 : parts < kHostParts ? (int)parts : kHostParts;
+}
+// First token of part `part`: whole groups of 128 tokens dealt evenly, a short last group joined to the last part.
+int part_begin(int M, int parts, int part) { return part == parts ? M : M / 128 * part / parts * 128; }
+
 bool overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
     const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
     return x < y + b_bytes && y < x + a_bytes;
 }
 
-int host_parts(const void* X_host, const void* Y_host, const void* X_dev, const void* Y_dev, int M, int N, int K,
-               cudaStream_t st) {
-    if (M < 256) return 1;
+// Whether the parts of a pass between these buffers may run beside each other.
+bool parts_allowed(const void* X_host, const void* Y_host, const void* X_dev, const void* Y_dev, int M, int N, int K,
+                   cudaStream_t st) {
     // Y in the place of X (on either side) asks for all of X to be read before the first of Y is written, unless each
     // row of Y takes the place of its own row of X
     const size_t x_bytes = (size_t)M * K * 2, y_bytes = (size_t)M * N * 2;
-    if (overlap(X_host, x_bytes, Y_host, y_bytes) && !(X_host == Y_host && N == K)) return 1;
-    if (overlap(X_dev, x_bytes, Y_dev, y_bytes) && !(X_dev == Y_dev && N == K)) return 1;
+    if (overlap(X_host, x_bytes, Y_host, y_bytes) && !(X_host == Y_host && N == K)) return false;
+    if (overlap(X_dev, x_bytes, Y_dev, y_bytes) && !(X_dev == Y_dev && N == K)) return false;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { cudaGetLastError(); return 1; }
-    if (cap != cudaStreamCaptureStatusNone) return 1;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { cudaGetLastError(); return false; }
+    if (cap != cudaStreamCaptureStatusNone) return false;
     for (const void* p : {X_host, Y_host}) {      // a copy from pageable memory holds the calling thread
         cudaPointerAttributes a;
-        if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return 1; }
-        if (a.type != cudaMemoryTypeHost) return 1;
+        if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return false; }
+        if (a.type != cudaMemoryTypeHost) return false;
     }
-    const int parts = M / 128;
-    return parts < kHostParts ? parts : kHostParts;
+    return true;
 }
 
 }  // namespace
@@ -709,6 +722,13 @@ int aser_forward(const void* X_f16, const float* s, const void* LA_f16, const vo
                          /*overlap_prev=*/true);
 }
 
+int aser_forward_host_parts(int M, int N, int K, int* first_token) {
+    if (!shape_ok(M, N, K, 0) || M == 0 || N == 0) return 0;
+    const int parts = host_parts(M, N, K);
+    for (int i = 0; first_token != nullptr && i <= parts; ++i) first_token[i] = part_begin(M, parts, i);
+    return parts;
+}
+
 int aser_forward_host(const void* X_host_f16, void* Y_host_f16, void* X_dev, int8_t* Xq_dev,
                       float* a_scale_dev, void* T_dev, void* Y_dev, const float* s,
                       const void* LA_f16, const void* Wk, const float* w_scale, const void* LB_f16,
@@ -723,8 +743,8 @@ int aser_forward_host(const void* X_host_f16, void* Y_host_f16, void* X_dev, int
                               T_dev, Y_dev, workspace, workspace_bytes);
     if (rc != ASER_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int parts = host_parts(X_host_f16, Y_host_f16, X_dev, Y_dev, M, N, K, st);
-    CopyLane* lane = parts > 1 ? copy_lane(st) : nullptr;
+    const int parts = host_parts(M, N, K);
+    CopyLane* lane = parts > 1 && parts_allowed(X_host_f16, Y_host_f16, X_dev, Y_dev, M, N, K, st) ? copy_lane(st) : nullptr;
     if (lane == nullptr) {
         cudaError_t e = cudaMemcpyAsync(X_dev, X_host_f16, (size_t)M * K * 2, cudaMemcpyHostToDevice, st);
         if (e != cudaSuccess) return record_cuda_error(e, "copy X to device");
@@ -737,21 +757,18 @@ int aser_forward_host(const void* X_host_f16, void* Y_host_f16, void* X_dev, int
     }
     // Parts of the tokens: X of a part comes in, the part before it is computed on `stream`, Y of an earlier one goes
     // out.  The copies' streams begin behind `stream` and `stream` ends behind them, whatever fails between.
-    const int rows = ((M + parts - 1) / parts + 127) / 128 * 128;
     cudaError_t e = cudaEventRecord(lane->begin, st);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(lane->in, lane->begin, 0);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(lane->out, lane->begin, 0);
-    int part = 0;
-    for (int m = 0; m < M && e == cudaSuccess; m += rows, ++part) {
-        const int Mp = M - m < rows ? M - m : rows;
+    for (int part = 0; part < parts && e == cudaSuccess; ++part) {
+        const int m = part_begin(M, parts, part), Mp = part_begin(M, parts, part + 1) - m;
         const size_t x0 = (size_t)m * K, xn = (size_t)Mp * K;
         e = cudaMemcpyAsync(static_cast<__half*>(X_dev) + x0, static_cast<const __half*>(X_host_f16) + x0, xn * 2,
                             cudaMemcpyHostToDevice, lane->in);
         if (e == cudaSuccess) e = cudaEventRecord(lane->landed[part], lane->in);
     }
-    part = 0;
-    for (int m = 0; m < M && e == cudaSuccess && rc == ASER_OK; m += rows, ++part) {
-        const int Mp = M - m < rows ? M - m : rows;
+    for (int part = 0; part < parts && e == cudaSuccess && rc == ASER_OK; ++part) {
+        const int m = part_begin(M, parts, part), Mp = part_begin(M, parts, part + 1) - m;
         const size_t x0 = (size_t)m * K, y0 = (size_t)m * N, yn = (size_t)Mp * N;
         e = cudaStreamWaitEvent(st, lane->landed[part], 0);
         if (e != cudaSuccess) break;

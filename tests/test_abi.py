@@ -89,3 +89,22 @@ def test_binding_refuses_cpu_tensors(lib):
     import paper_2411_07762_b200 as aser
     with pytest.raises(TypeError):
         aser.pack_w4(torch.zeros(128, 128, dtype=torch.float16), None)
+
+
+def test_forward_host_parts(lib):
+    """Whole 128-token groups dealt evenly, a short rest joined to the last part, no part below 128 tokens or below
+    1.5 MiB in the smaller direction."""
+    first = (C.c_int * 5)()
+    for N, K in ((264, 512), (1024, 4096), (4096, 4096), (4104, 14336), (28672, 8192)):
+        for M in (1, 127, 128, 255, 256, 257, 260, 384, 385, 512, 513, 640, 1024, 1030, 2047, 4096, 70001):
+            parts = lib.aser_forward_host_parts(M, N, K, first)
+            assert parts == lib.aser_forward_host_parts(M, N, K, None)
+            assert parts == max(1, min(4, M // 128, M * 2 * min(N, K) // (3 << 19)))
+            begin = list(first)[:parts + 1]
+            assert begin[0] == 0 and begin[-1] == M
+            if parts > 1:
+                sizes = [b - a for a, b in zip(begin, begin[1:])]
+                assert min(sizes) >= 128 and max(sizes) - min(sizes) < 256
+                assert all(b % 128 == 0 for b in begin[:-1])
+    assert lib.aser_forward_host_parts(0, 128, 128, None) == 0
+    assert lib.aser_forward_host_parts(512, 128, 100, None) == 0

@@ -741,11 +741,11 @@ def test_quant_act_bits_rejects_other_widths(aser):
 @pytest.mark.gpu
 @pytest.mark.parametrize("M", [200, 256, 333, 700, 1030])
 def test_forward_host_in_parts(aser, M):
-    """Pinned buffers: one part below 256 tokens, then two to four parts of whole 128-token groups with a ragged
-    last one; pageable buffers take the undivided path.  Both against the oracle, and again on two streams in turn
-    and from two threads at once (each with a layer of its own)."""
+    """Pinned buffers: one part, two and four with a ragged last one; pageable buffers take the undivided path.  Both
+    against the oracle, and again on two streams in turn and from two threads at once (each with a layer of its own)."""
     import threading
-    N, K, r = 264, 512, 32
+    N, K, r = 6152, 6144, 32
+    assert aser.lib.aser_forward_host_parts(M, N, K, None) == {200: 1, 256: 2, 333: 2, 700: 4, 1030: 4}[M]
     lay = synth.make_layer(M, N, K, seed=1200 + M, n_cal=8)
     s, Wq, w_scale, L_A, L_B = oracle_layer(lay, r, construct=False)
     ref = F.forward(lay.X, s, Wq, w_scale, L_A, L_B, use_dgemm=True)
@@ -795,11 +795,12 @@ def test_forward_host_in_parts(aser, M):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("host,device", [(True, False), (False, True), (True, True)])
-@pytest.mark.parametrize("N,K", [(1024, 512), (512, 1024), (512, 512)])
+@pytest.mark.parametrize("N,K", [(4096, 3072), (3072, 4096), (3072, 3072)])
 def test_forward_host_output_in_the_place_of_the_input(aser, N, K, host, device):
     """Y over X in the pinned host buffer, in the device staging buffer, or both: no row of X is overwritten before it
     is read, whether or not the pass is cut into parts."""
     M, r = 512, 32
+    assert aser.lib.aser_forward_host_parts(M, N, K, None) == 2
     lay = synth.make_layer(M, N, K, seed=1300 + N + K, n_cal=8)
     s, Wq, w_scale, L_A, L_B = oracle_layer(lay, r, construct=False)
     ref = F.forward(lay.X, s, Wq, w_scale, L_A, L_B, use_dgemm=True)
