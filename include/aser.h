@@ -304,9 +304,8 @@ int aser_forward_shared_cat(const void* X_f16, const float* s, const void* LA_st
  * staging buffers are the caller's.  All arguments are checked before the first copy is
  * enqueued.  With pinned buffers a large pass is cut into up to four parts of at least 128 tokens
  * whose copies run on streams of the library's own (a few per calling thread), begun behind `stream` and
- * joined to it at the end; each part is an aser_forward of its own.  A pass is not cut while `stream` is being
- * captured, nor where Y lies over X with rows of another length.  A thread whose last passes went to three
- * streams or more overlaps them itself: its passes are not cut.
+ * joined to it at the end.  A pass is not cut while `stream` is being captured, nor where Y lies over X with rows
+ * of another length.  Cut or not, the result has the bits of one aser_forward of all M tokens.
  * aser_forward_host_parts: the number of parts that a pass of this size is cut into where its buffers allow it, and
  * (first_token not NULL, of five entries) the first token of each part, then M.
  */

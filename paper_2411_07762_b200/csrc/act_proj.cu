@@ -609,12 +609,12 @@ int quant_act_ws_launches(int M, int K) {
 
 int launch_quant_act_ws(const __half* X, const float* s, const __half* LA, int M, int K, int r,
                         int8_t* Xq, float* a_scale, __nv_bfloat16* T, void* scratch, size_t scratch_bytes,
-                        cudaStream_t st, int act_bits, bool t_pair) {
+                        cudaStream_t st, int act_bits, bool t_pair, int M_pass) {
     const float qmax = (float)((1 << (act_bits - 1)) - 1);
     const int ldt = t_pair ? 2 * r : r, lo_off = t_pair ? r : 0;
     const int groups = (r + 127) / 128;
     if (groups > kPMaxGroups) return record_error(ASER_ERR_SHAPE, "quant_act: r beyond 512");
-    const ProjPlan plan = proj_plan(M, K, kProjPlanSms);
+    const ProjPlan plan{M, proj_plan(M_pass > 0 ? M_pass : M, K, kProjPlanSms).KS};
     if (scratch == nullptr || misaligned16(scratch) ||
         scratch_bytes < (proj_amax_floats(plan) + (size_t)plan.KS * plan.Mc * groups * 128) * sizeof(float))
         return record_error(ASER_ERR_WORKSPACE, "quant_act: scratch missing or too small");

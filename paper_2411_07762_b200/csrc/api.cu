@@ -155,17 +155,19 @@ bool forward_act_uses_scratch(int M, int K, int r) {
 
 // The activation step of a forward pass (the scratch of the two-kernel path sits behind the
 // workspace's zeroed prefix, where the linear kernel later keeps its partial sums).
-int quant_with_workspace(const void* X_f16, const float* s, const void* LA_f16, int M, int K, int r,
+// M_pass: the tokens of the whole pass where these M are a part of it; the kernels and their split of K are those of
+// the whole, so every token gets the same bits.
+int quant_with_workspace(const void* X_f16, const float* s, const void* LA_f16, int M, int M_pass, int K, int r,
                          int act_bits, bool t_pair, int8_t* Xq, float* a_scale, void* T_bf16,
                          void* workspace, size_t workspace_bytes, void* stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (!forward_act_uses_scratch(M, K, r))
+    if (!forward_act_uses_scratch(M_pass, K, r))
         return launch_quant_act(static_cast<const __half*>(X_f16), s, static_cast<const __half*>(LA_f16), M, K, r,
-                                Xq, a_scale, static_cast<__nv_bfloat16*>(T_bf16), st, act_bits, t_pair);
+                                Xq, a_scale, static_cast<__nv_bfloat16*>(T_bf16), st, act_bits, t_pair, M_pass);
     return launch_quant_act_ws(static_cast<const __half*>(X_f16), s, static_cast<const __half*>(LA_f16), M, K, r,
                                Xq, a_scale, static_cast<__nv_bfloat16*>(T_bf16),
                                static_cast<uint8_t*>(workspace) + kWsZeroedBytes,
-                               workspace_bytes - kWsZeroedBytes, st, act_bits, t_pair);
+                               workspace_bytes - kWsZeroedBytes, st, act_bits, t_pair, M_pass);
 }
 
 // ---- aser_forward_host: copies beside the computation ----
@@ -206,31 +208,15 @@ struct CopyLane {
 struct CopyLanes {
     CopyLane lane[kCopyLanes];
     int next = 0;
-    cudaStream_t recent[8] = {};       // the streams of the thread's last passes
-    int passes = 0;
-    // Whether the thread spreads its passes over three streams or more: their copies overlap already, and parts only
-    // add to them (a block step of 4096 tokens on four streams 7.7 -> 8.1 ms; 10.2 -> 9.1 on two, 13.5 -> 10.7 on one).
-    bool many_streams(cudaStream_t st) {
-        recent[passes++ & 7] = st;
-        int distinct = 0;
-        for (int i = 0; i < 8 && i < passes; ++i) {
-            bool seen = false;
-            for (int j = 0; j < i; ++j) seen = seen || recent[j] == recent[i];
-            distinct += seen ? 0 : 1;
-        }
-        if (passes >= 1 << 30) passes = 8;
-        return distinct >= 3;
-    }
     ~CopyLanes() {
         for (CopyLane& l : lane) l.destroy();
     }
 };
 
 // The calling thread's lane for work on `st`, created on first use and again after a change of device; nullptr
-// (and no error left behind) where that fails or the pass should not be cut.
+// (and no error left behind) where that fails.
 CopyLane* copy_lane(cudaStream_t st) {
     static thread_local CopyLanes lanes;
-    if (lanes.many_streams(st)) return nullptr;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return nullptr; }
     for (CopyLane& l : lanes.lane)
@@ -555,7 +541,7 @@ int aser_forward_shared(const void* X_f16, const float* s, const void* LA_stacke
             rc = linear_tc_check(M, N[l], K, r[l], workspace_bytes);
             if (rc != ASER_OK) return rc;
         }
-    rc = quant_with_workspace(X_f16, s, LA_stacked_f16, M, K, r_total, 8, false, Xq, a_scale, T_bf16,
+    rc = quant_with_workspace(X_f16, s, LA_stacked_f16, M, M, K, r_total, 8, false, Xq, a_scale, T_bf16,
                               workspace, workspace_bytes, stream);
     if (rc != ASER_OK) return rc;
     int col = 0;
@@ -645,7 +631,7 @@ int aser_forward_shared_cat(const void* X_f16, const float* s, const void* LA_st
         rc = linear_tc_check(M, n_total, K, r, workspace_bytes);
         if (rc != ASER_OK) return rc;
     }
-    rc = quant_with_workspace(X_f16, s, LA_stacked_f16, M, K, r_total, 8, false, Xq, a_scale, T_bf16,
+    rc = quant_with_workspace(X_f16, s, LA_stacked_f16, M, M, K, r_total, 8, false, Xq, a_scale, T_bf16,
                               workspace, workspace_bytes, stream);
     if (rc != ASER_OK) return rc;
     return linear_common(Xq, a_scale, Wk_cat, w_scale_cat, r > 0 ? T_bf16 : nullptr, r > 0 ? LB_cat_f16 : nullptr,
@@ -705,6 +691,19 @@ static int forward_validate(const void* X_f16, const float* s, const void* LA_f1
     return rc;
 }
 
+// The launches of a pass for M of its M_pass tokens.  (Which linear kernel serves a part makes no difference to the
+// bits: integer sums, then the low-rank chunks in order.)
+static int forward_tokens(const void* X_f16, const float* s, const void* LA_f16, const void* Wk, const float* w_scale,
+                          const void* LB_f16, int M, int M_pass, int N, int K, int r, int8_t* Xq, float* a_scale,
+                          void* T_bf16, void* Y_f16, void* workspace, size_t workspace_bytes, void* stream) {
+    const int rc = quant_with_workspace(X_f16, s, LA_f16, M, M_pass, K, r, 8, false, Xq, a_scale, T_bf16, workspace,
+                                        workspace_bytes, stream);
+    if (rc != ASER_OK) return rc;
+    return linear_common(Xq, a_scale, Wk, w_scale, r > 0 ? T_bf16 : nullptr, r > 0 ? LB_f16 : nullptr,
+                         M, N, K, r, Y_f16, nullptr, workspace, workspace_bytes, stream,
+                         /*overlap_prev=*/true);
+}
+
 int aser_forward(const void* X_f16, const float* s, const void* LA_f16, const void* Wk,
                  const float* w_scale, const void* LB_f16, int M, int N, int K, int r,
                  int8_t* Xq, float* a_scale, void* T_bf16, void* Y_f16, void* workspace,
@@ -714,12 +713,8 @@ int aser_forward(const void* X_f16, const float* s, const void* LA_f16, const vo
     int rc = forward_validate(X_f16, s, LA_f16, Wk, w_scale, LB_f16, M, N, K, r, Xq, a_scale, T_bf16,
                               Y_f16, workspace, workspace_bytes);
     if (rc != ASER_OK) return rc;
-    rc = quant_with_workspace(X_f16, s, LA_f16, M, K, r, 8, false, Xq, a_scale, T_bf16, workspace,
-                              workspace_bytes, stream);
-    if (rc != ASER_OK) return rc;
-    return linear_common(Xq, a_scale, Wk, w_scale, r > 0 ? T_bf16 : nullptr, r > 0 ? LB_f16 : nullptr,
-                         M, N, K, r, Y_f16, nullptr, workspace, workspace_bytes, stream,
-                         /*overlap_prev=*/true);
+    return forward_tokens(X_f16, s, LA_f16, Wk, w_scale, LB_f16, M, M, N, K, r, Xq, a_scale, T_bf16, Y_f16, workspace,
+                          workspace_bytes, stream);
 }
 
 int aser_forward_host_parts(int M, int N, int K, int* first_token) {
@@ -772,9 +767,9 @@ int aser_forward_host(const void* X_host_f16, void* Y_host_f16, void* X_dev, int
         const size_t x0 = (size_t)m * K, y0 = (size_t)m * N, yn = (size_t)Mp * N;
         e = cudaStreamWaitEvent(st, lane->landed[part], 0);
         if (e != cudaSuccess) break;
-        rc = aser_forward(static_cast<__half*>(X_dev) + x0, s, LA_f16, Wk, w_scale, LB_f16, Mp, N, K, r, Xq_dev + x0,
-                          a_scale_dev + m, r > 0 ? static_cast<__nv_bfloat16*>(T_dev) + (size_t)m * r : nullptr,
-                          static_cast<__half*>(Y_dev) + y0, workspace, workspace_bytes, stream);
+        rc = forward_tokens(static_cast<__half*>(X_dev) + x0, s, LA_f16, Wk, w_scale, LB_f16, Mp, M, N, K, r, Xq_dev + x0,
+                            a_scale_dev + m, r > 0 ? static_cast<__nv_bfloat16*>(T_dev) + (size_t)m * r : nullptr,
+                            static_cast<__half*>(Y_dev) + y0, workspace, workspace_bytes, stream);
         if (rc != ASER_OK) break;
         e = cudaEventRecord(lane->computed[part], st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(lane->out, lane->computed[part], 0);

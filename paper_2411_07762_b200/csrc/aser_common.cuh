@@ -34,16 +34,18 @@ int launch_pack_w4(const __half* W, const float* s, int N, int K, uint8_t* Wq, f
 int launch_repack_w4(const uint8_t* Wq, int N, int K, uint8_t* Wk, bool inverse, cudaStream_t st);
 // act_bits: width of the symmetric activation codes (2..8); they are stored in int8 either way.
 // t_pair: T is written as [M, 2r], a bf16 value and the bf16 remainder of each entry.
+// M_pass: tokens of the pass that these M are a part of (0: these are all); the split of K, and with it the order of T's
+// sums, is chosen for the pass.  A part has more than 32 tokens.
 int launch_quant_act(const __half* X, const float* s, const __half* LA, int M, int K, int r,
                      int8_t* Xq, float* a_scale, __nv_bfloat16* T, cudaStream_t st, int act_bits = 8,
-                     bool t_pair = false);
+                     bool t_pair = false, int M_pass = 0);
 // The same with caller-provided scratch (quant_act_ws_scratch_bytes): the two-kernel path for more
 // than 32 tokens, ranks up to 512 (stacked down projections of layers that share X).
 size_t quant_act_ws_scratch_bytes(int M, int K, int r);
 int quant_act_ws_launches(int M, int K);     // kernels one call enqueues
 int launch_quant_act_ws(const __half* X, const float* s, const __half* LA, int M, int K, int r,
                         int8_t* Xq, float* a_scale, __nv_bfloat16* T, void* scratch, size_t scratch_bytes,
-                        cudaStream_t st, int act_bits = 8, bool t_pair = false);
+                        cudaStream_t st, int act_bits = 8, bool t_pair = false, int M_pass = 0);
 // Device-side construction of a layer's factors (construct.cu); synchronises the stream.
 constexpr int kConstructIterations = 22;     // applications of A A^T unless the caller says otherwise
 size_t construct_workspace_bytes(int N, int K, int Tcal, int r, int n_split);

@@ -1125,7 +1125,7 @@ int pick_tma_cluster(int M, int K, int r, int max_ck) {
     return best;
 }
 
-int launch_tma(const __half* X, const float* s, const __half* LA, int M, int K, int r,
+int launch_tma(const __half* X, const float* s, const __half* LA, int M, int M_pass, int K, int r,
                int8_t* Xq, float* a_scale, __nv_bfloat16* T, int ldt, int lo_off, float qmax,
                cudaStream_t st, bool* unsupported) {
     *unsupported = false;
@@ -1141,8 +1141,8 @@ int launch_tma(const __half* X, const float* s, const __half* LA, int M, int K, 
         if (e != cudaSuccess) (void)cudaGetLastError();
     }
     const int max_ck = max_ck_all[dev];
-    if ((M + kTTok - 1) / kTTok > 65535 || r > kTMaxRank) { *unsupported = true; return ASER_OK; }
-    const int ck = pick_tma_cluster(M, K, r, max_ck);
+    if ((M_pass + kTTok - 1) / kTTok > 65535 || r > kTMaxRank) { *unsupported = true; return ASER_OK; }
+    const int ck = pick_tma_cluster(M_pass, K, r, max_ck);
     if (ck == 0) { *unsupported = true; return ASER_OK; }
     const int kc = K / ck;
     const size_t smem = (size_t)tma_smem(kc, r, ck).total;
@@ -1205,7 +1205,7 @@ int launch_large(const __half* X, const float* s, const __half* LA, int M, int K
 
 int launch_quant_act(const __half* X, const float* s, const __half* LA, int M, int K, int r,
                      int8_t* Xq, float* a_scale, __nv_bfloat16* T, cudaStream_t st, int act_bits,
-                     bool t_pair) {
+                     bool t_pair, int M_pass) {
     // symmetric codes of act_bits bits in the int8 container: +-127 for 8 bits, +-31 for 6
     const float qmax = (float)((1 << (act_bits - 1)) - 1);
     if (M == 0) return ASER_OK;
@@ -1218,15 +1218,16 @@ int launch_quant_act(const __half* X, const float* s, const __half* LA, int M, i
         return launch_small<512, 8>(X, s, LA, M, K, r, Xq, a_scale, T, ldt, lo_off, qmax, st);
     }
     bool unsupported = false;
+    if (M_pass == 0) M_pass = M;
     if (r > kTMaxRank && r <= 2 * kTMaxRank) {
         // Two launches of the cluster kernel, each for one half of L_A's rows and the matching
         // columns of T.  Both write the same codes and scales (the arithmetic is deterministic),
         // which costs one extra sweep over X but keeps the projection on the tensor cores.
         const int r1 = r - kTMaxRank;
-        int rc = launch_tma(X, s, LA, M, K, kTMaxRank, Xq, a_scale, T, ldt, lo_off, qmax, st, &unsupported);
+        int rc = launch_tma(X, s, LA, M, M_pass, K, kTMaxRank, Xq, a_scale, T, ldt, lo_off, qmax, st, &unsupported);
         if (!unsupported) {
             if (rc != ASER_OK) return rc;
-            rc = launch_tma(X, s, LA + (size_t)kTMaxRank * K, M, K, r1, Xq, a_scale, T + kTMaxRank, ldt, lo_off,
+            rc = launch_tma(X, s, LA + (size_t)kTMaxRank * K, M, M_pass, K, r1, Xq, a_scale, T + kTMaxRank, ldt, lo_off,
                             qmax, st, &unsupported);
             // the shape test is the same for both halves, so the second cannot be refused alone
             if (!unsupported) return rc;
@@ -1234,7 +1235,7 @@ int launch_quant_act(const __half* X, const float* s, const __half* LA, int M, i
         }
         return launch_large<4>(X, s, LA, M, K, r, Xq, a_scale, T, ldt, lo_off, qmax, st);
     }
-    const int rc = launch_tma(X, s, LA, M, K, r, Xq, a_scale, T, ldt, lo_off, qmax, st, &unsupported);
+    const int rc = launch_tma(X, s, LA, M, M_pass, K, r, Xq, a_scale, T, ldt, lo_off, qmax, st, &unsupported);
     if (!unsupported) return rc;
     if (r <= 64) return launch_large<1>(X, s, LA, M, K, r, Xq, a_scale, T, ldt, lo_off, qmax, st);
     if (r <= 128) return launch_large<2>(X, s, LA, M, K, r, Xq, a_scale, T, ldt, lo_off, qmax, st);

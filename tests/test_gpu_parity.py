@@ -794,6 +794,40 @@ def test_forward_host_in_parts(aser, M):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("M,N,K,r,parts", [
+    (1024, 4096, 5120, 64, 4),      # whole: two-kernel activation path; a quarter alone would take the cluster kernel
+    (2050, 1032, 1024, 48, 2),      # cluster kernel, whose split of K depends on the number of tokens; a ragged last part
+    (520, 6144, 14336, 16, 4),      # long rows; parts of 128 tokens share tiles of the linear kernel
+    (700, 3072, 7168, 256, 2),      # four low-rank chunks; two-kernel path, whose split depends on the number too
+])
+def test_forward_host_bits_do_not_depend_on_the_cut(aser, M, N, K, r, parts):
+    """A pass from pinned buffers, cut into parts on any number of streams, has the bits of one undivided pass."""
+    assert aser.lib.aser_forward_host_parts(M, N, K, None) == parts
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + N)
+    W = torch.randn(N, K, device="cuda", generator=g).half() * 0.02
+    # the second half of K all but cancels the first, so that T shows the order in which it was summed
+    half = torch.randn(M, K // 2, device="cuda", generator=g).half()
+    X = torch.cat([half, half], dim=1)
+    a = torch.randn(r, K // 2, device="cuda", generator=g).half()
+    L_A = torch.cat([a, 0.01 * torch.randn(r, K // 2, device="cuda", generator=g).half() - a], dim=1)
+    L_B = torch.randn(N, r, device="cuda", generator=g).half()
+    layer = aser.AserLinear(W, None, L_A, L_B, M)
+    whole, whole_T = layer(X).cpu(), layer.T.clone()
+    X_pin, Y_pin = X.cpu().pin_memory(), torch.empty((M, N), dtype=torch.float16).pin_memory()
+    torch.cuda.synchronize()
+    for st in [torch.cuda.Stream() for _ in range(6)]:       # more streams than a thread keeps copy streams for
+        for _ in range(2):
+            Y_pin.zero_()
+            with torch.cuda.stream(st):
+                layer.forward_host(X_pin, Y_pin)
+            st.synchronize()
+            assert torch.equal(layer.T, whole_T)
+            assert torch.equal(Y_pin, whole)
+    aser.check_status(layer.ws)
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("host,device", [(True, False), (False, True), (True, True)])
 @pytest.mark.parametrize("N,K", [(4096, 3072), (3072, 4096), (3072, 3072)])
 def test_forward_host_output_in_the_place_of_the_input(aser, N, K, host, device):
