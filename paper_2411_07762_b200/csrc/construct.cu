@@ -588,9 +588,11 @@ ConstructLayout construct_layout(int N, int K, int Tcal, int r, int n_split) {
     L.lda = wide;
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t o = off; off += (bytes + 255) / 256 * 256; return o; };
-    L.A = take((size_t)N * wide * 8);
-    L.E = take((size_t)N * K * 8);
-    L.G = take((size_t)K * K * 8);
+    // the wide error matrix, or (through the whitening factor) A, E and G: never both
+    const size_t nk = (size_t)N * K * 8, apart = 2 * nk + (size_t)K * K * 8, joined = (size_t)N * wide * 8;
+    L.A = take(joined > apart ? joined : apart);
+    L.E = L.A + nk;
+    L.G = L.E + nk;
     L.Xs = take((size_t)L.tokens * K * 8);
     for (int i = 0; i < 4; ++i) L.T[i] = take((size_t)p * N * 8);
     L.Y = take((size_t)p * wide * 8);

@@ -108,3 +108,15 @@ def test_forward_host_parts(lib):
                 assert all(b % 128 == 0 for b in begin[:-1])
     assert lib.aser_forward_host_parts(0, 128, 128, None) == 0
     assert lib.aser_forward_host_parts(512, 128, 100, None) == 0
+
+
+def test_construct_workspace_of_large_layers(lib):
+    """What one way through the construction holds at a time: through the whitening factor A, E [N, K], G [K, K] and
+    the tokens, or the matrix [N, K + tokens] and the tokens; the iterated vectors and split sums come to less than a
+    tenth of that and half a gigabyte."""
+    for N, K, tokens, r in ((8192, 28672, 512, 64), (14336, 4096, 4096, 128), (32768, 32768, 512, 64),
+                            (32768, 32768, 32768, 256), (4096, 4096, 262144, 64)):
+        wide = N * (K + tokens) if tokens <= K else 0
+        held = 8 * (max(2 * N * K + K * K, wide) + tokens * K)
+        got = lib.aser_construct_workspace_bytes(N, K, tokens, r, 0)
+        assert held <= got <= 1.1 * held + (1 << 29), (N, K, tokens, r, got / held)
