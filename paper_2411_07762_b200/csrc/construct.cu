@@ -769,6 +769,15 @@ int launch_construct(const __half* W, const float* s, const __half* Xcal, int N,
         ASER_STEP(product(ctx, false, p, kc, N, t0, N, A, kc, Y, kc));
         ASER_STEP(product(ctx, true, p, N, kc, Y, kc, A, kc, f0, N));
         swap(t0, f0);
+        if (done == 0) {
+            // The start vectors mix the whole spectrum, and the Gram matrix of Y A^T has its spread to the fourth power; with
+            // the factor of Y Y^T taken out first it is the second.  Later bases come near the singular vectors in
+            // descending order, whose Gram matrices are graded and factorise at any spread.
+            ASER_STEP(product(ctx, true, p, p, kc, Y, kc, Y, kc, C, p));
+            ASER_STEP(chol_inverse(ctx, C, p, Li, V));
+            ASER_STEP(product(ctx, false, p, N, p, Li, p, t0, N, f0, N));
+            swap(t0, f0);
+        }
         ASER_STEP(normalize(false));
     }
     const int cycles = (iters - done + 11) / 12;

@@ -145,3 +145,30 @@ def test_construct_reports_operands_that_are_not_numbers(aser, where):
         with pytest.raises(aser.AserError) as err:
             aser.construct(to_dev(ops["W"]), to_dev(ops["s"]), to_dev(ops["X"]), 32, damping=damping)
         assert err.value.code == -3
+
+
+@pytest.mark.parametrize("N,K,r,n_cal,top,w_top", [
+    (512, 512, 16, 256, 1000, 10),      # sigma_1 / sigma_r = 5.6e3
+    (640, 512, 48, 512, 300, 10),       # 3.3e3; as many tokens as channels
+    (512, 512, 48, 600, 300, 10),       # 3.2e3; more tokens than channels
+    (768, 640, 160, 512, 10000, 10),    # 7.9e3 with 240 vectors: the factorisation in three blocks
+])
+def test_construct_wide_spectrum(aser, N, K, r, n_cal, top, w_top):
+    """Outlier columns left to the factors (the split of Eq. 12) with gains that spread the singular values; no
+    smoothing, no S asked for.  The singular values are fp64 outputs: at these gaps to the next value the iteration has
+    converged, and what is left is rounding, 1e-14 to 1e-12 seen."""
+    rng = np.random.default_rng(5)
+    n_out = min(r, 48)
+    W = rng.standard_normal((N, K)) * 0.005
+    X = rng.standard_normal((n_cal, K)) / 32
+    idx = np.sort(rng.permutation(K)[:n_out])
+    X[:, idx] *= np.geomspace(1.0, top, n_out)
+    W[:, idx] *= np.geomspace(0.3, w_top, n_out)
+    W, X = W.astype(np.float16), X.astype(np.float16)
+    L = Cn.construct_layer(W, X, np.ones(K, np.float32), r=r, split_outliers=idx)
+    out = aser.construct(to_dev(W), None, to_dev(X), r, split_idx=to_dev(idx.astype(np.int32)))
+    assert np.array_equal(out["Wq"].cpu().numpy(), L.Wq)
+    assert np.allclose(out["sigma"].cpu().numpy(), L.sigma[:r], rtol=1e-10)
+    prod_gpu = out["L_B"].cpu().numpy().astype(np.float64) @ out["L_A"].cpu().numpy().astype(np.float64)
+    prod_ref = L.L_B.astype(np.float64) @ L.L_A.astype(np.float64)
+    assert np.linalg.norm(prod_gpu - prod_ref) < 2e-3 * np.linalg.norm(prod_ref)
