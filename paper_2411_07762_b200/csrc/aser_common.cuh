@@ -85,7 +85,8 @@ int launch_linear_decode(const int8_t* Xq, const float* a_scale, const uint8_t* 
                          int M, int N, int K, int r, __half* Y, int32_t* acc_debug,
                          cudaStream_t st, bool overlap_prev = false, int ldt = 0, CatSplit cat = CatSplit());
 // Many-token kernel on pairs of CTAs (linear_pair.cu); uses the workspace's status word only.
-// linear_pair_prefers: the shapes for which it is faster than linear_tc (estimates of both, in cycles).
+// linear_pair_prefers: the shapes for which it is faster than linear_tc (estimates of both, in cycles), where it can
+// run at all.  To be asked before every launch: it also sets the kernel up on its first yes.
 constexpr int kLinearPairMinTokens = 65;
 bool linear_pair_prefers(int M, int N, int K, const CatSplit& cat);
 int launch_linear_pair(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const float* w_scale,

@@ -624,19 +624,20 @@ Plan make_plan(int M, int N, int pairs) {
     return best;
 }
 
+// Whether the kernel can run as it was built: the warpgroups' budgets add up to what the block is launched with and to
+// nothing else, so a compiler that gives a thread another number of registers leaves every shape to linear_tc.
 template <bool DEBUG_ACC>
-int configure(int dev) {
-    static bool configured[kMaxDevices] = {false};
-    if (configured[dev]) return ASER_OK;
-    cudaFuncAttributes a;
-    cudaError_t e = cudaFuncGetAttributes(&a, linear_pair_kernel<DEBUG_ACC>);
-    if (e != cudaSuccess) return record_cuda_error(e, "linear_pair attributes");
-    // the warpgroups' budgets add up to what the block is launched with, and to nothing else
-    if (a.numRegs != kRegsLaunch) return record_error(ASER_ERR_LAUNCH, "linear_pair: built with an unexpected register count");
-    e = cudaFuncSetAttribute(linear_pair_kernel<DEBUG_ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return record_cuda_error(e, "linear_pair smem attribute");
-    configured[dev] = true;
-    return ASER_OK;
+bool configure(int dev) {
+    static int state[kMaxDevices] = {0};         // 1: ready, 2: not usable
+    if (state[dev] == 0) {
+        cudaFuncAttributes a;
+        cudaError_t e = cudaFuncGetAttributes(&a, linear_pair_kernel<DEBUG_ACC>);
+        const bool fits = e == cudaSuccess && a.numRegs == kRegsLaunch;
+        if (fits) e = cudaFuncSetAttribute(linear_pair_kernel<DEBUG_ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+        if (e != cudaSuccess) (void)cudaGetLastError();
+        state[dev] = fits && e == cudaSuccess ? 1 : 2;
+    }
+    return state[dev] == 1;
 }
 
 }  // namespace
@@ -648,19 +649,18 @@ int configure(int dev) {
 bool linear_pair_prefers(int M, int N, int K, const CatSplit& cat) {
     if (M < kLinearPairMinTokens) return false;
     if (cat.layers > 1 && ((cat.b1 | (cat.layers > 2 ? cat.b2 : 0) | (cat.layers > 3 ? cat.b3 : 0)) & 255)) return false;
-    int num_sms = 0;
-    if (device_sm_count(&num_sms) != ASER_OK || num_sms < 2) return false;
+    int num_sms = 0, dev = 0;
+    if (device_sm_count(&num_sms) != ASER_OK || num_sms < 2 || current_device(&dev) != ASER_OK) return false;
     const long long stages = (K / kWkCols + kKS - 1) / kKS;
-    return make_plan(M, N, num_sms / 2).cost * stages + 12000 < linear_tc_estimate(M, N, K, num_sms);
+    if (make_plan(M, N, num_sms / 2).cost * stages + 12000 >= linear_tc_estimate(M, N, K, num_sms)) return false;
+    return configure<false>(dev) && configure<true>(dev);
 }
 
 int launch_linear_pair(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const float* w_scale,
                        const __nv_bfloat16* T, const __half* LB, int M, int N, int K, int r, __half* Y,
                        int32_t* acc_debug, void* workspace, cudaStream_t st, bool overlap_prev, int ldt, CatSplit cat) {
-    int num_sms = 0, dev = 0;
+    int num_sms = 0;
     int rc = device_sm_count(&num_sms);
-    if (rc == ASER_OK) rc = current_device(&dev);
-    if (rc == ASER_OK) rc = acc_debug ? configure<true>(dev) : configure<false>(dev);
     if (rc != ASER_OK) return rc;
     const int pairs = num_sms / 2 > 0 ? num_sms / 2 : 1;
     const Plan plan = make_plan(M, N, pairs);
