@@ -141,14 +141,16 @@ bool act_shape_ok(int M, int K, int r) {
 // Which activation kernels a forward pass runs.  The two-kernel path with scratch reads X once
 // from HBM whatever the rank; it is the only one above rank 128 (stacked down projections of a
 // shared-input group).  The one-launch cluster kernel reads X twice (the second time from L2) and has one
-// launch less of fixed cost.  Measured at rank 128, cluster against two-kernel path: 400 x 4096 11.4 / 13.6 us, 512 x
-// 4096 14.9 / 14.0, 1000 x 4096 23 / 16, 400 x 14336 22.5 / 22.5, 512 x 14336 35 / 25, 1000 x 14336 63 / 30, 4096 x 14336
-// 125 / 83; rows of 1024 columns 9.1 / 11.3 at 512 tokens and still 16.3 / 16.8 at 4096.  Up to 32 tokens the few-token
-// kernel serves every rank.
+// launch less of fixed cost; up to seven of its 64-token clusters of 16 CTAs are resident at once, and at the eighth its
+// time steps up.  Measured at rank 128, cluster against two-kernel path, us: 448 / 449 x 4096 11.4 | 13.9 and 15.9 | 13.8,
+// 448 / 449 x 8192 15.5 | 17.8 and 24.8 | 18.1, 448 / 449 x 14336 21.8 | 23.4 and 35.0 | 22.6, 1024 x 4096 23.4 | 15.9, 4096 x
+// 14336 124 | 84; shorter rows step up later: 896 / 1000 x 3072 13.6 | 14.4 and 19.1 | 15.3, 896 / 1000 x 2048 10.9 | 12.2 and
+// 15.3 | 12.6, 1024 x 1536 12.7 | 13.4; rows of 1024 columns 9.4 | 11.1 at 512 tokens and still 15.3 | 16.8 at 4096.
+// Up to 32 tokens the few-token kernel serves every rank.
 bool forward_act_uses_scratch(int M, int K, int r) {
     if (M <= 32) return false;
     if (r > 128) return true;
-    if (K >= 4096) return M >= 448;
+    if (K >= 4096) return M > 448;
     if (K <= 1024) return M > 4096;
     return M >= 1024;
 }

@@ -120,3 +120,13 @@ def test_construct_workspace_of_large_layers(lib):
         held = 8 * (max(2 * N * K + K * K, wide) + tokens * K)
         got = lib.aser_construct_workspace_bytes(N, K, tokens, r, 0)
         assert held <= got <= 1.1 * held + (1 << 29), (N, K, tokens, r, got / held)
+
+
+def test_activation_path_of_a_forward_pass(lib):
+    """One launch (few-token or cluster kernel) or two: the cluster kernel serves whole 64-token clusters, seven of
+    them at 4096 columns and more."""
+    for K in (4096, 8192, 14336):
+        assert [lib.aser_forward_act_launches(M, K, 128) for M in (1, 32, 33, 447, 448, 449, 4096)] == [1, 1, 1, 1, 1, 2, 2]
+    assert [lib.aser_forward_act_launches(M, 2048, 128) for M in (1023, 1024)] == [1, 2]
+    assert [lib.aser_forward_act_launches(M, 1024, 128) for M in (4096, 4097)] == [1, 2]
+    assert [lib.aser_forward_act_launches(M, 4096, 144) for M in (32, 33)] == [1, 2]
