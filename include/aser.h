@@ -134,7 +134,7 @@ int aser_quant_act_ex(const void* X_f16, const float* s, const void* LA_f16,
  * `stream` that still uses the workspace when the call is made must precede it on `stream`.
  */
 size_t aser_quant_workspace_bytes(int M, int K, int r);
-/* Number of kernels one aser_quant_act_ws call enqueues (two per chunk of tokens; 0 for bad shapes). */
+/* Number of kernels one aser_quant_act_ws call enqueues (1 up to 32 tokens, else 2; 0 for bad shapes). */
 int aser_quant_act_ws_launches(int M, int K);
 int aser_quant_act_ws(const void* X_f16, const float* s, const void* LA_f16,
                       int M, int K, int r, int act_bits, int t_pair,
@@ -157,7 +157,11 @@ int aser_quant_act_ws(const void* X_f16, const float* s, const void* LA_f16,
  * packed weights the call runs a streaming kernel that leaves the workspace untouched; the
  * argument is validated all the same, so callers need not know which kernel serves a shape.
  * aser_linear_w4a8 is the same without the low-rank term (the plain W4A8 control).
+ * aser_linear_kernel: which kernel serves a shape on the current device: 0 the streaming kernel, 1 the one whose CTAs
+ * may share tiles through the workspace, 2 the one on pairs of CTAs; a negative error code for bad shapes.  The last two
+ * give the same bits.
  */
+int aser_linear_kernel(int M, int N, int K);
 int aser_linear_w4a8_lr(const int8_t* Xq, const float* a_scale, const void* Wk,
                         const float* w_scale, const void* T_bf16, const void* LB_f16,
                         int M, int N, int K, int r, void* Y_f16, int32_t* acc_debug,
@@ -235,8 +239,8 @@ int aser_check_status(void* workspace, void* stream);
  * quantization still runs, streams the weights (which that kernel does not write) and waits
  * for its completion before it reads Xq, a_scale or T.  The activation step is whichever of
  * aser_quant_act's kernels and aser_quant_act_ws's (on the same workspace) is faster at the
- * shape: the latter from 1024 tokens on and for every rank above 128;
- * aser_forward_act_launches tells how many kernels that is.  Results are those of the separate
+ * shape: the latter for many tokens (more than 448 of 4096 columns and more, 4096 of 1024 and fewer, from 1024 on
+ * between) and, above 32 tokens, for every rank above 128; aser_forward_act_launches tells how many kernels that is.  Results are those of the separate
  * calls.
  * X_f16 [M,K], s [K] or NULL, LA_f16 [r,K] / LB_f16 [N,r] (NULL when r == 0), Wk and w_scale as
  * for aser_linear_w4a8_lr.  Xq [M,K], a_scale [M], T_bf16 [M,r] (NULL when r == 0) are the

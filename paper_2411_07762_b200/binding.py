@@ -12,7 +12,7 @@ lib_path = os.path.join(_HERE, "libaser.so")
 EXPORTED_SYMBOLS = (
     "aser_pack_w4", "aser_repacked_bytes", "aser_repack_w4", "aser_unrepack_w4",
     "aser_quant_act", "aser_quant_act_bits", "aser_quant_act_ex", "aser_quant_act_ws",
-    "aser_quant_workspace_bytes", "aser_quant_act_ws_launches", "aser_forward_act_launches", "aser_forward_host_parts", "aser_linear_w4a8_lr_ld", "aser_forward_shared",
+    "aser_quant_workspace_bytes", "aser_quant_act_ws_launches", "aser_forward_act_launches", "aser_forward_host_parts", "aser_linear_kernel", "aser_linear_w4a8_lr_ld", "aser_forward_shared",
     "aser_linear_w4a8_lr_cat", "aser_forward_shared_cat_workspace_bytes", "aser_forward_shared_cat",
     "aser_forward_shared_workspace_bytes", "aser_construct", "aser_construct_workspace_bytes", "aser_linear_w4a8_lr", "aser_linear_w4a8", "aser_linear_w4a8_lr_simt", "aser_linear_w4a8_lr_static",
     "aser_workspace_bytes", "aser_workspace_init", "aser_check_status", "aser_forward",
@@ -40,6 +40,7 @@ lib.aser_quant_workspace_bytes.restype = _Z
 lib.aser_forward_act_launches.argtypes = [_I, _I, _I]
 lib.aser_forward_act_launches.restype = _I
 lib.aser_forward_host_parts.argtypes = [_I, _I, _I, _P]
+lib.aser_linear_kernel.argtypes = [_I, _I, _I]
 lib.aser_quant_act_ws_launches.argtypes = [_I, _I]
 lib.aser_quant_act_ws_launches.restype = _I
 lib.aser_quant_act_ws.argtypes = [_P, _P, _P, _I, _I, _I, _I, _I, _P, _P, _P, _P, _Z, _P]

@@ -354,6 +354,11 @@ int aser_quant_act_ex(const void* X_f16, const float* s, const void* LA_f16, int
                             static_cast<cudaStream_t>(stream), act_bits, t_pair != 0);
 }
 
+int aser_linear_kernel(int M, int N, int K) {
+    if (!shape_ok(M, N, K, 0) || M == 0 || N == 0) return ASER_ERR_SHAPE;
+    return linear_decode_prefers(M, N, K) ? 0 : linear_pair_prefers(M, N, K, CatSplit()) ? 2 : 1;
+}
+
 int aser_linear_w4a8_lr(const int8_t* Xq, const float* a_scale, const void* Wk,
                         const float* w_scale, const void* T_bf16, const void* LB_f16, int M, int N,
                         int K, int r, void* Y_f16, int32_t* acc_debug, void* workspace,

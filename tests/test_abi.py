@@ -130,3 +130,9 @@ def test_activation_path_of_a_forward_pass(lib):
     assert [lib.aser_forward_act_launches(M, 2048, 128) for M in (1023, 1024)] == [1, 2]
     assert [lib.aser_forward_act_launches(M, 1024, 128) for M in (4096, 4097)] == [1, 2]
     assert [lib.aser_forward_act_launches(M, 4096, 144) for M in (32, 33)] == [1, 2]
+
+
+def test_linear_kernel_rejects_bad_shapes(lib):
+    assert lib.aser_linear_kernel(8, 4096, 4096) == 0
+    for bad in ((8, 4096, 4100), (8, 4100, 4096), (0, 4096, 4096), (-1, 128, 128)):
+        assert lib.aser_linear_kernel(*bad) == -3

@@ -172,3 +172,19 @@ def test_construct_wide_spectrum(aser, N, K, r, n_cal, top, w_top):
     prod_gpu = out["L_B"].cpu().numpy().astype(np.float64) @ out["L_A"].cpu().numpy().astype(np.float64)
     prod_ref = L.L_B.astype(np.float64) @ L.L_A.astype(np.float64)
     assert np.linalg.norm(prod_gpu - prod_ref) < 2e-3 * np.linalg.norm(prod_ref)
+
+
+@pytest.mark.parametrize("iterations,damping", [(48, 0.01), (30, 1e-5), (0, 1e-7)])
+def test_construct_options_without_the_whitening_factor(aser, iterations, damping):
+    """A given number of iterations and small dampings (1e-7 goes through the factor all the same), the paper's smoothing
+    rule and outlier split, no S asked for.  Bounds as in _check; the remainder of 30 iterations is below them."""
+    lay = synth.make_layer(4, 392, 512, seed=88, n_cal=300)
+    s, idx = Cn.smoothing_vector_paper(lay.X_cal, lay.W, f=len(lay.outlier_idx))
+    L = Cn.construct_layer(lay.W, lay.X_cal, s, r=32, split_outliers=idx, damping=damping)
+    out = aser.construct(to_dev(lay.W), to_dev(s), to_dev(lay.X_cal), 32, damping=damping, iterations=iterations,
+                         split_idx=to_dev(idx.astype(np.int32)))
+    assert np.array_equal(out["Wq"].cpu().numpy(), L.Wq)
+    assert np.allclose(out["sigma"].cpu().numpy(), L.sigma[:32], rtol=1e-6)
+    prod_gpu = out["L_B"].cpu().numpy().astype(np.float64) @ out["L_A"].cpu().numpy().astype(np.float64)
+    prod_ref = L.L_B.astype(np.float64) @ L.L_A.astype(np.float64)
+    assert np.linalg.norm(prod_gpu - prod_ref) < 2e-3 * np.linalg.norm(prod_ref)

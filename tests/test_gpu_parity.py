@@ -96,6 +96,9 @@ ACT_CASES = [  # M, K, r
     # cluster kernel: one stage per CTA, r = 0, ranks that leave accumulator rows unused, ragged
     # last token tile, every cluster size
     (65, 128, 0), (200, 128, 48), (96, 8192, 32), (1000, 2048, 112), (2049, 512, 16), (40, 28672, 64),
+    # few tokens, long rows (two to eight chunks per thread, the last partly missing), with one, two
+    # and four tokens per projection CTA and a last CTA that has fewer
+    (1, 8320, 64), (5, 14336, 256), (17, 16512, 48), (32, 32768, 64), (3, 14336, 256), (7, 32768, 256), (31, 8320, 64), (2, 16384, 0),
 ]
 
 
@@ -324,7 +327,47 @@ PAIR_CASES = [  # M, N, K, r: shapes the kernel on CTA pairs serves (256 channel
 
 @pytest.mark.parametrize("M,N,K,r", PAIR_CASES)
 def test_pair_kernel_edges(aser, M, N, K, r):
+    assert aser.lib.aser_linear_kernel(M, N, K) == 2
     lay = synth.make_layer(M, N, K, seed=900 + M + N + K + r, n_cal=16, n_out=max(1, K // 100))
+    s, Wq, w_scale, L_A, L_B = oracle_layer(lay, r, construct=False)
+    if r == 0:
+        L_A = L_B = None
+    run_path(aser, lay, s, Wq, w_scale, L_A, L_B, "tc", timed_config=True, use_dgemm=True)
+
+
+SHARED_TILE_CASES = [  # M, N, K, r: more than 64 tokens on the kernel whose CTAs may share tiles
+    (130, 3080, 512, 64),       # whole tiles, ragged tokens and channels
+    (257, 2056, 512, 128),      # whole tiles; one token in the last token tile
+    (513, 1160, 512, 0),
+    (77, 136, 7168, 80),        # every tile shared by many CTAs; two chunks, the second 16 wide
+    (130, 392, 7168, 144),      # three chunks
+    (257, 264, 7168, 0),
+    (333, 264, 7168, 256),      # four chunks
+    (263, 9480, 6144, 80),      # shared tiles before and after whole ones in a CTA's range
+    (263, 9480, 8192, 32),      # the same with the shared tiles first
+]
+
+
+@pytest.mark.parametrize("M,N,K,r", SHARED_TILE_CASES)
+def test_shared_tile_kernel_edges(aser, M, N, K, r):
+    assert aser.lib.aser_linear_kernel(M, N, K) == 1
+    lay = synth.make_layer(M, N, K, seed=950 + M + N + K + r, n_cal=16, n_out=max(1, K // 100))
+    s, Wq, w_scale, L_A, L_B = oracle_layer(lay, r, construct=False)
+    if r == 0:
+        L_A = L_B = None
+    run_path(aser, lay, s, Wq, w_scale, L_A, L_B, "tc", timed_config=True, use_dgemm=True)
+
+
+@pytest.mark.parametrize("M", [1, 8])
+@pytest.mark.parametrize("N,K,r", [(14336, 384, 128), (14344, 640, 0), (18944, 384, 16), (14216, 512, 64)])
+def test_streaming_kernel_four_ctas_per_sm(aser, M, N, K, r):
+    """Up to eight tokens and three to four 32-channel tiles for every SM of the part (445 to 592 on 148), with odd
+    numbers of column blocks and a ragged last tile."""
+    assert aser.lib.aser_linear_kernel(M, N, K) == 0
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    if sms == 148:
+        assert 3 * sms < (N + 31) // 32 <= 4 * sms
+    lay = synth.make_layer(M, N, K, seed=970 + M + N + K + r, n_cal=16, n_out=max(1, K // 100))
     s, Wq, w_scale, L_A, L_B = oracle_layer(lay, r, construct=False)
     if r == 0:
         L_A = L_B = None
@@ -859,6 +902,7 @@ def test_fused_group_is_bit_identical_across_the_two_tensor_core_kernels(aser, r
     a layer alone by the kernel that may share tiles.  Both add the low-rank chunks in order, so the bits agree."""
     import ctypes as C
     M, K, N = 1024, 4096, 2048
+    assert [aser.lib.aser_linear_kernel(M, n, K) for n in (N, 2 * N)] == [1, 2]
     g = torch.Generator(device="cuda")
     g.manual_seed(77 + r)
     Xq = torch.randint(-127, 128, (M, K), device="cuda", dtype=torch.int8, generator=g)
