@@ -18,9 +18,11 @@
  * on error nothing has been launched unless stated.  Every data pointer is a
  * DEVICE pointer owned by the caller unless its name ends in _host; arrays are
  * row-major and contiguous; pointers must be 16-byte aligned.  The library
- * allocates no memory, never synchronises (except aser_check_status), and
- * enqueues all work on the cudaStream_t passed as `stream` (NULL = the legacy
- * default stream).  A process may use the library on several devices (the one current at the
+ * allocates no memory, never synchronises (except aser_check_status and
+ * aser_construct), and enqueues all work on the cudaStream_t passed as `stream`
+ * (NULL = the legacy default stream); aser_forward_host, which allocates no
+ * memory either, creates a few streams and events per calling thread for its copies on
+ * first use and joins them to `stream`.  A process may use the library on several devices (the one current at the
  * call is used; per-device set-up is done on first use).  NaN/Inf inputs give unspecified
  * values but never a fault.
  * Shapes: M >= 0, K % 128 == 0, N % 8 == 0, r % 16 == 0, 0 <= r <= 256.

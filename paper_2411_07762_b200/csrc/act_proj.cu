@@ -94,7 +94,9 @@ act_proj_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     const int la_box_rows = r / la_boxes;
     const uint32_t la_stage_bytes = (uint32_t)r * 128u;
     extern __shared__ uint8_t smem_raw[];
-    // a programmatic dependent of whatever precedes it; what depends on it starts only after its wait
+    // A programmatic dependent of whatever precedes it.  The signal must stay behind the wait: act_quant_kernel reads X
+    // and s, and the linear kernel after it the weights, before waits of their own, which is sound because neither
+    // starts until everything before this kernel is done.
     grid_dep_wait();
     grid_dep_launch();
     const uint32_t sraw = smem_u32(smem_raw);
@@ -140,8 +142,7 @@ act_proj_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
             prefetch_tensormap(&map_x);
             if (r > 0) prefetch_tensormap(&map_la);
             // The first round of the ring is requested before the other warps are ready: it needs
-            // only the barriers set up above.  X may come from the kernel before this one.
-            grid_dep_wait();
+            // only the barriers set up above.
             for (int i = 0; i < NS && i < nst; ++i) {
                 mbar_arrive_expect_tx(bar_full(i), (uint32_t)kPTileBytes);
                 tma_load_3d(sb + i * stage_bytes, &map_x, 0, m_first + row0, (k0 + i * kPCols) / kPCols, bar_full(i));
@@ -425,7 +426,8 @@ __device__ __forceinline__ uint2 codes8_unit(const uint4& x, float sc, float rcp
 // vector with more such columns than the list holds takes the general loop, which tests every
 // group of eight divisors.
 // Launched as a programmatic dependent of act_proj_kernel: the list and the first loads of X
-// (inputs of the whole step, not products of that kernel) are done before the dependency wait.
+// (inputs of the whole step, not products of that kernel; written before it started, see its signal) are
+// done before the dependency wait.
 constexpr int kQRows = 4;
 constexpr int kQList = 512;             // columns with a divisor the fix-up pass can take
 __global__ void __launch_bounds__(256, 4)
