@@ -45,6 +45,13 @@ __device__ __forceinline__ uint2 quant8(const float (&v)[8], float sc, bool nonz
 // ---------------------------------------------------------------------------
 constexpr int kRowsPerCta = 4;  // L_A rows handled by one projection CTA
 
+// 1 / v to about one unit in the last place, for v in the normal range.
+__device__ __forceinline__ float rcp_approx(float v) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+
 // CTAs 0 .. M - 1 quantize one token each, the others compute kRowsPerCta entries of T for TOK tokens.
 // What bounds it is the chain of loads: launch, one round trip per batch of chunks, a reduction.  So a thread
 // has at most CPT 8-column chunks of a row (TH threads by the row length), the quantizing CTA keeps them in
@@ -110,7 +117,7 @@ quant_act_small_kernel(const __half* __restrict__ X, const float* __restrict__ s
     for (int jj = 0; jj < kRowsPerCta; ++jj)
 #pragma unroll
         for (int k = 0; k < TOK; ++k) acc[jj][k] = 0.f;
-    bool far = false;           // a divisor so far from 1 that the parts of its reciprocal may leave the normal range
+    float nearest = 1.f, farthest = 1.f;        // magnitudes of the divisors met, from zero
 #pragma unroll 2
     for (int c = threadIdx.x; c < chunks; c += TH) {
         RawChunk rc[TOK];
@@ -125,25 +132,19 @@ quant_act_small_kernel(const __half* __restrict__ X, const float* __restrict__ s
         for (int jj = 0; jj < kRowsPerCta; ++jj)
             la[jj] = (j0 + jj < r) ? *reinterpret_cast<const uint4*>(LA + (size_t)(j0 + jj) * K + c * 8)
                                    : make_uint4(0, 0, 0, 0);
-        // x~ = fp32(x) / s as for the codes, without a division per token: the reciprocal of a divisor as two numbers
-        // (the first truncated, so the remainder has its sign and an infinite x stays infinite), once for all tokens;
-        // x * high + x * low is rounded once and differs from the quotient only where that lies within 2^-20 of a
-        // unit in the last place from a tie.  A remainder of zero is replaced by one that no sum sees.
+        // x~ = fp32(x) / s as for the codes, without a division per token: the reciprocal of a divisor as a double-length
+        // number (Dekker), once for all tokens.  The first part is taken a little short, so that the second is never
+        // zero and has its sign (an infinite x stays infinite); x * first + x * second is rounded once, to the quotient
+        // but for one case in millions next to a tie.
         const float sv[8] = {rc[0].s0.x, rc[0].s0.y, rc[0].s0.z, rc[0].s0.w, rc[0].s1.x, rc[0].s1.y, rc[0].s1.z, rc[0].s1.w};
-        constexpr float kUnseen = 0x1p-40f;
         float inv[8], low[8];
-        bool ones = true;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) { ones = ones && sv[i] == 1.f; inv[i] = 1.f; low[i] = kUnseen; }
-        if (!ones) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const float a = fabsf(sv[i]);
-                far = far || !(a > 0x1p-80f && a < 0x1p80f);
-                inv[i] = __frcp_rz(sv[i]);
-                const float rem = fmaf(-sv[i], inv[i], 1.f);
-                low[i] = inv[i] * (rem > 0.f ? rem : kUnseen);
-            }
+        for (int i = 0; i < 8; ++i) {
+            nearest = fminf(nearest, fabsf(sv[i]));
+            farthest = fmaxf(farthest, fabsf(sv[i]));
+            inv[i] = rcp_approx(sv[i]) * (1.f - 0x1p-21f);
+            const float rem = fmaf(-sv[i], inv[i], 1.f);
+            low[i] = inv[i] * fmaf(rem, rem, rem);
         }
 #pragma unroll
         for (int k = 0; k < TOK; ++k) {
@@ -169,7 +170,9 @@ quant_act_small_kernel(const __half* __restrict__ X, const float* __restrict__ s
             }
         }
     }
-    if (far) {                  // the thread's sums once more, every column divided
+    // A divisor so far from 1 that the parts of its reciprocal may leave the normal range: the thread's sums once more,
+    // every column divided.  (NaN needs no care: its quotients are NaN either way.)
+    if (!(nearest > 0x1p-80f && farthest < 0x1p80f)) {
 #pragma unroll
         for (int k = 0; k < TOK; ++k) {
 #pragma unroll
