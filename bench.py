@@ -76,19 +76,19 @@ EXTRA_POINTS = ("c2_decode_m8", "c2_decode_m1", "c3_prefill_gate_up", "c3_prefil
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel under ncu, taken with
 # the kernel as it stands in this tree; the summary with the command is
 # profiles/launches_c4_decoder_block_step.txt.  The workload's figure is the average over its
-# linear_tc launches; "<workload>/<layers>" is the launch of that layer or fused group.  Workloads
+# linear_pair launches; "<workload>/<layers>" is the launch of that layer or fused group.  Workloads
 # without a capture of the current kernel report null.
 NCU_DRAM_BYTES_PER_LAUNCH = {
-    "c4_decoder_block": 1056.9e6 / 5,
-    "c4_decoder_block/q+k+v": 36.8e6, "c4_decoder_block/o": 27.6e6, "c4_decoder_block/gate": 166.7e6,
-    "c4_decoder_block/up": 189.1e6, "c4_decoder_block/down": 636.9e6,
+    "c4_decoder_block": 465.4e6 / 5,
+    "c4_decoder_block/q+k+v": 43.7e6, "c4_decoder_block/o": 28.5e6, "c4_decoder_block/gate": 127.3e6,
+    "c4_decoder_block/up": 127.4e6, "c4_decoder_block/down": 138.6e6,
 }
 
 
 def dominant_kernel(M, N, K):
-    """Name of the kernel the library runs for the integer product at this shape (few tokens and
-    at most 64 MB of packed weights: the streaming kernel; otherwise the tensor-core kernel)."""
-    return "linear_decode_kernel" if M <= 16 and N * K // 2 <= (64 << 20) else "linear_tc_kernel"
+    """Name of the kernel the library runs for the integer product at this shape, as it says itself."""
+    import paper_2411_07762_b200 as aser
+    return ("linear_decode_kernel", "linear_tc_kernel", "linear_pair_kernel")[aser.lib.aser_linear_kernel(M, N, K)]
 
 
 def load_peaks():
