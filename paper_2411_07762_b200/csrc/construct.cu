@@ -23,7 +23,7 @@
 // on [0, b], b the smallest Ritz value (from below an estimate of sigma_p^2, so nothing wanted is
 // damped): the recurrence is linear in the rows, so both of its terms may be multiplied by the
 // inverse Cholesky factor after every step and it keeps its accuracy whatever the spread of the
-// spectrum.  b is estimated anew every dozen steps.  With x = sigma_r^2 / sigma_p^2, a step of the
+// spectrum (the first step, from vectors that mix the whole of it, is normalised in two stages).  b is estimated anew every dozen steps.  With x = sigma_r^2 / sigma_p^2, a step of the
 // recurrence gains exp(acosh(2 x - 1)), a plain one x: at x = 1.2 ... 1.6, where quantization errors
 // lie, 22 steps reach what 60 to 90 plain ones would.  Measured against the exact triplets (2048 x
 // 2048, 512 tokens, r = 64): product 5e-5 after 18 such steps, 9e-5 after 48 plain ones.
@@ -33,7 +33,7 @@
 // 4096 x 4096, 512 tokens, r = 64 took 236.8 ms with plain iteration on A, a 64 x 64 fma product
 // (157 ms), one thread per column in the triangular solves (46 ms) and one launch per Jacobi round
 // (11 ms); now 11.0 ms: Y and Z 5.8 (at 28 of 37 TFLOP/s), Cholesky factors 1.1, Jacobi 1.4.  2048 x
-// 1024, r = 256: 784 -> 46 ms.
+// 1024, r = 256: 784 -> 47 ms.
 #include "aser_common.cuh"
 #include "gemm64.cuh"
 

@@ -307,8 +307,9 @@ int launch_nt(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const f
     // measured 7 % slower at 8192 x 8192 than two blocks and three CTAs per SM.  Loading the next block's
     // activation fragment ahead made the kernel alone up to 8 % faster and a whole step of 4096 x 4096 9 % slower:
     // its first load is then two deep behind the dependency wait.)  Up to eight tokens, where the tiles are a few
-    // too many for three CTAs per SM, four with half the bytes in flight each take them in one wave (14336 x 4096:
-    // 448 tiles for 444 places; a step of eight tokens 14.5 -> 12.9 us).
+    // too many for three CTAs per SM, four with half the bytes in flight each take them in one wave (kernel alone, one /
+    // eight tokens: 14336 x 4096, 448 tiles for 444 places, 11.5 / 11.5 -> 7.6 / 8.9 us; 16384 x 1024, 512 tiles, 6.5 / 6.3 -> 4.5 /
+    // 4.8).
     const int tiles = (N + 31) / 32;
     if (NT == 1 && tiles > 3 * num_sms && tiles <= 4 * num_sms)
         return launch_cfg<1, 2, 1>(Xq, a_scale, Wk, w_scale, T, LB, M, N, K, r, Y, acc_debug, st, overlap_prev, ldt, cat);

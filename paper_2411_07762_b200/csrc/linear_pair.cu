@@ -33,9 +33,10 @@
 // partial sums and no workspace beyond the status word.
 // Every wait is bounded: on expiry the CTA sets the status word and winds down.
 //
-// Measured against linear_tc_kernel<128> (tokens x channels x K, rank; us): 2048 x 14336 x 4096, 64: 136 -> 112;
-// 4096 x 14336 x 4096, 128: 271 -> 211; 4096 x 4096 x 14336, 128: 233 -> 170 (2.8 POP/s); 4096 x 28672 x 8192,
-// 256: 1188 -> 851; 1024 x 4096 x 4096, 128: 44 -> 27; 333 x 14336 x 4096, 64: 49 -> 37.  A stage takes 1230 cycles
+// Measured against linear_tc_kernel<128>, the linear step alone, both in graphs on one box (tokens x channels x K, rank 64;
+// us): 2048 x 14336 x 4096 133 -> 110; 4096 x 14336 x 4096 242 -> 197; 4096 x 4096 x 14336 204 -> 163; 4096 x 8192 x 8192
+// 236 -> 181; 1500 x 4096 x 4096 37.6 -> 33.3; 1024 x 4096 x 4096 28.4 -> 23.7; 333 x 14336 x 4096 36.0 -> 32.6; 4096 x 28672 x
+// 8192 at rank 256, under the power cap, 1173 -> 777.  A stage takes 1230 cycles
 // against 1024 of MMAs (4096 x 4096 x 14336, rank 0); a tile of K = 4096 pays 5000 more for its turn-around, 11000
 // with a low-rank term.  Sixteen epilogue warps (72 registers at launch) or both halves' sums read at once cost
 // more in spilled registers than they saved there (gate projection 116 -> 122 ... 139 us).
@@ -644,8 +645,11 @@ bool configure(int dev) {
 
 // The estimates were fitted to whole forward passes (M 48 ... 2048, seven layer shapes): pairs win from about
 // 600 tokens on nearly everywhere and below that where they fill the part or where linear_tc would have to
-// share its tiles (333 x 2048 x 2048: 24 against 38 us, 160 x 8192 x 28672: 81 / 91), linear_tc where few long
-// tiles have to be split over the part (256 x 4096 x 14336: 50 against 60 us), which pairs do not do.
+// share its tiles (linear step, 333 x 2048 x 2048: 14.0 against 25.5 us, 160 x 28672 x 8192: 70 / 77), linear_tc where few long
+// tiles have to be split over the part (256 x 4096 x 14336: 31 us; the whole pass was 10 us longer with pairs),
+// which pairs do not do.  Looked at again on 920 points (18 layer shapes of 1152 to 28672 columns, 65 to 4096 tokens drawn,
+// ranks 0, 64 and 128; linear step in a graph): 1.153 times as fast as linear_tc alone in the geometric mean, four points slower
+// by more than 1.5 %, the worst 6 % (1027 x 8192 x 28672: a short column of three tokens costs a pass over its weights).
 bool linear_pair_prefers(int M, int N, int K, const CatSplit& cat) {
     if (M < kLinearPairMinTokens) return false;
     if (cat.layers > 1 && ((cat.b1 | (cat.layers > 2 ? cat.b2 : 0) | (cat.layers > 3 ? cat.b3 : 0)) & 255)) return false;
