@@ -782,13 +782,15 @@ def test_quant_act_bits_rejects_other_widths(aser):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("N,K", [(264, 512), (6152, 6144)])
 @pytest.mark.parametrize("M", [200, 256, 333, 700, 1030])
-def test_forward_host_in_parts(aser, M):
-    """Pinned buffers: one part, two and four with a ragged last one; pageable buffers take the undivided path.  Both
-    against the oracle, and again on two streams in turn and from two threads at once (each with a layer of its own)."""
+def test_forward_host_in_parts(aser, M, N, K):
+    """Pinned buffers: undivided where there is too little to overlap, else one part, two and four with a ragged last
+    one; pageable buffers take the undivided path.  Both against the oracle, and again on two streams in turn
+    and from two threads at once (each with a layer of its own)."""
     import threading
-    N, K, r = 6152, 6144, 32
-    assert aser.lib.aser_forward_host_parts(M, N, K, None) == {200: 1, 256: 2, 333: 2, 700: 4, 1030: 4}[M]
+    r = 32
+    assert aser.lib.aser_forward_host_parts(M, N, K, None) == (1 if K == 512 else {200: 1, 256: 2, 333: 2, 700: 4, 1030: 4}[M])
     lay = synth.make_layer(M, N, K, seed=1200 + M, n_cal=8)
     s, Wq, w_scale, L_A, L_B = oracle_layer(lay, r, construct=False)
     ref = F.forward(lay.X, s, Wq, w_scale, L_A, L_B, use_dgemm=True)
