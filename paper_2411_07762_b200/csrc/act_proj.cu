@@ -388,35 +388,6 @@ act_proj_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     }
 }
 
-// Eight codes of a row whose divisors are all 1: fp16 pairs widened by the conversion unit, then on
-// packed fp32 pairs su = x * (1 / sc) + 1.5 * 2^23 (one rounding: the low byte of su is the code),
-// -w = 1.5 * 2^23 - su (exact) and d = x * (1 / sc) - w, the distance of the product to its integer.
-// rne(x / sc) can differ from that integer only where the product is within 1e-4 of a tie (the
-// quotient and the product differ by less than 3.1e-5): such a group takes the exact division.
-__device__ __forceinline__ uint2 codes8_unit(const uint4& x, float sc, float rcp, float qmax) {
-    const float kMagic = 12582912.0f;
-    const float2 m2 = make_float2(kMagic, kMagic), neg1 = make_float2(-1.f, -1.f), r2 = make_float2(rcp, rcp);
-    const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
-    float2 f[4];
-    uint32_t u[8];
-    float far = 0.f;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        f[i] = __half22float2(*reinterpret_cast<const __half2*>(&xw[i]));
-        const float2 su = __ffma2_rn(f[i], r2, m2);
-        const float2 nw = __ffma2_rn(su, neg1, m2);
-        const float2 d = __ffma2_rn(f[i], r2, nw);
-        u[2 * i] = __float_as_uint(su.x);
-        u[2 * i + 1] = __float_as_uint(su.y);
-        far = fmaxf(far, fmaxf(fabsf(d.x), fabsf(d.y)));
-    }
-    if (far > 0.4999f)
-        return quant8_exact(f[0].x, f[0].y, f[1].x, f[1].y, f[2].x, f[2].y, f[3].x, f[3].y, sc, qmax);
-    const uint32_t a01 = __byte_perm(u[0], u[1], 0x0040), a23 = __byte_perm(u[2], u[3], 0x0040);
-    const uint32_t a45 = __byte_perm(u[4], u[5], 0x0040), a67 = __byte_perm(u[6], u[7], 0x0040);
-    return make_uint2(__byte_perm(a01, a23, 0x5410), __byte_perm(a45, a67, 0x5410));
-}
-
 // grid = ceil(rows of the chunk / kQRows), 256 threads; a CTA takes kQRows token rows, several
 // 16-byte loads per thread are in flight, and the per-row scales are computed once per CTA (one
 // warp per row).  The kernel is bound by instruction issue, not by bytes, so the common case is

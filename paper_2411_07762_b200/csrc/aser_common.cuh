@@ -39,6 +39,10 @@ int launch_repack_w4(const uint8_t* Wq, int N, int K, uint8_t* Wk, bool inverse,
 int launch_quant_act(const __half* X, const float* s, const __half* LA, int M, int K, int r,
                      int8_t* Xq, float* a_scale, __nv_bfloat16* T, cudaStream_t st, int act_bits = 8,
                      bool t_pair = false, int M_pass = 0);
+// One launch for 33 to a few hundred tokens (act_mid.cu); quant_act_mid_prefers: where launch_quant_act takes it.
+bool quant_act_mid_prefers(int M, int K, int r);
+int launch_quant_act_mid(const __half* X, const float* s, const __half* LA, int M, int K, int r, int8_t* Xq, float* a_scale,
+                         __nv_bfloat16* T, int ldt, int lo_off, float qmax, cudaStream_t st);
 // The same with caller-provided scratch (quant_act_ws_scratch_bytes): the two-kernel path for more
 // than 32 tokens, ranks up to 512 (stacked down projections of layers that share X).
 size_t quant_act_ws_scratch_bytes(int M, int K, int r);

@@ -1222,6 +1222,7 @@ int launch_quant_act(const __half* X, const float* s, const __half* LA, int M, i
     }
     bool unsupported = false;
     if (M_pass == 0) M_pass = M;
+    if (quant_act_mid_prefers(M_pass, K, r)) return launch_quant_act_mid(X, s, LA, M, K, r, Xq, a_scale, T, ldt, lo_off, qmax, st);
     if (r > kTMaxRank && r <= 2 * kTMaxRank) {
         // Two launches of the cluster kernel, each for one half of L_A's rows and the matching
         // columns of T.  Both write the same codes and scales (the arithmetic is deterministic),

@@ -241,6 +241,34 @@ def test_quant_act_ws_dense_smoothing_and_6_bits(aser):
         assert_T_close(T.float().cpu().numpy(), F.down_proj(xs, L_A), xs, L_A)
 
 
+@pytest.mark.parametrize("entry,M,K,r,divided,act_bits,t_pair", [
+    # one launch (33 to a few hundred tokens): every cluster size and chunk count, one, two and four rows per CTA
+    ("one", 33, 128, 16, 1, 8, False), ("one", 129, 1152, 48, 3, 8, True), ("one", 600, 1024, 16, 10, 6, False),
+    ("one", 200, 2176, 64, 513, 8, False), ("one", 131, 4224, 80, 42, 8, False), ("one", 65, 8192, 32, 8192, 6, True),
+    ("one", 40, 14336, 112, 143, 8, False), ("one", 34, 28672, 16, 600, 8, False), ("one", 47, 512, 0, 5, 8, False)])
+def test_quant_act_beside_projection(aser, entry, M, K, r, divided, act_bits, t_pair):
+    """Codes and scales bit-exact and T within the derived bound where codes and T are made by different CTAs
+    (or kernels), with none, a few, a full list of and more divided columns than the list holds."""
+    rng = np.random.default_rng(7 * M + K + r)
+    X = rng.standard_normal((M, K)).astype(np.float16)
+    X[1] = 0
+    X[M - 1, :6] = np.array([127, .5, 1.5, 2.5, -2.5, -126.5], np.float16)
+    X[M - 1, 6:] = 0
+    s = np.ones(K, np.float32)
+    cols = rng.choice(K, divided, replace=False)
+    s[cols] = rng.uniform(0.02, 40.0, divided).astype(np.float32)
+    X[:, cols[:3]] *= np.float16(30)
+    L_A = synth.standin_factors(8, K, r, seed=M, scale_a=0.05)[0] if r else None
+    xs = F.smooth_act(X, s)
+    Xq_ref, sc_ref = F.quant_act(xs, act_bits=act_bits)
+    fn = aser.quant_act if entry == "one" else aser.quant_act_ws
+    Xq, sc, T = fn(to_dev(X), to_dev(s), None if L_A is None else to_dev(L_A), act_bits=act_bits, t_pair=t_pair)
+    assert np.array_equal(Xq.cpu().numpy(), Xq_ref)
+    assert np.array_equal(bits(sc.cpu().numpy()), bits(sc_ref))
+    if r:
+        assert_T_close(T[:, :r].float().cpu().numpy(), F.down_proj(xs, L_A), xs, L_A)
+
+
 # ---------------------------------------------------------------------------
 # whole path: quant_act -> linear
 # ---------------------------------------------------------------------------
