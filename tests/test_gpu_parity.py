@@ -245,7 +245,11 @@ def test_quant_act_ws_dense_smoothing_and_6_bits(aser):
     # one launch (33 to a few hundred tokens): every cluster size and chunk count, one, two and four rows per CTA
     ("one", 33, 128, 16, 1, 8, False), ("one", 129, 1152, 48, 3, 8, True), ("one", 600, 1024, 16, 10, 6, False),
     ("one", 200, 2176, 64, 513, 8, False), ("one", 131, 4224, 80, 42, 8, False), ("one", 65, 8192, 32, 8192, 6, True),
-    ("one", 40, 14336, 112, 143, 8, False), ("one", 34, 28672, 16, 600, 8, False), ("one", 47, 512, 0, 5, 8, False)])
+    ("one", 40, 14336, 112, 143, 8, False), ("one", 34, 28672, 16, 600, 8, False), ("one", 47, 512, 0, 5, 8, False),
+    # rows quantized beside the projection, and without one: every number of warps per row, ragged last rows
+    ("ws", 35, 128, 16, 2, 8, False), ("ws", 1201, 1152, 16, 70, 8, True), ("ws", 333, 4096, 144, 512, 8, False),
+    ("ws", 50, 4224, 16, 513, 6, False), ("ws", 1187, 8192, 32, 81, 8, False), ("ws", 305, 14336, 0, 143, 8, False),
+    ("ws", 37, 28672, 0, 28672, 8, False), ("ws", 2500, 640, 0, 0, 8, False)])
 def test_quant_act_beside_projection(aser, entry, M, K, r, divided, act_bits, t_pair):
     """Codes and scales bit-exact and T within the derived bound where codes and T are made by different CTAs
     (or kernels), with none, a few, a full list of and more divided columns than the list holds."""
