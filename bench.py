@@ -88,7 +88,7 @@ NCU_DRAM_BYTES_PER_LAUNCH = {
 def dominant_kernel(M, N, K):
     """Name of the kernel the library runs for the integer product at this shape, as it says itself."""
     import paper_2411_07762_b200 as aser
-    return ("linear_decode_kernel", "linear_tc_kernel", "linear_pair_kernel")[aser.lib.aser_linear_kernel(M, N, K)]
+    return ("linear_decode_kernel", "linear_tc_kernel", "linear_pair_kernel", "linear_split_kernel")[aser.lib.aser_linear_kernel(M, N, K)]
 
 
 def load_peaks():

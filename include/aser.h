@@ -160,8 +160,8 @@ int aser_quant_act_ws(const void* X_f16, const float* s, const void* LA_f16,
  * argument is validated all the same, so callers need not know which kernel serves a shape.
  * aser_linear_w4a8 is the same without the low-rank term (the plain W4A8 control).
  * aser_linear_kernel: which kernel serves a shape on the current device: 0 the streaming kernel, 1 the one whose CTAs
- * may share tiles through the workspace, 2 the one on pairs of CTAs; a negative error code for bad shapes.  The last two
- * give the same bits.
+ * may share tiles through the workspace, 2 the one on pairs of CTAs, 3 the one whose tiles are split along K over
+ * clusters; a negative error code for bad shapes.  The last three give the same bits.
  */
 int aser_linear_kernel(int M, int N, int K);
 int aser_linear_w4a8_lr(const int8_t* Xq, const float* a_scale, const void* Wk,

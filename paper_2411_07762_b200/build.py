@@ -13,7 +13,7 @@ INCLUDE = os.path.join(ROOT, "include")
 OBJ_DIR = os.path.join(_HERE, "_build")
 LIB = os.path.join(_HERE, "libaser.so")
 
-SOURCES = ["api.cu", "pack_w4.cu", "quant_act.cu", "act_mid.cu", "act_proj.cu", "linear_simt.cu", "linear_tc.cu", "linear_pair.cu",
+SOURCES = ["api.cu", "pack_w4.cu", "quant_act.cu", "act_mid.cu", "act_proj.cu", "linear_simt.cu", "linear_tc.cu", "linear_pair.cu", "linear_split.cu",
            "linear_decode.cu", "linear_static.cu", "construct.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]

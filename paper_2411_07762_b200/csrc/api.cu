@@ -118,9 +118,15 @@ int linear_common(const int8_t* Xq, const float* a_scale, const void* Wk, const 
                                     static_cast<const __half*>(LB_f16), M, N, K, r,
                                     static_cast<__half*>(Y_f16), acc_debug,
                                     static_cast<cudaStream_t>(stream), overlap_prev, ldt, cat);
-    if (linear_pair_prefers(M, N, K, cat)) {
-        rc = linear_tc_check(M, N, K, r, workspace_bytes);      // the limits are the same for both kernels
+    const bool split = linear_split_prefers(M, N, K);
+    if (split || linear_pair_prefers(M, N, K, cat)) {
+        rc = linear_tc_check(M, N, K, r, workspace_bytes);      // the limits are the same for all three kernels
         if (rc != ASER_OK) return rc;
+        if (split)
+            return launch_linear_split(Xq, a_scale, static_cast<const uint8_t*>(Wk), w_scale,
+                                       static_cast<const __nv_bfloat16*>(T_bf16), static_cast<const __half*>(LB_f16),
+                                       M, N, K, r, static_cast<__half*>(Y_f16), acc_debug, workspace,
+                                       static_cast<cudaStream_t>(stream), overlap_prev, ldt, cat);
         return launch_linear_pair(Xq, a_scale, static_cast<const uint8_t*>(Wk), w_scale,
                                   static_cast<const __nv_bfloat16*>(T_bf16), static_cast<const __half*>(LB_f16),
                                   M, N, K, r, static_cast<__half*>(Y_f16), acc_debug, workspace,
@@ -356,7 +362,7 @@ int aser_quant_act_ex(const void* X_f16, const float* s, const void* LA_f16, int
 
 int aser_linear_kernel(int M, int N, int K) {
     if (!shape_ok(M, N, K, 0) || M == 0 || N == 0) return ASER_ERR_SHAPE;
-    return linear_decode_prefers(M, N, K) ? 0 : linear_pair_prefers(M, N, K, CatSplit()) ? 2 : 1;
+    return linear_decode_prefers(M, N, K) ? 0 : linear_split_prefers(M, N, K) ? 3 : linear_pair_prefers(M, N, K, CatSplit()) ? 2 : 1;
 }
 
 int aser_linear_w4a8_lr(const int8_t* Xq, const float* a_scale, const void* Wk,

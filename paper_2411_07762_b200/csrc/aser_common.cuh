@@ -96,6 +96,11 @@ bool linear_pair_prefers(int M, int N, int K, const CatSplit& cat);
 int launch_linear_pair(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const float* w_scale,
                        const __nv_bfloat16* T, const __half* LB, int M, int N, int K, int r, __half* Y,
                        int32_t* acc_debug, void* workspace, cudaStream_t st, bool overlap_prev, int ldt, CatSplit cat);
+// Tiles split along K over clusters (linear_split.cu), 17 to 512 tokens; uses the workspace's status word only.
+bool linear_split_prefers(int M, int N, int K);
+int launch_linear_split(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const float* w_scale,
+                        const __nv_bfloat16* T, const __half* LB, int M, int N, int K, int r, __half* Y,
+                        int32_t* acc_debug, void* workspace, cudaStream_t st, bool overlap_prev, int ldt, CatSplit cat);
 // Estimated cycles of launch_linear_tc with 128-token tiles (M > 64): 530 per 128 x 128 x 128 unit of the
 // fullest CTA, and 8000 of fixed cost, or where tiles are shared between CTAs as much as 32 to 64 more units.
 long long linear_tc_estimate(int M, int N, int K, int num_sms);

@@ -390,6 +390,27 @@ def test_shared_tile_kernel_edges(aser, M, N, K, r):
     run_path(aser, lay, s, Wq, w_scale, L_A, L_B, "tc", timed_config=True, use_dgemm=True)
 
 
+SPLIT_CASES = [  # M, N, K, r: 17 to 512 tokens, a tile's slices of K in a cluster
+    (17, 520, 1024, 16),        # two CTAs of a cluster finish sixteen tokens each, the others none; ragged channels
+    (33, 18944, 1024, 64),      # as many tiles as SMs: not split
+    (64, 2056, 2176, 0),        # an odd number of column blocks, slices of unequal length
+    (101, 4104, 4096, 80),      # the last CTA of a cluster has fewer tokens to finish; two chunks, the second 16 wide
+    (128, 1160, 7168, 256),     # four chunks, eight slices
+    (257, 2048, 1152, 144),     # three token tiles, three chunks
+    (512, 1032, 1024, 128),     # four full token tiles
+]
+
+
+@pytest.mark.parametrize("M,N,K,r", SPLIT_CASES)
+def test_split_kernel_edges(aser, M, N, K, r):
+    assert aser.lib.aser_linear_kernel(M, N, K) == 3
+    lay = synth.make_layer(M, N, K, seed=990 + M + N + K + r, n_cal=16, n_out=max(1, K // 100))
+    s, Wq, w_scale, L_A, L_B = oracle_layer(lay, r, construct=False)
+    if r == 0:
+        L_A = L_B = None
+    run_path(aser, lay, s, Wq, w_scale, L_A, L_B, "tc", timed_config=True, use_dgemm=True)
+
+
 @pytest.mark.parametrize("M", [1, 8])
 @pytest.mark.parametrize("N,K,r", [(14336, 384, 128), (14344, 640, 0), (18944, 384, 16), (14216, 512, 64)])
 def test_streaming_kernel_four_ctas_per_sm(aser, M, N, K, r):
