@@ -32,7 +32,9 @@
 //
 // 4096 x 4096, 512 tokens, r = 64 took 236.8 ms with plain iteration on A, a 64 x 64 fma product
 // (157 ms), one thread per column in the triangular solves (46 ms) and one launch per Jacobi round
-// (11 ms); now 11.0 ms: Y and Z 5.8 (at 28 of 37 TFLOP/s), Cholesky factors 1.1, Jacobi 1.4.  2048 x
+// (11 ms); then 11.0 ms: Y and Z 5.8 (at 28 of 37 TFLOP/s), Cholesky factors 1.1, Jacobi 1.4; with the Gram matrix and its
+// factorisation beside the products of the next step, and a Jacobi round that keeps up the norms of its rows
+// instead of summing them, 9.8 ms (2000 x 1536, r = 16: 2.84 -> 2.51, 3000 x 3840, r = 48: 7.90 -> 6.71).  2048 x
 // 1024, r = 256: 784 -> 47 ms.
 #include "aser_common.cuh"
 #include "gemm64.cuh"
@@ -341,7 +343,7 @@ jacobi_round_kernel(double* __restrict__ Bt, int N, double* __restrict__ Qt, int
 // ---------------------------------------------------------------------------
 constexpr int kMaxP = 112;
 
-// H [p, p] symmetric -> Linv = L^-1 (lower, zeros above) with H = L L^T, and L itself if G is given.
+// H [p, p] symmetric (or `pieces` that add up to it, contiguous) -> Linv = L^-1 (lower, zeros above) with H = L L^T, and L itself if G is given.
 // 16 x 16 threads hold the matrix cyclically (row ti + 16 a, column tj + 16 b).  Elimination step j
 // needs row j alone (the multipliers of column j are its entries, by symmetry): its owners write it to
 // shared memory, then every thread updates its T x T entries; columns below j, done with, hold the
@@ -349,8 +351,9 @@ constexpr int kMaxP = 112;
 // barriers took 74 for each block of 64, and the inverse another 310).
 template <int T>
 __global__ void __launch_bounds__(256)
-chol_inverse_kernel(const double* __restrict__ H, long long ldh, int p, double* __restrict__ Linv, long long ldl,
+chol_inverse_kernel(const double* __restrict__ H, long long ldh, int p, int pieces, double* __restrict__ Linv, long long ldl,
                     double* __restrict__ G, long long ldg, int* __restrict__ fail) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // (only a launch made for it makes use of this)
     __shared__ double row[2][16 * T];
     __shared__ double piv[16 * T];
     const int ti = threadIdx.x >> 4, tj = threadIdx.x & 15;
@@ -362,6 +365,14 @@ chol_inverse_kernel(const double* __restrict__ H, long long ldh, int p, double* 
             const int i = ti + 16 * a, j = tj + 16 * b;
             w[a][b] = (i < p && j < p) ? H[(long long)i * ldh + j] : (i == j ? 1.0 : 0.0);
         }
+    for (int q = 1; q < pieces; ++q)         // H is the sum of its pieces, p * p apart
+#pragma unroll
+        for (int a = 0; a < T; ++a)
+#pragma unroll
+            for (int b = 0; b < T; ++b) {
+                const int i = ti + 16 * a, j = tj + 16 * b;
+                if (i < p && j < p) w[a][b] += H[(long long)q * p * p + (long long)i * ldh + j];
+            }
     bool bad = false;
 #pragma unroll
     for (int ja = 0; ja < T; ++ja) {
@@ -470,6 +481,7 @@ jacobi_kernel(double* __restrict__ G, double* __restrict__ V, int p) {
     extern __shared__ __align__(16) double jsm[];
     double* g = jsm;
     double* v = jsm + p * p;
+    __shared__ double sq[kMaxP];             // squared norms of the rows: summed at the start of a sweep, then kept up
     __shared__ int rotated;
     const int pair = threadIdx.x >> 4, lane = threadIdx.x & 15;
     for (int e = threadIdx.x; e < p * p; e += kJacobiThreads) { g[e] = G[e]; v[e] = (e / p == e % p) ? 1.0 : 0.0; }
@@ -477,6 +489,14 @@ jacobi_kernel(double* __restrict__ G, double* __restrict__ V, int p) {
     for (int sweep = 0; sweep < 20; ++sweep) {
         __syncthreads();
         if (threadIdx.x == 0) rotated = 0;
+        for (int i0 = 0; i0 < p; i0 += kJacobiThreads / 16) {
+            const int i = i0 + pair;
+            double a = 0.0;
+            if (i < p)
+                for (int k = lane; k < p; k += 16) a = fma(g[i * p + k], g[i * p + k], a);
+            for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (i < p && lane == 0) sq[i] = a;
+        }
         __syncthreads();
         for (int round = 0; round < m; ++round) {
             // round-robin tournament over p (even) players: player p - 1 stays, the others rotate
@@ -485,23 +505,22 @@ jacobi_kernel(double* __restrict__ G, double* __restrict__ V, int p) {
             const bool have = pair < p / 2;
             double* gi = g + i * p;
             double* gj = g + j * p;
-            double a = 0.0, b = 0.0, c = 0.0;
+            double c = 0.0;
             if (have)
-                for (int k = lane; k < p; k += 16) {
-                    const double x = gi[k], y = gj[k];
-                    a = fma(x, x, a); b = fma(y, y, b); c = fma(x, y, c);
-                }
-            for (int o = 8; o > 0; o >>= 1) {
-                a += __shfl_xor_sync(0xffffffffu, a, o);
-                b += __shfl_xor_sync(0xffffffffu, b, o);
-                c += __shfl_xor_sync(0xffffffffu, c, o);
-            }
+                for (int k = lane; k < p; k += 16) c = fma(gi[k], gj[k], c);
+            for (int o = 8; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+            const double a = have ? sq[i] : 0.0, b = have ? sq[j] : 0.0;
             if (have && c * c > 1e-28 * a * b) {
-                if (lane == 0) rotated = 1;
-                const float zeta = (float)((b - a) / (2.0 * c)), z = fabsf(zeta);
+                // (b - a) / 2c in fp32, both brought near 1 by the larger exponent
+                const double diff = b - a, twice = 2.0 * c;
+                const int top = max(__double2hiint(diff) & 0x7ff00000, __double2hiint(twice) & 0x7ff00000);
+                const double scale = __hiloint2double(min(max(0x7fe00000 - top, 0x00100000), 0x7fe00000), 0);
+                const float zeta = __fdividef((float)(diff * scale), (float)(twice * scale)), z = fabsf(zeta);
                 const float tf = z > 1e9f ? 0.5f / z : 1.f / (z + sqrtf(1.f + z * z));
                 const double t = zeta >= 0.f ? (double)tf : -(double)tf;
                 const double cs = rsqrt(1.0 + t * t), sn = cs * t;
+                __syncwarp(__activemask());
+                if (lane == 0) { rotated = 1; sq[i] = a - t * c; sq[j] = b + t * c; }
                 double* vi = v + i * p;
                 double* vj = v + j * p;
                 for (int k = lane; k < p; k += 16) {
@@ -573,6 +592,7 @@ constexpr int kSplitSms = 148;
 struct ConstructLayout {
     int p, tokens;                // tokens padded to 16 rows
     long long lda;                // columns of the wide error matrix, at most
+    int pieces;                   // of the Gram matrix that is made beside the products of the next step (0: p is too large)
     size_t A, E, G, Xs, T[4], Y, part, C, L, V, Vsel, sigma, row_sq, scalars, fail, Wm, total;     // byte offsets
 };
 
@@ -596,9 +616,13 @@ ConstructLayout construct_layout(int N, int K, int Tcal, int r, int n_split) {
     L.Xs = take((size_t)L.tokens * K * 8);
     for (int i = 0; i < 4; ++i) L.T[i] = take((size_t)p * N * 8);
     L.Y = take((size_t)p * wide * 8);
+    // as many pieces as the product beside it has splits, of k = N both
+    L.pieces = 0;
+    for (int q = 4; p <= 96 && q <= 16 && L.pieces == 0; q *= 2)
+        if (q == 16 || gemm64::split_count(p, wide, N, kSplitSms - q) <= q) L.pieces = q;
     size_t part = 0;
-    auto need = [&](int m, int n, int k) {
-        const size_t b = gemm64::partial_bytes(m, n, k, kSplitSms);
+    auto need = [&](int m, int n, int k, int sms = kSplitSms) {
+        const size_t b = gemm64::partial_bytes(m, n, k, sms);
         if (b > part) part = b;
     };
     need(N, L.tokens, K); need(N, K, K);
@@ -608,8 +632,9 @@ ConstructLayout construct_layout(int N, int K, int Tcal, int r, int n_split) {
         const int nb = p - i0 < kMaxP ? p - i0 : kMaxP;
         need(p - i0, kMaxP, kMaxP); need(p - i0, p - i0, kMaxP); need(nb, i0, i0); need(nb, i0, nb);
     }
+    for (int kc : {K, wide}) { need(p, kc, N, kSplitSms - L.pieces); need(p, N, kc, kSplitSms - 1); }
     L.part = take(part);
-    L.C = take((size_t)p * p * 8);
+    L.C = take((size_t)p * p * 8 * (L.pieces > 1 ? L.pieces : 1));
     L.L = take((size_t)p * p * 8);
     L.V = take((size_t)p * p * 8);
     L.Vsel = take((size_t)(r > 0 ? r : 1) * p * 8);
@@ -634,11 +659,12 @@ struct Ctx {
 // C[m, n] = a0 / *div * A B (+ a1 X1 + a2 X2)
 int product(const Ctx& c, bool tb, int m, int n, int k, const double* A, long long lda, const double* B, long long ldb,
             double* C, long long ldc, double a0 = 1.0, const double* div = nullptr, const double* X1 = nullptr, double a1 = 0.0,
-            const double* X2 = nullptr, double a2 = 0.0) {
+            const double* X2 = nullptr, double a2 = 0.0, int beside_ctas = 0) {
     gemm64::Args g = {};
     g.A = A; g.B = B; g.C = C; g.lda = lda; g.ldb = ldb; g.ldc = ldc; g.m = m; g.n = n; g.k = k;
     g.a0 = a0; g.a0_div = div; g.X1 = X1; g.a1 = a1; g.X2 = X2; g.a2 = a2;
-    return gemm64::run(g, tb, c.part, kSplitSms, c.st);
+    g.beside = beside_ctas > 0;                 // the launch before has this many SMs to itself
+    return gemm64::run(g, tb, c.part, kSplitSms - beside_ctas, c.st);
 }
 
 #define ASER_STEP(call)                        \
@@ -647,15 +673,16 @@ int product(const Ctx& c, bool tb, int m, int n, int k, const double* A, long lo
         if (step_rc != ASER_OK) return step_rc; \
     } while (0)
 
-int chol_inverse_block(const Ctx& c, const double* H, long long ldh, int p, double* Linv, long long ldl, double* G, long long ldg) {
+int chol_inverse_block(const Ctx& c, const double* H, long long ldh, int p, double* Linv, long long ldl, double* G, long long ldg,
+                       int pieces = 1) {
     switch ((p + 15) / 16) {
-        case 1: chol_inverse_kernel<1><<<1, 256, 0, c.st>>>(H, ldh, p, Linv, ldl, G, ldg, c.fail); break;
-        case 2: chol_inverse_kernel<2><<<1, 256, 0, c.st>>>(H, ldh, p, Linv, ldl, G, ldg, c.fail); break;
-        case 3: chol_inverse_kernel<3><<<1, 256, 0, c.st>>>(H, ldh, p, Linv, ldl, G, ldg, c.fail); break;
-        case 4: chol_inverse_kernel<4><<<1, 256, 0, c.st>>>(H, ldh, p, Linv, ldl, G, ldg, c.fail); break;
-        case 5: chol_inverse_kernel<5><<<1, 256, 0, c.st>>>(H, ldh, p, Linv, ldl, G, ldg, c.fail); break;
-        case 6: chol_inverse_kernel<6><<<1, 256, 0, c.st>>>(H, ldh, p, Linv, ldl, G, ldg, c.fail); break;
-        default: chol_inverse_kernel<7><<<1, 256, 0, c.st>>>(H, ldh, p, Linv, ldl, G, ldg, c.fail); break;
+        case 1: chol_inverse_kernel<1><<<1, 256, 0, c.st>>>(H, ldh, p, pieces, Linv, ldl, G, ldg, c.fail); break;
+        case 2: chol_inverse_kernel<2><<<1, 256, 0, c.st>>>(H, ldh, p, pieces, Linv, ldl, G, ldg, c.fail); break;
+        case 3: chol_inverse_kernel<3><<<1, 256, 0, c.st>>>(H, ldh, p, pieces, Linv, ldl, G, ldg, c.fail); break;
+        case 4: chol_inverse_kernel<4><<<1, 256, 0, c.st>>>(H, ldh, p, pieces, Linv, ldl, G, ldg, c.fail); break;
+        case 5: chol_inverse_kernel<5><<<1, 256, 0, c.st>>>(H, ldh, p, pieces, Linv, ldl, G, ldg, c.fail); break;
+        case 6: chol_inverse_kernel<6><<<1, 256, 0, c.st>>>(H, ldh, p, pieces, Linv, ldl, G, ldg, c.fail); break;
+        default: chol_inverse_kernel<7><<<1, 256, 0, c.st>>>(H, ldh, p, pieces, Linv, ldl, G, ldg, c.fail); break;
     }
     return check_launch("chol_inverse_kernel");
 }
@@ -749,10 +776,8 @@ int launch_construct(const __half* W, const float* s, const __half* Xcal, int N,
     // subspace iteration on A A^T with the basis as rows: t0 the current basis, t1 the term before it
     double *t0 = at(L.T[0]), *t1 = at(L.T[1]), *f0 = at(L.T[2]), *f1 = at(L.T[3]);
     auto swap = [](double*& x, double*& y) { double* t = x; x = y; y = t; };
-    // t0 <- L^-1 t0 with L L^T = t0 t0^T; the same factor applied to t1 if it is still needed
-    auto normalize = [&](bool both) {
-        ASER_STEP(product(ctx, true, p, p, N, t0, N, t0, N, C, p));
-        ASER_STEP(chol_inverse(ctx, C, p, Li, V));
+    // normalize: t0 <- L^-1 t0 with L L^T = t0 t0^T; apply: with the factor there is; the same to t1 if it is still needed
+    auto apply = [&](bool both) {
         gemm64::Args g = {};
         g.A = Li; g.lda = p; g.B = t0; g.ldb = N; g.C = f0; g.ldc = N; g.m = p; g.n = N; g.k = p; g.a0 = 1.0;
         if (both) { g.B2 = t1; g.C2 = f1; }
@@ -760,6 +785,11 @@ int launch_construct(const __half* W, const float* s, const __half* Xcal, int N,
         else { ASER_STEP(product(ctx, false, p, N, p, Li, p, t0, N, f0, N)); }
         swap(t0, f0);
         return (int)ASER_OK;
+    };
+    auto normalize = [&](bool both) {
+        ASER_STEP(product(ctx, true, p, p, N, t0, N, t0, N, C, p));
+        ASER_STEP(chol_inverse(ctx, C, p, Li, V));
+        return apply(both);
     };
     init_basis_kernel<<<blocks_for((long long)p * N, 256), 256, 0, st>>>(t0, (long long)p * N);
     ASER_STEP(normalize(false));
@@ -784,6 +814,22 @@ int launch_construct(const __half* W, const float* s, const __half* Xcal, int N,
     for (int cycle = 0; cycle < cycles; ++cycle) {
         const int steps = (iters - done) / (cycles - cycle);
         for (int i = 0; i < steps; ++i, ++done) {
+            if (i > 0 && L.pieces > 0) {
+                // The basis of the step before is still as its product left it.  Its Gram matrix is made beside the first
+                // product of this step and factorised beside the second (40 us of one CTA), then the factor is applied to both
+                // terms: the rows that the products see have the growth of one step, as their Gram matrix always had.
+                gemm64::Args h = {};
+                h.A = h.B = t0; h.lda = h.ldb = N; h.ldc = p; h.m = h.n = p; h.k = N; h.a0 = 1.0; h.side = true;
+                ASER_STEP(gemm64::run_pieces(h, C, L.pieces, st));
+                ASER_STEP(product(ctx, false, p, kc, N, t0, N, A, kc, Y, kc, 1.0, nullptr, nullptr, 0.0, nullptr, 0.0, L.pieces));
+                ASER_STEP(chol_inverse_block(ctx, C, p, p, Li, p, nullptr, p, L.pieces));
+                ASER_STEP(product(ctx, true, p, N, kc, Y, kc, A, kc, f0, N, 4.0, bound, t0, -2.0, t1, -1.0, 1));
+                swap(t1, f0);
+                swap(t0, t1);
+                ASER_STEP(apply(i + 1 < steps));
+                if (i + 1 == steps) ASER_STEP(normalize(false));
+                continue;
+            }
             ASER_STEP(product(ctx, false, p, kc, N, t0, N, A, kc, Y, kc));
             if (i == 0) {       // the basis is orthonormal here: Y Y^T holds its Ritz values
                 ASER_STEP(product(ctx, true, p, p, kc, Y, kc, Y, kc, C, p));
@@ -795,7 +841,7 @@ int launch_construct(const __half* W, const float* s, const __half* Xcal, int N,
             }
             swap(t1, f0);       // the new term to t1 ...
             swap(t0, t1);       // ... and into its place, the old basis behind it
-            ASER_STEP(normalize(i + 1 < steps));
+            if (L.pieces == 0 || i + 1 == steps) ASER_STEP(normalize(i + 1 < steps));
         }
     }
     ASER_STEP(normalize(false));

@@ -35,6 +35,8 @@ struct Args {
     const double *X1, *X2;           // [m, n] with pitch ldc, or null
     double a0, a1, a2;
     const double* a0_div;            // a0 is divided by *a0_div (or null)
+    bool side;                       // the launch after this one may run beside it
+    bool beside;                     // launched to run beside a side launch, and not over before that one is
 };
 
 template <int MT, bool TB>
@@ -52,6 +54,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const Args g) {
     constexpr int TM = 16 * MT;
     constexpr int kAElems = TM * kLdK, kBElems = TB ? kTN * kLdK : kTK * kLdN;
     extern __shared__ __align__(16) double sm[];
+    if (g.side) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
     const int n0 = blockIdx.x * kTN, m0 = blockIdx.y * TM;
     const int split = g.splits > 1 ? (int)blockIdx.z : 0;
@@ -157,6 +160,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const Args g) {
                 }
                 *reinterpret_cast<double2*>(Cp + o) = v;
             }
+    if (g.beside && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // C = a0 * (sum of the pieces, in order) + a1 X1 + a2 X2; C and X1, X2 have the pitch ldc.
@@ -225,8 +229,18 @@ int launch_mt(const Args& g, int batch, cudaStream_t st) {
         configured[dev] = true;
     }
     const dim3 grid((g.n + kTN - 1) / kTN, (g.m + 16 * MT - 1) / (16 * MT), g.splits > 1 ? g.splits : batch);
-    gemm_kernel<MT, TB><<<grid, kThreads, smem_bytes<MT, TB>(), st>>>(g);
-    return check_launch("gemm64");
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem_bytes<MT, TB>();
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = g.beside ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_kernel<MT, TB>, g);
+    return e == cudaSuccess ? (int)ASER_OK : record_cuda_error(e, "gemm64");
 }
 
 template <bool TB>
@@ -237,6 +251,15 @@ int launch_tb(const Args& g, int batch, cudaStream_t st) {
         case 5: return launch_mt<5, TB>(g, batch, st);
         default: return launch_mt<6, TB>(g, batch, st);
     }
+}
+
+// C = A B^T in `pieces` parts of k, raw, one after the other at `part` (pieces * m * n doubles): who reads them sums them in order.
+inline int run_pieces(Args g, double* part, int pieces, cudaStream_t st) {
+    const int steps = (g.k + kTK - 1) / kTK;
+    g.splits = pieces;
+    g.k_per_split = (steps + pieces - 1) / pieces * kTK;
+    g.C = part;
+    return launch_tb<true>(g, 1, st);
 }
 
 // n, k, all pitches even; pointers 16-byte aligned; `part` holds partial_bytes(m, n, k).  With
