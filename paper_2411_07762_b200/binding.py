@@ -386,7 +386,7 @@ class AserLinear:
                               self.T.data_ptr() if r else None, Y.data_ptr(), ws.data_ptr(), ws.numel(), _stream())
         if rc != 0:
             raise AserError(rc, "aser_forward")
-        return Y.narrow(0, 0, M)
+        return Y[:M]                       # (a slice: narrow costs a microsecond more)
 
     def forward_host(self, X_host: torch.Tensor, Y_host: torch.Tensor):
         """Host fp16 X [M,K] (pinned) -> host fp16 Y [M,N] through aser_forward_host."""
@@ -449,7 +449,7 @@ class AserSharedInput:
                                      self._LB, self._N, self._r, M, self.K, _ptr(self.Xq),
                                      _ptr(self.a_scale), _ptr(self.T) if self.r_total else None, self._Y,
                                      _ptr(self.ws), self.ws.numel(), _stream()), "aser_forward_shared")
-        return [y.narrow(0, 0, M) for y in self.Y]
+        return [y[:M] for y in self.Y]
 
 
 
