@@ -7,41 +7,41 @@ namespace aser {
 
 namespace {
 
-// A CTA quantizes whole rows, one after the other; thread t keeps the chunks t, t + TH, ... of a row
-// and their smoothing factors in registers, so W is read once and s once per CTA.  The next row is
-// loaded before the current one is reduced.  Codes: v * (1 / scale) is within 4e-6 of the quotient
-// (|quotient| <= 7), so its rounding is that of the IEEE quotient unless it lies within 1e-5 of a
-// tie; such chunks (one in ten thousand) are divided, as are rows with a scale whose reciprocal is
-// not safely a normal number.
-// HBM-bound by design: 2 K bytes in, K / 2 out per row.  28672 x 8192: 246 us with two passes over
-// the row, both multiplying by s from L1 and one dividing every element; 135 us now (4.3 TB/s).
+// Largest magnitude of three: a NaN does not count, or makes the result NaN.
+__device__ __forceinline__ float max3_abs(float a, float b, float c) {
+    float d;
+    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+__device__ __forceinline__ float max3_abs_nan(float a, float b, float c) {
+    float d;
+    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+// Low nibbles of four words, one after the other in sixteen bits.
+__device__ __forceinline__ uint32_t nibbles4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    uint32_t x = __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410) & 0x0F0F0F0Fu;
+    x = (x | (x >> 4)) & 0x00FF00FFu;
+    return (x | (x >> 8)) & 0x0000FFFFu;
+}
+
+// A CTA quantizes whole rows, one after the other; thread t takes the chunks t, t + TH, ... of a row, s
+// stays in shared memory, so W is read once and s once per CTA.  The next row is loaded before the current one
+// is reduced; the products w s are kept in registers between the maximum and the codes.  Codes: one fused multiply-add
+// v * (1 / scale) + 1.5 * 2^23 on packed fp32 pairs (the low nibble is the code), two more give the distance of the product
+// to its integer.  v * (1 / scale) is within 4e-6 of the quotient (|quotient| <= 7), so its rounding is that of the
+// IEEE quotient unless it lies within 1e-5 of a tie; such chunks (one in ten thousand), and those with a NaN, are
+// divided, as are rows with a scale whose reciprocal is not safely a normal number.
+// What bounds it is instruction issue as much as HBM (2 K bytes in, K / 2 out per row): 28672 x 8192 246 us with two
+// passes over the row, 134 with the row and s in registers, every step on single floats and the products made twice,
+// 123 now (4.8 TB/s); 4096 x 4096 14.0 -> 12.4.
 template <int TH, int V>
 __global__ void __launch_bounds__(TH)
 pack_w4_kernel(const __half* __restrict__ W, const float* __restrict__ s, int N, int K,
                uint8_t* __restrict__ Wq, float* __restrict__ w_scale) {
+    extern __shared__ float4 s_sm[];          // [K / 4]
     __shared__ float red[2][TH / 32];
     const int chunks = K / 8, tid = threadIdx.x;
-    constexpr bool kKeepS = V <= 4;           // else (rows above 16384) s is read again, from L1
-    float kept[kKeepS ? V : 1][8];
-    auto load_s = [&](int v, float (&f)[8]) {
-        const int c = tid + v * TH;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) f[i] = 1.f;
-        if (s && c < chunks) {
-            const float4 s0 = __ldg(reinterpret_cast<const float4*>(s + c * 8)), s1 = __ldg(reinterpret_cast<const float4*>(s + c * 8 + 4));
-            f[0] = s0.x; f[1] = s0.y; f[2] = s0.z; f[3] = s0.w;
-            f[4] = s1.x; f[5] = s1.y; f[6] = s1.z; f[7] = s1.w;
-        }
-    };
-    if constexpr (kKeepS) {
-#pragma unroll
-        for (int v = 0; v < V; ++v) load_s(v, kept[v]);
-    }
-    auto get_s = [&](int v, float (&f)[8]) {
-        if (!kKeepS) { load_s(v, f); return; }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) f[i] = kept[kKeepS ? v : 0][i];
-    };
     uint4 next[V];
     auto load = [&](int n) {
 #pragma unroll
@@ -52,24 +52,42 @@ pack_w4_kernel(const __half* __restrict__ W, const float* __restrict__ s, int N,
         }
     };
     load(blockIdx.x);
+    // Up to two chunks per thread s stays in registers (one barrier and one trip through shared memory less, which counts
+    // where a CTA has two rows: 1024 x 4096 6.5 -> 5.6 us), above that in shared memory (the two float4s of a chunk lie K / 8
+    // apart: consecutive threads read consecutive ones).
+    constexpr bool kKeepS = V <= 2;
+    float4 kept[kKeepS ? V : 1][2];
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        const int c = tid + v * TH;
+        float4 s0 = make_float4(1.f, 1.f, 1.f, 1.f), s1 = s0;
+        if (s && c < chunks) {
+            s0 = __ldg(reinterpret_cast<const float4*>(s) + 2 * c);
+            s1 = __ldg(reinterpret_cast<const float4*>(s) + 2 * c + 1);
+        }
+        if (kKeepS) { kept[kKeepS ? v : 0][0] = s0; kept[kKeepS ? v : 0][1] = s1; }
+        else if (c < chunks) { s_sm[c] = s0; s_sm[chunks + c] = s1; }
+    }
+    if (!kKeepS) __syncthreads();
     int buf = 0;
     for (int n = blockIdx.x; n < N; n += gridDim.x, buf ^= 1) {
-        uint4 raw[V];
+        float2 x[V][4];
         float amax = 0.f;
 #pragma unroll
-        for (int v = 0; v < V; ++v) raw[v] = next[v];
-        load(n + gridDim.x);
-#pragma unroll
         for (int v = 0; v < V; ++v) {
-            const __half2* h = reinterpret_cast<const __half2*>(&raw[v]);
-            float sv[8];
-            get_s(v, sv);
+            const int c = tid + v * TH;
+            float4 s0 = make_float4(1.f, 1.f, 1.f, 1.f), s1 = s0;
+            if (kKeepS) { s0 = kept[kKeepS ? v : 0][0]; s1 = kept[kKeepS ? v : 0][1]; }
+            else if (c < chunks) { s0 = s_sm[c]; s1 = s_sm[chunks + c]; }
+            const float2 sv[4] = {make_float2(s0.x, s0.y), make_float2(s0.z, s0.w), make_float2(s1.x, s1.y), make_float2(s1.z, s1.w)};
+            const __half2* h = reinterpret_cast<const __half2*>(&next[v]);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const float2 w = __half22float2(h[i]);          // s == NULL: times 1, exact
-                amax = fmaxf(amax, fmaxf(fabsf(__fmul_rn(w.x, sv[2 * i])), fabsf(__fmul_rn(w.y, sv[2 * i + 1]))));
+                x[v][i] = __fmul2_rn(__half22float2(h[i]), sv[i]);          // s == NULL: times 1, exact
+                amax = max3_abs(amax, x[v][i].x, x[v][i].y);
             }
         }
+        load(n + gridDim.x);
         amax = warp_max(amax);
         if ((tid & 31) == 0) red[buf][tid >> 5] = amax;
         __syncthreads();
@@ -80,32 +98,28 @@ pack_w4_kernel(const __half* __restrict__ W, const float* __restrict__ s, int N,
         if (tid == 0) w_scale[n] = sc;
         const bool divide = !(sc > 1e-30f && sc < 1e30f);
         const float inv = __fdiv_rn(1.f, sc);
+        const float2 inv2 = make_float2(inv, inv), m2 = make_float2(12582912.f, 12582912.f), neg1 = make_float2(-1.f, -1.f);
         uint32_t* out = reinterpret_cast<uint32_t*>(Wq + (size_t)n * (K / 2));
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             const int c = tid + v * TH;
-            const __half2* h = reinterpret_cast<const __half2*>(&raw[v]);
-            float sv[8];
-            get_s(v, sv);
-            constexpr float kMagic = 12582912.f;                // 1.5 * 2^23: rounds to an integer in the low bits
-            uint32_t word = 0;
-            bool near = true;                                   // every element within 0.49999 of its code (false for NaN)
+            uint32_t u[8];
+            float far = 0.f;                                                // largest distance to a code
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const float2 w = __half22float2(h[i]);
-                const float a = __fmul_rn(__fmul_rn(w.x, sv[2 * i]), inv), b = __fmul_rn(__fmul_rn(w.y, sv[2 * i + 1]), inv);
-                const float ra = __fadd_rn(a, kMagic), rb = __fadd_rn(b, kMagic);
-                near = near && fabsf(a - __fsub_rn(ra, kMagic)) < 0.49999f && fabsf(b - __fsub_rn(rb, kMagic)) < 0.49999f;
-                word |= (__float_as_uint(ra) & 0xFu) << (8 * i);         // column 2j -> low nibble of byte j
-                word |= (__float_as_uint(rb) & 0xFu) << (8 * i + 4);
+                const float2 su = __ffma2_rn(x[v][i], inv2, m2);
+                const float2 d = __ffma2_rn(x[v][i], inv2, __ffma2_rn(su, neg1, m2));
+                far = max3_abs_nan(far, d.x, d.y);
+                u[2 * i] = __float_as_uint(su.x);
+                u[2 * i + 1] = __float_as_uint(su.y);
             }
-            if (divide || !near) {
+            uint32_t word = nibbles4(u[0], u[1], u[2], u[3]) | (nibbles4(u[4], u[5], u[6], u[7]) << 16);
+            if (divide || !(far < 0.49999f)) {
                 word = 0;
-                const __half* e = reinterpret_cast<const __half*>(&raw[v]);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    const float x = __fmul_rn(__half2float(e[i]), sv[i]);
-                    const int q = amax > 0.f ? rne_clamp(__fdiv_rn(x, sc), -8.f, 7.f) : 0;
+                    const float f = i & 1 ? x[v][i >> 1].y : x[v][i >> 1].x;
+                    const int q = amax > 0.f ? rne_clamp(__fdiv_rn(f, sc), -8.f, 7.f) : 0;
                     word |= (uint32_t)(q & 0xF) << (4 * i);
                 }
             }
@@ -180,12 +194,14 @@ int launch_pack_cfg(const __half* W, const float* s, int N, int K, uint8_t* Wq, 
     if (rc != ASER_OK) return rc;
     if (resident[dev] == 0) {
         int per_sm = 0;
-        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pack_w4_kernel<TH, V>, TH, 0);
+        const int most = V <= 2 ? 0 : TH * V * 32;       // for the longest rows of this configuration: shared memory holds s
+        cudaError_t e = cudaFuncSetAttribute(pack_w4_kernel<TH, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pack_w4_kernel<TH, V>, TH, most);
         if (e != cudaSuccess || per_sm < 1) return record_cuda_error(e, "pack_w4 occupancy");
         resident[dev] = per_sm * sms;
     }
     const int grid = N < resident[dev] ? N : resident[dev];
-    pack_w4_kernel<TH, V><<<grid, TH, 0, st>>>(W, s, N, K, Wq, w_scale);
+    pack_w4_kernel<TH, V><<<grid, TH, V <= 2 ? 0 : (size_t)K * 4, st>>>(W, s, N, K, Wq, w_scale);
     return check_launch("pack_w4_kernel");
 }
 
