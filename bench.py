@@ -457,11 +457,14 @@ class Model:
     def launches_per_step(self):
         """Kernels of this library launched by one step: per input group the activation pass
         (as many kernels as the library says it runs at that shape) and one linear kernel per layer
-        (one per group where the group is stored fused)."""
+        (one per group where the group is stored fused, or where the streaming kernel or the one on CTA pairs
+        serves each of its two to four layers)."""
         n = 0
         for g, idx in self.members.items():
             K = self.w["layers"][idx[0]][1]
-            n += self.aser.forward_act_launches(self.M, K, self.r * len(idx)) + (1 if self.fused.get(g) else len(idx))
+            kernels = {self.aser.lib.aser_linear_kernel(self.M, self.w["layers"][i][2], K) for i in idx}
+            one = self.fused.get(g) or (2 <= len(idx) <= 4 and kernels in ({0}, {2}))
+            n += self.aser.forward_act_launches(self.M, K, self.r * len(idx)) + (1 if one else len(idx))
         return n
 
     def check(self):

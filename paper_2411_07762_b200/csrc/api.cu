@@ -557,7 +557,27 @@ int aser_forward_shared(const void* X_f16, const float* s, const void* LA_stacke
     rc = quant_with_workspace(X_f16, s, LA_stacked_f16, M, M, K, r_total, 8, false, Xq, a_scale, T_bf16,
                               workspace, workspace_bytes, stream);
     if (rc != ASER_OK) return rc;
+    // one launch for all layers where the kernel that serves each of them can (a launch has its start-up and a last, emptying
+    // wave)
     int col = 0;
+    if (n_layers > 1 && n_layers <= kMaxGroup) {
+        LinearGroup group = {};
+        group.layers = n_layers;
+        bool few = true;
+        for (int l = 0; l < n_layers; ++l) {
+            few = few && N[l] > 0 && linear_decode_prefers(M, N[l], K);
+            group.N[l] = N[l]; group.r[l] = r[l]; group.t_col[l] = col;
+            group.Wk[l] = static_cast<const uint8_t*>(Wk[l]); group.w_scale[l] = w_scale[l];
+            group.LB[l] = static_cast<const __half*>(LB_f16[l]); group.Y[l] = static_cast<__half*>(Y_f16[l]);
+            col += r[l];
+        }
+        const __nv_bfloat16* T = static_cast<const __nv_bfloat16*>(T_bf16);
+        cudaStream_t st = static_cast<cudaStream_t>(stream);
+        if (few) return launch_linear_decode_group(Xq, a_scale, T, M, K, group, nullptr, st, /*overlap_prev=*/true, r_total);
+        if (linear_pair_groups(group, M, K))
+            return launch_linear_pair_group(Xq, a_scale, T, M, K, group, nullptr, workspace, st, /*overlap_prev=*/true, r_total);
+        col = 0;
+    }
     for (int l = 0; l < n_layers; ++l) {
         const void* Tl = r[l] > 0 ? static_cast<const void*>(static_cast<const __nv_bfloat16*>(T_bf16) + col) : nullptr;
         rc = linear_common(Xq, a_scale, Wk[l], w_scale[l], Tl, r[l] > 0 ? LB_f16[l] : nullptr, M, N[l], K,

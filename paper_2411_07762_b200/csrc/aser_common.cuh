@@ -80,6 +80,17 @@ int launch_linear_tc(const int8_t* Xq, const float* a_scale, const uint8_t* Wk,
                      int M, int N, int K, int r, __half* Y, int32_t* acc_debug,
                      void* workspace, size_t workspace_bytes, cudaStream_t st,
                      bool overlap_prev = false, int ldt = 0, CatSplit cat = CatSplit());
+// Layers that read the same codes, each with operands of its own, served by one launch; layer l takes the columns
+// [t_col, t_col + r) of T.
+constexpr int kMaxGroup = 4;
+struct LinearGroup {
+    int layers;
+    int N[kMaxGroup], r[kMaxGroup], t_col[kMaxGroup];
+    const uint8_t* Wk[kMaxGroup];
+    const float* w_scale[kMaxGroup];
+    const __half* LB[kMaxGroup];
+    __half* Y[kMaxGroup];
+};
 // Few-token kernel (M <= kLinearDecodeMaxTokens): streams the weights once, no workspace.
 // linear_decode_prefers: the shapes for which it is faster than the tensor-core kernel.
 constexpr int kLinearDecodeMaxTokens = 16;
@@ -88,6 +99,9 @@ int launch_linear_decode(const int8_t* Xq, const float* a_scale, const uint8_t* 
                          const float* w_scale, const __nv_bfloat16* T, const __half* LB,
                          int M, int N, int K, int r, __half* Y, int32_t* acc_debug,
                          cudaStream_t st, bool overlap_prev = false, int ldt = 0, CatSplit cat = CatSplit());
+int launch_linear_decode_group(const int8_t* Xq, const float* a_scale, const __nv_bfloat16* T, int M, int K,
+                               const LinearGroup& group, int32_t* acc_debug, cudaStream_t st, bool overlap_prev, int ldt,
+                               CatSplit cat = CatSplit());
 // Many-token kernel on pairs of CTAs (linear_pair.cu); uses the workspace's status word only.
 // linear_pair_prefers: the shapes for which it is faster than linear_tc (estimates of both, in cycles), where it can
 // run at all.  To be asked before every launch: it also sets the kernel up on its first yes.
@@ -96,6 +110,11 @@ bool linear_pair_prefers(int M, int N, int K, const CatSplit& cat);
 int launch_linear_pair(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const float* w_scale,
                        const __nv_bfloat16* T, const __half* LB, int M, int N, int K, int r, __half* Y,
                        int32_t* acc_debug, void* workspace, cudaStream_t st, bool overlap_prev, int ldt, CatSplit cat);
+// linear_pair_groups: whether one launch serves these layers (it also sets the kernel up on its first yes).
+bool linear_pair_groups(const LinearGroup& g, int M, int K);
+int launch_linear_pair_group(const int8_t* Xq, const float* a_scale, const __nv_bfloat16* T, int M, int K, const LinearGroup& g,
+                             int32_t* acc_debug, void* workspace, cudaStream_t st, bool overlap_prev, int ldt,
+                             CatSplit cat = CatSplit());
 // Tiles split along K over clusters (linear_split.cu), 17 to 512 tokens; uses the workspace's status word only.
 bool linear_split_prefers(int M, int N, int K);
 int launch_linear_split(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const float* w_scale,

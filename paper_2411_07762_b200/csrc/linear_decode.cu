@@ -86,10 +86,8 @@ struct DecCfg {
 
 template <int NT, int R, int B>
 __global__ void __launch_bounds__(kDecThreads, DecCfg<NT, R, B>::MinCtas)
-linear_decode_kernel(const int8_t* Xq, const float* a_scale, const uint8_t* __restrict__ Wk,
-                     const float* __restrict__ w_scale, const __nv_bfloat16* T,
-                     const __half* __restrict__ LB, int M, int N, int K, int r, int ldt,
-                     __half* __restrict__ Y, int32_t* __restrict__ acc_debug, const CatSplit cat) {
+linear_decode_kernel(const int8_t* Xq, const float* a_scale, const __nv_bfloat16* T, int M, int K, int ldt,
+                     int32_t* __restrict__ acc_debug, const CatSplit cat, const __grid_constant__ LinearGroup group) {
     using C = DecCfg<NT, R, B>;
     constexpr int BATCH = C::Batch;
     // partial sums of the eight warps: integer accumulators and fp32 accumulators of the low-rank term
@@ -98,8 +96,20 @@ linear_decode_kernel(const int8_t* Xq, const float* a_scale, const uint8_t* __re
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;       // fragment row group / k quarter
     const int KB = K / kWkCols;
-    const int n0 = blockIdx.x * C::Rows;
-    T += cat_layer(cat, n0) * r;        // a CTA's rows lie inside one layer (16 R divides 128)
+    // this CTA's layer of the group, and its rows there (layers that share their input are one launch: a launch has its
+    // start-up and a last, emptying wave)
+    int first = 0, layer = 0;
+#pragma unroll
+    for (int l = 1; l < kMaxGroup; ++l) {
+        const int next = first + (group.N[l - 1] + C::Rows - 1) / C::Rows;
+        if (layer == l - 1 && l < group.layers && (int)blockIdx.x >= next) { layer = l; first = next; }
+    }
+    const uint8_t* __restrict__ Wk = group.Wk[layer];
+    const float* __restrict__ w_scale = group.w_scale[layer];
+    const __half* __restrict__ LB = group.LB[layer];
+    __half* __restrict__ Y = group.Y[layer];
+    const int N = group.N[layer], r = group.r[layer], n0 = ((int)blockIdx.x - first) * C::Rows;
+    T += group.t_col[layer] + cat_layer(cat, n0) * r;        // a CTA's rows lie inside one layer (16 R divides 128)
     // Rows n0 + 16 rt + g and + 8 of sub-block t (columns 32 t .. 32 t + 31 of a block).  The
     // blocked layout pads the last 128-row tile with zero codes, so rows past N inside that tile
     // read as zeros; a CTA never reaches past the tile (16 R divides 128).
@@ -273,11 +283,12 @@ linear_decode_kernel(const int8_t* Xq, const float* a_scale, const uint8_t* __re
 }
 
 template <int NT, int R, int B>
-int launch_cfg(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const float* w_scale,
-               const __nv_bfloat16* T, const __half* LB, int M, int N, int K, int r, __half* Y,
-               int32_t* acc_debug, cudaStream_t st, bool overlap_prev, int ldt, CatSplit cat) {
+int launch_cfg(const int8_t* Xq, const float* a_scale, const __nv_bfloat16* T, int M, int K, int32_t* acc_debug,
+               cudaStream_t st, bool overlap_prev, int ldt, const CatSplit& cat, const LinearGroup& group) {
+    int tiles = 0;
+    for (int l = 0; l < group.layers; ++l) tiles += (group.N[l] + DecCfg<NT, R, B>::Rows - 1) / DecCfg<NT, R, B>::Rows;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((N + DecCfg<NT, R, B>::Rows - 1) / DecCfg<NT, R, B>::Rows, 1, 1);
+    cfg.gridDim = dim3(tiles, 1, 1);
     cfg.blockDim = dim3(kDecThreads, 1, 1);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = st;
@@ -286,16 +297,14 @@ int launch_cfg(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = overlap_prev ? 1 : 0;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, linear_decode_kernel<NT, R, B>, Xq, a_scale, Wk, w_scale, T, LB,
-                                       M, N, K, r, ldt, Y, acc_debug, cat);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, linear_decode_kernel<NT, R, B>, Xq, a_scale, T, M, K, ldt, acc_debug, cat, group);
     if (e != cudaSuccess) return record_cuda_error(e, "linear_decode_kernel");
     return check_launch("linear_decode_kernel");
 }
 
 template <int NT>
-int launch_nt(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const float* w_scale,
-              const __nv_bfloat16* T, const __half* LB, int M, int N, int K, int r, __half* Y,
-              int32_t* acc_debug, cudaStream_t st, bool overlap_prev, int ldt, CatSplit cat) {
+int launch_nt(const int8_t* Xq, const float* a_scale, const __nv_bfloat16* T, int M, int K, int32_t* acc_debug,
+              cudaStream_t st, bool overlap_prev, int ldt, const CatSplit& cat, const LinearGroup& group) {
     // Rows per CTA: 32 where that still gives every SM about one and a half CTAs (activation
     // fragments reused twice), else 16 (few output channels: latency matters, every SM gets work).
     int num_sms = 0;
@@ -310,12 +319,13 @@ int launch_nt(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const f
     // too many for three CTAs per SM, four with half the bytes in flight each take them in one wave (kernel alone, one /
     // eight tokens: 14336 x 4096, 448 tiles for 444 places, 11.5 / 11.5 -> 7.6 / 8.9 us; 16384 x 1024, 512 tiles, 6.5 / 6.3 -> 4.5 /
     // 4.8).
-    const int tiles = (N + 31) / 32;
+    int tiles = 0, rows = 0;
+    for (int l = 0; l < group.layers; ++l) { tiles += (group.N[l] + 31) / 32; rows += group.N[l]; }
     if (NT == 1 && tiles > 3 * num_sms && tiles <= 4 * num_sms)
-        return launch_cfg<1, 2, 1>(Xq, a_scale, Wk, w_scale, T, LB, M, N, K, r, Y, acc_debug, st, overlap_prev, ldt, cat);
-    if (N >= 32 * 3 * num_sms / 2)
-        return launch_cfg<NT, 2, 2>(Xq, a_scale, Wk, w_scale, T, LB, M, N, K, r, Y, acc_debug, st, overlap_prev, ldt, cat);
-    return launch_cfg<NT, 1, 4>(Xq, a_scale, Wk, w_scale, T, LB, M, N, K, r, Y, acc_debug, st, overlap_prev, ldt, cat);
+        return launch_cfg<1, 2, 1>(Xq, a_scale, T, M, K, acc_debug, st, overlap_prev, ldt, cat, group);
+    if (rows >= 32 * 3 * num_sms / 2)
+        return launch_cfg<NT, 2, 2>(Xq, a_scale, T, M, K, acc_debug, st, overlap_prev, ldt, cat, group);
+    return launch_cfg<NT, 1, 4>(Xq, a_scale, T, M, K, acc_debug, st, overlap_prev, ldt, cat, group);
 }
 
 }  // namespace
@@ -324,14 +334,24 @@ bool linear_decode_prefers(int M, int N, int K) {
     return M <= kLinearDecodeMaxTokens && (long long)N * K / 2 <= (64ll << 20);
 }
 
+int launch_linear_decode_group(const int8_t* Xq, const float* a_scale, const __nv_bfloat16* T, int M, int K,
+                               const LinearGroup& group, int32_t* acc_debug, cudaStream_t st, bool overlap_prev, int ldt,
+                               CatSplit cat) {
+    if (M > kLinearDecodeMaxTokens) return record_error(ASER_ERR_SHAPE, "linear_decode: more than 16 tokens");
+    if (M <= 8) return launch_nt<1>(Xq, a_scale, T, M, K, acc_debug, st, overlap_prev, ldt, cat, group);
+    return launch_nt<2>(Xq, a_scale, T, M, K, acc_debug, st, overlap_prev, ldt, cat, group);
+}
+
 int launch_linear_decode(const int8_t* Xq, const float* a_scale, const uint8_t* Wk,
                          const float* w_scale, const __nv_bfloat16* T, const __half* LB,
                          int M, int N, int K, int r, __half* Y, int32_t* acc_debug,
                          cudaStream_t st, bool overlap_prev, int ldt, CatSplit cat) {
     if (ldt <= 0) ldt = r * cat.layers;
-    if (M > kLinearDecodeMaxTokens) return record_error(ASER_ERR_SHAPE, "linear_decode: more than 16 tokens");
-    if (M <= 8) return launch_nt<1>(Xq, a_scale, Wk, w_scale, T, LB, M, N, K, r, Y, acc_debug, st, overlap_prev, ldt, cat);
-    return launch_nt<2>(Xq, a_scale, Wk, w_scale, T, LB, M, N, K, r, Y, acc_debug, st, overlap_prev, ldt, cat);
+    LinearGroup group = {};
+    group.layers = 1;
+    group.Wk[0] = Wk; group.w_scale[0] = w_scale; group.LB[0] = LB; group.Y[0] = Y;
+    group.N[0] = N; group.r[0] = r;
+    return launch_linear_decode_group(Xq, a_scale, T, M, K, group, acc_debug, st, overlap_prev, ldt, cat);
 }
 
 }  // namespace aser

@@ -84,23 +84,27 @@ static_assert(kNumBars * 8 + 8 <= 256, "barrier area");
 constexpr int kEpiWarps = 8, kEpiThreads = 256;
 
 struct Params {
-    const uint8_t* Wk;
+    LinearGroup g;         // one layer, or (GROUP) several of one rank
+    int tile0[kMaxGroup];  // first tile of 256 rows of each layer
     const float* a_scale;
-    const float* w_scale;
     int32_t* acc_debug;
     uint32_t* status;
-    int M, N, r;
-    int KB, NB;            // 128-column blocks, 128-row blocks
+    int M, r;
+    int KB;                // 128-column blocks
     int NT, TT;            // tiles of 256 rows, whole token columns (see Plan)
     int full, cut, items;  // items [0, full): whole tiles; [full, full + 2 cut): the halves of further tiles; then the short ones
     int tt_outer;          // tile numbering: 1 = token tile outer
     CatSplit cat;
 };
 
+struct Maps { CUtensorMap lb[kMaxGroup], y[kMaxGroup]; };
+
 // `step` tokens lie between the rows of the two CTAs: a whole tile's tokens are [CTA][half][rows], a
 // single half's [CTA][rows].
-struct Item { int nt, tok0, halves, step; };
+// nt is the tile inside its layer.
+struct Item { int nt, tok0, halves, step, layer; };
 
+template <bool GROUP>
 __device__ __forceinline__ Item get_item(const Params& p, int i) {
     Item w;
     int tt, part = 0;
@@ -117,6 +121,13 @@ __device__ __forceinline__ Item get_item(const Params& p, int i) {
     w.tok0 = (2 * tt + part) * kHalf;
     w.halves = single ? 1 : 2;
     w.step = single ? kHw : kHalf;
+    w.layer = 0;
+    if (GROUP) {
+#pragma unroll
+        for (int l = 1; l < kMaxGroup; ++l)
+            if (l < p.g.layers && w.nt >= p.tile0[l]) w.layer = l;
+        w.nt -= p.tile0[w.layer];
+    }
     return w;
 }
 
@@ -163,11 +174,10 @@ __device__ __forceinline__ void let_copies_land() {
     while (clock64() - t0 < 2000000) {}
 }
 
-template <bool DEBUG_ACC>
+template <bool DEBUG_ACC, bool GROUP>
 __global__ void __launch_bounds__(kThreads, 1)
-linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_lb,
-                   const __grid_constant__ CUtensorMap map_t, const __grid_constant__ CUtensorMap map_y,
-                   const Params p) {
+linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_t,
+                   const __grid_constant__ Maps maps, const __grid_constant__ Params p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t sbase = smem_u32(smem), bar0 = sbase + kOffBar;
@@ -182,9 +192,11 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     const int stages = (p.KB + kKS - 1) / kKS;      // per item
 
     auto weights_of = [&](int item) {
-        int nb = 2 * get_item(p, item).nt + (int)rank;
-        if (nb >= p.NB) nb = p.NB - 1;             // rows past N: any weights, the results are dropped
-        return p.Wk + (size_t)nb * p.KB * kWkBlockBytes;
+        const Item w = get_item<GROUP>(p, item);
+        const int NB = (p.g.N[w.layer] + kWkRows - 1) / kWkRows;
+        int nb = 2 * w.nt + (int)rank;
+        if (nb >= NB) nb = NB - 1;                 // rows past N: any weights, the results are dropped
+        return p.g.Wk[w.layer] + (size_t)nb * p.KB * kWkBlockBytes;
     };
     auto load_weights = [&](const uint8_t* src, int kb, uint32_t s) {
         const uint32_t bytes = (p.KB - kb < kKS ? p.KB - kb : kKS) * kWkBlockBytes;
@@ -217,8 +229,8 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     }
     if (warp == 1 && lane == 0) {
         prefetch_tensormap(&map_x);
-        prefetch_tensormap(&map_y);
-        if (p.r > 0) { prefetch_tensormap(&map_lb); prefetch_tensormap(&map_t); }
+        prefetch_tensormap(&maps.y[0]);
+        if (p.r > 0) { prefetch_tensormap(&maps.lb[0]); prefetch_tensormap(&map_t); }
     }
     tc_fence_before();
     __syncthreads();
@@ -251,7 +263,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             uint32_t c = 0;
             bool ok = true;
             for (int i = pair; i < p.items && ok; i += pairs) {
-                const Item w = get_item(p, i);
+                const Item w = get_item<GROUP>(p, i);
                 for (int kb = 0; kb < p.KB; kb += kKS, ++c) {
                     const uint32_t s = c % kNS;
                     ok = wait(bar(B_FREE + s), ((c / kNS) & 1) ^ 1, stop);
@@ -284,7 +296,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                 }
             };
             for (int i = pair; i < p.items && ok; i += pairs) {
-                const Item w = get_item(p, i);
+                const Item w = get_item<GROUP>(p, i);
                 const bool mine = h < w.halves;
                 if (mine) ok = wait(bar(B_ACC_EMPTY + h), (done & 1) ^ 1, stop);
                 if (!ok) break;
@@ -401,13 +413,13 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         grid_dep_wait();           // a_scale and T come from the kernel launched before this one
         // a set of low-rank operands: chunks [c0, c1), T of the halves in the mask (one thread)
         auto load_set = [&](const Item& w, int c0, int c1, int mask) {
-            const int row0 = (2 * w.nt + (int)rank) * 128, layer = cat_layer(p.cat, w.nt * 256) * p.r;
+            const int row0 = (2 * w.nt + (int)rank) * 128, t_col = p.g.t_col[w.layer] + cat_layer(p.cat, w.nt * 256) * p.r;
             mbar_arrive_expect_tx(bar(B_LR_FULL), (c1 - c0) * (kLbBytes + ((mask & 1) + (mask >> 1)) * kHw * 128));
             for (int c = c0; c < c1; ++c) {
-                tma_load_2d(sbase + kOffLr + (c & 1) * kLbBytes, &map_lb, c * 64, row0, bar(B_LR_FULL));
+                tma_load_2d(sbase + kOffLr + (c & 1) * kLbBytes, &maps.lb[w.layer], c * 64, row0, bar(B_LR_FULL));
                 for (int h = 0; h < 2; ++h)
                     if (mask >> h & 1)
-                        tma_load_2d(sbase + kOffT + (h * 2 + (c & 1)) * kTBytes, &map_t, c * 64 + layer,
+                        tma_load_2d(sbase + kOffT + (h * 2 + (c & 1)) * kTBytes, &map_t, c * 64 + t_col,
                                     w.tok0 + (int)rank * w.step + h * kHw, bar(B_LR_FULL));
             }
         };
@@ -444,16 +456,16 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             return true;
         };
         int i = pair;
-        Item w = {0, 0, 0, 0};
-        if (i < p.items) w = get_item(p, i);
+        Item w = {};
+        if (i < p.items) w = get_item<GROUP>(p, i);
         if (chunks > 0 && i < p.items && et == 0) load_first(w);
         while (i < p.items && ok) {
             // the item after this one (its first operands are loaded as soon as their place is free)
             const int i_next = i + pairs;
-            Item next = {0, 0, 0, 0};
-            if (i_next < p.items) next = get_item(p, i_next);
-            const int n0 = (2 * w.nt + (int)rank) * 128, n = n0 + q * 32 + lane;
-            const float ws16 = (n < p.N ? __ldg(p.w_scale + n) : 0.f) * 0.0625f;      // the sums hold 16 q x
+            Item next = {};
+            if (i_next < p.items) next = get_item<GROUP>(p, i_next);
+            const int n0 = (2 * w.nt + (int)rank) * 128, n = n0 + q * 32 + lane, N = p.g.N[w.layer];
+            const float ws16 = (n < N ? __ldg(p.g.w_scale[w.layer] + n) : 0.f) * 0.0625f;      // the sums hold 16 q x
             {   // token scales in the order of the accumulator's columns: [half][CTA][rows]
                 const int h = et >= kHalf ? 1 : 0, col = et - h * kHalf, cta = col >= kHw ? 1 : 0;
                 const int tok = w.tok0 + cta * w.step + h * kHw + (col - cta * kHw);
@@ -494,8 +506,8 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                         for (int c = 0; c < 4; ++c)
 #pragma unroll
                             for (int j = 0; j < 16; ++j)
-                                if (tok + c * 16 + j < p.M && n < p.N)
-                                    p.acc_debug[(size_t)(tok + c * 16 + j) * p.N + n] = ((int)v[c][j]) >> 4;
+                                if (tok + c * 16 + j < p.M && n < N)
+                                    p.acc_debug[(size_t)(tok + c * 16 + j) * N + n] = ((int)v[c][j]) >> 4;
                     }
                 }
                 if (chunks > 2) {
@@ -563,10 +575,10 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             ok = named_bar_all(1, kEpiThreads, ok);
             if (!ok) break;
             if (et == 0) {
-                if (n0 < p.N) {
+                if (n0 < N) {
                     for (int b = 0; b < 2 * w.halves; ++b) {
                         const int tok = w.tok0 + (b & 1) * w.step + (b >> 1) * kHw;
-                        if (tok < p.M) tma_store_2d_tile(&map_y, n0, tok, sbase + kOffLr + b * kHw * kYRow);
+                        if (tok < p.M) tma_store_2d_tile(&maps.y[w.layer], n0, tok, sbase + kOffLr + b * kHw * kYRow);
                     }
                     bulk_store_commit();
                     bulk_store_wait_read();
@@ -602,10 +614,10 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
 // spread over the stages; narrower tiles, bound by the unpacking, cost no less).
 struct Plan { int NT, TT, full, cut, items; long long cost; };
 
-Plan make_plan(int M, int N, int pairs) {
+Plan make_plan(int M, int NT, int pairs) {
     constexpr long long whole = 1500, single = 1300;
     const int columns = (M + 2 * kHalf - 1) / (2 * kHalf), last = M - (columns - 1) * 2 * kHalf;
-    const int NT = (N + 255) / 256, TT = last <= kHalf ? columns - 1 : columns, tiles = NT * TT;
+    const int TT = last <= kHalf ? columns - 1 : columns, tiles = NT * TT;
     const int shorts = last <= kHalf ? NT : 0;
     Plan best = {};
     for (int cut = 0; cut <= 1; ++cut) {
@@ -627,14 +639,14 @@ Plan make_plan(int M, int N, int pairs) {
 
 // Whether the kernel can run as it was built: the warpgroups' budgets add up to what the block is launched with and to
 // nothing else, so a compiler that gives a thread another number of registers leaves every shape to linear_tc.
-template <bool DEBUG_ACC>
+template <bool DEBUG_ACC, bool GROUP>
 bool configure(int dev) {
     static int state[kMaxDevices] = {0};         // 1: ready, 2: not usable
     if (state[dev] == 0) {
         cudaFuncAttributes a;
-        cudaError_t e = cudaFuncGetAttributes(&a, linear_pair_kernel<DEBUG_ACC>);
+        cudaError_t e = cudaFuncGetAttributes(&a, linear_pair_kernel<DEBUG_ACC, GROUP>);
         const bool fits = e == cudaSuccess && a.numRegs == kRegsLaunch;
-        if (fits) e = cudaFuncSetAttribute(linear_pair_kernel<DEBUG_ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+        if (fits) e = cudaFuncSetAttribute(linear_pair_kernel<DEBUG_ACC, GROUP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
         if (e != cudaSuccess) (void)cudaGetLastError();
         state[dev] = fits && e == cudaSuccess ? 1 : 2;
     }
@@ -656,41 +668,64 @@ bool linear_pair_prefers(int M, int N, int K, const CatSplit& cat) {
     int num_sms = 0, dev = 0;
     if (device_sm_count(&num_sms) != ASER_OK || num_sms < 2 || current_device(&dev) != ASER_OK) return false;
     const long long stages = (K / kWkCols + kKS - 1) / kKS;
-    if (make_plan(M, N, num_sms / 2).cost * stages + 12000 >= linear_tc_estimate(M, N, K, num_sms)) return false;
-    return configure<false>(dev) && configure<true>(dev);
+    if (make_plan(M, (N + 255) / 256, num_sms / 2).cost * stages + 12000 >= linear_tc_estimate(M, N, K, num_sms)) return false;
+    return configure<false, false>(dev) && configure<true, false>(dev);
 }
 
-int launch_linear_pair(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const float* w_scale,
-                       const __nv_bfloat16* T, const __half* LB, int M, int N, int K, int r, __half* Y,
-                       int32_t* acc_debug, void* workspace, cudaStream_t st, bool overlap_prev, int ldt, CatSplit cat) {
+// Layers that would each be served by this kernel, of one rank: one launch deals the tiles of all of them (two layers of 14336 x
+// 4096, 333 tokens: 56 whole and 56 half tiles each on 74 pairs, so a whole and a half for the busiest pair, twice; together
+// 112 and 112, three items at most).
+bool linear_pair_groups(const LinearGroup& g, int M, int K) {
+    int dev = 0;
+    if (g.layers < 2 || g.layers > kMaxGroup || current_device(&dev) != ASER_OK) return false;
+    for (int l = 0; l < g.layers; ++l)
+        if (g.r[l] != g.r[0] || g.N[l] <= 0 || linear_split_prefers(M, g.N[l], K) || !linear_pair_prefers(M, g.N[l], K, CatSplit()))
+            return false;
+    return configure<false, true>(dev);
+}
+
+int launch_linear_pair_group(const int8_t* Xq, const float* a_scale, const __nv_bfloat16* T, int M, int K, const LinearGroup& g,
+                             int32_t* acc_debug, void* workspace, cudaStream_t st, bool overlap_prev, int ldt, CatSplit cat) {
     int num_sms = 0;
     int rc = device_sm_count(&num_sms);
     if (rc != ASER_OK) return rc;
-    const int pairs = num_sms / 2 > 0 ? num_sms / 2 : 1;
-    const Plan plan = make_plan(M, N, pairs);
-    CUtensorMap mx, mlb, mt, my;
-    rc = encode_map_2d(&my, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, Y, M, N, kHw, 128, CU_TENSOR_MAP_SWIZZLE_NONE);
-    if (rc != ASER_OK) return rc;
+    const int pairs = num_sms / 2 > 0 ? num_sms / 2 : 1, r = g.r[0];
+    Params p = {};
+    p.g = g;
+    int NT = 0, t_cols = 0;
+    long long rows = 0;
+    for (int l = 0; l < g.layers; ++l) {
+        p.tile0[l] = NT;
+        NT += (g.N[l] + 255) / 256;
+        rows += g.N[l];
+        if (g.t_col[l] + r * cat.layers > t_cols) t_cols = g.t_col[l] + r * cat.layers;
+    }
+    const Plan plan = make_plan(M, NT, pairs);
+    CUtensorMap mx, mt;
+    Maps maps;
     rc = encode_map_blocks(&mx, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Xq, M, K, kHalf, kKS);
     if (rc != ASER_OK) return rc;
+    mt = mx;
     if (r > 0) {
-        rc = encode_map_2d(&mlb, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, LB, N, r, 128, 64, CU_TENSOR_MAP_SWIZZLE_128B);
+        rc = encode_map_2d_ld(&mt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, T, M, t_cols, ldt > 0 ? ldt : t_cols, kHw, 64,
+                              CU_TENSOR_MAP_SWIZZLE_128B);
         if (rc != ASER_OK) return rc;
-        rc = encode_map_2d_ld(&mt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, T, M, r * cat.layers, ldt > 0 ? ldt : r * cat.layers,
-                              kHw, 64, CU_TENSOR_MAP_SWIZZLE_128B);
-        if (rc != ASER_OK) return rc;
-    } else {
-        mlb = mx;
-        mt = mx;
     }
-    Params p = {};
-    p.Wk = Wk; p.a_scale = a_scale; p.w_scale = w_scale; p.acc_debug = acc_debug;
+    for (int l = 0; l < kMaxGroup; ++l) {
+        if (l >= g.layers) { maps.y[l] = maps.y[0]; maps.lb[l] = maps.lb[0]; continue; }
+        rc = encode_map_2d(&maps.y[l], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, g.Y[l], M, g.N[l], kHw, 128, CU_TENSOR_MAP_SWIZZLE_NONE);
+        if (rc != ASER_OK) return rc;
+        maps.lb[l] = mx;
+        if (r > 0) rc = encode_map_2d(&maps.lb[l], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, g.LB[l], g.N[l], r, 128, 64, CU_TENSOR_MAP_SWIZZLE_128B);
+        if (rc != ASER_OK) return rc;
+    }
+    p.a_scale = a_scale; p.acc_debug = acc_debug;
     p.status = static_cast<uint32_t*>(workspace);
-    p.M = M; p.N = N; p.r = r;
-    p.KB = K / kWkCols; p.NB = (N + kWkRows - 1) / kWkRows;
+    p.M = M; p.r = r;
+    p.KB = K / kWkCols;
     p.NT = plan.NT; p.TT = plan.TT; p.full = plan.full; p.cut = plan.cut; p.items = plan.items;
     // the smaller of the two operand sets stays in L2 while the other is streamed (as in linear_tc.cu)
-    p.tt_outer = ((long long)M * K > (long long)N * K / 2) ? 1 : 0;
+    p.tt_outer = ((long long)M * K > rows * K / 2) ? 1 : 0;
     p.cat = cat;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (plan.items < pairs ? plan.items : pairs), 1, 1);
@@ -704,10 +739,21 @@ int launch_linear_pair(const int8_t* Xq, const float* a_scale, const uint8_t* Wk
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = overlap_prev ? 2 : 1;
-    const cudaError_t e = acc_debug ? cudaLaunchKernelEx(&cfg, linear_pair_kernel<true>, mx, mlb, mt, my, p)
-                                    : cudaLaunchKernelEx(&cfg, linear_pair_kernel<false>, mx, mlb, mt, my, p);
+    const cudaError_t e = g.layers > 1 ? cudaLaunchKernelEx(&cfg, linear_pair_kernel<false, true>, mx, mt, maps, p)
+                          : acc_debug  ? cudaLaunchKernelEx(&cfg, linear_pair_kernel<true, false>, mx, mt, maps, p)
+                                       : cudaLaunchKernelEx(&cfg, linear_pair_kernel<false, false>, mx, mt, maps, p);
     if (e != cudaSuccess) return record_cuda_error(e, "linear_pair_kernel");
     return check_launch("linear_pair_kernel");
+}
+
+int launch_linear_pair(const int8_t* Xq, const float* a_scale, const uint8_t* Wk, const float* w_scale,
+                       const __nv_bfloat16* T, const __half* LB, int M, int N, int K, int r, __half* Y,
+                       int32_t* acc_debug, void* workspace, cudaStream_t st, bool overlap_prev, int ldt, CatSplit cat) {
+    LinearGroup g = {};
+    g.layers = 1;
+    g.Wk[0] = Wk; g.w_scale[0] = w_scale; g.LB[0] = LB; g.Y[0] = Y;
+    g.N[0] = N; g.r[0] = r;
+    return launch_linear_pair_group(Xq, a_scale, T, M, K, g, acc_debug, workspace, st, overlap_prev, ldt, cat);
 }
 
 }  // namespace aser

@@ -951,6 +951,35 @@ def test_forward_host_output_in_the_place_of_the_input(aser, N, K, host, device)
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("M,K,spec", [
+    (5, 640, [(520, 16), (24, 0), (2056, 48)]), (16, 1024, [(9480, 64), (9480, 64)]),               # few tokens: any ranks
+    (333, 384, [(264, 48)] * 4), (1300, 512, [(2056, 144)] * 2), (513, 640, [(768, 0)] * 3),      # CTA pairs: one rank
+])
+def test_shared_group_in_one_launch_has_the_bits_of_its_layers(aser, M, K, spec):
+    """Layers that read the same codes, each with operands of its own, served by one launch: ragged channels in every
+    layer, so that tiles end inside the group."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + K)
+    s = torch.ones(K, device="cuda")
+    s[::97] = 3.0
+    half = lambda *shape, scale: (torch.randn(*shape, device="cuda", generator=g) * scale).half()
+    layers = [aser.AserLinear(half(n, K, scale=0.02), s, half(r, K, scale=0.02) if r else None,
+                              half(n, r, scale=0.02) if r else None, M) for n, r in spec]
+    assert len({aser.lib.aser_linear_kernel(M, n, K) for n, _ in spec}) == 1
+    group = aser.AserSharedInput(layers, M)
+    Ys = [y.clone() for y in group(half(M, K, scale=1.0))]
+    aser.check_status(group.ws)
+    col = 0
+    for (n, r), lay, Y in zip(spec, layers, Ys):
+        if r:
+            ref = aser.binding.linear_w4a8_lr_ld(group.Xq, group.a_scale, lay.Wk, lay.w_scale, group.T, col, lay.L_B, n, group.ws)
+        else:
+            ref = aser.linear_w4a8(group.Xq, group.a_scale, lay.Wk, lay.w_scale, n, group.ws)
+        assert torch.equal(Y, ref)
+        col += r
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("r", [128, 192])
 def test_fused_group_is_bit_identical_across_the_two_tensor_core_kernels(aser, r):
     """1024 tokens, K = 4096, two layers of 2048 channels: the fused launch (4096 channels) is served by CTA pairs,
