@@ -472,8 +472,10 @@ smallest_eigenvalue_kernel(const double* __restrict__ Linv, long long ldl, int p
 // One-sided Jacobi on the rows of G [p, p], the rotations applied to V (the identity at first):
 // V G has orthogonal rows.  All rounds in one CTA, rows in shared memory, half a warp per pair; ends
 // with the first sweep that finds every pair orthogonal to rounding.  The tangent of an angle is
-// taken in fp32 (its error only leaves the pair for a later sweep), cosine and sine in fp64, so the
-// rotations are orthogonal to fp64 rounding.
+// taken in fp32 from an fp64 quotient (its error only leaves the pair for a later sweep), cosine and sine in fp64, so the
+// rotations are orthogonal to fp64 rounding.  The squared norms of the rows are summed when a sweep begins and then follow the
+// rotations, in fp64 and for the angle as it was taken: good to a few roundings of the larger norm of a pair.
+// A sweep that rotates nothing, which ends the loop, has only seen norms that were summed in it.
 constexpr int kJacobiThreads = 896;          // kMaxP / 2 half warps
 static_assert(kJacobiThreads / 16 >= kMaxP / 2, "a half warp per pair");
 __global__ void __launch_bounds__(kJacobiThreads)
@@ -505,22 +507,23 @@ jacobi_kernel(double* __restrict__ G, double* __restrict__ V, int p) {
             const bool have = pair < p / 2;
             double* gi = g + i * p;
             double* gj = g + j * p;
+            // Both norms are read before the shuffles: every lane of the warp has them when one of its pairs writes new ones.
+            const double a = have ? sq[i] : 0.0, b = have ? sq[j] : 0.0;
             double c = 0.0;
             if (have)
                 for (int k = lane; k < p; k += 16) c = fma(gi[k], gj[k], c);
             for (int o = 8; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-            const double a = have ? sq[i] : 0.0, b = have ? sq[j] : 0.0;
+            __syncwarp();
             if (have && c * c > 1e-28 * a * b) {
-                // (b - a) / 2c in fp32, both brought near 1 by the larger exponent
-                const double diff = b - a, twice = 2.0 * c;
-                const int top = max(__double2hiint(diff) & 0x7ff00000, __double2hiint(twice) & 0x7ff00000);
-                const double scale = __hiloint2double(min(max(0x7fe00000 - top, 0x00100000), 0x7fe00000), 0);
-                const float zeta = __fdividef((float)(diff * scale), (float)(twice * scale)), z = fabsf(zeta);
+                const float zeta = (float)((b - a) / (2.0 * c)), z = fabsf(zeta);
                 const float tf = z > 1e9f ? 0.5f / z : 1.f / (z + sqrtf(1.f + z * z));
                 const double t = zeta >= 0.f ? (double)tf : -(double)tf;
                 const double cs = rsqrt(1.0 + t * t), sn = cs * t;
-                __syncwarp(__activemask());
-                if (lane == 0) { rotated = 1; sq[i] = a - t * c; sq[j] = b + t * c; }
+                if (lane == 0) {            // the norms of the rows as they are rotated, whatever the angle
+                    rotated = 1;
+                    sq[i] = fmax(cs * cs * fma(t, fma(t, b, -2.0 * c), a), 0.0);
+                    sq[j] = fmax(cs * cs * fma(t, fma(t, a, 2.0 * c), b), 0.0);
+                }
                 double* vi = v + i * p;
                 double* vj = v + j * p;
                 for (int k = lane; k < p; k += 16) {
