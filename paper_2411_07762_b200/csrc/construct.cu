@@ -596,6 +596,7 @@ struct ConstructLayout {
     int p, tokens;                // tokens padded to 16 rows
     long long lda;                // columns of the wide error matrix, at most
     int pieces;                   // of the Gram matrix that is made beside the products of the next step (0: p is too large)
+    bool sum_pieces;              // they are summed by a launch of their own, ahead of the factorisation
     size_t A, E, G, Xs, T[4], Y, part, C, L, V, Vsel, sigma, row_sq, scalars, fail, Wm, total;     // byte offsets
 };
 
@@ -623,6 +624,11 @@ ConstructLayout construct_layout(int N, int K, int Tcal, int r, int n_split) {
     L.pieces = 0;
     for (int q = 4; p <= 96 && q <= 16 && L.pieces == 0; q *= 2)
         if (q == 16 || gemm64::split_count(p, wide, N, kSplitSms - q) <= q) L.pieces = q;
+    // The factorisation in one CTA takes 4.9e-3 p^2 us, each piece that it sums itself 3.1e-4 p^2 more, the product beside it 2 p N
+    // `wide` at 28 TFLOP/s; a launch that sums them first takes 3.6.  22 steps, ms, all in order / the CTA sums / summed first: 768 x 768,
+    // r = 64 4.47 / 5.22 / 3.99; 1536 x 1536, r = 64 5.24 / 5.80 / 4.50; 2048 x 2048, r = 16 3.07 / 2.62 / 2.70, r = 64 5.99 / 5.46 / 5.01;
+    // 4096 x 4096, r = 64 10.67 / 9.60 / 9.68.
+    L.sum_pieces = 4.9e-3 * p * p + 3.1e-4 * (L.pieces - 1) * p * p > 2.0 * p * N * (double)wide / 28e6 + 3.6;
     size_t part = 0;
     auto need = [&](int m, int n, int k, int sms = kSplitSms) {
         const size_t b = gemm64::partial_bytes(m, n, k, sms);
@@ -819,13 +825,18 @@ int launch_construct(const __half* W, const float* s, const __half* Xcal, int N,
         for (int i = 0; i < steps; ++i, ++done) {
             if (i > 0 && L.pieces > 0) {
                 // The basis of the step before is still as its product left it.  Its Gram matrix is made beside the first
-                // product of this step and factorised beside the second (40 us of one CTA), then the factor is applied to both
+                // product of this step, summed and factorised beside the second (40 us of one CTA), then the factor is applied to both
                 // terms: the rows that the products see have the growth of one step, as their Gram matrix always had.
                 gemm64::Args h = {};
                 h.A = h.B = t0; h.lda = h.ldb = N; h.ldc = p; h.m = h.n = p; h.k = N; h.a0 = 1.0; h.side = true;
                 ASER_STEP(gemm64::run_pieces(h, C, L.pieces, st));
                 ASER_STEP(product(ctx, false, p, kc, N, t0, N, A, kc, Y, kc, 1.0, nullptr, nullptr, 0.0, nullptr, 0.0, L.pieces));
-                ASER_STEP(chol_inverse_block(ctx, C, p, p, Li, p, nullptr, p, L.pieces));
+                if (L.sum_pieces) {
+                    ASER_STEP(gemm64::sum_pieces(C, p, p, L.pieces, V, p, st));
+                    ASER_STEP(chol_inverse_block(ctx, V, p, p, Li, p, nullptr, p));
+                } else {
+                    ASER_STEP(chol_inverse_block(ctx, C, p, p, Li, p, nullptr, p, L.pieces));
+                }
                 ASER_STEP(product(ctx, true, p, N, kc, Y, kc, A, kc, f0, N, 4.0, bound, t0, -2.0, t1, -1.0, 1));
                 swap(t1, f0);
                 swap(t0, t1);

@@ -262,6 +262,15 @@ inline int run_pieces(Args g, double* part, int pieces, cudaStream_t st) {
     return launch_tb<true>(g, 1, st);
 }
 
+// Their sum, [m, n] (n even).
+inline int sum_pieces(const double* part, int m, int n, int pieces, double* C, long long ldc, cudaStream_t st) {
+    Args g = {};
+    g.C = C; g.ldc = ldc; g.m = m; g.n = n; g.splits = pieces; g.a0 = 1.0;
+    const long long pairs = (long long)m * n / 2;
+    reduce_kernel<<<(unsigned)((pairs + 255) / 256), 256, 0, st>>>(part, g);
+    return check_launch("gemm64 sum");
+}
+
 // n, k, all pitches even; pointers 16-byte aligned; `part` holds partial_bytes(m, n, k).  With
 // B2 (and C2) the same A is applied to two matrices and k is not split.
 inline int run(Args g, bool tb, double* part, int num_sms, cudaStream_t st) {

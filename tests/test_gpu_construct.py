@@ -188,3 +188,23 @@ def test_construct_options_without_the_whitening_factor(aser, iterations, dampin
     prod_gpu = out["L_B"].cpu().numpy().astype(np.float64) @ out["L_A"].cpu().numpy().astype(np.float64)
     prod_ref = L.L_B.astype(np.float64) @ L.L_A.astype(np.float64)
     assert np.linalg.norm(prod_gpu - prod_ref) < 2e-3 * np.linalg.norm(prod_ref)
+
+
+@pytest.mark.parametrize("N,K,r,n_cal", [
+    (16, 512, 16, 64),        # sixteen vectors: four pieces, three of them empty, added by the factorising CTA
+    (40, 640, 16, 100),       # two pieces of sixteen columns, one of eight, one empty, summed ahead of it
+    (1000, 384, 48, 40),      # sixteen pieces
+    (2048, 2048, 16, 64),     # eight pieces, added by the factorising CTA beside a longer product
+])
+def test_construct_gram_matrix_in_pieces(aser, N, K, r, n_cal):
+    """The Gram matrix that is made beside the products, summed by a launch of its own or by the CTA that factorises it.
+    Bounds as in _check."""
+    lay = synth.make_layer(4, N, K, seed=synth.seed_for(2, N + K + r), n_cal=n_cal)
+    s = Cn.smoothing_vector_config(lay.X_cal, lay.W, lay.outlier_idx)
+    L = Cn.construct_layer(lay.W, lay.X_cal, s, r=r)
+    out = aser.construct(to_dev(lay.W), to_dev(s), to_dev(lay.X_cal), r)
+    assert np.array_equal(out["Wq"].cpu().numpy(), L.Wq)
+    assert np.allclose(out["sigma"].cpu().numpy(), L.sigma[:r], rtol=1e-6)
+    prod_gpu = out["L_B"].cpu().numpy().astype(np.float64) @ out["L_A"].cpu().numpy().astype(np.float64)
+    prod_ref = L.L_B.astype(np.float64) @ L.L_A.astype(np.float64)
+    assert np.linalg.norm(prod_gpu - prod_ref) < 2e-3 * np.linalg.norm(prod_ref)
