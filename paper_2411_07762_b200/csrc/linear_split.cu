@@ -10,24 +10,23 @@
 //  * The packed weights do not go through shared memory: sixteen warps load them straight into registers (two blocks of
 //    8 KB per group of four warps ahead, the first before anything else, while the activation kernel still runs), turn them
 //    into int8 (value 16 q) and write them to tensor memory.  Shared memory carries the activations alone.
-//  * Activations come two blocks to a copy, two threads issue the products of alternate blocks into the same sums; a block's
-//    products free its activations and its A operand by one commit.
+//  * A stage is two blocks: their activations in one copy, one barrier that counts the copy's bytes and the eight warps that
+//    unpack, one commit that frees both operands.  One thread issues all integer products: those of one thread into the same
+//    sums run in order, those of two only if each waits for the other's issue.
 //  * Partial sums: each CTA stages its int32 sums as [token][128 channels] where the activations were and sends every peer
 //    the tokens that this peer finishes, one bulk copy each into a buffer of its own (16 n tokens per CTA).  Integer sums:
 //    the order does not matter.
-//  * The low-rank product of the tokens that a CTA finishes is issued by the first of the two threads when its operands are
-//    there (looked at once per block, waited for at the end only); two warps load and convert them (T bf16 -> fp16, exact
-//    in the fp16 normal range).  Chunks of 64 in order: the same sums as in the other kernels.
+//  * The low-rank product of the tokens that a CTA finishes has sums and an issuing thread of its own; two warps load and
+//    convert its operands (T bf16 -> fp16, exact in the fp16 normal range).  Chunks of 64 in order: the same sums as in the
+//    other kernels.
 //  * The sixteen warps are the epilogue as well; outputs leave through shared memory as tensor stores of 16 tokens.
 // Every wait is bounded: on expiry the CTA sets the status word and winds down.
 //
 // Measured against linear_tc_kernel (or linear_pair_kernel, whichever the shape had), the linear step alone in graphs on one box
-// (tokens x channels x K, us): 17 x 4096 x 4096 13.2 -> 10.0; 32 x 14336 x 4096 20.4 -> 13.7; 64 x 4096 x 14336 21.1 -> 15.7;
-// 101 x 8192 x 8192 26.5 -> 18.4; 128 x 14336 x 4096 20.9 -> 16.9; 200 x 8192 x 2048 14.7 -> 12.4; 400 x 4096 x 4096 19.6 -> 16.8;
-// 256 x 4096 x 14336 32.4 -> 24.1.  What bounds it: at 101 x 8192 x 8192 a block takes 265 ns, in which the 128 SMs at
-// work fetch 22 KB each, 10 TB/s out of L2 (activations are read once per 128 channels); set-up 1.2 us, exchange
-// and outputs 3 us.  With one block to a copy and one issuing thread the same launch took 22.5 us: each of
-// the two then needs 770 cycles a block.
+// (tokens x channels x K, us): 17 x 4096 x 4096 13.2 -> 8.4; 32 x 14336 x 4096 20.4 -> 10.0; 64 x 4096 x 14336 21.1 -> 12.8;
+// 101 x 8192 x 8192 26.5 -> 16.7; 128 x 14336 x 4096 20.9 -> 14.3; 200 x 8192 x 2048 14.7 -> 10.5; 400 x 4096 x 4096 19.6 -> 13.3;
+// 256 x 4096 x 14336 32.4 -> 20.2.  (Repeats of one call: the weights come from L2.)  What bounds it: activations are read once
+// per 128 channels, 22 KB per SM and block at 101 x 8192 x 8192, so L2 -> SM traffic; set-up 1.2 us, exchange and outputs 3 us.
 #include "aser_common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -35,14 +34,14 @@ namespace aser {
 
 namespace {
 
-constexpr int kUnpackWarps = 16, kThreads = (kUnpackWarps + 5) * 32;   // + activation producer, two issuers, two of the low-rank operands
+constexpr int kUnpackWarps = 16, kThreads = (kUnpackWarps + 5) * 32;   // + activation producer, issuers of the integer and of the low-rank products, two of the low-rank operands
 constexpr int kWarpIssue = kUnpackWarps + 1, kWarpLr = kUnpackWarps + 3;
-constexpr int kSlots = 8, kPairs = kSlots / 2;   // A blocks in tensor memory = activation blocks in shared memory, two to a copy
+constexpr int kSlots = 8, kStages = kSlots / 2;  // A blocks in tensor memory = activation blocks in shared memory, two to a stage
 constexpr int kMaxTok = 128, kMaxSplit = 8;
 constexpr int kLbBytes = 128 * 128;
 constexpr long long kWaitClocks = 400000000ll;   // about 0.2 s of SM clocks per wait
 
-constexpr int B_FULL = 0, B_FREE = B_FULL + kSlots, B_X = B_FREE + kSlots, B_ACC = B_X + kPairs, B_RECV = B_ACC + 1,
+constexpr int B_FULL = 0, B_FREE = B_FULL + kStages, B_ACC = B_FREE + kStages, B_RECV = B_ACC + 1,
               B_LR_FULL = B_RECV + 1, B_LR_CONV = B_LR_FULL + 2, B_LR_FREE = B_LR_CONV + 2, B_LR_DONE = B_LR_FREE + 2,
               kNumBars = B_LR_DONE + 1;
 static_assert(kNumBars * 8 + 8 <= 256, "barrier area");
@@ -118,13 +117,6 @@ __device__ __forceinline__ void let_copies_land() {
     const long long t0 = clock64();
     while (clock64() - t0 < 2000000) {}
 }
-// A look at a barrier phase, without the time that try_wait may wait for it.
-__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
-}
 __device__ __forceinline__ uint4 ld_weights(const uint8_t* p) {
     uint4 v;
     asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
@@ -153,7 +145,7 @@ linear_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = (int)blockIdx.x % S, tile = (int)blockIdx.x / S, nt = tile / p.TT, tt = tile % p.TT;
     const int n0 = nt * 128, tok0 = tt * p.tok;
-    const int kb0 = p.KB * rank / S, nkb = p.KB * (rank + 1) / S - kb0;
+    const int kb0 = p.KB * rank / S, nkb = p.KB * (rank + 1) / S - kb0, stages = (nkb + 1) / 2;
     const int own0 = rank * p.own;                       // this CTA's tokens of the tile: [own0, own0 + owned)
     const int owned = p.tok - own0 < p.own ? (p.tok - own0 > 0 ? p.tok - own0 : 0) : p.own;
     const int chunks = owned > 0 ? (p.r + 63) / 64 : 0;
@@ -172,8 +164,8 @@ linear_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     } else if (warp == kUnpackWarps) {
         for (int i = lane; i < kNumBars; i += 32) {
             uint32_t count = 1;
-            if (i < B_FREE) count = 4;                   // four warps' A rows
-            if (i == B_ACC || (i >= B_LR_CONV && i < B_LR_FREE)) count = 2;
+            if (i < B_FREE) count = 9;                   // eight warps' A rows and the copy
+            if (i >= B_LR_CONV && i < B_LR_FREE) count = 2;
             mbar_init(bar(i), count);
         }
         if (lane == 0) *stop_flag = 0;
@@ -198,14 +190,6 @@ linear_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     if (S > 1) cluster_arrive();         // the peers' barriers are in place: waited for before sums are sent
     tc_fence_after();
     const uint32_t tmem = *tmem_slot, tm_lr = tmem + kMaxTok, tm_a = tmem + 2 * kMaxTok;
-    // The integer sums start at zero, so that the order of the two issuers' products does not matter.
-    if (warp < kUnpackWarps) {
-        for (int c = group * 16; c < p.tok; c += 64) tmem_zero16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c);
-        tmem_wait_st();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
 
     // The next activation kernel may be set up meanwhile: it waits for the end of this kernel before it reads anything, and
     // lets its own dependents start only then.
@@ -217,56 +201,65 @@ linear_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             // Two blocks to a copy: a copy costs its thread 500 cycles whatever its size.  (The second block of the last copy
             // may lie past the slice or past K.)
             bool ok = true;
-            for (int b = 0; b < nkb && ok; b += 2) {
-                const int s = b % kSlots, pr = s / 2;
-                if (b >= kSlots) {
-                    const uint32_t parity = (uint32_t)(b / kSlots - 1) & 1u;
-                    ok = wait(bar(B_FREE + s), parity, stop) && wait(bar(B_FREE + s + 1), parity, stop);
-                    if (!ok) break;
-                }
-                mbar_arrive_expect_tx(bar(B_X + pr), 2u * (uint32_t)L.x_block);
-                tma_load_3d(sb + s * L.x_block, &map_x, 0, tok0, kb0 + b, bar(B_X + pr));
+            for (int st = 0; st < stages && ok; ++st) {
+                const int s = st % kStages;
+                if (st >= kStages) ok = wait(bar(B_FREE + s), (uint32_t)(st / kStages - 1) & 1u, stop);
+                if (!ok) break;
+                mbar_arrive_expect_tx(bar(B_FULL + s), 2u * (uint32_t)L.x_block);
+                tma_load_3d(sb + 2 * s * L.x_block, &map_x, 0, tok0, kb0 + 2 * st, bar(B_FULL + s));
             }
             if (!ok || *stop_flag) let_copies_land();
         }
-    } else if (warp == kWarpIssue || warp == kWarpIssue + 1) {
-        // =================== MMA issuers: alternate blocks (two waits, four products and a commit take one thread longer than
-        // the tensor pipe); the first one also multiplies the low-rank chunks ===================
-        if (lane == 0) {
-            const bool lowrank = warp == kWarpIssue;
-            const uint32_t idesc_i8 = make_idesc(2, 1, 128, (uint32_t)p.tok), idesc_f16 = make_idesc(1, 0, 128, (uint32_t)p.own);
-            int c = 0;                   // low-rank chunks multiplied so far
-            bool ok = true;
-            auto chunk = [&]() {
-                tc_fence_after();
-                const uint32_t set = sb + (uint32_t)(L.lr + (c & 1) * L.lr_set);
-                const uint64_t ad = smem_desc_sw128(set), bd = smem_desc_sw128(set + kLbBytes);
-                const int steps = p.r - c * 64 >= 64 ? 4 : (p.r - c * 64) / 16;
-                for (int kk = 0; kk < steps; ++kk)
-                    mma_f16_ss(tm_lr, ad + 2 * kk, bd + 2 * kk, idesc_f16, (c | kk) != 0 ? 1u : 0u);
-                tc_commit(bar(B_LR_FREE + (c & 1)));
-                ++c;
-            };
-            for (int b = warp - kWarpIssue; b < nkb; b += 2) {
-                const int s = b % kSlots;
-                const uint32_t parity = (uint32_t)(b / kSlots) & 1u;
-                ok = wait(bar(B_X + s / 2), parity, stop) && wait(bar(B_FULL + s), parity, stop);
-                if (!ok) break;
-                tc_fence_after();
-                const uint64_t xdesc = smem_desc_sw128(sb + s * L.x_block);
+    } else if (warp == kWarpIssue) {
+        // =================== integer products ===================
+        // The whole warp goes through the loop and one lane is elected around the products (the same one every time), which
+        // keeps their operands in uniform registers: in a branch of lane 0 the same loop took 10 to 40 % longer, and two
+        // such threads with alternate blocks 11 %.
+        const uint32_t idesc = make_idesc(2, 1, 128, (uint32_t)p.tok);
+        bool ok = true;
+        for (int st = 0; st < stages; ++st) {
+            const int s = st % kStages;
+            ok = wait(bar(B_FULL + s), (uint32_t)(st / kStages) & 1u, stop);
+            ok = __all_sync(0xffffffffu, ok) != 0;
+            if (!ok) break;
+            tc_fence_after();
+            const uint64_t xdesc = smem_desc_sw128(sb + 2 * s * L.x_block);
+            const uint32_t a = tm_a + s * 64;
+            if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    mma_i8_ts(tmem, tm_a + s * 32 + kk * 8, xdesc + 2 * kk, idesc_i8, 1u);
+                for (int h = 0; h < 2; ++h)
+                    if (2 * st + h < nkb)
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk)
+                            mma_i8_ts(tmem, a + h * 32 + kk * 8, xdesc + (uint64_t)(h * (L.x_block >> 4) + 2 * kk), idesc,
+                                      (st | h | kk) != 0 ? 1u : 0u);
                 tc_commit(bar(B_FREE + s));
-                if (lowrank && b + 2 < nkb && c < chunks && mbar_test_wait(bar(B_LR_CONV + (c & 1)), (uint32_t)(c >> 1) & 1u)) chunk();
             }
-            if (ok) tc_commit(bar(B_ACC));
-            while (ok && lowrank && c < chunks) {
-                ok = wait(bar(B_LR_CONV + (c & 1)), (uint32_t)(c >> 1) & 1u, stop);
-                if (ok) chunk();
-            }
-            if (ok && lowrank && chunks > 0) tc_commit(bar(B_LR_DONE));
+            __syncwarp();
         }
+        if (ok && elect_one()) tc_commit(bar(B_ACC));
+        __syncwarp();
+    } else if (warp == kWarpIssue + 1) {
+        // =================== low-rank products ===================
+        const uint32_t idesc = make_idesc(1, 0, 128, (uint32_t)p.own);
+        bool ok = true;
+        for (int c = 0; c < chunks; ++c) {
+            ok = wait(bar(B_LR_CONV + (c & 1)), (uint32_t)(c >> 1) & 1u, stop);
+            ok = __all_sync(0xffffffffu, ok) != 0;
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t set = sb + (uint32_t)(L.lr + (c & 1) * L.lr_set);
+            const uint64_t ad = smem_desc_sw128(set), bd = smem_desc_sw128(set + kLbBytes);
+            const int steps = p.r - c * 64 >= 64 ? 4 : (p.r - c * 64) / 16;
+            if (elect_one()) {
+                for (int kk = 0; kk < steps; ++kk)
+                    mma_f16_ss(tm_lr, ad + 2 * kk, bd + 2 * kk, idesc, (c | kk) != 0 ? 1u : 0u);
+                tc_commit(bar(B_LR_FREE + (c & 1)));
+            }
+            __syncwarp();
+        }
+        if (ok && chunks > 0 && elect_one()) tc_commit(bar(B_LR_DONE));
+        __syncwarp();
     } else if (warp >= kWarpLr) {
         // =================== low-rank operands ===================
         const int w = warp - kWarpLr;
@@ -318,8 +311,12 @@ linear_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         bool ok = true;
         auto block = [&](int b, uint4 (&w)[4]) {
             const int s = b % kSlots;
-            if (b >= kSlots) ok = warp_wait(bar(B_FREE + s), (uint32_t)(b / kSlots - 1) & 1u, stop, lane);
+            if (b >= kSlots) ok = warp_wait(bar(B_FREE + s / 2), (uint32_t)(b / kSlots - 1) & 1u, stop, lane);
             if (!ok) return;
+            if (b == nkb) {              // the half of the last stage that is not there
+                if (lane == 0) mbar_arrive(bar(B_FULL + s / 2));
+                return;
+            }
             tc_fence_after();
             const uint32_t a = tm_a + s * 32 + ((uint32_t)(q * 32) << 16);
 #pragma unroll
@@ -340,11 +337,11 @@ linear_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar(B_FULL + s));
+            if (lane == 0) mbar_arrive(bar(B_FULL + s / 2));
         };
-        for (int b = group; b < nkb && ok; b += 8) {
+        for (int b = group; b < 2 * stages && ok; b += 8) {
             block(b, raw[0]);
-            if (ok && b + 4 < nkb) block(b + 4, raw[1]);
+            if (ok && b + 4 < 2 * stages) block(b + 4, raw[1]);
         }
 
         // =================== epilogue ===================

@@ -1006,3 +1006,36 @@ def test_fused_group_is_bit_identical_across_the_two_tensor_core_kernels(aser, r
         y = aser.linear_w4a8_lr_ld(Xq, a, Wk[i], packed[i][1], T, i * r, LB[i], N, ws)
         assert torch.equal(Y[:, i * N:(i + 1) * N], y)
     aser.check_status(ws)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,more,N,K,r,kernel", [
+    (17, 2000, 512, 1152, 48, 1),         # an odd number of column blocks: the last stage of a slice is half a stage
+    (101, 1200, 4096, 4096, 128, 2), (384, 900, 2048, 2176, 192, 1), (512, 2000, 1024, 1024, 256, 1), (32, 2048, 14336, 1024, 0, 2)])
+def test_split_kernel_has_the_bits_of_the_other_tensor_core_kernels(aser, M, more, N, K, r, kernel):
+    """The first tokens of a call that another kernel serves: integer sums, and the low-rank chunks in order."""
+    assert [aser.lib.aser_linear_kernel(m, N, K) for m in (M, more)] == [3, kernel]
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + N + r)
+    Xq = torch.randint(-127, 128, (more, K), device="cuda", dtype=torch.int8, generator=g)
+    a = torch.rand(more, device="cuda", generator=g) * 1e-3
+    T = torch.randn(more, max(r, 1), device="cuda", generator=g).bfloat16()
+    Wq, sc = aser.pack_w4(torch.randn(N, K, device="cuda", generator=g).half(), None)
+    Wk, LB = aser.repack_w4(Wq), torch.randn(N, max(r, 1), device="cuda", generator=g).half() * 0.1
+    ws = aser.new_workspace(more, N, K, r)
+    Y = [aser.linear_w4a8_lr(Xq[:m], a[:m], Wk, sc, T[:m], LB, N, ws) if r else aser.linear_w4a8(Xq[:m], a[:m], Wk, sc, N, ws)
+         for m in (M, more)]
+    assert torch.equal(Y[0], Y[1][:M])
+    if r and N % 256 == 0:          # the same channels as a fused group of two layers, each with its columns of T
+        import ctypes as C
+        T2 = torch.randn(M, 2 * r, device="cuda", generator=g).bfloat16()
+        P = lambda t: C.c_void_p(t.data_ptr())
+        Yc = torch.empty((M, N), device="cuda", dtype=torch.float16)
+        h = N // 2
+        rc = aser.lib.aser_linear_w4a8_lr_cat(P(Xq), P(a), P(Wk), P(sc), P(T2), P(LB), 2, (C.c_int * 2)(h, h), r, M, K, P(Yc),
+                                              P(ws), ws.numel(), C.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert rc == 0
+        for i in range(2):
+            y = aser.linear_w4a8_lr(Xq[:M], a[:M], Wk, sc, T2[:, i * r:(i + 1) * r].contiguous(), LB, N, ws)
+            assert torch.equal(Yc[:, i * h:(i + 1) * h], y[:, i * h:(i + 1) * h])
+    aser.check_status(ws)
