@@ -12,15 +12,16 @@
 // units is cut into equal contiguous ranges, one per CTA; tiles shared by several CTAs are
 // summed through the workspace by whichever CTA arrives last.
 //
-// Warp roles (512 threads for token tiles of 16/32, 640 above): 0 = weight producer, 1 and the
-// last warp = MMA issuers for even / odd stages (1 also owns the TMEM allocation and issues the
-// low-rank MMAs), 2..5 and 6..9 = two groups of int4 -> int8 unpack warps that take alternate
-// stages (group 0 also converts T), then 4 or 8 epilogue warps (two per tensor-memory lane
+// Warp roles (512 threads for token tiles of 16/32, 640 above): 0 = weight producer, 1 = issuer of the
+// integer MMAs (it also owns the TMEM allocation), the last = issuer of the low-rank MMAs up to 64
+// tokens, 2..5 and 6..9 = two groups of int4 -> int8 unpack warps that take alternate stages (group 0 also converts T), then 4 or 8 epilogue warps (two per tensor-memory lane
 // quarter take alternate 16-column chunks), then the activation / low-rank operand producer.
-// A single lane issues one tcgen05.mma per ~60-85 cycles, which bounds decode shapes (16 MMAs
-// per 32 KiB of weights); the integer accumulation is order-independent, so two lanes share the
-// issue work.  For that the accumulator is zeroed by the epilogue warps (tcgen05.st) when they
-// hand it back, and every integer MMA accumulates.
+// One thread issues all integer MMAs: those of one thread into the same accumulator run in order, those of two only
+// if each waits for the other's issue.  The whole issuing warp goes through its loop and one lane is elected around
+// the MMAs, which keeps their operands in uniform registers; the barriers of the next A slot are looked at while this
+// one's MMAs are issued.  Against two threads of a lane-0 branch with alternate stages, us: 12 x 20480 x 8192
+// 25.5 -> 25.0; 33 x 20000 x 4096 24.9 -> 24.0; 513 x 1024 x 8192 29.1 -> 28.2; 23 shapes 1.012 times as fast.  (640 threads
+// rather than 608 for 64 and 128 tokens: with 608 the finishing of shared tiles spills more, 1500 x 512 x 8192 33.5 -> 37.8.)
 // Every wait is bounded: on expiry the CTA sets the status word and winds down.
 #include "aser_common.cuh"
 #include "sm100_ptx.cuh"
@@ -43,13 +44,13 @@ struct Cfg {
     // Epilogue warps: one per tensor-memory lane quarter, two where a tile has many columns.
     static constexpr int EW = (BT >= 64) ? 8 : 4;
     static constexpr int EpiThreads = EW * 32;
-    static constexpr int WarpXProd = 10 + EW, WarpIssuer1 = 11 + EW;
+    static constexpr int WarpXProd = 10 + EW, WarpLrIssuer = 11 + EW;
     static constexpr int Threads = (12 + EW) * 32;
     static constexpr int KS = 2;
     static constexpr int NW = (BT == 128) ? 4 : (BT == 64 ? 6 : 8);     // weight ring depth (even)
     static constexpr int NX = 4;                                        // activation ring depth
     // A-operand ring (tensor memory).  All ring depths are even: stages alternate between two
-    // unpack groups and two MMA issuers, and a parity wait is only sound if the waiter sees every
+    // unpack groups, and a parity wait is only sound if the waiter sees every
     // phase of the barrier, i.e. if a ring slot always belongs to the same group.
     // An A slot holds KA column blocks.  With 128 tokens only 128 tensor-memory columns are left
     // for A, so a slot is one block there: each group then still owns two slots and can unpack
@@ -71,14 +72,11 @@ struct Cfg {
     static constexpr int OffT = OffLb + NL * LbBytes;
     static constexpr int OffBar = OffT + NL * TBytes;
     static constexpr int NumBars = 2 * NW + 2 * NX + 2 * NA + 3 * NL + 2 + 2 + 2;
-    // Who issues the low-rank MMAs.  The two integer issuers spend nine tenths of their time
-    // inside barrier and tensor-core instructions (a wait, MMA or commit costs its thread a few
-    // hundred cycles under copy traffic), so every operation of a low-rank chunk on one of them
-    // sets it back against the other and the whole pipeline with it.  A warp of its own for the
-    // job costs every thread 16 registers (21 warps: six on one scheduler); a second lane of the
-    // producer's warp as a third issuer measured the same as what is done here and leans on how the
-    // hardware shares a warp between two diverged spinning lanes.  So, with the one-slot chunk
-    // ring, the thread that loads the chunks also multiplies them: it runs a few stages ahead of
+    // Who issues the low-rank MMAs.  They have sums of their own, so any thread may, but not the integer issuer: it
+    // spends nine tenths of its time inside barrier and tensor-core instructions (a wait, MMA or commit costs its
+    // thread a few hundred cycles under copy traffic), so every operation of a low-rank chunk there sets the whole
+    // pipeline back.  With a ring of two chunks a warp of its own issues them.  With the one-slot ring of 128-token tiles
+    // the thread that loads the chunks also multiplies them: it runs a few stages ahead of
     // the MMAs, has slack, polls the chunk's barriers between its activation stages, and waits for
     // them only where nothing it still has to do is needed for them to complete (after the last
     // activation stage of the item).  For the same reason no other role waits for a chunk in
@@ -297,12 +295,12 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     // barrier indices
     //   W_FULL[s]  weight bytes of stage landed (tx)          -> unpack warps
     //   W_FREE[s]  unpack warps have the weights in registers -> weight producer
-    //   X_FULL[x]  activation bytes of stage landed (tx)      -> MMA issuer of the stage
+    //   X_FULL[x]  activation bytes of stage landed (tx)      -> MMA issuer
     //   X_FREE[x]  MMAs of the stage retired (commit)         -> activation producer
-    //   READY[a]   A operand of the stage written to tensor memory -> MMA issuer of the stage
+    //   READY[a]   A operand of the stage written to tensor memory -> MMA issuer
     //   FREE[a]    MMAs of the stage retired (commit)         -> unpack warps
     //   FULL_LR / CONV_LR / EMPTY_LR[l]  low-rank chunk landed / converted / multiplied
-    //   ACC_FULL / ACC_EMPTY[2]  integer accumulator complete / read and zeroed by the epilogue
+    //   ACC_FULL / ACC_EMPTY[2]  integer accumulator complete / read by the epilogue
     //   DLR_EMPTY  the epilogue has read the low-rank accumulator -> low-rank issuer
     //   LR_DONE    the item's low-rank MMAs retired (commit by the producer) -> epilogue
     constexpr int B_W_FULL = 0, B_W_FREE = B_W_FULL + C::NW, B_X_FULL = B_W_FREE + C::NW,
@@ -332,7 +330,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             const uint32_t count =
                 (i == B_LR_DONE) ? 1u
                 : (i >= B_ACC_EMPTY) ? (uint32_t)C::EW
-                : (i >= B_ACC_FULL && i < B_ACC_EMPTY) ? 2u : 1u;
+                : (i >= B_ACC_FULL && !C::ProducerLr) ? 2u : 1u;         // both issuers
             mbar_init(bar(i), count);
         }
         if (lane == 0) {
@@ -391,6 +389,8 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     }
     const uint32_t tm_dint0 = tmem, tm_dlr = tmem + 2 * BT, tm_a0 = tmem + 3 * BT;
     const int lr_chunks = (p.r + 63) / 64;
+
+    auto wait_all = [&](uint32_t b, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait(b, parity, ab)) != 0; };
 
     if (warp == 0) {
         // =================== weight producer (one lane) ===================
@@ -533,92 +533,102 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                     mbar_wait(bar(B_X_FULL + i % C::NX), (i / C::NX) & 1, Abort{never_flag, p.status});
             }
         }
-    } else if (warp == 1 || warp == C::WarpIssuer1) {
-        // =================== MMA issuers (one lane each; even / odd stages) ===================
-        const int issuer = (warp == 1) ? 0 : 1;
-        if (lane == 0) {
-            constexpr uint32_t idesc_i8 = make_idesc(2, 1, 128, BT);
-            constexpr uint32_t idesc_f16 = make_idesc(1, 0, 128, BT);
-            Cursor cur;
-            cur.init(u_begin, u_end, p);
-            Work w;
-            uint32_t ca = 0, cl = 0, ci = 0, clr_items = 0;
-            bool ok = true;
-            while (ok && next_work(cur, p, w)) {
-                const int buf = ci & 1;
-                const uint32_t d_int = tm_dint0 + buf * BT;
-                // the epilogue warps hand the accumulator over zeroed (first time: initial zeroing)
-                ok = mbar_wait(bar(B_ACC_EMPTY + buf), (ci >> 1) & 1, ab);
-                if (!ok) break;
-                tc_fence_after();
-                const int nst = (w.kb1 - w.kb0 + KS - 1) / KS;
-                const bool mid = !C::ProducerLr && MID && issuer == 0 && lr_mid_tile(C::NL, w.has_lr, lr_chunks, nst);
-                int lc = 0;                // low-rank chunks of this item multiplied so far
-                // one chunk: wait for its conversion, multiply, hand the slot back
-                auto lr_chunk = [&](int c) {
+    } else if (warp == 1) {
+        // =================== MMA issuer ===================
+        constexpr uint32_t idesc_i8 = make_idesc(2, 1, 128, BT);
+        Cursor cur;
+        cur.init(u_begin, u_end, p);
+        Work w;
+        uint32_t ca = 0, ci = 0;       // ca counts stages
+        bool ok = true;
+        while (ok && next_work(cur, p, w)) {
+            const int buf = ci & 1;
+            const uint32_t d_int = tm_dint0 + buf * BT;
+            ok = wait_all(bar(B_ACC_EMPTY + buf), (ci >> 1) & 1);        // the epilogue has read it
+            if (!ok) break;
+            tc_fence_after();
+            bool ready = false;          // the next A slot, and its activations, have been seen to be there
+            for (int kb = w.kb0; kb < w.kb1 && ok; kb += KS, ++ca) {
+                const int nkb = (w.kb1 - kb < KS) ? (w.kb1 - kb) : KS;
+                const int sx = ca % C::NX;
+                const uint64_t xdesc = smem_desc_sw128(sbase + C::OffX + sx * C::XBytes);
+#pragma unroll
+                for (int sub = 0; sub < C::SPS; ++sub) {
+                    const uint32_t cs = ca * C::SPS + sub;          // running A-slot counter
+                    const int sa = cs % C::NA;
+                    if (!ready) {
+                        ok = (sub > 0 || mbar_wait(bar(B_X_FULL + sx), (ca / C::NX) & 1, ab)) &&
+                             mbar_wait(bar(B_READY + sa), (cs / C::NA) & 1, ab);
+                        ok = __all_sync(0xffffffffu, ok) != 0;
+                    }
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t a_tm = tm_a0 + sa * C::ASlotCols, xn = sub == C::SPS - 1 ? ca + 1 : ca;
+#pragma unroll
+                    for (int jj = 0; jj < C::KA; ++jj) {
+                        const int j = sub * C::KA + jj;
+                        if (j < nkb) {
+                            const uint32_t acc = (kb != w.kb0 || j != 0) ? 1u : 0u;
+                            const uint64_t xd = xdesc + (uint64_t)(j * (C::XTile >> 4));
+                            if (jj == 0)
+                                ready = mma_i8_block_elect_look(d_int, a_tm, xd, idesc_i8, acc, bar(B_READY + (cs + 1) % C::NA), ((cs + 1) / C::NA) & 1,
+                                                                bar(B_X_FULL + xn % C::NX), (xn / C::NX) & 1);
+                            else
+                                mma_i8_block_elect(d_int, a_tm + jj * 32, xd, idesc_i8, acc);
+                        } else if (jj == 0) {
+                            ready = false;
+                        }
+                    }
+                    if (elect_one()) {
+                        tc_commit(bar(B_FREE + sa));   // an empty slot (ragged last stage) still hands over
+                        if (sub == C::SPS - 1) tc_commit(bar(B_X_FREE + sx));
+                    }
+                    ready = __all_sync(0xffffffffu, ready) != 0;
+                }
+            }
+            if (ok && elect_one()) tc_commit(bar(B_ACC_FULL + buf));
+            __syncwarp();
+            ++ci;
+        }
+        if (lane == 0 && *abort_flag) dump_role(p.status, 2, ca, 0u, ci, (uint32_t)w.tile, ((uint32_t)w.kb0 << 16) | (uint32_t)w.kb1);
+    } else if (!C::ProducerLr && warp == C::WarpLrIssuer) {
+        // =================== low-rank MMA issuer: sums of its own, in step with the items ===================
+        constexpr uint32_t idesc_f16 = make_idesc(1, 0, 128, BT);
+        Cursor cur;
+        cur.init(u_begin, u_end, p);
+        Work w;
+        uint32_t cl = 0, ci = 0, clr_items = 0;
+        bool ok = true;
+        while (ok && next_work(cur, p, w)) {
+            if (w.has_lr) {
+                ok = wait_all(bar(B_DLR_EMPTY), (clr_items & 1) ^ 1);    // the epilogue before has read them
+                for (int c = 0; c < lr_chunks && ok; ++c) {
                     const int s = cl % C::NL;
-                    if (!mbar_wait(bar(B_CONV_LR + s), (cl / C::NL) & 1, ab)) return false;
+                    ok = wait_all(bar(B_CONV_LR + s), (cl / C::NL) & 1);
+                    if (!ok) break;
                     tc_fence_after();
                     const uint64_t adesc = smem_desc_sw128(sbase + C::OffLb + s * C::LbBytes);
                     const uint64_t bdesc = smem_desc_sw128(sbase + C::OffT + s * C::TBytes);
                     int steps = (p.r - c * 64) / 16;
                     if (steps > 4) steps = 4;
-                    for (int kk = 0; kk < steps; ++kk)
-                        mma_f16_ss(tm_dlr, adesc + 2 * kk, bdesc + 2 * kk, idesc_f16,
-                                   (c != 0 || kk != 0) ? 1u : 0u);
-                    tc_commit(bar(B_EMPTY_LR + s));
+                    if (elect_one()) {
+                        for (int kk = 0; kk < steps; ++kk)
+                            mma_f16_ss(tm_dlr, adesc + 2 * kk, bdesc + 2 * kk, idesc_f16,
+                                       (c != 0 || kk != 0) ? 1u : 0u);
+                        tc_commit(bar(B_EMPTY_LR + s));
+                    }
+                    __syncwarp();
                     ++cl;
-                    return true;
-                };
-                int st_idx = 0;
-                for (int kb = w.kb0; kb < w.kb1 && ok; kb += KS, ++st_idx) {
-                    const int nkb = (w.kb1 - kb < KS) ? (w.kb1 - kb) : KS;
-                    const int sx = ca % C::NX;   // ca counts stages
-                    if (mid && lc < lr_chunks - 1 && st_idx == lr_mma_stage(lc, lr_chunks, nst)) {
-                        // the epilogue of the previous item has read the low-rank accumulator
-                        if (lc == 0) ok = mbar_wait(bar(B_DLR_EMPTY), (clr_items & 1) ^ 1, ab);
-                        ok = ok && lr_chunk(lc);
-                        if (!ok) break;
-                        ++lc;
-                    }
-                    if ((int)(ca & 1u) != issuer) { ++ca; continue; }
-                    ok = mbar_wait(bar(B_X_FULL + sx), (ca / C::NX) & 1, ab);
-                    if (!ok) break;
-                    const uint64_t xdesc = smem_desc_sw128(sbase + C::OffX + sx * C::XBytes);
-#pragma unroll
-                    for (int sub = 0; sub < C::SPS; ++sub) {
-                        const uint32_t cs = ca * C::SPS + sub;          // running A-slot counter
-                        const int sa = cs % C::NA;
-                        ok = ok && mbar_wait(bar(B_READY + sa), (cs / C::NA) & 1, ab);
-                        if (!ok) break;
-                        tc_fence_after();
-                        const uint32_t a_tm = tm_a0 + sa * C::ASlotCols;
-#pragma unroll
-                        for (int jj = 0; jj < C::KA; ++jj) {
-                            const int j = sub * C::KA + jj;
-                            if (j < nkb) {
-#pragma unroll
-                                for (int kk = 0; kk < 4; ++kk)
-                                    mma_i8_ts(d_int, a_tm + jj * 32 + kk * 8,
-                                              xdesc + (uint64_t)(j * (C::XTile >> 4) + 2 * kk), idesc_i8, 1u);
-                            }
-                        }
-                        tc_commit(bar(B_FREE + sa));   // an empty slot (ragged last stage) still hands over
-                    }
-                    if (!ok) break;
-                    tc_commit(bar(B_X_FREE + sx));
-                    ++ca;
                 }
-                if (!C::ProducerLr && ok && w.has_lr && issuer == 0) {
-                    if (lc == 0) ok = mbar_wait(bar(B_DLR_EMPTY), (clr_items & 1) ^ 1, ab);
-                    for (int c = lc; c < lr_chunks && ok; ++c) ok = lr_chunk(c);
-                    ++clr_items;
-                }
-                if (ok) tc_commit(bar(B_ACC_FULL + buf));
-                ++ci;
+                ++clr_items;
             }
-            if (*abort_flag) dump_role(p.status, 2 + issuer, ca, cl, ci, (uint32_t)w.tile, ((uint32_t)w.kb0 << 16) | (uint32_t)w.kb1);
+            // (An item without a low-rank term waits for the epilogue too: two arrivals must not fall into one phase.)
+            ok = ok && wait_all(bar(B_ACC_EMPTY + (ci & 1)), (ci >> 1) & 1);
+            if (ok && elect_one()) tc_commit(bar(B_ACC_FULL + (ci & 1)));
+            __syncwarp();
+            ++ci;
         }
+        if (lane == 0 && *abort_flag) dump_role(p.status, 3, 0u, cl, ci, (uint32_t)w.tile, ((uint32_t)w.kb0 << 16) | (uint32_t)w.kb1);
     } else if (warp < 10) {
         // =================== unpack warps: int4 -> int8 (x16) into tensor memory ===================
         const int q = warp & 3;                    // TMEM lane quarter this warp may touch
@@ -739,9 +749,6 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         uint32_t ci = 0, lr_seen = 0;
         int partial_idx = 0;                       // 0: first partial item of this CTA, 1: second
         bool ok = true;
-        // both integer accumulators start at zero: every integer MMA accumulates
-        for (int c0 = 16 * half; c0 < 2 * BT; c0 += kChunkStep) tmem_zero16(tm_dint0 + lane_sel + c0);
-        tmem_wait_st();
         grid_dep_wait();            // a_scale comes from the kernel launched before this one
         tc_fence_before();
         __syncwarp();
@@ -817,8 +824,6 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                     }
                 }
             }
-            for (int c0 = 16 * half; c0 < BT; c0 += kChunkStep) tmem_zero16(d_int + c0);   // hand it back zeroed
-            tmem_wait_st();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {

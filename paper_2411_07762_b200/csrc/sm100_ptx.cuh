@@ -102,6 +102,35 @@ __device__ __forceinline__ void mma_i8_ts(uint32_t d, uint32_t a, uint64_t bdesc
         ::"r"(d), "r"(a), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// The four products of a 128-column block (`accumulate` is for the first) by the elected lane of a converged warp; with a look at
+// two barrier phases that is issued before them and read after them.
+#define ASER_MMA_I8_BLOCK                                                          \
+    "elect.sync _|e, 0xffffffff;\n\t"                                              \
+    "setp.ne.b32 p, %5, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"                            \
+    "@e tcgen05.mma.cta_group::1.kind::i8 [%1], [%2], %3, %4, p;\n\t"             \
+    "add.u32 x, %2, 8;\n\tadd.u64 y, %3, 2;\n\t"                                  \
+    "@e tcgen05.mma.cta_group::1.kind::i8 [%1], [x], y, %4, t;\n\t"               \
+    "add.u32 x, %2, 16;\n\tadd.u64 y, %3, 4;\n\t"                                 \
+    "@e tcgen05.mma.cta_group::1.kind::i8 [%1], [x], y, %4, t;\n\t"               \
+    "add.u32 x, %2, 24;\n\tadd.u64 y, %3, 6;\n\t"                                 \
+    "@e tcgen05.mma.cta_group::1.kind::i8 [%1], [x], y, %4, t;\n\t"
+__device__ __forceinline__ void mma_i8_block_elect(uint32_t d, uint32_t a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+    uint32_t none;
+    asm volatile("{\n\t.reg .pred e, p, t;\n\t.reg .b32 x;\n\t.reg .b64 y;\n\t" ASER_MMA_I8_BLOCK "mov.u32 %0, 0;\n\t}"
+                 : "=r"(none) : "r"(d), "r"(a), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ bool mma_i8_block_elect_look(uint32_t d, uint32_t a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate,
+                                                        uint32_t bar0, uint32_t parity0, uint32_t bar1, uint32_t parity1) {
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred e, p, t, w, v;\n\t.reg .b32 x;\n\t.reg .b64 y;\n\t"
+                 "mbarrier.test_wait.parity.shared::cta.b64 w, [%6], %7;\n\t"
+                 "mbarrier.test_wait.parity.shared::cta.b64 v, [%8], %9;\n\t" ASER_MMA_I8_BLOCK
+                 "and.pred w, w, v;\n\tselp.u32 %0, 1, 0, w;\n\t}"
+                 : "=r"(done)
+                 : "r"(d), "r"(a), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(bar0), "r"(parity0), "r"(bar1), "r"(parity1)
+                 : "memory");
+    return done != 0;
+}
 // D[tmem] (+)= A[smem desc] * B[smem desc], fp16 x fp16 -> fp32
 __device__ __forceinline__ void mma_f16_ss(uint32_t d, uint64_t adesc, uint64_t bdesc,
                                            uint32_t idesc, uint32_t accumulate) {
@@ -211,15 +240,6 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16
         ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]),
         "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]),
         "r"(v[14]), "r"(v[15])
-        : "memory");
-}
-// Zero 16 consecutive columns of this warp's 32 lanes.
-__device__ __forceinline__ void tmem_zero16(uint32_t taddr) {
-    const uint32_t z = 0;
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-        "{%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};"
-        ::"r"(taddr), "r"(z)
         : "memory");
 }
 __device__ __forceinline__ void tmem_wait_st() {
