@@ -56,6 +56,10 @@ __device__ __forceinline__ void store_t2(__nv_bfloat16* row, int j, float t0, fl
             __floats2bfloat162_rn(t0 - __low2float(hi), t1 - __high2float(hi));
 }
 
+// The factor that stands in for the division by a row's scale: 0 for a row of zeros, and where 1 / sc may overflow.  Then
+// every undivided element is zero (the smallest fp16 magnitude over 127 is 4.7e-10); what smoothing divided goes by exact codes.
+__device__ __forceinline__ float code_rcp(float sc) { return sc > 0x1p-127f ? __frcp_rn(sc) : 0.f; }
+
 // Exact codes for eight values (the definition: IEEE quotient, round half to even, clamp).
 static __device__ __noinline__ uint2 quant8_exact(float v0, float v1, float v2, float v3, float v4, float v5,
                                            float v6, float v7, float sc, float qmax) {
@@ -68,7 +72,7 @@ static __device__ __noinline__ uint2 quant8_exact(float v0, float v1, float v2, 
     }
     return make_uint2(w[0], w[1]);
 }
-// Same codes as quant8 for sc > 0, on packed fp32 pairs: t = x~ * (1 / sc), rounded by adding
+// The same codes, with rcp = code_rcp(sc), on packed fp32 pairs: t = x~ * (1 / sc), rounded by adding
 // 1.5 * 2^23 (the low byte of the sum is the code); the distance of t to that integer tells the
 // near-ties, and a group with one takes the exact path as a whole.
 __device__ __forceinline__ uint2 quant8_pairs(const float (&v)[8], float sc, float rcp, float qmax) {
@@ -87,7 +91,7 @@ __device__ __forceinline__ uint2 quant8_pairs(const float (&v)[8], float sc, flo
         q[2 * i + 1] = __float_as_uint(u.y);
         far = fmaxf(far, fmaxf(fabsf(d.x), fabsf(d.y)));
     }
-    if (far > 0.4999f) return quant8_exact(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7], sc, qmax);
+    if (far > 0.4999f || (rcp == 0.f && sc > 0.f)) return quant8_exact(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7], sc, qmax);
     const uint32_t a01 = __byte_perm(q[0], q[1], 0x0040), a23 = __byte_perm(q[2], q[3], 0x0040);
     const uint32_t a45 = __byte_perm(q[4], q[5], 0x0040), a67 = __byte_perm(q[6], q[7], 0x0040);
     return make_uint2(__byte_perm(a01, a23, 0x5410), __byte_perm(a45, a67, 0x5410));
@@ -245,7 +249,7 @@ __device__ __forceinline__ void quantize_rows(const __half* __restrict__ X, cons
 #pragma unroll
     for (int rr = 0; rr < R; ++rr) {
         sc[rr] = __fdiv_rn(__uint_as_float(sh.rowmax[rr]), qmax);
-        rcp[rr] = sc[rr] > 0.f ? __frcp_rn(sc[rr]) : 0.f;
+        rcp[rr] = code_rcp(sc[rr]);
     }
 #pragma unroll
     for (int rr = 0; rr < R; ++rr)

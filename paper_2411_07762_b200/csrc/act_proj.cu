@@ -497,7 +497,7 @@ act_quant_kernel(const __half* __restrict__ X, const float* __restrict__ s, int 
         if (lane == 0) {
             const float sc = __fdiv_rn(a, qmax);
             sc_sm[warp] = sc;
-            rcp_sm[warp] = (sc > 0.f) ? __frcp_rn(sc) : 0.f;
+            rcp_sm[warp] = code_rcp(sc);
             a_scale[row0 + warp] = sc;
         }
     } else if (warp < kQRows && lane == 0) {
@@ -710,7 +710,7 @@ act_rows_kernel(const __half* __restrict__ X, const float* __restrict__ s, int M
             row_sync();
             for (int w = 0; w < W; ++w) top = max(top, part[flip][sub * W + w]);
         }
-        const float sc = __fdiv_rn(__uint_as_float(top), qmax), rcp = sc > 0.f ? __frcp_rn(sc) : 0.f;
+        const float sc = __fdiv_rn(__uint_as_float(top), qmax), rcp = code_rcp(sc);
         if (c0 == 0) a_scale[m] = sc;
         if (!(sc > 0.f)) {
 #pragma unroll

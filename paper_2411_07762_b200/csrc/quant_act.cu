@@ -966,8 +966,8 @@ quant_act_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
 
         // ---- sweep 2: int8 codes into the output tiles (they take the place of the L_A ring;
         // the wait on the accumulator above says the MMAs are done reading it) ----
-        const float rcp0 = (sc0 > 0.f) ? __frcp_rn(sc0) : 0.f;
-        const float rcp1 = (sc1 > 0.f) ? __frcp_rn(sc1) : 0.f;
+        const float rcp0 = code_rcp(sc0);
+        const float rcp1 = code_rcp(sc1);
         for (int jj = all_observe ? 0 : grp; jj < nst && ok; jj += all_observe ? 1 : 2) {
             const int i = nst + jj, st = i % NS, o = jj % kTOut;
             ok = qa_warp_wait(bar_full(st), (uint32_t)(i / NS) & 1u, abort_flag, lane);

@@ -273,6 +273,24 @@ def test_quant_act_beside_projection(aser, entry, M, K, r, divided, act_bits, t_
         assert_T_close(T[:, :r].float().cpu().numpy(), F.down_proj(xs, L_A), xs, L_A)
 
 
+@pytest.mark.parametrize("entry", ["one", "ws"])
+@pytest.mark.parametrize("M,K", [(20, 1024), (40, 8192), (300, 2048), (900, 4096), (333, 14336)])
+@pytest.mark.parametrize("divided,s_value", [(3, 1e36), (3, 3e37), (0, 3e37), (600, 1e-36)])
+def test_quant_act_rows_with_tiny_scales(aser, entry, M, K, divided, s_value):
+    """Rows whose only elements that are not zero were divided by huge factors: the reciprocal of the scale overflows.
+    divided 0: every column (the loop without a list)."""
+    rng = np.random.default_rng(M + K + divided)
+    X = rng.standard_normal((M, K)).astype(np.float16)
+    s = np.ones(K, np.float32)
+    cols = rng.choice(K, divided or K, replace=False)
+    s[cols] = s_value
+    X[::2, s == 1] = 0
+    Xq_ref, sc_ref = F.quant_act(F.smooth_act(X, s))
+    Xq, sc, _ = (aser.quant_act if entry == "one" else aser.quant_act_ws)(to_dev(X), to_dev(s), None)
+    assert np.array_equal(bits(sc.cpu().numpy()), bits(sc_ref))
+    assert np.array_equal(Xq.cpu().numpy(), Xq_ref)
+
+
 # ---------------------------------------------------------------------------
 # whole path: quant_act -> linear
 # ---------------------------------------------------------------------------
