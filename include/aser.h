@@ -136,8 +136,8 @@ int aser_quant_act_ex(const void* X_f16, const float* s, const void* LA_f16,
  * `stream` that still uses the workspace when the call is made must precede it on `stream`.
  */
 size_t aser_quant_workspace_bytes(int M, int K, int r);
-/* Number of kernels one aser_quant_act_ws call enqueues (1 up to 32 tokens, else 2, the
- * first of which a pass without a projection does not need; 0 for bad shapes). */
+/* Number of kernels one aser_quant_act_ws call with a projection (r > 0) enqueues: 1 up to 32 tokens, else 2; 0
+ * for bad shapes.  A call without one enqueues a single kernel. */
 int aser_quant_act_ws_launches(int M, int K);
 int aser_quant_act_ws(const void* X_f16, const float* s, const void* LA_f16,
                       int M, int K, int r, int act_bits, int t_pair,

@@ -352,7 +352,7 @@ class AserLinear:
         """The activation step alone, with the kernels aser_forward runs at this shape."""
         M = X.shape[0]
         r = self.r
-        if forward_act_launches(M, self.K, r) == 1:
+        if forward_act_launches(M, self.K, r or 16) == 1:       # (without a projection either step is one kernel: the same choice)
             _chk(lib.aser_quant_act(_ptr(X), _ptr(self.s), _ptr(self.L_A) if r else None, M, self.K, r,
                                     _ptr(self.Xq), _ptr(self.a_scale), _ptr(self.T) if r else None,
                                     _stream()), "aser_quant_act")
@@ -432,7 +432,7 @@ class AserSharedInput:
     def quant(self, X: torch.Tensor):
         """The activation pass of the group alone (aser_quant_act_ws with the stacked L_A)."""
         M = X.shape[0]
-        if forward_act_launches(M, self.K, self.r_total) == 1 and self.r_total <= 256:
+        if forward_act_launches(M, self.K, self.r_total or 16) == 1 and self.r_total <= 256:
             _chk(lib.aser_quant_act(_ptr(X), _ptr(self.s), _ptr(self.L_A), M, self.K, self.r_total,
                                     _ptr(self.Xq), _ptr(self.a_scale), _ptr(self.T) if self.r_total else None,
                                     _stream()), "aser_quant_act")

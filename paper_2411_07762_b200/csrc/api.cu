@@ -489,7 +489,7 @@ int aser_quant_act_ws(const void* X_f16, const float* s, const void* LA_f16, int
 
 int aser_forward_act_launches(int M, int K, int r) {
     if (!act_shape_ok(M, K, r) || M == 0) return 0;
-    return forward_act_uses_scratch(M, K, r) ? quant_act_ws_launches(M, K) : 1;
+    return forward_act_uses_scratch(M, K, r) && r > 0 ? quant_act_ws_launches(M, K) : 1;
 }
 
 int aser_linear_w4a8_lr_ld(const int8_t* Xq, const float* a_scale, const void* Wk,

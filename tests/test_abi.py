@@ -123,13 +123,20 @@ def test_construct_workspace_of_large_layers(lib):
 
 
 def test_activation_path_of_a_forward_pass(lib):
-    """One launch (few-token or cluster kernel) or two: the cluster kernel serves whole 64-token clusters, seven of
-    them at 4096 columns and more."""
+    """One launch or two (many tokens, and ranks above 128 from 33 on): 448 tokens are seven whole clusters of the
+    cluster kernel, the last of the one-launch kernels, at 4096 columns and more."""
     for K in (4096, 8192, 14336):
         assert [lib.aser_forward_act_launches(M, K, 128) for M in (1, 32, 33, 447, 448, 449, 4096)] == [1, 1, 1, 1, 1, 2, 2]
     assert [lib.aser_forward_act_launches(M, 2048, 128) for M in (1023, 1024)] == [1, 2]
     assert [lib.aser_forward_act_launches(M, 1024, 128) for M in (4096, 4097)] == [1, 2]
     assert [lib.aser_forward_act_launches(M, 4096, 144) for M in (32, 33)] == [1, 2]
+
+
+def test_activation_path_without_a_projection_is_one_launch(lib):
+    """The kernel that quantizes rows is the only one then, whatever the number of tokens."""
+    for K in (1024, 4096, 8192, 14336):
+        assert {lib.aser_forward_act_launches(M, K, 0) for M in (1, 32, 33, 448, 449, 4097)} == {1}
+    assert lib.aser_forward_act_launches(0, 4096, 0) == 0 and lib.aser_forward_act_launches(8, 4100, 0) == 0
 
 
 def test_linear_kernel_rejects_bad_shapes(lib):
