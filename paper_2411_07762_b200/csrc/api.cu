@@ -806,10 +806,14 @@ int aser_forward_host(const void* X_host_f16, void* Y_host_f16, void* X_dev, int
         if (rc != ASER_OK) break;
         e = cudaEventRecord(lane->computed[part], st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(lane->out, lane->computed[part], 0);
-        // A part goes out when the one after it has come in.  Otherwise its copy starts in the middle of the other direction's,
-        // and two copies at once are slower than one: 2048 tokens 4096 -> 4096 564 -> 520 us, 1024 302 -> 293; behind two further
-        // parts 582 and 319.  (Two parts: 177 as it is, 181 so.)
-        if (e == cudaSuccess && parts > 2) e = cudaStreamWaitEvent(lane->out, lane->landed[part + 1 < parts ? part + 1 : part], 0);
+        // A part goes out when the one after it has come in, so that its copy and the one after that in the other direction start
+        // together: a copy that starts in the middle of one in the other direction costs both 20 to 30 us.  That fits where a
+        // part's Y is no longer than its X; a longer one still goes out when the next X starts, and only loses the wait.  As soon as
+        // computed / so, us: 1024 x 4096 -> 4096 310 / 299; 2048 x 4096 -> 4096 565 / 526, -> 4104 568 / 528; 1024 x 6144 -> 4096 401 /
+        // 352; 2048 x 8192 -> 8192 1015 / 979; 1024 x 4096 -> 6144 343 / 362, -> 8192 417 / 446, -> 14336 647 / 651.  Behind two
+        // further parts 325 and 588 for the first two; with two parts no difference.
+        if (e == cudaSuccess && parts > 2 && N <= K + K / 8)
+            e = cudaStreamWaitEvent(lane->out, lane->landed[part + 1 < parts ? part + 1 : part], 0);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(static_cast<__half*>(Y_host_f16) + y0, static_cast<__half*>(Y_dev) + y0, yn * 2,
                                 cudaMemcpyDeviceToHost, lane->out);
