@@ -21,7 +21,7 @@
 //
 // (Sec. 4.2 smoothing M^-1 X of Eq. 10, Sec. 5.1 per-token round-to-nearest, Sec. 4.1 projection
 // V_r^T S^-1 of the reconstruction branch.)  All kernels are deterministic: no atomics on global memory.
-// Every mbarrier wait is bounded; a CTA that gives up makes its tokens' partial T NaN.
+// Every mbarrier wait is bounded; a CTA that gives up makes its tokens' partial T, and row maxima, NaN.
 #include "act_math.cuh"
 #include "aser_common.cuh"
 #include "sm100_ptx.cuh"
@@ -111,7 +111,7 @@ __device__ __forceinline__ void pj_stage_t(uint32_t tmem, int g, uint32_t buf, i
 
 // grid = (KS slices, token tiles).
 // MAXIMA: the row maxima of |x~| over the slice and the partial T go to the scratch,
-//   amax_part [KS][M]               fp32
+//   amax_part [KS][M]               fp32 (NaN: the CTA gave up)
 //   t_part    [KS][groups][M][128]  fp32, by 128-row group of L_A (rows past r: unspecified; NaN: the CTA gave up)
 // otherwise the slices of a tile are a cluster that sums the partial T through distributed shared memory and writes T.
 // map_x: X as fp16 [K / 64 blocks][M][64], box 1 block x 128 rows, 128-byte swizzle (rows past
@@ -359,6 +359,7 @@ act_proj_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
                 float a = amax_w[row];
 #pragma unroll
                 for (int w = 1; w < kPConsumerWarps; ++w) a = fmaxf(a, amax_w[w * kPTok + row]);
+                if (*abort_flag) a = __int_as_float(0x7fc00000);        // not all columns were seen
                 amax_part[(size_t)ks * M + row0 + row] = a;
             }
         }
