@@ -97,13 +97,6 @@ __device__ __forceinline__ uint2 quant8_pairs(const float (&v)[8], float sc, flo
     return make_uint2(__byte_perm(a01, a23, 0x5410), __byte_perm(a45, a67, 0x5410));
 }
 
-// Largest magnitude of three (a NaN does not count).
-__device__ __forceinline__ float max3_abs(float a, float b, float c) {
-    float d;
-    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-
 // Eight codes of a row whose divisors are all 1: fp16 pairs widened by the conversion unit, then on
 // packed fp32 pairs su = x * (1 / sc) + 1.5 * 2^23 (one rounding: the low byte of su is the code),
 // -w = 1.5 * 2^23 - su (exact) and d = x * (1 / sc) - w, the distance of the product to its integer.
@@ -159,7 +152,7 @@ struct RowsShared {
     int list_col[kRowsList];
 };
 
-// The code of a NaN is -1 (the low byte of its bits), also in a row whose scale is zero.
+// (Codes of a NaN are unspecified: -1 by the fast path, -qmax by the exact one.)
 template <int CPT, int R>
 __device__ __forceinline__ void quantize_rows(const __half* __restrict__ X, const float* __restrict__ s, int nrows, int K,
                                               int8_t* __restrict__ Xq, float* __restrict__ a_scale, float qmax,

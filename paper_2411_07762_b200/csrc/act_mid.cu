@@ -28,11 +28,6 @@ __device__ __forceinline__ void mid_mma(float (&d)[4], uint32_t a0, uint32_t a1,
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ float mid_ld_cluster(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-    return v;
-}
 
 // Grid: t_tiles * CL projecting CTAs (clusters of CL along K), then the quantizing CTAs, R rows each.
 // A sum (register 4 (4 mt + nt) + e of lane 4 g + t) is token 16 mt + g + 8 (e / 2), L_A row 8 nt + 2 t + e % 2.
@@ -145,7 +140,7 @@ quant_act_mid_kernel(const __half* __restrict__ X, const float* __restrict__ s, 
     for (int i = rank * per + tid; i < (rank + 1) * per; i += kMThreads) {
         float v[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = q < CL ? (CL > 1 ? mid_ld_cluster(map_to_rank(mine + 4u * i, q)) : part[i >> 5][i & 31]) : 0.f;
+        for (int q = 0; q < 8; ++q) v[q] = q < CL ? (CL > 1 ? ld_cluster_f32(map_to_rank(mine + 4u * i, q)) : part[i >> 5][i & 31]) : 0.f;
         float sum = v[0];
 #pragma unroll
         for (int q = 1; q < 8; ++q) sum += v[q];
@@ -203,11 +198,10 @@ bool quant_act_mid_prefers(int M, int K, int r) {
 
 int launch_quant_act_mid(const __half* X, const float* s, const __half* LA, int M, int K, int r, int8_t* Xq, float* a_scale,
                          __nv_bfloat16* T, int ldt, int lo_off, float qmax, cudaStream_t st) {
-    // chunks of eight columns per thread by the row length, one or two rows per quantizing CTA
+    // chunks of eight columns per thread by the row length, one, two or four rows per quantizing CTA
     const int chunks = (K / 8 + kMThreads - 1) / kMThreads, rows = mid_rows(M, K);
     auto go = [&](auto* kernel) { return launch_mid_cfg(kernel, rows, X, s, LA, M, K, r, Xq, a_scale, T, ldt, lo_off, qmax, st); };
-    if (rows == 4 && chunks <= 1) return go(quant_act_mid_kernel<1, 4>);
-    if (rows == 4 && chunks <= 2) return go(quant_act_mid_kernel<2, 4>);
+    if (rows == 4) return go(quant_act_mid_kernel<1, 4>);        // up to 2048 columns
     if (chunks <= 1) return rows == 2 ? go(quant_act_mid_kernel<1, 2>) : go(quant_act_mid_kernel<1, 1>);
     if (chunks <= 2) return rows == 2 ? go(quant_act_mid_kernel<2, 2>) : go(quant_act_mid_kernel<2, 1>);
     if (chunks <= 4) return rows == 2 ? go(quant_act_mid_kernel<4, 2>) : go(quant_act_mid_kernel<4, 1>);

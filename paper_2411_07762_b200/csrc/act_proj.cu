@@ -52,7 +52,7 @@ __host__ __device__ constexpr int proj_stages(int groups, int K, bool beside) {
     int ns = (beside ? 213 * 1024 - 2 * (K + 5300) : 208 * 1024) / per_stage;
     const int least = (131072 + per_stage - 1) / per_stage;
     ns = ns < least ? least : ns;
-    return ns > 8 ? 8 : ns;                 // 6, 4, 3, 2 stages for 1..4 groups
+    return ns > 8 ? 8 : ns;                 // 6, 4, 3, 2 stages for 1..4 groups; 5 beside rows of 8192 columns (one group)
 }
 
 __device__ __noinline__ bool pj_wait_slow(uint32_t bar, uint32_t parity, volatile int* flag) {
@@ -89,11 +89,6 @@ __device__ __forceinline__ void pj_sts128(uint32_t addr, uint4 v) {
     asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
-__device__ __forceinline__ float4 pj_ld_cluster128(uint32_t addr) {
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
-}
 // A group's partial sums, tensor memory -> `buf` as [token][128 rows of the group].  A warp reaches the 32 lanes (rows j) of
 // its quarter, warp % 4; the two warps of a quarter take 64 tokens each.  gave_up: NaN instead.
 __device__ __forceinline__ void pj_stage_t(uint32_t tmem, int g, uint32_t buf, int cw, int warp, int lane, bool gave_up) {
@@ -411,7 +406,7 @@ act_proj_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
                     float4 a[4];
 #pragma unroll
                     for (int q = 0; q < 4; ++q)
-                        a[q] = q0 + q < (int)gridDim.x ? pj_ld_cluster128(map_to_rank(sb + (uint32_t)e * 16u, (uint32_t)(q0 + q)))
+                        a[q] = q0 + q < (int)gridDim.x ? ld_cluster_f32x4(map_to_rank(sb + (uint32_t)e * 16u, (uint32_t)(q0 + q)))
                                                        : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                     for (int q = 0; q < 4; ++q) { v.x += a[q].x; v.y += a[q].y; v.z += a[q].z; v.w += a[q].w; }
@@ -584,7 +579,7 @@ act_quant_kernel(const __half* __restrict__ X, const float* __restrict__ s, int 
 // The codes and scales need nothing from act_proj_kernel, so the two kernels run beside each other.  Without a projection
 // it is the only kernel of the pass and waits for what precedes it first.
 //
-// A row belongs to W warps (one up to 4096 columns), a lane has at most C 8-column chunks of it in registers: all loads
+// A row belongs to W warps (one up to 2048 columns, two up to 4096), a lane has at most C 8-column chunks of it in registers: all loads
 // of a row leave together, its maximum is one warp reduction, and no block-wide barrier ties the warps of an SM together, so
 // some load while others compute.  (A block per two or four rows with two chunks per thread spent 155 instructions per chunk, two
 // thirds of them per-group overhead.)
@@ -764,7 +759,8 @@ act_rows_kernel(const __half* __restrict__ X, const float* __restrict__ s, int M
     if (beside && blockIdx.x == 0) grid_dep_wait();
 }
 
-// W warps per row and C chunks per lane: the fewest warps that need at most sixteen chunks.
+// W warps per row and C chunks per lane: the fewest warps that need at most eight chunks; sixteen where eight warps do not
+// suffice (rows above 16384).
 int launch_rows(cudaLaunchConfig_t cfg, const __half* X, const float* s, int M, int K, bool beside, int8_t* Xq,
                 float* a_scale, float qmax) {
     auto go = [&](auto* kernel, int W) {

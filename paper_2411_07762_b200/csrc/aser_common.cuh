@@ -160,6 +160,18 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 // Round-half-to-even to an integer-valued float, then clamp; returns the int.
+// Largest magnitude of three: a NaN does not count, or makes the result NaN.
+__device__ __forceinline__ float max3_abs(float a, float b, float c) {
+    float d;
+    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+__device__ __forceinline__ float max3_abs_nan(float a, float b, float c) {
+    float d;
+    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
 __device__ __forceinline__ int rne_clamp(float v, float lo, float hi) {
     float c = rintf(v);
     c = fminf(fmaxf(c, lo), hi);

@@ -338,6 +338,8 @@ int launch_linear_decode_group(const int8_t* Xq, const float* a_scale, const __n
                                const LinearGroup& group, int32_t* acc_debug, cudaStream_t st, bool overlap_prev, int ldt,
                                CatSplit cat) {
     if (M > kLinearDecodeMaxTokens) return record_error(ASER_ERR_SHAPE, "linear_decode: more than 16 tokens");
+    if (group.layers > 1 && (acc_debug || cat.layers > 1))
+        return record_error(ASER_ERR_SHAPE, "linear_decode: neither accumulators nor fused layers of a group");
     if (M <= 8) return launch_nt<1>(Xq, a_scale, T, M, K, acc_debug, st, overlap_prev, ldt, cat, group);
     return launch_nt<2>(Xq, a_scale, T, M, K, acc_debug, st, overlap_prev, ldt, cat, group);
 }

@@ -686,6 +686,8 @@ bool linear_pair_groups(const LinearGroup& g, int M, int K) {
 
 int launch_linear_pair_group(const int8_t* Xq, const float* a_scale, const __nv_bfloat16* T, int M, int K, const LinearGroup& g,
                              int32_t* acc_debug, void* workspace, cudaStream_t st, bool overlap_prev, int ldt, CatSplit cat) {
+    if (g.layers > 1 && (acc_debug || cat.layers > 1))
+        return record_error(ASER_ERR_SHAPE, "linear_pair: neither accumulators nor fused layers of a group");
     int num_sms = 0;
     int rc = device_sm_count(&num_sms);
     if (rc != ASER_OK) return rc;

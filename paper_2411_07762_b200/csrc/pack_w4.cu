@@ -7,17 +7,6 @@ namespace aser {
 
 namespace {
 
-// Largest magnitude of three: a NaN does not count, or makes the result NaN.
-__device__ __forceinline__ float max3_abs(float a, float b, float c) {
-    float d;
-    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-__device__ __forceinline__ float max3_abs_nan(float a, float b, float c) {
-    float d;
-    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
 // Low nibbles of four words, one after the other in sixteen bits.
 __device__ __forceinline__ uint32_t nibbles4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
     uint32_t x = __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410) & 0x0F0F0F0Fu;
