@@ -412,7 +412,9 @@ class Model:
                 S["layers"][idx[0]](S["xs"][g], lowrank)
 
     def linear_only(self, i, li=None, lowrank=True):
-        """The linear launches of a step (a fused group is one launch), or layer `li` on its own."""
+        """The linear products of a step, or layer `li` on its own.  A fused group is one launch, other layers are
+        launched one by one: a pass may serve such a group by one launch too (launches_per_step), for which the
+        binding has no entry of its own."""
         S = self.sets[i % self.n_sets]
         if li is not None:
             S["layers"][li].linear(self.M, lowrank)
@@ -454,16 +456,22 @@ class Model:
         else:
             S["layers"][idx[0]](S["xs"][g], lowrank)
 
+    def grouped(self, g):
+        """Whether a pass serves these layers, stored apart, by one linear launch: the streaming kernel or the one on CTA
+        pairs for each of two to four."""
+        idx = self.members[g]
+        K = self.w["layers"][idx[0]][1]
+        kernels = {self.aser.lib.aser_linear_kernel(self.M, self.w["layers"][i][2], K) for i in idx}
+        return not self.fused.get(g) and 2 <= len(idx) <= 4 and kernels in ({0}, {2})
+
     def launches_per_step(self):
         """Kernels of this library launched by one step: per input group the activation pass
         (as many kernels as the library says it runs at that shape) and one linear kernel per layer
-        (one per group where the group is stored fused, or where the streaming kernel or the one on CTA pairs
-        serves each of its two to four layers)."""
+        (one per group where the group is stored fused or served by one launch)."""
         n = 0
         for g, idx in self.members.items():
             K = self.w["layers"][idx[0]][1]
-            kernels = {self.aser.lib.aser_linear_kernel(self.M, self.w["layers"][i][2], K) for i in idx}
-            one = self.fused.get(g) or (2 <= len(idx) <= 4 and kernels in ({0}, {2}))
+            one = self.fused.get(g) or self.grouped(g)
             n += self.aser.forward_act_launches(self.M, K, self.r * len(idx)) + (1 if one else len(idx))
         return n
 
@@ -604,6 +612,9 @@ def measure(m, steps, peaks, lib_int8, barrier=None, max_over_ranks=lambda x: x,
                overhead=dict(linear=t_lin["median"] / t_lin_plain["median"] - 1.0,
                              step=t_step["median"] / t_step_plain["median"] - 1.0),
                roofline=roofline_of(w, m.name, t_lin["median"] * 1e3, peaks, lib_int8, launches=m.linear_launches()))
+    if any(m.grouped(g) for g in m.members):
+        out["roofline"]["timed"] = "layer by layer; in a step %s share one launch" % ", ".join(
+            " and ".join(w["layers"][i][0] for i in idx) for g, idx in m.members.items() if m.grouped(g))
     act_bytes = sum(algorithmic_bytes_act(w["M"], w["layers"][idx[0]][1], w["r"] * len(idx))
                     for idx in m.members.values())
     out["quant_act_gbs"] = act_bytes / (t_act["median"] * 1e-3) / 1e9
