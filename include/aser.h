@@ -121,9 +121,11 @@ int aser_quant_act_ex(const void* X_f16, const float* s, const void* LA_f16,
 /*
  * aser_quant_act_ws -- aser_quant_act_ex for callers that can spare scratch memory (same
  * passages of the paper; the scratch is an implementation matter).  With more than 32 tokens it
- * runs two kernels instead of one: the first reads X once, takes the row maxima and the
- * projection T on the tensor cores and leaves per-slice partial results in the scratch; the
- * second writes the scales, the codes and T.  Results are those of aser_quant_act_ex (Xq and
+ * runs two kernels instead of one, the first of which makes the projection T on the tensor cores.  Beside each other
+ * where that is faster (rows of up to 8192 columns, not too many rows of L_A for the number of tokens): the first then
+ * writes T, the second the scales and the codes.  Otherwise one after the other: the first also takes the row
+ * maxima and leaves per-slice partial results in the scratch, the second writes the scales, the codes and T.
+ * Results are those of aser_quant_act_ex (Xq and
  * a_scale bit-exact; T may differ in its last bf16 bit because the fp32 sums are formed in a
  * different order), at several times the throughput.  Two extensions:
  *   - r may go up to 512 (a multiple of 16): L_A may be the STACKED down projections of

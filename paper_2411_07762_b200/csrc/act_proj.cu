@@ -6,18 +6,21 @@
 //                      (kind::f16) with L_A on the M side (up to four groups of 128 rows, so the
 //                      down projections of several layers that share X are computed in one pass)
 //                      and the 128 tokens on the N side.  The slices' partial T are summed in order and rounded to bf16.
-//   act_rows_kernel    up to 8192 columns, and without a projection (then it is the only kernel): scales and codes of
+//   act_rows_kernel    up to 8192 columns (see below), and without a projection (then it is the only kernel): scales and codes of
 //                      whole rows, beside act_proj_kernel.
-//   act_quant_kernel   longer rows: the scale from row maxima that act_proj_kernel left in the scratch, the codes, and T
+//   act_quant_kernel   otherwise: the scale from row maxima that act_proj_kernel left in the scratch, the codes, and T
 //                      from the partial T beside them.
 //
-// Which of the two (rows_beside): running beside each other the kernels take little more than the longer one while X, which both
+// Which of the two (beside_from): running beside each other the kernels take little more than the longer one while X, which both
 // read, comes from L2 for the second; what bounds them then is the L2 -> SM traffic of X (twice) and L_A (once per 128
 // tokens), 4.5 TB/s.  Rows of more than 8192 columns exceed L2 at a few thousand tokens and both streams come from
-// HBM; many rows of L_A at 8192 columns are bound by their own traffic already.  The activation step, us, beside | after each
-// other: rank 128: 600 x 4096 12.5 | 13.9, 1500 x 4096 14.9 | 18.4, 4096 x 4096 24.9 | 30.9, 1024 x 8192 19.9 | 21.3, 4096 x 8192 47.5 |
-// 50.7, 1500 x 14336 46 | 41, 4096 x 14336 100 | 85; rank 256: 4096 x 4096 32.3 | 37.4, 1024 x 8192 28.6 | 25.9, 2048 x 8192 39.5 | 35.2;
-// 1500 x 4096 at rank 384 25.9 | 26.3, at rank 512 33.3 | 32.4.
+// HBM; many rows of L_A at 8192 columns are bound by their own traffic already.  Few tokens: beside, a tile has at most eight
+// slices of K, so with few tiles the projection is the longer chain the more rows of L_A there are.  The activation step, us, beside |
+// after each other: rank 128: 33 x 4096 12.4 | 11.9, 64 x 4096 12.3 | 12.5, 600 x 4096 12.7 | 14.1, 4096 x 4096 24.3 | 28.9, 33 x 3072 11.0 |
+// 12.3, 64 x 6144 14.8 | 13.9, 128 x 6144 14.0 | 14.8; rank 64: 300 x 8192 16.7 | 16.6, 449 x 8192 16.6 | 17.3, 4096 x 8192 45.8 | 46.7; rank 128:
+// 1500 x 14336 46 | 41, 4096 x 14336 100 | 85; rank 256: 64 x 4096 17.3 | 15.5, 449 x 4096 17.8 | 17.0, 800 x 4096 18.7 | 19.3, 4096 x 4096 30.6 |
+// 36.7, 100 x 2048 14.2 | 14.2, 600 x 2048 14.9 | 15.4, 600 x 8192 28.2 | 22.2; rank 384: 64 x 4096 22.3 | 17.6, 800 x 4096 24.1 | 22.8, 1600 x 4096 26.4 |
+// 26.4, 4096 x 4096 36.8 | 43.3, 600 x 2048 19.7 | 18.2, 300 x 512 17.8 | 18.0, 200 x 3584 22.0 | 23.9.  (Rank 512 would gain from 2500 tokens on.)
 //
 // (Sec. 4.2 smoothing M^-1 X of Eq. 10, Sec. 5.1 per-token round-to-nearest, Sec. 4.1 projection
 // V_r^T S^-1 of the reconstruction branch.)  All kernels are deterministic: no atomics on global memory.
@@ -40,7 +43,16 @@ constexpr int kPMaxGroups = 4;              // 128-row groups of L_A: r <= 512
 constexpr int kProjPlanSms = 148;           // chunks and slices are planned for this many SMs (the
                                             // scratch size must not depend on the device)
 constexpr long long kPWaitLimitClocks = 400000000ll;   // about 0.2 s of SM clocks per wait
-__host__ __device__ constexpr bool rows_beside(int K, int r) { return K <= 4096 ? r <= 384 : K <= 8192 && r <= 128; }
+// Tokens from which the kernels run beside each other (see above).
+constexpr int kNever = 0x7fffffff;
+constexpr int beside_from(int K, int r) {
+    if (K > 8192 || r > 384) return kNever;
+    if (K > 4096) return r > 128 ? kNever : K < 8192 ? 100 : 400;
+    if (r <= 128) return K < 4096 ? 0 : 64;
+    if (r <= 256) return K <= 3584 ? 100 : 600;
+    return K < 1024 || (K > 2048 && K <= 3584) ? 100 : 1600;
+}
+constexpr bool rows_beside(int M, int K, int r) { return M >= beside_from(K, r); }
 constexpr int kPMaxCluster = 8;             // CTAs of a cluster
 constexpr int kPCacheUnits = 254;           // 8-column units with a divisor whose divisors are kept in shared memory
 constexpr int kPUncached = 255;             // tag of such a unit beyond the cache: its divisors are read from global memory
@@ -427,7 +439,7 @@ act_proj_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     }
 }
 
-// Where rows_beside says no.  grid = ceil(M / kQRows), 256 threads; a CTA takes kQRows token rows, several
+// Where the kernels run one after the other.  grid = ceil(M / kQRows), 256 threads; a CTA takes kQRows token rows, several
 // 16-byte loads per thread are in flight, and the per-row scales are computed once per CTA (one
 // warp per row).  The kernel is bound by instruction issue, not by bytes, so the common case is
 // kept free of per-column work: the CTA first lists the columns whose divisor is not 1 (the few
@@ -784,11 +796,11 @@ int launch_rows(cudaLaunchConfig_t cfg, const __half* X, const float* s, int M, 
 // two waves, 24 us).  Otherwise as many equal slices as keep the grid within one wave.
 // Cutting long inputs into chunks of tokens whose X stays in L2 for the second kernel cost more in fixed time per
 // launch pair than the L2 hits saved (4096 x 14336 at rank 128: 140 us in three chunks, 95 us in one).
-int proj_slices(int M, int K, int r, int num_sms) {
+int proj_slices(int M, int K, bool beside, int num_sms) {
     const int blocks = K / kPCols;
     const int tiles = (M + kPTok - 1) / kPTok;
     int ks_best = 1;
-    if (rows_beside(K, r)) {
+    if (beside) {
         constexpr int fit[kPMaxCluster + 1] = {0, kProjPlanSms, 72, 44, 32, 24, 20, 14, 14};
         for (int ks = 2; ks <= kPMaxCluster && ks <= blocks / 4; ++ks)
             if (tiles <= fit[ks]) ks_best = ks;
@@ -803,16 +815,24 @@ int proj_slices(int M, int K, int r, int num_sms) {
 // a 128-byte boundary (it is written by bulk copies, which need 16-byte alignment).
 size_t proj_amax_floats(int M, int slices) { return ((size_t)slices * M + 31) & ~(size_t)31; }
 
-size_t proj_scratch_bytes(int M, int K, int r, int slices) {
-    if (rows_beside(K, r) || r == 0) return 0;         // nothing goes through the scratch
+// What M tokens leave in the scratch, one kernel after the other.
+size_t proj_scratch_bytes(int M, int r, int slices) {
     return (proj_amax_floats(M, slices) + (size_t)slices * M * ((r + 127) / 128) * 128) * sizeof(float);
 }
 
 }  // namespace
 
+// Enough for any pass of up to M tokens where the two orders meet, so that a caller may size it for his largest: nothing goes through the
+// scratch from beside_from tokens on; below, the slices of all tiles are at most one wave.
 size_t quant_act_ws_scratch_bytes(int M, int K, int r) {
-    if (M <= 32) return 0;
-    return proj_scratch_bytes(M, K, r, proj_slices(M, K, r, kProjPlanSms));
+    if (M <= 32 || r == 0) return 0;
+    const int from = beside_from(K, r);
+    if (from == kNever) return proj_scratch_bytes(M, r, proj_slices(M, K, false, kProjPlanSms));
+    const int few = M < from ? M : from - 1;
+    if (few <= 32) return 0;
+    const int most = K / kPCols / 4 > 1 ? K / kPCols / 4 : 1;            // slices of a pass
+    const long long rows = (long long)most * few;
+    return proj_scratch_bytes((int)(rows < (long long)kProjPlanSms * kPTok ? rows : (long long)kProjPlanSms * kPTok), r, 1);
 }
 
 int quant_act_ws_launches(int M, int K) { return M <= 32 ? 1 : 2; }
@@ -824,10 +844,11 @@ int launch_quant_act_ws(const __half* X, const float* s, const __half* LA, int M
     const int ldt = t_pair ? 2 * r : r, lo_off = t_pair ? r : 0;
     const int groups = (r + 127) / 128;
     if (groups > kPMaxGroups) return record_error(ASER_ERR_SHAPE, "quant_act: r beyond 512");
-    const int KS = proj_slices(M_pass > 0 ? M_pass : M, K, r, kProjPlanSms);
-    if (scratch == nullptr || misaligned16(scratch) || scratch_bytes < proj_scratch_bytes(M, K, r, KS))
+    if (M_pass == 0) M_pass = M;
+    const bool beside = r > 0 && rows_beside(M_pass, K, r);
+    const int KS = proj_slices(M_pass, K, beside, kProjPlanSms);
+    if (scratch == nullptr || misaligned16(scratch) || (r > 0 && !beside && scratch_bytes < proj_scratch_bytes(M, r, KS)))
         return record_error(ASER_ERR_WORKSPACE, "quant_act: scratch missing or too small");
-    const bool beside = rows_beside(K, r);
     float* amax_part = static_cast<float*>(scratch);
     float* t_part = amax_part + proj_amax_floats(M, KS);
     cudaLaunchAttribute attr[1];

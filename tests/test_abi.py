@@ -139,6 +139,19 @@ def test_activation_path_without_a_projection_is_one_launch(lib):
     assert lib.aser_forward_act_launches(0, 4096, 0) == 0 and lib.aser_forward_act_launches(8, 4100, 0) == 0
 
 
+def test_activation_scratch_of_a_larger_pass_is_enough_for_a_smaller_one(lib):
+    """A caller sizes it once, for his largest pass, although only few tokens go through it up to 8192 columns."""
+    for K in (128, 512, 1024, 3072, 4096, 6144, 7680, 8192):
+        for r in (0, 16, 128, 144, 256, 384):
+            if K > 4096 and r > 128:
+                continue            # partial sums at every size
+            sizes = [lib.aser_quant_workspace_bytes(M, K, r) for M in (1, 32, 33, 63, 64, 100, 333, 399, 400, 599, 600, 1599, 1600, 4096, 70000)]
+            assert sizes == sorted(sizes) and sizes[0] > 0
+            slices = max(k for k in range(1, max(1, K // 256) + 1) if (K // 64) % k == 0)       # of one tile: the most there are
+            if r > 128 and K <= 2048:
+                assert sizes[3] >= 1024 + slices * 63 * (1 + (r + 127) // 128 * 128) * 4
+
+
 def test_linear_kernel_rejects_bad_shapes(lib):
     assert lib.aser_linear_kernel(8, 4096, 4096) == 0
     for bad in ((8, 4096, 4100), (8, 4100, 4096), (0, 4096, 4096), (-1, 128, 128)):

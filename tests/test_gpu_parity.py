@@ -273,6 +273,28 @@ def test_quant_act_beside_projection(aser, entry, M, K, r, divided, act_bits, t_
         assert_T_close(T[:, :r].float().cpu().numpy(), F.down_proj(xs, L_A), xs, L_A)
 
 
+@pytest.mark.parametrize("M,K,r", [
+    (63, 4096, 48), (64, 4096, 48), (99, 2048, 144), (100, 2048, 144), (599, 3712, 256), (600, 3712, 256),
+    (99, 512, 384), (100, 512, 384), (1599, 1024, 272), (1600, 1024, 272), (99, 6144, 32), (100, 6144, 32), (99, 3200, 384),
+    (100, 3200, 384), (399, 8192, 80), (400, 8192, 80)])
+def test_quant_act_ws_on_both_sides_of_each_line(aser, M, K, r):
+    """The two kernels one after the other below, beside each other above, with the scratch of a larger pass."""
+    rng = np.random.default_rng(M + K + r)
+    X = rng.standard_normal((M, K)).astype(np.float16)
+    s = np.ones(K, np.float32)
+    cols = rng.choice(K, K // 100, replace=False)
+    s[cols] = 4.0
+    X[:, cols] *= np.float16(20)
+    L_A = synth.standin_factors(8, K, r, seed=M, scale_a=0.05)[0]
+    ws = torch.full((aser.quant_workspace_bytes(4096, K, r),), 0x7f, dtype=torch.uint8, device="cuda")
+    Xq, sc, T = aser.quant_act_ws(to_dev(X), to_dev(s), to_dev(L_A), ws=ws)
+    xs = F.smooth_act(X, s)
+    Xq_ref, sc_ref = F.quant_act(xs)
+    assert np.array_equal(Xq.cpu().numpy(), Xq_ref)
+    assert np.array_equal(bits(sc.cpu().numpy()), bits(sc_ref))
+    assert_T_close(T.float().cpu().numpy(), F.down_proj(xs, L_A), xs, L_A)
+
+
 @pytest.mark.parametrize("entry", ["one", "ws"])
 @pytest.mark.parametrize("M,K", [(20, 1024), (40, 8192), (300, 2048), (900, 4096), (333, 14336)])
 @pytest.mark.parametrize("divided,s_value", [(3, 1e36), (3, 3e37), (0, 3e37), (600, 1e-36)])
