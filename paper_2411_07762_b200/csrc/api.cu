@@ -144,15 +144,16 @@ bool act_shape_ok(int M, int K, int r) {
     return M >= 0 && K > 0 && K % 128 == 0 && K <= 32768 && r >= 0 && r <= 512 && r % 16 == 0;
 }
 
-// Which activation kernels a forward pass runs.  The two-kernel path with scratch reads X once
-// from HBM whatever the rank; it is the only one above rank 128 (stacked down projections of a
-// shared-input group).  The one-launch cluster kernel reads X twice (the second time from L2) and has one
-// launch less of fixed cost; up to seven of its 64-token clusters of 16 CTAs are resident at once, and at the eighth its
-// time steps up.  Measured at rank 128, cluster against two-kernel path, us: 448 / 449 x 4096 11.4 | 13.9 and 15.9 | 13.8,
-// 448 / 449 x 8192 15.5 | 17.8 and 24.8 | 18.1, 448 / 449 x 14336 21.8 | 23.4 and 35.0 | 22.6, 1024 x 4096 23.4 | 15.9, 4096 x
-// 14336 124 | 84; shorter rows step up later: 896 / 1000 x 3072 13.6 | 14.4 and 19.1 | 15.3, 896 / 1000 x 2048 10.9 | 12.2 and
-// 15.3 | 12.6, 1024 x 1536 12.7 | 13.4; rows of 1024 columns 9.4 | 11.1 at 512 tokens and still 15.3 | 16.8 at 4096.
-// Up to 32 tokens the few-token kernel serves every rank.
+// Which activation kernels a forward pass runs.  The two kernels with scratch are the only path above rank 128 (stacked down
+// projections of a shared-input group).  Below, one launch (quant_act_mid while its CTAs are about one wave, else the cluster
+// kernel) has less fixed cost; up to seven of the cluster kernel's 64-token clusters of 16 CTAs are resident at once,
+// and at the eighth its time steps up.  One launch | two kernels, us, rank 32: 448 / 449 x 4096 9.0 | 11.1 and 12.7 | 10.8, 448 / 449 x 8192 13.6 |
+// 16.1 and 18.5 | 15.8, 448 / 449 x 14336 18.5 | 20.7 and 26.2 | 21.0, 1024 x 4096 18.6 | 12.1; rank 128: 448 / 449 x 4096 11.1 | 12.0 and 15.8 |
+// 12.0, 448 / 449 x 8192 15.6 | 17.2 and 23.2 | 16.8, 448 / 449 x 14336 22.4 | 22.1 and 35.5 | 23.7.  Shorter rows step up later, but not all at the
+// same number of tokens: rank 32: 700 / 1024 x 3072 9.1 | 10.4 and 15.4 | 10.9, 1024 x 2048 9.1 | 9.4, 1023 x 1536 7.9 | 9.3, 1000 / 4096 x 1024
+// 7.7 | 8.8 and 13.6 | 11.5; rank 128: 700 / 1000 x 3072 12.6 | 11.5 and 18.7 | 12.2, 896 / 1000 x 2048 11.2 | 10.8 and 15.3 | 10.8, 1023 x
+// 1536 12.9 | 10.5, 1000 / 4096 x 1024 10.8 | 9.8 and 16.4 | 11.9, 448 x 5120 17.0 | 13.6, 448 x 7168 21.0 | 15.6: between these lines two kernels would
+// gain, most at rank 128.  Up to 32 tokens the few-token kernel serves every rank.
 bool forward_act_uses_scratch(int M, int K, int r) {
     if (M <= 32) return false;
     if (r > 128) return true;
