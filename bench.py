@@ -73,16 +73,11 @@ EXTRA_POINTS = ("c2_decode_m8", "c2_decode_m1", "c3_prefill_gate_up", "c3_prefil
                 "c5_decode_m16_8192", "c5_decode_m16_28672", "c5_prefill_m4096_8192",
                 "c5_prefill_m4096_28672")
 
-# dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel under ncu, taken with
-# the kernel as it stands in this tree; the summary with the command is
-# profiles/launches_c4_decoder_block_step.txt.  The workload's figure is the average over its
-# linear_pair launches; "<workload>/<layers>" is the launch of that layer or fused group.  Workloads
-# without a capture of the current kernel report null.
-NCU_DRAM_BYTES_PER_LAUNCH = {
-    "c4_decoder_block": 465.4e6 / 5,
-    "c4_decoder_block/q+k+v": 43.7e6, "c4_decoder_block/o": 28.5e6, "c4_decoder_block/gate": 127.3e6,
-    "c4_decoder_block/up": 127.4e6, "c4_decoder_block/down": 138.6e6,
-}
+# dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel under ncu, by "<workload>" (the average over
+# its launches) or "<workload>/<layers>" (the launch of that layer or fused group).  Only captures of the kernel as it stands
+# in this tree belong here; what has none reports null.  (profiles/launches_c4_decoder_block_step.txt was taken
+# before gate and up became one launch.)
+NCU_DRAM_BYTES_PER_LAUNCH = {}
 
 
 def dominant_kernel(M, N, K):

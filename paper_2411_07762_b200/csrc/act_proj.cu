@@ -793,7 +793,8 @@ int launch_rows(cudaLaunchConfig_t cfg, const __half* X, const float* s, int M, 
 
 // Slices of K, of at least four 64-column stages.  Beside act_rows_kernel the slices are one cluster: the size of at most eight that
 // gives the most CTAs while all clusters fit at once (a GPC has 16 to 20 SMs; 2048 x 4096, rank 64: 16 clusters of eight took
-// two waves, 24 us).  Otherwise as many equal slices as keep the grid within one wave.
+// two waves, 24 us); how many fit is written down for a part of 148 SMs rather than asked for, since the slices decide the order of
+// T's sums, which should not depend on the device.  Otherwise as many equal slices as keep the grid within one wave.
 // Cutting long inputs into chunks of tokens whose X stays in L2 for the second kernel cost more in fixed time per
 // launch pair than the L2 hits saved (4096 x 14336 at rank 128: 140 us in three chunks, 95 us in one).
 int proj_slices(int M, int K, bool beside, int num_sms) {
