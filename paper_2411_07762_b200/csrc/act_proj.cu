@@ -12,8 +12,8 @@
 //                      from the partial T beside them.
 //
 // Which of the two (beside_from): running beside each other the kernels take little more than the longer one while X, which both
-// read, comes from L2 for the second; what bounds them then is the L2 -> SM traffic of X (twice) and L_A (once per 128
-// tokens), 4.5 TB/s.  Rows of more than 8192 columns exceed L2 at a few thousand tokens and both streams come from
+// read, comes from L2 for the second; they move X twice and L_A once per 128 tokens to the SMs, at 4.5 TB/s (each alone, cold,
+// has L2 15 % and HBM 20 % busy: latency of the loads in flight).  Rows of more than 8192 columns exceed L2 at a few thousand tokens and both streams come from
 // HBM; many rows of L_A at 8192 columns are bound by their own traffic already.  Few tokens: beside, a tile has at most eight
 // slices of K, so with few tiles the projection is the longer chain the more rows of L_A there are.  The activation step, us, beside |
 // after each other: rank 128: 33 x 4096 12.4 | 11.9, 64 x 4096 12.3 | 12.5, 600 x 4096 12.7 | 14.1, 4096 x 4096 24.3 | 28.9, 33 x 3072 11.0 |

@@ -25,8 +25,9 @@
 // Measured against linear_tc_kernel (or linear_pair_kernel, whichever the shape had), the linear step alone in graphs on one box
 // (tokens x channels x K, us): 17 x 4096 x 4096 13.2 -> 8.4; 32 x 14336 x 4096 20.4 -> 10.0; 64 x 4096 x 14336 21.1 -> 12.8;
 // 101 x 8192 x 8192 26.5 -> 16.7; 128 x 14336 x 4096 20.9 -> 14.3; 200 x 8192 x 2048 14.7 -> 10.5; 400 x 4096 x 4096 19.6 -> 13.3;
-// 256 x 4096 x 14336 32.4 -> 20.2.  (Repeats of one call: the weights come from L2.)  What bounds it: activations are read once
-// per 128 channels, 22 KB per SM and block at 101 x 8192 x 8192, so L2 -> SM traffic; set-up 1.2 us, exchange and outputs 3 us.
+// 256 x 4096 x 14336 32.4 -> 20.2.  (Repeats of one call: the weights come from L2.)  What bounds it is latency: at 101 x 8192 x
+// 8192, cold, L2 is 18 % busy, HBM 22, the SM 22; set-up takes 1.2 us, exchange and outputs 3, and between them a stage brings 44 KB
+// to every SM (activations are read once per 128 channels).
 #include "aser_common.cuh"
 #include "sm100_ptx.cuh"
 
